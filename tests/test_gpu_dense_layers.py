@@ -1,0 +1,103 @@
+"""Element-wise and reduction kernels of the dense layers at the sizes where their
+vector width, their cluster split and their tails change, and on arrays that are not
+16-byte aligned, against FP64 numpy.  A sum of n FP32 products in any order differs
+from the exact one by at most n 2^-24 of the sum of magnitudes."""
+import ctypes as C
+
+import numpy as np
+import pytest
+
+from tests.gpu_common import need_gpu, to_dev, torch
+
+pytestmark = pytest.mark.gpu
+
+U = 2.0 ** -24
+
+
+@pytest.fixture(autouse=True)
+def _gpu():
+    need_gpu()
+
+
+def _lib():
+    from paper_2405_12380_gb300 import _lib as L
+    return L.lib()
+
+
+def _p(t):
+    # (data_ptr() of an empty tensor is null, which the calls refuse)
+    return C.c_void_p(t.untyped_storage().data_ptr() + 4 * t.storage_offset())
+
+
+def _off(a, off):
+    """A device copy of `a` that starts `off` floats past an aligned address."""
+    t = torch.empty(a.size + off + 1, dtype=torch.float32, device="cuda")
+    t[off:off + a.size] = to_dev(a.reshape(-1))
+    return t[off:off + a.size]
+
+
+@pytest.mark.parametrize("off", [0, 1])
+@pytest.mark.parametrize("rows,cols", [(1, 1), (7, 3), (255, 33), (256, 32), (257, 100), (300, 31), (5000, 260), (0, 5)])
+def test_bias_grad(rows, cols, off):
+    dY = np.random.default_rng(rows + cols).standard_normal((rows, cols)).astype(np.float32)
+    d, db = _off(dY, off), torch.full((cols,), 7.0, device="cuda")
+    assert _lib().nn_bias_grad(rows, cols, _p(d), _p(db), None) == 0
+    err = np.abs(db.cpu().numpy() - dY.astype(np.float64).sum(0))
+    assert np.all(err <= max(rows, 1) * U * np.abs(dY).astype(np.float64).sum(0))
+
+
+@pytest.mark.parametrize("off", [0, 1])
+@pytest.mark.parametrize("B,P2", [(1, 1), (3, 4095), (2, 4096), (5, 4097), (4, 4099), (33, 20000)])
+def test_rel_l2(B, P2, off):
+    rng = np.random.default_rng(B + P2)
+    pr, tg = (rng.standard_normal((B, P2)).astype(np.float32) for _ in range(2))
+    a, b = _off(pr, off), _off(tg, off)
+    d, lo = torch.empty(B * P2, device="cuda"), torch.empty(B, device="cuda")
+    assert _lib().nn_rel_l2(B, P2, _p(a), _p(b), _p(d), _p(lo), None) == 0
+    df, t64 = pr.astype(np.float64) - tg, tg.astype(np.float64)
+    den = (t64 ** 2).sum(1)
+    loss = (df ** 2).sum(1) / den
+    assert np.all(np.abs(lo.cpu().numpy() - loss) <= (2 * P2 + 8) * U * loss)
+    ref = 2.0 / (den[:, None] * B) * df
+    err = np.abs(d.cpu().numpy().reshape(B, P2) - ref)
+    scale = 2.0 / (den[:, None] * B) * (np.abs(pr) + np.abs(tg))      # the subtraction rounds once
+    assert np.all(err <= (P2 + 8) * U * np.abs(ref) + 2 * U * scale)
+
+
+@pytest.mark.parametrize("off", [0, 1])
+@pytest.mark.parametrize("n", [0, 1, 3, 4, 1027, 70001])
+def test_adam_and_act_backward(n, off):
+    rng = np.random.default_rng(n)
+    p, g, m = (rng.standard_normal(n).astype(np.float32) for _ in range(3))
+    v = rng.uniform(0, 2, n).astype(np.float32)
+    P, G, M, V = (_off(a, off) for a in (p, g, m, v))
+    lr, t = 1e-3, 7
+    assert _lib().nn_adam(n, _p(P), _p(G), _p(M), _p(V), lr, 0.9, 0.999, 1e-8, t, None) == 0
+    m1 = 0.9 * m.astype(np.float64) + 0.1 * g
+    v1 = 0.999 * v.astype(np.float64) + 0.001 * g.astype(np.float64) ** 2
+    # 1 - beta and 1 - beta^t carry the FP32 rounding of beta: up to 2^-24 / 1e-3 relative
+    assert np.all(np.abs(M.cpu().numpy() - m1) <= 4 * U * (np.abs(m) + np.abs(g)))
+    assert np.all(np.abs(V.cpu().numpy() - v1) <= 4 * U * v + 1e-4 * 0.001 * g ** 2)
+    step = lr * (m1 / (1 - 0.9 ** t)) / (np.sqrt(v1 / (1 - 0.999 ** t)) + 1e-8)
+    assert np.all(np.abs(P.cpu().numpy() - (p - step)) <= 2 * U * np.abs(p) + 1e-3 * np.abs(step) + 8 * U * lr * 10)
+    for act in (0, 1, 2, 3):
+        d, y = _off(g, off), _off(np.tanh(m), off)
+        assert _lib().nn_act_backward(n, _p(d), _p(y), act, None) == 0
+        y64 = np.tanh(m).astype(np.float64)
+        f = [np.ones_like(y64), y64 > 0, 1 - y64 * y64, np.where(y64 > 0, 1.0, 0.01)][act]
+        assert np.all(np.abs(d.cpu().numpy() - g * f) <= 4 * U * np.abs(g))
+
+
+@pytest.mark.parametrize("off", [0, 1])
+@pytest.mark.parametrize("rows,cols", [(1, 1), (3, 4), (5, 255), (4099, 256), (2, 1028), (33, 70000)])
+def test_bias_act(rows, cols, off):
+    rng = np.random.default_rng(rows * 3 + cols)
+    X, b = rng.standard_normal((rows, cols)).astype(np.float32), rng.standard_normal(cols).astype(np.float32)
+    for act, f in ((0, lambda z: z), (1, lambda z: np.maximum(z, 0)), (2, np.tanh), (3, lambda z: np.where(z > 0, z, 0.01 * z))):
+        x, bb = _off(X, off), _off(b, 1 - off)
+        assert _lib().nn_bias_act(rows, cols, _p(x), _p(bb), act, None) == 0
+        ref = f(X.astype(np.float64) + b)
+        assert np.all(np.abs(x.cpu().numpy().reshape(rows, cols) - ref) <= 4 * U * (np.abs(X) + np.abs(b) + 1e-6))
+    x = _off(X, off)
+    assert _lib().nn_bias_act(rows, cols, _p(x), None, 1, None) == 0
+    assert np.array_equal(x.cpu().numpy().reshape(rows, cols), np.maximum(X, 0))
