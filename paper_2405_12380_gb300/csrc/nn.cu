@@ -1,10 +1,8 @@
 // Dense layers of the DeepONet (App. B): FP32 GEMM, bias + activation and their
 // gradients, the relative-L2 loss of the DeepONet output, and Adam.
 //
-// Row-major matrices throughout.  The GEMM computes C = alpha op(A) op(B) + beta C
-// with 64 x 64 output tiles, a 16-deep K slab in shared memory and a 4 x 4
-// register tile per thread; long-K products are split over blockIdx.z and
-// combined with atomic adds (training tolerates the summation order).
+// Row-major matrices throughout.  Long-K products of the GEMM are split over
+// blockIdx.z and combined with atomic adds (training tolerates the summation order).
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
@@ -14,68 +12,173 @@
 
 namespace {
 
-constexpr int GBM = 64, GBN = 64, GBK = 16;
+// ---- FP32 GEMM: C += alpha op(A) op(B) over a slice of K (blockIdx.z)
+//
+// A block of (BM / 8)(BN / 8) threads owns a BM x BN tile of C, 8 x 8 per thread; a warp
+// covers 32 x 64 of it (4 x 8 threads), so that one K step of a warp reads four 128-byte
+// wavefronts of shared memory for 64 FMA instructions per scheduler.  Slabs of SBK K
+// values of both operands are held K-major in two shared buffers; the next slab's global
+// loads are issued before the current one is used, 16 bytes per thread where the operand
+// allows it (VA / VB: leading dimension a multiple of 4 and a 16-byte aligned base).
+// Bound by the FP32 pipe for square products (16384 x 256 x 256: 93 -> 30 us, 72 of the
+// pipe's 80 TFLOP/s), by the FP32 pipe and HBM about equally for the branch's first layer
+// at 64^3 (32 x 256 x 524288, 537 MB of weights read: 1060 -> 206 us; its weight gradient,
+// 537 MB written: 842 -> 181 us).  Before: 64 x 64 tiles, 4 x 4 per thread, 4-byte loads,
+// no prefetch, and 64-row tiles half empty at a batch of 32.  fma.rn.f32x2 measured the
+// same rate per multiply-add as scalar FMA but half the issue slots.
+constexpr int SBK = 16;
 
-__global__ void __launch_bounds__(256) k_sgemm(int transA, int transB, int M, int N, int K, float alpha,
-                                               const float* __restrict__ A, int lda, const float* __restrict__ B,
-                                               int ldb, float* __restrict__ C, int ldc, int kslice, int atomic) {
-    __shared__ float As[GBK][GBM + 4];
-    __shared__ float Bs[GBK][GBN + 4];
-    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-    const int m0 = blockIdx.y * GBM, n0 = blockIdx.x * GBN;
-    const int k0 = blockIdx.z * kslice;
-    const int k1 = min(K, k0 + kslice);
-    float acc[4][4];
+__device__ __forceinline__ unsigned long long pack2(float a, float b) {
+    unsigned long long v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(a), "f"(b));
+    return v;
+}
+__device__ __forceinline__ void unpack2(unsigned long long v, float& a, float& b) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+// two FP32 fused multiply-adds in one instruction (each rounded as fmaf)
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+
+// one SBK x R slab of an operand, global -> registers -> shared [SBK][R + 4].
+// KC: stored with K contiguous (element (r, k) at X[r ld + k]); else (r, k) at X[k ld + r]
+template <int R, int T, bool KC>
+struct Slab {
+    static constexpr int Q = R * SBK / 4 / T;              // groups of four values per thread
+    static_assert(Q * T * 4 == R * SBK, "the slab divides among the threads");
+    float4 v[Q];
+
+    __device__ __forceinline__ void load(const float* __restrict__ X, long long ld, int r0, int rows, int k0, int k1,
+                                         bool vec) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-    for (int kb = k0; kb < k1; kb += GBK) {
-        // A tile: GBM x GBK (op(A)[m][k]); B tile: GBK x GBN (op(B)[k][n])
-        for (int t = threadIdx.x; t < GBM * GBK; t += 256) {
-            int mm, kk;
-            if (transA) { mm = t % GBM; kk = t / GBM; }        // A stored K x M: contiguous in m
-            else { kk = t % GBK; mm = t / GBK; }               // A stored M x K: contiguous in k
-            const int gm = m0 + mm, gk = kb + kk;
-            float v = 0.f;
-            if (gm < M && gk < k1) v = transA ? A[(long long)gk * lda + gm] : A[(long long)gm * lda + gk];
-            As[kk][mm] = v;
+        for (int q = 0; q < Q; ++q) {
+            const int t = threadIdx.x + q * T;
+            const int r = KC ? t / (SBK / 4) : (t % (R / 4)) * 4, k = KC ? (t % (SBK / 4)) * 4 : t / (R / 4);
+            const int gr = r0 + r, gk = k0 + k;
+            float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+            const int n = KC ? (gr < rows ? k1 - gk : 0) : (gk < k1 ? rows - gr : 0);   // values that exist
+            const float* p = X + (KC ? (long long)gr * ld + gk : (long long)gk * ld + gr);
+            if (n >= 4 && vec) {
+                x = __ldg(reinterpret_cast<const float4*>(p));
+            } else if (n > 0) {
+                x.x = __ldg(p);
+                if (n > 1) x.y = __ldg(p + 1);
+                if (n > 2) x.z = __ldg(p + 2);
+                if (n > 3) x.w = __ldg(p + 3);
+            }
+            v[q] = x;
         }
-        for (int t = threadIdx.x; t < GBK * GBN; t += 256) {
-            int kk, nn;
-            if (transB) { kk = t % GBK; nn = t / GBK; }        // B stored N x K: contiguous in k
-            else { nn = t % GBN; kk = t / GBN; }               // B stored K x N: contiguous in n
-            const int gk = kb + kk, gn = n0 + nn;
-            float v = 0.f;
-            if (gn < N && gk < k1) v = transB ? B[(long long)gn * ldb + gk] : B[(long long)gk * ldb + gn];
-            Bs[kk][nn] = v;
+    }
+    __device__ __forceinline__ void store(float (*S)[R + 4]) const {
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const int t = threadIdx.x + q * T;
+            if (KC) {
+                const int r = t / (SBK / 4), k = (t % (SBK / 4)) * 4;
+                S[k][r] = v[q].x;
+                S[k + 1][r] = v[q].y;
+                S[k + 2][r] = v[q].z;
+                S[k + 3][r] = v[q].w;
+            } else {
+                *reinterpret_cast<float4*>(&S[t / (R / 4)][(t % (R / 4)) * 4]) = v[q];
+            }
         }
-        __syncthreads();
+    }
+};
+
+template <int BM, int BN, bool AKC, bool BKC>
+__global__ void __launch_bounds__(BM * BN / 64, BM * BN / 64 >= 256 ? 2 : 3)
+    k_sgemm(int M, int N, int K, float alpha, const float* __restrict__ A, int lda, const float* __restrict__ B,
+            int ldb, float* __restrict__ C, int ldc, int kslice, int vecs, int add) {
+    constexpr int T = BM * BN / 64;
+    __shared__ __align__(16) float As[2][SBK][BM + 4];
+    __shared__ __align__(16) float Bs[2][SBK][BN + 4];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    constexpr int WN = BN / 64;                            // warps along N
+    const int rm = (w / WN) * 32 + (lane >> 3) * 4, rn = (w % WN) * 64 + (lane & 7) * 4;
+    const int tiles_m = (M + BM - 1) / BM;
+    const int m0 = (blockIdx.x % tiles_m) * BM, n0 = (blockIdx.x / tiles_m) * BN;
+    const int k0 = blockIdx.z * kslice, k1 = min(K, k0 + kslice);
+    unsigned long long acc[8][4];
 #pragma unroll
-        for (int kk = 0; kk < GBK; ++kk) {
-            float a[4], b[4];
+    for (int i = 0; i < 8; ++i)
 #pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
+        for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
+    Slab<BM, T, AKC> sa;
+    Slab<BN, T, BKC> sb;
+    sa.load(A, lda, m0, M, k0, k1, vecs & 1);
+    sb.load(B, ldb, n0, N, k0, k1, vecs & 2);
+    sa.store(As[0]);
+    sb.store(Bs[0]);
+    __syncthreads();
+    int buf = 0;
+    for (int kb = k0; kb < k1; kb += SBK, buf ^= 1) {
+        const bool more = kb + SBK < k1;
+        if (more) {
+            sa.load(A, lda, m0, M, kb + SBK, k1, vecs & 1);
+            sb.load(B, ldb, n0, N, kb + SBK, k1, vecs & 2);
+        }
 #pragma unroll
-            for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx + 16 * j];
+        for (int kk = 0; kk < SBK; ++kk) {
+            float a[8];
+            unsigned long long b[4];
+            *reinterpret_cast<float4*>(a) = *reinterpret_cast<const float4*>(&As[buf][kk][rm]);
+            *reinterpret_cast<float4*>(a + 4) = *reinterpret_cast<const float4*>(&As[buf][kk][rm + 16]);
+            *reinterpret_cast<ulonglong2*>(b) = *reinterpret_cast<const ulonglong2*>(&Bs[buf][kk][rn]);
+            *reinterpret_cast<ulonglong2*>(b + 2) = *reinterpret_cast<const ulonglong2*>(&Bs[buf][kk][rn + 32]);
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int i = 0; i < 8; ++i) {
+                const unsigned long long aa = pack2(a[i], a[i]);
 #pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+                for (int j = 0; j < 4; ++j) acc[i][j] = fma2(aa, b[j], acc[i][j]);
+            }
+        }
+        if (more) {
+            sa.store(As[buf ^ 1]);
+            sb.store(Bs[buf ^ 1]);
         }
         __syncthreads();
     }
+    // add: 0 C = alpha acc, 1 C += alpha acc (one block per tile), 2 atomically (K split)
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < 8; ++i) {
+        const int gm = m0 + rm + (i < 4 ? i : 12 + i);
+        if (gm >= M) continue;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int gm = m0 + ty + 16 * i, gn = n0 + tx + 16 * j;
-            if (gm < M && gn < N) {
-                float* c = C + (long long)gm * ldc + gn;
-                if (atomic) atomicAdd(c, alpha * acc[i][j]);
-                else *c += alpha * acc[i][j];
+        for (int h = 0; h < 2; ++h) {
+            const int gn = n0 + rn + 32 * h;
+            float v[4];
+            unpack2(acc[i][2 * h], v[0], v[1]);
+            unpack2(acc[i][2 * h + 1], v[2], v[3]);
+            float* c = C + (long long)gm * ldc + gn;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) v[q] *= alpha;
+            if (gn + 4 <= N && (vecs & 4)) {
+                if (add == 2) {
+                    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(c), "f"(v[0]), "f"(v[1]),
+                                 "f"(v[2]), "f"(v[3])
+                                 : "memory");
+                } else {
+                    float4 t = make_float4(v[0], v[1], v[2], v[3]);
+                    if (add) {
+                        const float4 o = *reinterpret_cast<const float4*>(c);
+                        t = make_float4(o.x + t.x, o.y + t.y, o.z + t.z, o.w + t.w);
+                    }
+                    *reinterpret_cast<float4*>(c) = t;
+                }
+            } else {
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (gn + q < N) {
+                        if (add == 2) atomicAdd(c + q, v[q]);
+                        else c[q] = add ? c[q] + v[q] : v[q];
+                    }
             }
         }
+    }
 }
 
 __global__ void k_scale_matrix(int M, int N, float beta, float* __restrict__ C, int ldc) {
@@ -447,17 +550,52 @@ helm_status nn_gemm(int transA, int transB, int M, int N, int K, float alpha, co
     if (M < 0 || N < 0 || K < 0 || !C || (K > 0 && (!A || !B))) return HELM_BAD_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (M == 0 || N == 0) return HELM_OK;
-    if (beta != 1.f) k_scale_matrix<<<grid_for((long long)M * N), 256, 0, s>>>(M, N, beta, C, ldc);
-    if (K == 0 || alpha == 0.f) return cudaGetLastError() == cudaSuccess ? HELM_OK : HELM_CUDA_ERROR;
-    const int gx = (N + GBN - 1) / GBN, gy = (M + GBM - 1) / GBM;
-    // split K until there are about two blocks per SM
-    int splits = 1;
-    while ((long long)gx * gy * splits < 2 * 152 && K / (splits * 2) >= 4 * GBK) splits *= 2;
-    int kslice = (K + splits - 1) / splits;
-    kslice = ((kslice + GBK - 1) / GBK) * GBK;
+    if (K == 0 || alpha == 0.f) {
+        if (beta != 1.f) k_scale_matrix<<<grid_for((long long)M * N), 256, 0, s>>>(M, N, beta, C, ldc);
+        return cudaGetLastError() == cudaSuccess ? HELM_OK : HELM_CUDA_ERROR;
+    }
+    // 128 x 128 tiles where M fills them; 32 rows for the batch-sized products (a row of
+    // the batch per 8 threads wastes nothing on padding), 256 columns wide while that
+    // still gives two blocks per SM with K unsplit or K is long enough to split
+    const int bm = M <= 64 ? 32 : 128;
+    const int bn = bm == 32 && N > 128 ? 256 : 128;
+    const long long tiles = (long long)((M + bm - 1) / bm) * ((N + bn - 1) / bn);
+    if (tiles > 0x7fffffffLL) return HELM_BAD_ARG;
+    // K split until every SM holds its resident blocks once (2 of 256 threads, 3 of 128, 5
+    // of 64: a part of a second wave would cost a whole one), at least 2 slabs each; the
+    // split parts add into C atomically
+    const long long want = (bm == 128 ? 2 : bn == 256 ? 3 : 5) * 152;
+    int splits = (int)std::max<long long>(1, std::min<long long>(want / tiles, K / (2 * SBK)));
+    int kslice = ((K + splits - 1) / splits + SBK - 1) / SBK * SBK;
     splits = (K + kslice - 1) / kslice;
-    k_sgemm<<<dim3(gx, gy, splits), 256, 0, s>>>(transA, transB, M, N, K, alpha, A, lda, B, ldb, C, ldc, kslice,
-                                                 splits > 1);
+    int add = splits > 1 ? 2 : (beta != 0.f);
+    if (beta != 1.f && add) {
+        if (beta == 0.f && (M == 1 || ldc == N)) {
+            if (cudaMemsetAsync(C, 0, sizeof(float) * N * (size_t)M, s) != cudaSuccess) return HELM_CUDA_ERROR;
+        } else if (beta == 0.f && ldc > N) {
+            if (cudaMemset2DAsync(C, sizeof(float) * ldc, 0, sizeof(float) * N, M, s) != cudaSuccess)
+                return HELM_CUDA_ERROR;
+        } else {
+            k_scale_matrix<<<grid_for((long long)M * N), 256, 0, s>>>(M, N, beta, C, ldc);
+        }
+    }
+    const int vecs = (lda % 4 == 0 && al16(A) ? 1 : 0) | (ldb % 4 == 0 && al16(B) ? 2 : 0) |
+                     (ldc % 4 == 0 && al16(C) ? 4 : 0);
+    const dim3 g((unsigned)tiles, 1, (unsigned)splits);
+#define SG(BM, BN, AKC, BKC)                                                                                   \
+    k_sgemm<BM, BN, AKC, BKC><<<g, BM * BN / 64, 0, s>>>(M, N, K, alpha, A, lda, B, ldb, C, ldc, kslice, vecs, add)
+#define SGT(BM, BN)                                                      \
+    do {                                                                 \
+        if (!transA && transB) SG(BM, BN, true, true);                   \
+        else if (!transA) SG(BM, BN, true, false);                       \
+        else if (transB) SG(BM, BN, false, true);                        \
+        else SG(BM, BN, false, false);                                   \
+    } while (0)
+    if (bm == 128) SGT(128, 128);
+    else if (bn == 256) SGT(32, 256);
+    else SGT(32, 128);
+#undef SGT
+#undef SG
     return cudaGetLastError() == cudaSuccess ? HELM_OK : HELM_CUDA_ERROR;
 }
 

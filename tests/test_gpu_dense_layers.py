@@ -101,3 +101,29 @@ def test_bias_act(rows, cols, off):
     x = _off(X, off)
     assert _lib().nn_bias_act(rows, cols, _p(x), None, 1, None) == 0
     assert np.array_equal(x.cpu().numpy().reshape(rows, cols), np.maximum(X, 0))
+
+
+@pytest.mark.parametrize("ta", [0, 1])
+@pytest.mark.parametrize("tb", [0, 1])
+@pytest.mark.parametrize("M,N,K", [(1, 1, 1), (33, 129, 15), (64, 128, 16), (65, 257, 17), (32, 256, 4101), (128, 128, 300),
+                                   (130, 3, 2049), (5, 700, 128)])
+def test_gemm_tiles(ta, tb, M, N, K):
+    """Edges of the GEMM's tiles (32 and 128 rows, 128 and 256 columns), slabs and K
+    splits, leading dimensions with and without 16-byte rows, beta 0, 1 and general.
+    |C - exact| <= (K + 4) 2^-24 (|A| |B|) + a few ulps of beta C."""
+    rng = np.random.default_rng(M + 3 * N + 7 * K)
+    for pad, beta in ((0, 0.0), (4 - (M + N + K) % 4, 1.0), (1, -0.75)):
+        A = rng.standard_normal((K, M + pad) if ta else (M, K + pad)).astype(np.float32)
+        B = rng.standard_normal((N, K + pad) if tb else (K, N + pad)).astype(np.float32)
+        C0 = rng.standard_normal((M, N + pad)).astype(np.float32)
+        opA = (A[:, :M].T if ta else A[:, :K]).astype(np.float64)
+        opB = (B[:, :K].T if tb else B[:, :N]).astype(np.float64)
+        Ad, Bd, Cd = _off(A, pad % 2), to_dev(B), to_dev(C0)
+        if beta == 0.0:
+            Cd[:, :N] = float("nan")                      # not read
+        assert _lib().nn_gemm(ta, tb, M, N, K, 1.5, _p(Ad), A.shape[1], _p(Bd), B.shape[1], beta, _p(Cd), N + pad, None) == 0
+        got = Cd.cpu().numpy()
+        ref = 1.5 * (opA @ opB) + beta * C0[:, :N]
+        bound = (K + 4) * U * 1.5 * (np.abs(opA) @ np.abs(opB)) + 4 * U * abs(beta) * np.abs(C0[:, :N])
+        assert np.all(np.abs(got[:, :N] - ref) <= bound)
+        assert np.array_equal(got[:, N:], C0[:, N:])      # nothing outside the matrix
