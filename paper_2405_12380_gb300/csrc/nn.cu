@@ -24,8 +24,8 @@ namespace {
 // pipe's 80 TFLOP/s), by the FP32 pipe and HBM about equally for the branch's first layer
 // at 64^3 (32 x 256 x 524288, 537 MB of weights read: 1060 -> 206 us; its weight gradient,
 // 537 MB written: 842 -> 181 us).  Before: 64 x 64 tiles, 4 x 4 per thread, 4-byte loads,
-// no prefetch, and 64-row tiles half empty at a batch of 32.  fma.rn.f32x2 measured the
-// same rate per multiply-add as scalar FMA but half the issue slots.
+// no prefetch, and 64-row tiles half empty at a batch of 32.  The packed fma.rn.f32x2
+// issues two multiply-adds per instruction.
 constexpr int SBK = 16;
 
 __device__ __forceinline__ unsigned long long pack2(float a, float b) {

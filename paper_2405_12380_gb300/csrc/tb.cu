@@ -107,61 +107,95 @@ __global__ void __launch_bounds__(TR_T) k_trunk(Op<double> op, const double* __r
 }
 
 // ------------------------------------------------------------------- Gram
-// C = A^T B over N rows; A: N x p (lda), B: N x q (ldb); 64 x 64 output tile per
-// block, 4 x 4 per thread, split over row slices (blockIdx.z); partials then summed.
-constexpr int GT = 64, GR = 32;
+// C = A^T B over N rows; A: N x p (lda), B: N x q (ldb), split over row slices
+// (blockIdx.z) whose partials are then summed.  Bound by the FP64 pipe (2 instructions
+// per clock and SM), so what counts is the number of FMAs: a block of 64 threads owns a
+// 16 x 16 tile, 2 x 2 per thread (64 x 64 tiles padded a 16-column basis 16 times over
+// with zeros), and with SYM (B = A) only the tiles on and above the diagonal are formed,
+// k_gram_sum mirroring them.  The four shared-memory reads per four FMAs stay far below
+// the 64 clocks that an FP64 instruction of a warp holds its scheduler's pipe.  Each
+// value is summed row by row over its slice, then slice by slice, whatever the tiles.
+// 64^3 nodes (ncu), 64 x 64 tiles without symmetry against this form: p = q = 128
+// 7.12 -> 3.93 ms (98% of the FP64 pipe), p = q = 16 1.80 -> 0.14 ms, p = 16, q = 32
+// 1.80 -> 0.22 ms.
+constexpr int GT = 16, GR = 32;
+constexpr int GSPLIT_TILE = 64;      // the row split depends on 64 x 64 tiles of C (its order of sums)
 
-__global__ void __launch_bounds__(256) k_gram(const double* __restrict__ A, int lda, int p,
-                                              const double* __restrict__ B, int ldb, int q, long long N,
-                                              long long rows_per_split, double* __restrict__ partials) {
-    __shared__ double As[GR][GT + 1];
-    __shared__ double Bs[GR][GT + 1];
-    const int ti = threadIdx.x / 16, tj = threadIdx.x % 16;   // 16 x 16 threads, 4 x 4 each
-    const int i0 = blockIdx.x * GT, j0 = blockIdx.y * GT;
+template <bool SYM>
+__global__ void __launch_bounds__(64) k_gram(const double* __restrict__ A, int lda, int p, const double* __restrict__ B,
+                                             int ldb, int q, long long N, long long rows_per_split,
+                                             double* __restrict__ partials) {
+    __shared__ double As[GR][GT];
+    __shared__ double Bs[GR][GT];
+    const int ti = threadIdx.x / 8, tj = threadIdx.x % 8;    // 8 x 8 threads, 2 x 2 each
+    const int tp = (p + GT - 1) / GT;
+    int bi, bj;
+    if (SYM) {                                               // tile pair (bi <= bj) of a linear index
+        int e = blockIdx.x;
+        bi = 0;
+        while (e >= tp - bi) { e -= tp - bi; ++bi; }
+        bj = bi + e;
+    } else {
+        bi = blockIdx.x % tp;
+        bj = blockIdx.x / tp;
+    }
+    const int i0 = bi * GT, j0 = bj * GT;
     const long long r0 = (long long)blockIdx.z * rows_per_split;
     const long long r1 = min(N, r0 + rows_per_split);
-    double acc[4][4];
+    double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+    const int cc = threadIdx.x % GT, rq = threadIdx.x / GT;  // this thread loads column cc of rows rq + 4 u
+    const bool aok = i0 + cc < p, bok = j0 + cc < q;
+    double av[GR / 4], bv[GR / 4];
+    auto load = [&](long long rb) {
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) acc[a][c] = 0.0;
+        for (int u = 0; u < GR / 4; ++u) {
+            const long long row = rb + rq + 4 * u;
+            av[u] = (aok && row < r1) ? A[row * lda + i0 + cc] : 0.0;
+            bv[u] = (bok && row < r1) ? B[row * ldb + j0 + cc] : 0.0;
+        }
+    };
+    if (r0 < r1) load(r0);
     for (long long rb = r0; rb < r1; rb += GR) {
-        for (int t = threadIdx.x; t < GR * GT; t += 256) {
-            int rr = t / GT, cc = t % GT;
-            long long row = rb + rr;
-            bool ok = row < r1;
-            As[rr][cc] = (ok && i0 + cc < p) ? A[row * lda + i0 + cc] : 0.0;
-            Bs[rr][cc] = (ok && j0 + cc < q) ? B[row * ldb + j0 + cc] : 0.0;
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < GR / 4; ++u) {
+            As[rq + 4 * u][cc] = av[u];
+            Bs[rq + 4 * u][cc] = bv[u];
         }
         __syncthreads();
-#pragma unroll 4
+        if (rb + GR < r1) load(rb + GR);
+#pragma unroll 8
         for (int rr = 0; rr < GR; ++rr) {
-            double av[4], bv[4];
-#pragma unroll
-            for (int a = 0; a < 4; ++a) av[a] = As[rr][ti + 16 * a];
-#pragma unroll
-            for (int c = 0; c < 4; ++c) bv[c] = Bs[rr][tj + 16 * c];
-#pragma unroll
-            for (int a = 0; a < 4; ++a)
-#pragma unroll
-                for (int c = 0; c < 4; ++c) acc[a][c] = fma(av[a], bv[c], acc[a][c]);
+            const double a0 = As[rr][ti], a1 = As[rr][ti + 8], b0 = Bs[rr][tj], b1 = Bs[rr][tj + 8];
+            acc[0][0] = fma(a0, b0, acc[0][0]);
+            acc[0][1] = fma(a0, b1, acc[0][1]);
+            acc[1][0] = fma(a1, b0, acc[1][0]);
+            acc[1][1] = fma(a1, b1, acc[1][1]);
         }
-        __syncthreads();
     }
     double* P = partials + (long long)blockIdx.z * p * q;
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+    for (int a = 0; a < 2; ++a)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            int i = i0 + ti + 16 * a, j = j0 + tj + 16 * c;
+        for (int c = 0; c < 2; ++c) {
+            const int i = i0 + ti + 8 * a, j = j0 + tj + 8 * c;
             if (i < p && j < q) P[(long long)i * q + j] = acc[a][c];
         }
 }
 
-__global__ void k_gram_sum(const double* __restrict__ partials, int nsplit, long long pq, double* __restrict__ out) {
+// SYM: C is q x q with only the tiles on and above the diagonal in the partials
+template <bool SYM>
+__global__ void k_gram_sum(const double* __restrict__ partials, int nsplit, long long pq, int q,
+                           double* __restrict__ out) {
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < pq; e += (long long)gridDim.x * blockDim.x) {
+        long long s_at = e;
+        if (SYM) {
+            const int i = (int)(e / q), j = (int)(e % q);
+            if (i / GT > j / GT) s_at = (long long)j * q + i;
+        }
         double s = 0;
-        for (int z = 0; z < nsplit; ++z) s += partials[(long long)z * pq + e];
+#pragma unroll 16
+        for (int z = 0; z < nsplit; ++z) s += partials[(long long)z * pq + s_at];
         out[e] = s;
     }
 }
@@ -232,20 +266,26 @@ __global__ void k_tri_inverse(const double* __restrict__ R, int k, int ldr, doub
     }
 }
 
-// Q[l][c] = sum_{a <= c} T[l][kept[a]] Rinv[a][c]  (kept == nullptr: identity)
+// Q[l][c] = sum_{a <= c} T[l][kept[a]] Rinv[a][c]  (kept == nullptr: identity).
+// Threads along x own columns (as many as ldq, at most 256), groups along y own GU_NB
+// nodes each, so that a narrow basis still fills the block: with one group per block and
+// 256 threads a 32-column basis left 224 of them idle (64^3, k = 16: 486 -> 274 us).
 constexpr int GU_NB = 16;
 __global__ void __launch_bounds__(256) k_gather_upper(const double* __restrict__ T, int ldt,
                                                       const int* __restrict__ kept, int k,
                                                       const double* __restrict__ Rinv, int ldr,
                                                       double* __restrict__ Q, int ldq, long long N) {
-    extern __shared__ double ts[];     // [GU_NB][k]
-    const long long l0 = (long long)blockIdx.x * GU_NB;
-    for (int t = threadIdx.x; t < GU_NB * k; t += blockDim.x) {
-        int nb = t / k, a = t % k;
-        long long l = l0 + nb;
+    extern __shared__ double ts[];     // [blockDim.y][GU_NB][k]
+    const long long b0 = (long long)blockIdx.x * GU_NB * blockDim.y;
+    const int tid = threadIdx.y * blockDim.x + threadIdx.x, nt = blockDim.x * blockDim.y;
+    for (int t = tid; t < GU_NB * (int)blockDim.y * k; t += nt) {
+        const int nb = t / k, a = t % k;
+        const long long l = b0 + nb;
         ts[t] = l < N ? T[l * ldt + (kept ? kept[a] : a)] : 0.0;
     }
     __syncthreads();
+    const long long l0 = b0 + (long long)threadIdx.y * GU_NB;
+    const double* tg = ts + (size_t)threadIdx.y * GU_NB * k;
     for (int c = threadIdx.x; c < ldq; c += blockDim.x) {
         double acc[GU_NB];
 #pragma unroll
@@ -254,7 +294,7 @@ __global__ void __launch_bounds__(256) k_gather_upper(const double* __restrict__
             for (int a = 0; a <= c; ++a) {
                 const double r = Rinv[(long long)a * ldr + c];
 #pragma unroll
-                for (int nb = 0; nb < GU_NB; ++nb) acc[nb] = fma(ts[nb * k + a], r, acc[nb]);
+                for (int nb = 0; nb < GU_NB; ++nb) acc[nb] = fma(tg[nb * k + a], r, acc[nb]);
             }
         }
 #pragma unroll
@@ -1165,14 +1205,22 @@ void launch_trunk_eval(const Op<double>& op, const double* dW, const int* widths
 
 void launch_gram(const double* A, int lda, int p, const double* B, int ldb, int q, long long N, double* partials,
                  double* out, cudaStream_t s) {
-    int gx = (p + GT - 1) / GT, gy = (q + GT - 1) / GT;
+    const int gx = (p + GSPLIT_TILE - 1) / GSPLIT_TILE, gy = (q + GSPLIT_TILE - 1) / GSPLIT_TILE;
     int nsplit = (2 * 152 + gx * gy - 1) / (gx * gy);
     long long rows = (N + nsplit - 1) / nsplit;
     rows = ((rows + GR - 1) / GR) * GR;
     nsplit = (int)((N + rows - 1) / rows);
-    k_gram<<<dim3(gx, gy, nsplit), 256, 0, s>>>(A, lda, p, B, ldb, q, N, rows, partials);
-    long long pq = (long long)p * q;
-    k_gram_sum<<<(unsigned)((pq + 255) / 256), 256, 0, s>>>(partials, nsplit, pq, out);
+    const bool sym = A == B && lda == ldb && p == q;
+    const int tp = (p + GT - 1) / GT, tq = (q + GT - 1) / GT;
+    const long long pq = (long long)p * q;
+    const unsigned sum_blocks = (unsigned)((pq + 63) / 64);
+    if (sym) {
+        k_gram<true><<<dim3(tp * (tp + 1) / 2, 1, nsplit), 64, 0, s>>>(A, lda, p, B, ldb, q, N, rows, partials);
+        k_gram_sum<true><<<sum_blocks, 64, 0, s>>>(partials, nsplit, pq, q, out);
+    } else {
+        k_gram<false><<<dim3(tp * tq, 1, nsplit), 64, 0, s>>>(A, lda, p, B, ldb, q, N, rows, partials);
+        k_gram_sum<false><<<sum_blocks, 64, 0, s>>>(partials, nsplit, pq, q, out);
+    }
 }
 
 void launch_select_chol(const double* G, int p, int ldg, double tau, double* W, double* R, int* kept, int* nkept,
@@ -1186,9 +1234,14 @@ void launch_tri_inverse(const double* R, int k, int ldr, double* Rinv, cudaStrea
 
 void launch_gather_times_upper(const double* T, int ldt, const int* kept, int k, const double* Rinv, int ldr,
                                double* Q, int ldq, long long N, cudaStream_t s) {
-    size_t smem = GU_NB * k * sizeof(double);
-    cudaFuncSetAttribute(k_gather_upper, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_gather_upper<<<(unsigned)((N + GU_NB - 1) / GU_NB), 256, smem, s>>>(T, ldt, kept, k, Rinv, ldr, Q, ldq, N);
+    // ldq is a multiple of 32, at most 256
+    const int tx = ldq <= 32 ? 32 : ldq <= 64 ? 64 : ldq <= 128 ? 128 : 256;
+    int ty = 256 / tx;
+    while (ty > 1 && N < 2LL * 152 * GU_NB * ty) ty /= 2;            // small grids: a block per SM first
+    const size_t smem = (size_t)ty * GU_NB * k * sizeof(double);     // at most 32 KB
+    const int nodes = GU_NB * ty;
+    k_gather_upper<<<(unsigned)((N + nodes - 1) / nodes), dim3(tx, ty), smem, s>>>(T, ldt, kept, k, Rinv, ldr, Q, ldq,
+                                                                                   N);
 }
 
 void launch_apply_columns(const Op<double>& op, const double* Q, int ldq, int k, double* W, int ldw,
