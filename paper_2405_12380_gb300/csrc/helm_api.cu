@@ -206,6 +206,37 @@ bool fused_sweeps32(helm_handle* h, int kind, double omega, int sweeps, const fl
     return true;
 }
 
+// `sweeps` damped-Jacobi sweeps on A x = f, the result in x (from zero, or from x); tmp is
+// the other buffer of the out-of-place sweeps.  Small 2D grids take several sweeps per
+// launch; there the launch count is made even unless from zero (one launch from zero, or
+// an even number from x, ends in x without a copy).
+template <typename R>
+helm_status jacobi_run(helm_handle* h, const Op<R>& op, double omega, int sweeps, const typename CT<R>::T* f,
+                       typename CT<R>::T* x, typename CT<R>::T* tmp, int conj, bool from_zero, cudaStream_t s) {
+    using C = typename CT<R>::T;
+    if (sweeps <= 0) return HELM_OK;
+    const int per = jacobi_tile_sweeps(op);
+    int L = per ? (sweeps + per - 1) / per : sweeps;
+    if (per && !from_zero && sweeps > 1) L += L & 1;
+    // the last launch writes x, unless an odd number starts from x: then it writes tmp
+    const bool to_tmp = !from_zero && (L & 1);
+    const C* in = from_zero ? nullptr : x;
+    for (int q = 0, done = 0; q < L; ++q) {
+        const int n = per ? (sweeps - done + L - q - 1) / (L - q) : 1;
+        C* out = (((L - 1 - q) & 1) == 0) != to_tmp ? x : tmp;
+        const bool mark = in != nullptr;                   // (a launch that reads neighbours)
+        if (mark) ev_mark(h, 2, 0);
+        if (per) launch_jacobi_tile<R>(op, omega, n, f, in, out, conj, s);
+        else launch_jacobi<R>(op, omega, f, in, out, conj, in == nullptr, s);
+        if (mark) ev_mark(h, 2, 1);
+        in = out;
+        done += n;
+    }
+    if (to_tmp) CK(cudaMemcpyAsync(x, tmp, sizeof(C) * op.N, cudaMemcpyDeviceToDevice, s));
+    h->launches += L;
+    return HELM_OK;
+}
+
 // z = n sweeps of the relaxation on A z = r from z = 0 (FP64)
 helm_status relax_from_zero(helm_handle* h, int kind, double omega, int sweeps, const double2* r, double2* z,
                             int conj) {
@@ -216,17 +247,7 @@ helm_status relax_from_zero(helm_handle* h, int kind, double omega, int sweeps, 
     }
     if (kind == HELM_JACOBI) {
         TRY(ensure_tmp(h, 1));
-        // sweep 1 from zero writes z; later sweeps ping-pong so that the last lands in z
-        double2* a = (sweeps % 2 == 1) ? z : h->tmp[0];
-        double2* b = (sweeps % 2 == 1) ? h->tmp[0] : z;
-        launch_jacobi<double>(h->op64, omega, r, nullptr, a, conj, true, s);
-        for (int q = 1; q < sweeps; ++q) {
-            ev_mark(h, 2, 0);
-            launch_jacobi<double>(h->op64, omega, r, a, b, conj, false, s);
-            ev_mark(h, 2, 1);
-            std::swap(a, b);
-        }
-        h->launches += sweeps;
+        TRY(jacobi_run<double>(h, h->op64, omega, sweeps, r, z, h->tmp[0], conj, true, s));
         CKL();
         return HELM_OK;
     }
@@ -311,14 +332,7 @@ helm_status precond32(helm_handle* h, const helm_solve_opts* o, const float2* v,
         CK(cudaMemsetAsync(z, 0, sizeof(float2) * h->N, s));
     } else if (o->relax == HELM_JACOBI) {
         TRY(ensure_tmp32(h, 4));
-        float2* a = (o->n_r % 2 == 1) ? z : h->tmp32[3];
-        float2* b = (o->n_r % 2 == 1) ? h->tmp32[3] : z;
-        launch_jacobi<float>(h->op32, o->omega, v, nullptr, a, conj, true, s);
-        for (int q = 1; q < o->n_r; ++q) {
-            launch_jacobi<float>(h->op32, o->omega, v, a, b, conj, false, s);
-            std::swap(a, b);
-        }
-        h->launches += o->n_r;
+        TRY(jacobi_run<float>(h, h->op32, o->omega, o->n_r, v, z, h->tmp32[3], conj, true, s));
     } else {
         TRY(ensure_tmp32(h, 4));
         if (!fused_sweeps32(h, o->relax, o->omega, o->n_r, v, z, h->tmp32[3], conj, true)) {
@@ -411,25 +425,11 @@ helm_status precond_rbgs_tb_df(helm_handle* h, const helm_solve_opts* o, const d
 }
 
 // ---------------------------------------------------------------- multigrid
-// `sweeps` damped-Jacobi sweeps on A z = r on handle H, z from zero if `zero`; the
-// sweeps alternate between z and jt so that the last one lands in z
+// `sweeps` damped-Jacobi sweeps on A z = r on handle H, z from zero if `zero`
 helm_status jacobi_sweeps(helm_handle* h, double omega, int sweeps, const double2* r, double2* z, double2* jt,
                           int conj, bool zero, cudaStream_t s) {
-    if (sweeps <= 0) {
-        if (zero) CK(cudaMemsetAsync(z, 0, sizeof(double2) * h->N, s));
-        return HELM_OK;
-    }
-    double2* bufs[2] = {z, jt};
-    int src = zero ? -1 : 0;
-    for (int q = 0; q < sweeps; ++q) {
-        const int dst = ((sweeps - 1 - q) % 2 == 0) ? 0 : 1;
-        if (src == dst) {
-            CK(cudaMemcpyAsync(bufs[1 - src], bufs[src], sizeof(double2) * h->N, cudaMemcpyDeviceToDevice, s));
-            src = 1 - src;
-        }
-        launch_jacobi<double>(h->op64, omega, r, src < 0 ? nullptr : bufs[src], bufs[dst], conj, src < 0, s);
-        src = dst;
-    }
+    if (sweeps <= 0 && zero) CK(cudaMemsetAsync(z, 0, sizeof(double2) * h->N, s));
+    TRY(jacobi_run<double>(h, h->op64, omega, sweeps, r, z, jt, conj, zero, s));
     CKL();
     return HELM_OK;
 }
@@ -570,14 +570,7 @@ helm_status solve_relax(helm_handle* h, const helm_solve_opts* o, const double2*
         if (cycles >= o->maxit) { st->status = HELM_NOT_CONVERGED; break; }
         if (o->relax == HELM_JACOBI) {
             TRY(ensure_tmp(h, 1));
-            double2* a = x;
-            double2* b = h->tmp[0];
-            for (int q = 0; q < o->n_r; ++q) {
-                launch_jacobi<double>(h->op64, o->omega, f, a, b, o->conj, false, h->stream);
-                std::swap(a, b);
-            }
-            h->launches += o->n_r;
-            if (a != x) CK(cudaMemcpyAsync(x, a, sizeof(double2) * h->N, cudaMemcpyDeviceToDevice, h->stream));
+            TRY(jacobi_run<double>(h, h->op64, o->omega, o->n_r, f, x, h->tmp[0], o->conj, false, h->stream));
         } else if (red_black(o->relax)) {
             red_black_sweeps<double>(h, h->op64, o->relax, o->omega, o->n_r, f, x, o->conj, false);
         }
@@ -1510,26 +1503,14 @@ helm_status helm_relax(helm_handle* h, int kind, double omega, int sweeps, const
     if (dtype == HELM_C128) {
         if (kind == HELM_JACOBI) {
             TRY(ensure_tmp(h, 1));
-            double2* a = (double2*)x;
-            double2* b = h->tmp[0];
-            for (int q = 0; q < sweeps; ++q) {
-                launch_jacobi<double>(h->op64, omega, (const double2*)f, a, b, conj, false, s);
-                std::swap(a, b);
-            }
-            if (a != x) CK(cudaMemcpyAsync(x, a, sizeof(double2) * h->N, cudaMemcpyDeviceToDevice, s));
+            TRY(jacobi_run<double>(h, h->op64, omega, sweeps, (const double2*)f, (double2*)x, h->tmp[0], conj, false, s));
         } else {
             red_black_sweeps<double>(h, h->op64, kind, omega, sweeps, (const double2*)f, (double2*)x, conj, false);
         }
     } else if (dtype == HELM_C64) {
         if (kind == HELM_JACOBI) {
             TRY(ensure_tmp32(h, 1));
-            float2* a = (float2*)x;
-            float2* b = h->tmp32[0];
-            for (int q = 0; q < sweeps; ++q) {
-                launch_jacobi<float>(h->op32, omega, (const float2*)f, a, b, conj, false, s);
-                std::swap(a, b);
-            }
-            if (a != x) CK(cudaMemcpyAsync(x, a, sizeof(float2) * h->N, cudaMemcpyDeviceToDevice, s));
+            TRY(jacobi_run<float>(h, h->op32, omega, sweeps, (const float2*)f, (float2*)x, h->tmp32[0], conj, false, s));
         } else {
             TRY(ensure_tmp32(h, 1));
             if (!fused_sweeps32(h, kind, omega, sweeps, (const float2*)f, (float2*)x, h->tmp32[0], conj, false))

@@ -149,6 +149,13 @@ template <typename R>
 void launch_jacobi(const Op<R>& op, double omega, const typename CT<R>::T* f,
                    const typename CT<R>::T* xin, typename CT<R>::T* xout, int conj, bool xzero,
                    cudaStream_t s);
+// several sweeps in one launch (2D grids): at most jacobi_tile_sweeps(op) of them, which is
+// 0 where the tiled form is not used; xin = nullptr: from zero; xin != xout
+template <typename R>
+int jacobi_tile_sweeps(const Op<R>& op);
+template <typename R>
+void launch_jacobi_tile(const Op<R>& op, double omega, int sweeps, const typename CT<R>::T* f,
+                        const typename CT<R>::T* xin, typename CT<R>::T* xout, int conj, cudaStream_t s);
 // omega: 1 = Gauss-Seidel; otherwise SOR (each node moves by omega times its GS step)
 template <typename R>
 void launch_rbgs_half(const Op<R>& op, int colour, const typename CT<R>::T* f, typename CT<R>::T* x,

@@ -12,6 +12,7 @@
 //   k_sweep_c64      3D complex64 full red-black sweep in one launch (old planes
 //                    staged in shared memory by cp.async, halo rows recomputed)
 //   k_apply, k_jacobi, k_rbgs   the general forms (2D, no tables, complex128)
+//   k_jacobi_tile    several 2D Jacobi sweeps per launch (small grids)
 //   k_apply_bicg(_df)           the BiCGStab operator with its fused reduction
 //   k_cycle_df       the red-black part of the FP64 trunk-basis hybrid cycle in
 //                    double-float arithmetic, one cooperative launch
@@ -29,6 +30,7 @@ namespace helm {
 namespace {
 
 constexpr int BX = 32, BY = 8;
+constexpr int kJacobiTileSweeps = 5;      // sweeps of one tiled Jacobi launch (at most 26^2 threads)
 
 __device__ __forceinline__ int layer_index(int i, int n, int L) {
     int d = min(i, n - 1 - i);
@@ -897,6 +899,63 @@ __global__ void __launch_bounds__(BX * BY) k_jacobi(Op<R> op, R omega, const typ
     if (op.dim == 3 && k0 + 1 < op.n) jacobi_point<R, XZERO>(op, omega, f, xin, xout, conj, i, j, k0 + 1);
 }
 
+// Several damped-Jacobi sweeps of a 2D grid in one launch (small grids, where a sweep
+// costs its launch: 5.3 us at 64 x 64 against 0.1 us of FP64 arithmetic).  A block owns
+// TI x TI nodes and recomputes a halo of S nodes around them, one node per thread
+// (blockDim = TI + 2 S per side): S sweeps run in shared memory, each on a region one
+// node smaller per side, and only the block's own nodes are written.  The sweep is
+// x <- (1 - omega) x + omega D^-1 f - omega h^-2 D^-1 s with the two products of D^-1
+// formed once per node (12 FP64 instructions a sweep against 16 when D^-1 (f - h^-2 s)
+// is formed each time); a masked node has s's factor zero, and is zero to its
+// neighbours.  xin = nullptr: from zero.
+template <typename R>
+__global__ void k_jacobi_tile(Op<R> op, R omega, int S, const typename CT<R>::T* __restrict__ f,
+                              const typename CT<R>::T* __restrict__ xin, typename CT<R>::T* __restrict__ xout,
+                              int conj) {
+    using C = typename CT<R>::T;
+    extern __shared__ __align__(16) unsigned char jt_smem[];
+    const int E = blockDim.x, TI = E - 2 * S, tx = threadIdx.x, ty = threadIdx.y, t = ty * E + tx;
+    C* buf = reinterpret_cast<C*>(jt_smem);                // [2][E * E]
+    const int i = blockIdx.x * TI - S + tx, j = blockIdx.y * TI - S + ty;
+    const bool in = i >= 0 && j >= 0 && i < op.n && j < op.n;
+    const int l = in ? i + op.n * j : 0;
+    C zero;
+    zero.x = 0; zero.y = 0;
+    C x = zero, fp = zero, c = zero;
+    bool fluid = false;
+    if (in) {
+        fluid = !(op.nbm[HCHK(l, op.N)] & kMasked);
+        const C fv = f[HCHK(l, op.N)];
+        if (xin) x = xin[HCHK(l, op.N)];
+        if (fluid) {
+            const C id = cscale(omega, invd_of(op, l, op.lidx[HCHK(l, op.N)], conj));
+            fp = cmul(id, fv);
+            c = cscale(op.hinv2, id);
+        } else {
+            fp = cscale(omega, fv);
+        }
+    }
+    const int rim = min(min(tx, E - 1 - tx), min(ty, E - 1 - ty));
+    const R w1 = (R)1 - omega;
+    for (int q = 0; q < S; ++q) {
+        C* b = buf + (q & 1) * E * E;
+        b[t] = fluid ? x : zero;
+        __syncthreads();
+        if (rim > q) {
+            C y;
+            y.x = fp.x + w1 * x.x;
+            y.y = fp.y + w1 * x.y;
+            if (fluid) {
+                const C s = cadd(cadd(b[t - 1], b[t + 1]), cadd(b[t - E], b[t + E]));
+                y.x -= c.x * s.x - c.y * s.y;
+                y.y -= c.x * s.y + c.y * s.x;
+            }
+            x = y;
+        }
+    }
+    if (rim >= S && in) xout[HCHK(l, op.N)] = x;
+}
+
 // red-black Gauss-Seidel update of one node of the swept colour, in place:
 // x_l = D_l^-1 (f_l - h^-2 sum of fluid neighbours) on fluid nodes (the Gauss-Seidel
 // value x + D^-1 (f - A x) with the diagonal term cancelled), f_l on masked nodes;
@@ -1666,6 +1725,33 @@ void launch_jacobi(const Op<R>& op, double omega, const typename CT<R>::T* f, co
     if (xzero) k_jacobi<R, true><<<g, b, 0, s>>>(op, (R)omega, f, xin, xout, conj);
     else k_jacobi<R, false><<<g, b, 0, s>>>(op, (R)omega, f, xin, xout, conj);
 }
+
+// sweeps per launch of the tiled form for this operator, 0 where it does not apply (3D,
+// outer-boundary rows, no tables) or does not pay: with the halo an FP64 node costs about
+// twice its arithmetic, so the tiles win while a sweep is bound by its launch (64^2: 5.3 us
+// a launch; a 512^2 FP64 sweep is already bound by the FP64 pipe)
+template <typename R>
+int jacobi_tile_sweeps(const Op<R>& op) {
+    const int limit = std::is_same<R, double>::value ? 384 : 768;
+    return (op.dim == 2 && op.nbm && op.lidx && !op.face && op.n <= limit) ? kJacobiTileSweeps : 0;
+}
+
+template <typename R>
+void launch_jacobi_tile(const Op<R>& op, double omega, int sweeps, const typename CT<R>::T* f,
+                        const typename CT<R>::T* xin, typename CT<R>::T* xout, int conj, cudaStream_t s) {
+    // about 12 x 12 blocks (one per SM), of 6 x 6 to 16 x 16 nodes (more has less halo, but a
+    // node per thread)
+    const int TI = std::max(6, std::min(16, (op.n + 11) / 12)), E = TI + 2 * sweeps;
+    const dim3 g((op.n + TI - 1) / TI, (op.n + TI - 1) / TI), b(E, E);
+    k_jacobi_tile<R><<<g, b, 2 * (size_t)E * E * sizeof(typename CT<R>::T), s>>>(op, (R)omega, sweeps, f, xin, xout, conj);
+}
+
+template int jacobi_tile_sweeps<double>(const Op<double>&);
+template int jacobi_tile_sweeps<float>(const Op<float>&);
+template void launch_jacobi_tile<double>(const Op<double>&, double, int, const double2*, const double2*, double2*, int,
+                                         cudaStream_t);
+template void launch_jacobi_tile<float>(const Op<float>&, double, int, const float2*, const float2*, float2*, int,
+                                        cudaStream_t);
 
 template <typename R>
 void launch_rbgs_half(const Op<R>& op, int colour, const typename CT<R>::T* f, typename CT<R>::T* x, int conj,
