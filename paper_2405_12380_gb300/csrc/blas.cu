@@ -250,71 +250,21 @@ __global__ void __launch_bounds__(kFinThreads) k_bicg_scalar(int recipe, const d
 }
 
 // ------------------------------------------------------------------ FGMRES
-constexpr int MD_TILE = 512;
-
-// partials[b * nv + i] = sum over this block's tiles of conj(V_i) . w
-__global__ void __launch_bounds__(TB) k_mdot(const double2* __restrict__ V, int nv, const double2* __restrict__ w,
-                                             long long N, double2* partials) {
-    __shared__ double2 ws[MD_TILE];
-    __shared__ double2 acc[kMaxRestart + 1];
-    for (int i = threadIdx.x; i < nv; i += TB) acc[i] = make_double2(0, 0);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (long long t0 = (long long)blockIdx.x * MD_TILE; t0 < N; t0 += (long long)gridDim.x * MD_TILE) {
-        const int rows = (int)min((long long)MD_TILE, N - t0);
-        __syncthreads();
-        for (int r = threadIdx.x; r < rows; r += TB) ws[r] = w[t0 + r];
-        __syncthreads();
-        for (int i = warp; i < nv; i += TB / 32) {
-            const double2* Vi = V + (long long)i * N + t0;
-            double2 a = make_double2(0, 0);
-            for (int r = lane; r < rows; r += 32) {
-                double2 u = Vi[r], b = ws[r];
-                a.x += u.x * b.x + u.y * b.y;
-                a.y += u.x * b.y - u.y * b.x;
-            }
-            a = warp_sum(a);
-            if (lane == 0) acc[i] = cadd(acc[i], a);
-        }
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < nv; i += TB) partials[(long long)blockIdx.x * nv + i] = acc[i];
-}
-
-// out[i] (+)= sum_b partials[b * nv + i]; one warp per vector, fixed order
-__global__ void k_mdot_fin(const double2* __restrict__ partials, int nparts, int nv, double2* out, int accumulate,
-                           double2* copy) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int i = warp; i < nv; i += blockDim.x / 32) {
-        double2 a = make_double2(0, 0);
-        for (int b = lane; b < nparts; b += 32) a = cadd(a, partials[(long long)b * nv + i]);
-        a = warp_sum(a);
-        if (lane == 0) {
-            if (copy) copy[i] = a;
-            out[i] = accumulate ? cadd(out[i], a) : a;
-        }
-    }
-}
-
-// w += sign * sum_i V_i coef_i; optional ||w||^2 partials
+// w += sign * sum_i V_i coef_i (the solution update of FGMRES)
 __global__ void __launch_bounds__(TB) k_mupdate(const double2* __restrict__ V, int nv, const double2* __restrict__ coef,
-                                                double sign, double2* __restrict__ w, long long N, double* partials) {
+                                                double sign, double2* __restrict__ w, long long N) {
     __shared__ double2 c[kMaxRestart + 1];
     for (int i = threadIdx.x; i < nv; i += TB) c[i] = cscale(sign, coef[i]);
     __syncthreads();
-    double acc = 0;
     for (long long l = blockIdx.x * (long long)TB + threadIdx.x; l < N; l += (long long)gridDim.x * TB) {
         double2 s = w[l];
+#pragma unroll 4
         for (int i = 0; i < nv; ++i) {
             double2 v = V[(long long)i * N + l];
             s.x += c[i].x * v.x - c[i].y * v.y;
             s.y += c[i].x * v.y + c[i].y * v.x;
         }
         w[l] = s;
-        acc += s.x * s.x + s.y * s.y;
-    }
-    if (partials) {
-        acc = block_sum(acc);
-        if (threadIdx.x == 0) partials[blockIdx.x] = acc;
     }
 }
 
@@ -326,6 +276,7 @@ __global__ void __launch_bounds__(TB) k_mupdate32(const float2* __restrict__ V, 
     __syncthreads();
     for (long long l = blockIdx.x * (long long)TB + threadIdx.x; l < N; l += (long long)gridDim.x * TB) {
         double2 s = w[l];
+#pragma unroll 4
         for (int i = 0; i < nv; ++i) {
             float2 vf = V[(long long)i * N + l];
             double2 v = make_double2(vf.x, vf.y);
@@ -334,69 +285,6 @@ __global__ void __launch_bounds__(TB) k_mupdate32(const float2* __restrict__ V, 
         }
         w[l] = s;
     }
-}
-
-__global__ void __launch_bounds__(TB) k_scale_vec(const double2* __restrict__ w, double2* __restrict__ v,
-                                                  const double* norm2, long long N) {
-    const double nn = sqrt(*norm2);
-    if (nn == 0) return;
-    const double inv = 1.0 / nn;
-    for (long long l = blockIdx.x * (long long)TB + threadIdx.x; l < N; l += (long long)gridDim.x * TB)
-        v[l] = cscale(inv, w[l]);
-}
-
-// Givens step for column j of the Hessenberg matrix (column-major, ldh rows).
-// H[0..j, j] holds h = V^H w; wnorm2 = ||w||^2 after orthogonalisation.
-__global__ void k_givens(double2* H, int ldh, int j, double* cs, double2* sn, double2* g, const double* wnorm2,
-                         double* est) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double2* col = H + (long long)j * ldh;
-    const double hn = sqrt(*wnorm2);
-    col[j + 1] = make_double2(hn, 0);
-    for (int i = 0; i < j; ++i) {
-        double2 a = col[i], b = col[i + 1];
-        double2 s = sn[i];
-        double c = cs[i];
-        col[i] = cadd(cscale(c, a), cmul(s, b));
-        col[i + 1] = csub(cscale(c, b), cmulc(s, a));
-    }
-    double2 a = col[j], b = col[j + 1];
-    double c;
-    double2 s, r;
-    double ab = hypot(a.x, a.y), bb = hypot(b.x, b.y);
-    if (bb == 0) {
-        c = 1; s = make_double2(0, 0); r = a;
-    } else if (ab == 0) {
-        c = 0; s = make_double2(b.x / bb, -b.y / bb); r = make_double2(bb, 0);
-    } else {
-        double t = sqrt(ab * ab + bb * bb);
-        double2 ph = make_double2(a.x / ab, a.y / ab);
-        c = ab / t;
-        s = cscale(1.0 / t, cmul(ph, make_double2(b.x, -b.y)));
-        r = cscale(t, ph);
-    }
-    cs[j] = c;
-    sn[j] = s;
-    col[j] = r;
-    col[j + 1] = make_double2(0, 0);
-    double2 gj = g[j];
-    g[j + 1] = cscale(-1.0, cmulc(s, gj));
-    g[j] = cscale(c, gj);
-    *est = hypot(g[j + 1].x, g[j + 1].y);
-}
-
-__global__ void k_hsolve(const double2* H, int ldh, int k, const double2* g, double2* y) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    for (int i = k - 1; i >= 0; --i) {
-        double2 s = g[i];
-        for (int q = i + 1; q < k; ++q) s = csub(s, cmul(H[(long long)q * ldh + i], y[q]));
-        y[i] = cdiv(s, H[(long long)i * ldh + i]);
-    }
-}
-
-__global__ void k_init_g(double2* g, int m1, const double* beta2) {
-    int i = threadIdx.x;
-    if (i < m1) g[i] = make_double2(i == 0 ? sqrt(*beta2) : 0.0, 0);
 }
 
 __global__ void __launch_bounds__(TB) k_set_masked(double2* __restrict__ x, const double2* __restrict__ f,
@@ -448,34 +336,13 @@ void launch_bicg_scalar(int recipe, const double* partials, int nparts, double2*
                         cudaStream_t s) {
     k_bicg_scalar<<<1, kFinThreads, 0, s>>>(recipe, partials, nparts, sc, tol_abs);
 }
-void launch_mdot(const double2* V, int nv, const double2* w, long long N, double2* partials, cudaStream_t s) {
-    k_mdot<<<kRedBlocks, TB, 0, s>>>(V, nv, w, N, partials);
-}
 void launch_mupdate(const double2* V, int nv, const double2* coef, double sign, double2* w, long long N,
-                    double* norm_partials, cudaStream_t s) {
-    k_mupdate<<<norm_partials ? kRedBlocks : stream_blocks(N), TB, 0, s>>>(V, nv, coef, sign, w, N,
-                                                                            norm_partials);
-}
-void launch_mdot_finalize(const double2* partials, int nparts, int nv, double2* out, int accumulate,
-                          double2* copy, cudaStream_t s) {
-    k_mdot_fin<<<1, 512, 0, s>>>(partials, nparts, nv, out, accumulate, copy);
+                    cudaStream_t s) {
+    k_mupdate<<<stream_blocks(N), TB, 0, s>>>(V, nv, coef, sign, w, N);
 }
 void launch_mupdate32(const float2* V, int nv, const double2* coef, double sign, double2* w, long long N,
                       cudaStream_t s) {
     k_mupdate32<<<stream_blocks(N), TB, 0, s>>>(V, nv, coef, sign, w, N);
-}
-void launch_scale_vec(const double2* w, double2* v, const double* norm2, long long N, cudaStream_t s) {
-    k_scale_vec<<<stream_blocks(N), TB, 0, s>>>(w, v, norm2, N);
-}
-void launch_givens(double2* H, int ldh, int j, double* cs, double2* sn, double2* g, const double* wnorm2,
-                   double* est, cudaStream_t s) {
-    k_givens<<<1, 32, 0, s>>>(H, ldh, j, cs, sn, g, wnorm2, est);
-}
-void launch_hsolve(const double2* H, int ldh, int k, const double2* g, double2* y, cudaStream_t s) {
-    k_hsolve<<<1, 32, 0, s>>>(H, ldh, k, g, y);
-}
-void launch_init_g(double2* g, int m1, const double* beta2, cudaStream_t s) {
-    k_init_g<<<1, 128, 0, s>>>(g, m1, beta2);
 }
 void launch_set_masked(double2* x, const double2* f, const uint8_t* mask, long long N, cudaStream_t s) {
     k_set_masked<<<stream_blocks(N), TB, 0, s>>>(x, f, mask, N);

@@ -625,8 +625,35 @@ helm_status solve_fgmres(helm_handle* h, const helm_solve_opts* o, const double2
             h->m32_alloc = m;
         }
     }
-    double2* h2 = h->y + (kMaxRestart + 1);
+    double2* coef = h->y;                        // 2 (kMaxRestart + 1) coefficients
     int iters = 0, cycles = 0;
+    // one Arnoldi step; ends by copying the scalars into a pinned snapshot
+    auto enqueue_step = [&](int j, int slot) -> helm_status {
+        double2* Vj = h->V + (long long)j * N;
+        double2* w = h->V + (long long)(j + 1) * N;
+        const float2* w32 = nullptr;
+        if (mixed) {
+            // complex64 preconditioner and matvec (V_j rounded when it was normalised);
+            // the product is widened inside the orthogonalisation
+            float2* Z32j = h->Z32 + (long long)j * N;
+            TRY(precond32(h, o, h->tmp32[0], Z32j, o->conj));
+            launch_apply<float>(h->op32, Z32j, nullptr, h->tmp32[2], nullptr, o->conj, false, s);
+            w32 = h->tmp32[2];
+        } else {
+            double2* Zj = h->Z + (long long)j * N;
+            TRY(precond(h, o, Vj, Zj, o->conj));
+            launch_apply<double>(h->op64, Zj, nullptr, w, nullptr, o->conj, false, s);
+        }
+        // CGS2 against V_0..V_j, H column j, its Givens rotation, the normalised V_{j+1}
+        NvtxRange nvtx_a("Arnoldi CGS2 + Givens");
+        CK(launch_arnoldi(h->V, j, N, w32, w, h->Hm, ldh, h->cs, h->sn, h->g, coef, scal(h, S_WN2), scal(h, S_EST),
+                          h->hpart, h->counter, mixed ? h->tmp32[0] : nullptr, s));
+        h->launches += 5;
+        CK(cudaMemcpyAsync(h->hring + 2 * S_NSLOTS * slot, h->sc, S_NSLOTS * sizeof(double2), cudaMemcpyDeviceToHost, s));
+        CK(cudaEventRecord(h->evring[slot], s));
+        CKL();
+        return HELM_OK;
+    };
     while (true) {
         double2* V0 = h->V;
         TRY(residual_norm(h, f, x, V0, o->conj, S_BETA2));
@@ -639,60 +666,43 @@ helm_status solve_fgmres(helm_handle* h, const helm_solve_opts* o, const double2
         if (!std::isfinite(beta)) { st->status = HELM_DIVERGED; break; }
         if (iters >= o->maxit) { st->status = HELM_NOT_CONVERGED; break; }
         ++cycles;
-        launch_init_g(h->g, m + 1, scal(h, S_BETA2), s);
-        launch_scale_vec(V0, V0, scal(h, S_BETA2), N, s);
-        h->launches += 2;
-        CK(cudaMemsetAsync(h->Hm, 0, sizeof(double2) * (m + 1) * m, s));
-        int kdim = 0;
+        launch_gs_scale(V0, V0, mixed ? h->tmp32[0] : nullptr, scal(h, S_BETA2), N, h->g, m + 1, s);
+        h->launches += 1;
+        // Lagged polling: step j + 1 is queued before the host waits for the estimate of
+        // step j, so the GPU does not idle while the host decides (about 20 us a step on
+        // small grids).  If step j ends the cycle, the queued step is surplus: it writes
+        // V_{j+2}, column j + 1 of H and of the rotations, and g_{j+1}, g_{j+2}, none of
+        // which the k = j + 1 solve reads.  (Not with profiling on, whose event counts
+        // are those of the steps taken.)
+        int kdim = 0, queued = 0;
         for (int j = 0; j < m; ++j) {
-            double2* Vj = h->V + (long long)j * N;
-            double2* Zj = h->Z + (long long)j * N;
-            double2* w = h->V + (long long)(j + 1) * N;
-            double2* Hcol = h->Hm + (long long)j * ldh;
-            if (mixed) {
-                // complex64 preconditioner and matvec; the product is widened before CGS2
-                float2* Z32j = h->Z32 + (long long)j * N;
-                launch_cvt_f64_to_f32(Vj, h->tmp32[0], N, s);
-                TRY(precond32(h, o, h->tmp32[0], Z32j, o->conj));
-                launch_apply<float>(h->op32, Z32j, nullptr, h->tmp32[2], nullptr, o->conj, false, s);
-                launch_cvt_f32_to_f64(h->tmp32[2], w, N, s);
-                h->launches += 3;
-            } else {
-                TRY(precond(h, o, Vj, Zj, o->conj));
-                launch_apply<double>(h->op64, Zj, nullptr, w, nullptr, o->conj, false, s);
-                h->launches += 1;
+            if (queued == j) {
+                TRY(enqueue_step(j, j & 1));
+                queued = j + 1;
+            }
+            if (!h->profile && j + 1 < m && iters + 1 < o->maxit) {
+                TRY(enqueue_step(j + 1, (j + 1) & 1));
+                queued = j + 2;
             }
             ++st->precond_applies;
             ++st->matvecs;
-            // CGS2: h = V^H w, w -= V h, h2 = V^H w, w -= V h2, h += h2
-            NvtxRange nvtx_a("Arnoldi CGS2 + Givens");
-            launch_mdot(h->V, j + 1, w, N, h->hpart, s);
-            launch_mdot_finalize(h->hpart, kRedBlocks, j + 1, Hcol, 0, nullptr, s);
-            launch_mupdate(h->V, j + 1, Hcol, -1.0, w, N, nullptr, s);
-            launch_mdot(h->V, j + 1, w, N, h->hpart, s);
-            launch_mdot_finalize(h->hpart, kRedBlocks, j + 1, Hcol, 1, h2, s);
-            launch_mupdate(h->V, j + 1, h2, -1.0, w, N, h->red, s);
-            launch_sum_real(h->red, kRedBlocks, scal(h, S_WN2), s);
-            launch_givens(h->Hm, ldh, j, h->cs, h->sn, h->g, scal(h, S_WN2), scal(h, S_EST), s);
-            launch_scale_vec(w, w, scal(h, S_WN2), N, s);
-            h->launches += 10;
-            CKL();
             ++iters;
             kdim = j + 1;
-            TRY(poll(h));
-            if (barrier_timed_out(h)) { st->status = HELM_TIMEOUT; break; }
-            const double est = hs(h, S_EST) / bnorm;
+            CK(cudaEventSynchronize(h->evring[j & 1]));
+            const double* snap = h->hring + 2 * S_NSLOTS * (j & 1);
+            if (snap[2 * S_FLAGS + 1] == 4.0) { st->status = HELM_TIMEOUT; break; }
+            const double est = snap[2 * S_EST] / bnorm;
             hist.push(est);
-            const double wn2 = hs(h, S_WN2);
+            const double wn2 = snap[2 * S_WN2];
             if (!std::isfinite(est)) break;
             if (wn2 == 0.0 || est <= o->tol || iters >= o->maxit) break;
         }
         if (st->status == HELM_TIMEOUT) break;
-        launch_hsolve(h->Hm, ldh, kdim, h->g, h->y, s);
+        CK(launch_hsolve(h->Hm, ldh, kdim, h->g, h->y, s));
         if (mixed)
             launch_mupdate32(h->Z32, kdim, h->y, 1.0, x, N, s);
         else
-            launch_mupdate(h->Z, kdim, h->y, 1.0, x, N, nullptr, s);
+            launch_mupdate(h->Z, kdim, h->y, 1.0, x, N, s);
         h->launches += 2;
         CKL();
     }

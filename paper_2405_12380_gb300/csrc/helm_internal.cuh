@@ -84,6 +84,15 @@ __host__ __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
 __host__ __device__ __forceinline__ double2 cmulc(double2 a, double2 b) {
     return make_double2(a.x * b.x + a.y * b.y, a.x * b.y - a.y * b.x);
 }
+// c + a b and c + conj(a) b, two fused multiply-adds a component (written as c + (p q - r s)
+// the compiler needs a product, a fused multiply-add and an add)
+__device__ __forceinline__ double2 cfma(double2 a, double2 b, double2 c) {
+    return make_double2(fma(a.x, b.x, fma(-a.y, b.y, c.x)), fma(a.x, b.y, fma(a.y, b.x, c.y)));
+}
+__device__ __forceinline__ double2 cfmac(double2 a, double2 b, double2 c) {
+    return make_double2(fma(a.x, b.x, fma(a.y, b.y, c.x)), fma(a.x, b.y, fma(-a.y, b.x, c.y)));
+}
+__device__ __forceinline__ double cnorm2(double2 a, double s) { return fma(a.x, a.x, fma(a.y, a.y, s)); }
 __host__ __device__ __forceinline__ double2 cadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
 __host__ __device__ __forceinline__ double2 csub(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
 __host__ __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
@@ -243,17 +252,18 @@ void launch_bicg_update_p(const double2* r, const double2* v, double2* p, const 
 void launch_bicg_scalar(int recipe, const double* partials, int nparts, double2* sc, double tol_abs,
                         cudaStream_t s);
 // FGMRES pieces
-void launch_mdot(const double2* V, int nv, const double2* w, long long N, double2* partials,
-                 cudaStream_t s);
 void launch_mupdate(const double2* V, int nv, const double2* coef, double sign, double2* w, long long N,
-                    double* norm_partials, cudaStream_t s);
-void launch_mdot_finalize(const double2* partials, int nparts, int nv, double2* out, int accumulate,
-                          double2* copy, cudaStream_t s);
-void launch_scale_vec(const double2* w, double2* v, const double* norm2, long long N, cudaStream_t s);
-void launch_givens(double2* H, int ldh, int j, double* cs, double2* sn, double2* g, const double* wnorm2,
-                   double* est, cudaStream_t s);
-void launch_hsolve(const double2* H, int ldh, int k, const double2* g, double2* y, cudaStream_t s);
-void launch_init_g(double2* g, int m1, const double* beta2, cudaStream_t s);
+                    cudaStream_t s);
+// arnoldi.cu: column j of the Arnoldi relation.  w (or, given w32, its complex64 form,
+// widened into w) is orthogonalised against V_0..V_j by CGS2 and normalised in place;
+// H column j, the Givens rotation, g, *wnorm2 = ||w||^2 and *est follow.  coef: 2
+// (kMaxRestart + 1) entries; partials: kRedBlocks (j + 1); v32: complex64 copy or null
+cudaError_t launch_arnoldi(const double2* V, int j, long long N, const float2* w32, double2* w, double2* H, int ldh,
+                           double* cs, double2* sn, double2* g, double2* coef, double* wnorm2, double* est,
+                           double2* partials, unsigned* counter, float2* v32, cudaStream_t s);
+void launch_gs_scale(const double2* w, double2* v, float2* v32, const double* norm2, long long N, double2* g, int m1,
+                     cudaStream_t s);
+cudaError_t launch_hsolve(const double2* H, int ldh, int k, const double2* g, double2* y, cudaStream_t s);
 void launch_set_masked(double2* x, const double2* f, const uint8_t* mask, long long N, cudaStream_t s);
 void launch_cvt_f64_to_f32(const double2* a, float2* b, long long N, cudaStream_t s);
 void launch_cvt_f32_to_f64(const float2* a, double2* b, long long N, cudaStream_t s);
