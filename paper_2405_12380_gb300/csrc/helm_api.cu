@@ -342,31 +342,22 @@ helm_status precond32(helm_handle* h, const helm_solve_opts* o, const float2* v,
     }
     if (o->correction == HELM_CORR_TB) {
         if (!h->Qbf) return fail(h, HELM_NOT_READY, "trunk basis not loaded (don_load)");
-        int nblk = restrict_blocks(h->N);
         ev_mark(h, 0, 0);
-        // after the black half-sweep v - A z vanishes on black and masked rows: with
-        // the pair layout the red rows' residual is stored compactly (in the sweep
-        // buffer, free again) and projected by a plain tall-skinny product
-        if (!no_relax && o->relax == HELM_RBGS && h->Qbr &&
-            launch_red_residual32(h->op32, v, z, h->tmp32[3], conj, s)) {
-            nblk = launch_restrict32_rr(h->Qbr, basis_ld((h->N + 1) / 2), h->k, h->tmp32[3], (h->N + 1) / 2,
-                                        h->partials32, h->N, s);
-            h->launches += 1;
-        } else if (!no_relax && o->relax == HELM_RBGS && h->Qbr) {
-            // after the black half-sweep v - A z vanishes on black and masked rows:
-            // project the red rows only
-            nblk = launch_restrict32_red(h->op32, h->Qbr, basis_ld((h->N + 1) / 2), h->k, v, z, conj,
-                                         h->partials32, s);
-        } else {
-            launch_restrict32(h->op32, h->Qbf, basis_ld(h->N), h->k, v, no_relax ? nullptr : z, conj,
-                              h->partials32, nblk, s);
-        }
+        // the residual after the sweeps, stored (in the sweep buffer, free again), then a
+        // plain tall-skinny product.  After the black half-sweep of red-black Gauss-Seidel
+        // it vanishes on black and masked rows: the red rows only, compactly
+        const bool red = !no_relax && o->relax == HELM_RBGS;
+        const long long M = red ? (h->N + 1) / 2 : h->N;
+        TRY(ensure_tmp32(h, 4));
+        if (!red || !launch_red_residual32(h->op32, v, z, h->tmp32[3], conj, s))
+            launch_residual32(h->op32, v, no_relax ? nullptr : z, red, conj, h->tmp32[3], s);
+        const int nblk = launch_restrict32(red ? h->Qbr : h->Qbf, basis_ld(M), h->k, h->tmp32[3], M, h->partials32, s);
         ev_mark(h, 0, 1);
         launch_coarse_apply32(h->partials32, nblk, h->k, h->Ainv, conj, h->y32, h->cbuf, s);
         ev_mark(h, 1, 0);
         launch_prolong32(h->Qbf, basis_ld(h->N), h->k, h->y32, z, h->N, s);
         ev_mark(h, 1, 1);
-        h->launches += 4;
+        h->launches += 5;
     }
     CKL();
     return HELM_OK;
@@ -1663,11 +1654,10 @@ helm_status don_load(helm_handle* h, const double* weights, const int* widths, i
         dfree(h->Q); dfree(h->Qr); dfree(h->Ainv);
         return st;
     }
-    STEP(dalloc(h, &h->coarse_partials, (size_t)std::max(restrict_blocks(N), project_blocks(N)) * k));
+    STEP(dalloc(h, &h->coarse_partials, (size_t)project_blocks(N) * k));
     if (h->precision == HELM_MIXED) {
         dfree(h->partials32); dfree(h->y32);
-        STEP(dalloc(h, &h->partials32,
-                    (size_t)std::max({restrict_blocks(N), restrict32_red_blocks(N), restrict32_rr_ranges(N)}) * k));
+        STEP(dalloc(h, &h->partials32, (size_t)restrict32_ranges(N) * k));
         STEP(dalloc(h, &h->y32, (size_t)kMaxP));
     }
     STEP(dalloc(h, &h->cbuf, (size_t)kMaxP));

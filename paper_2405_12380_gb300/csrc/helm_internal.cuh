@@ -344,25 +344,21 @@ void launch_nl_prolong(const float* T, int p, const float* b, const double* s2, 
 // padding), complex64 vectors, FP32 accumulation
 void launch_round_bf16(double* A, int ld, int k, long long N, cudaStream_t s);
 void launch_rm_to_cm_bf16(const double* A, int ld, int k, void* B, long long ldb, long long N, cudaStream_t s);
-void launch_restrict32(const Op<float>& op, const void* Q, long long ldq, int k, const float2* v, const float2* z,
-                       int conj, float2* partials, int nblk, cudaStream_t s);
 void launch_coarse_apply32(const float2* partials, int nblk, int k, const double2* Ainv, int conj, float2* y,
                            double2* cbuf, cudaStream_t s);
 void launch_prolong32(const void* Q, long long ldq, int k, const float2* y, float2* z, long long N, cudaStream_t s);
 // the red rows of the BF16 basis (k x ceil(N / 2), stride basis_ld(ceil(N / 2)))
 void launch_red_rows_bf16(const void* Q, long long ldq, int k, long long N, int n, void* Qr, long long ldr,
                           cudaStream_t s);
-// c = Q_red^T (v - A z) over the red rows (the residual after a red-black sweep that
-// ends with the black half-sweep); returns the number of block partials written
-int restrict32_red_blocks(long long N);
-// c partials = Q_red^T r_red from a stored red-row residual (M = red rows): returns
-// the number of partial rows written (restrict32_rr_ranges(N))
-int restrict32_rr_ranges(long long N);
-int launch_restrict32_rr(const void* Qr, long long ldr, int k, const float2* r_red, long long M, float2* partials,
-                         long long N, cudaStream_t s);
-int launch_restrict32_red(const Op<float>& op, const void* Qr, long long ldr, int k, const float2* v,
-                          const float2* z, int conj, float2* partials, cudaStream_t s);
-int restrict_blocks(long long N);
+// r = v - A z (zero on masked nodes; z may be null: v) on every row, or on the red row of
+// each node pair; then c partials = Q^T r over its M rows with the BF16 basis (all rows:
+// stride basis_ld(N); red rows: basis_ld(ceil(N / 2))): returns the number of partial
+// rows written, restrict32_ranges(M)
+void launch_residual32(const Op<float>& op, const float2* v, const float2* z, bool red, int conj, float2* r,
+                       cudaStream_t s);
+int restrict32_ranges(long long M);
+int launch_restrict32(const void* Q, long long ld, int k, const float2* r, long long M, float2* partials,
+                      cudaStream_t s);
 
 // mg.cu: grid transfers of the multigrid V-cycle (n_f = 2 n_c - 1, coarse node I at fine 2I)
 void launch_inject_mask(int dim, int nf, const uint8_t* fine, uint8_t* coarse, cudaStream_t s);

@@ -435,8 +435,6 @@ __global__ void __launch_bounds__(1024) k_gauss_jordan(const double* __restrict_
 
 // ---------------------------------------------------------- per application
 // Q is column-major here: basis vector j occupies Q[j*N .. j*N + N).
-constexpr int RS_T = 256;        // threads per restriction block
-constexpr int RS_TILE = 256;     // rows per tile (one residual per thread)
 
 // ---------------------------------------------- FP32-pair (df64) projection
 // GB300 issues FP32 FMAs 64x faster than FP64 ones, so the FP64 restriction and
@@ -838,85 +836,6 @@ __global__ void k_rm_to_cm_bf16(const double* __restrict__ A, int ld, int k, __n
     }
 }
 
-// complex64 restriction with a BF16 basis, FP32 accumulation: same structure as k_restrict
-template <int KPW>
-__global__ void __launch_bounds__(RS_T) k_restrict32(Op<float> op, const __nv_bfloat16* __restrict__ Q, long long ldq, int k,
-                                                     const float2* __restrict__ v, const float2* __restrict__ z,
-                                                     int conj, float2* __restrict__ partials,
-                                                     long long rows_per_block) {
-    __shared__ float2 rs[RS_TILE];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    constexpr int NW = RS_T / 32;
-    const long long r0 = (long long)blockIdx.x * rows_per_block;
-    const long long r1 = min(op.N, r0 + rows_per_block);
-    const long long N = op.N;
-    float2 acc[KPW];
-#pragma unroll
-    for (int c = 0; c < KPW; ++c) acc[c] = make_float2(0.f, 0.f);
-    const long long sy = op.n, sz = (long long)op.n * op.n;
-    for (long long t0 = r0; t0 < r1; t0 += RS_TILE) {
-        const long long l = t0 + threadIdx.x;
-        float2 r = make_float2(0.f, 0.f);
-        if (l < r1 && !op.mask[l]) {
-            r = v[l];
-            if (z) {
-                float2 s = make_float2(0.f, 0.f);
-                const uint8_t* mk = op.mask;
-                if (!mk[l - 1]) s = cadd(s, z[l - 1]);
-                if (!mk[l + 1]) s = cadd(s, z[l + 1]);
-                if (!mk[l - sy]) s = cadd(s, z[l - sy]);
-                if (!mk[l + sy]) s = cadd(s, z[l + sy]);
-                if (op.dim == 3) {
-                    if (!mk[l - sz]) s = cadd(s, z[l - sz]);
-                    if (!mk[l + sz]) s = cadd(s, z[l + sz]);
-                }
-                float2 d;
-                if (op.k2) {
-                    d = op.k2[l];
-                    d.x -= 2.0f * op.dim * op.hinv2;
-                } else {
-                    d = make_float2(op.dre, op.im[op.lidx[l]]);
-                }
-                if (conj) d.y = -d.y;
-                const float2 zc = z[l];
-                r.x -= op.hinv2 * s.x + (d.x * zc.x - d.y * zc.y);
-                r.y -= op.hinv2 * s.y + (d.x * zc.y + d.y * zc.x);
-            }
-        }
-        __syncthreads();
-        rs[threadIdx.x] = r;
-        __syncthreads();
-        const int rows = (int)min((long long)RS_TILE, r1 - t0);
-#pragma unroll
-        for (int c = 0; c < KPW; ++c) {
-            const int j = warp + NW * c;
-            if (j < k) {
-                const __nv_bfloat16* Qj = Q + (long long)j * ldq + t0;
-                float ax = acc[c].x, ay = acc[c].y;
-                for (int q = lane; q < rows; q += 32) {
-                    const float qv = __bfloat162float(Qj[q]);
-                    const float2 rr = rs[q];
-                    ax = fmaf(qv, rr.x, ax);
-                    ay = fmaf(qv, rr.y, ay);
-                }
-                acc[c].x = ax;
-                acc[c].y = ay;
-            }
-        }
-    }
-#pragma unroll
-    for (int c = 0; c < KPW; ++c) {
-        const int j = warp + NW * c;
-        float sx = acc[c].x, sy2 = acc[c].y;
-        for (int o = 16; o > 0; o >>= 1) {
-            sx += __shfl_xor_sync(0xffffffffu, sx, o);
-            sy2 += __shfl_xor_sync(0xffffffffu, sy2, o);
-        }
-        if (lane == 0 && j < k) partials[(long long)blockIdx.x * k + j] = make_float2(sx, sy2);
-    }
-}
-
-
 __global__ void __launch_bounds__(256) k_prolong32(const __nv_bfloat16* __restrict__ Q, long long ldq, int k,
                                                    const float2* __restrict__ y, float2* __restrict__ z, long long N) {
     __shared__ float2 ys[kMaxP];
@@ -961,10 +880,9 @@ __global__ void k_red_rows_bf16(const __nv_bfloat16* __restrict__ Q, long long l
     }
 }
 
-// (v - A z) at the red node of pair m (complex64); zero on masked nodes and past N
-__device__ __forceinline__ float2 red_residual32(const Op<float>& op, const float2* __restrict__ v,
-                                                 const float2* __restrict__ z, long long m, int conj) {
-    const long long l = 2 * m + node_colour(2 * m, op.n);
+// (v - A z) at node l (complex64); zero on masked nodes and past N
+__device__ __forceinline__ float2 row_residual32(const Op<float>& op, const float2* __restrict__ v,
+                                                 const float2* __restrict__ z, long long l, int conj) {
     if (l >= op.N) return make_float2(0.f, 0.f);
     const unsigned code = op.nbm[l];
     if (code & 0x80u) return make_float2(0.f, 0.f);
@@ -991,88 +909,23 @@ __device__ __forceinline__ float2 red_residual32(const Op<float>& op, const floa
                        vv.y - (op.hinv2 * s.y + (d.x * zc.y + d.y * zc.x)));
 }
 
-constexpr int RR_T = 256;     // threads of the red-row restriction
-constexpr int RR_ROWS = 8;    // consecutive red rows per thread (one 16-byte basis load per column)
-constexpr int RR_KC = 8;      // columns per chunk (registers)
-
-// c = Q_red^T r with r = v - A z on the red rows (after a red-black sweep that ends
-// with the black half-sweep the residual vanishes on black and masked rows).  A
-// warp takes 32 x 8 consecutive red rows; per chunk of 8 columns each lane sums its
-// 8 rows in FP32, the warp adds its lanes (fixed butterfly) and lane 0 adds the
-// chunk into the warp's row of shared memory; at the end the block sums its warps
-// in a fixed order into partials[block][j].  Deterministic.
-__global__ void __launch_bounds__(RR_T, 4) k_restrict32_red(Op<float> op, const __nv_bfloat16* __restrict__ Qr,
-                                                         long long ldr, int k, const float2* __restrict__ v,
-                                                         const float2* __restrict__ z, int conj,
-                                                         float2* __restrict__ partials, long long M) {
-    constexpr int NW = RR_T / 32;
-    constexpr int WROWS = 32 * RR_ROWS;            // red rows of one warp tile
-    __shared__ float2 sacc[NW][kMaxP];
-    // the warp tile's residuals, 8 rows per lane with one padding slot per lane
-    __shared__ float2 rsm[NW][32 * (RR_ROWS + 1)];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int j = lane; j < k; j += 32) sacc[warp][j] = make_float2(0.f, 0.f);
-    __syncwarp();
-    const long long groups = (M + RR_ROWS - 1) / RR_ROWS;
-    const long long wtiles = (groups + 31) / 32;
-    for (long long wt = blockIdx.x * (long long)NW + warp; wt < wtiles; wt += (long long)gridDim.x * NW) {
-        // residuals of the tile's rows computed with consecutive rows on consecutive
-        // lanes (coalesced neighbour loads), then read back eight consecutive rows per lane
-        const long long mt = wt * WROWS;
-#pragma unroll
-        for (int q = 0; q < RR_ROWS; ++q) {
-            const int row = lane + 32 * q;
-            const long long m = mt + row;
-            rsm[warp][row + row / RR_ROWS] = (m < M) ? red_residual32(op, v, z, m, conj) : make_float2(0.f, 0.f);
-        }
-        __syncwarp();
-        const long long m0 = mt + (long long)lane * RR_ROWS;
-        float2 r[RR_ROWS];
-#pragma unroll
-        for (int q = 0; q < RR_ROWS; ++q) r[q] = rsm[warp][lane * (RR_ROWS + 1) + q];
-        __syncwarp();
-        for (int c0 = 0; c0 < k; c0 += RR_KC) {
-            float ax[RR_KC], ay[RR_KC];
-#pragma unroll
-            for (int c = 0; c < RR_KC; ++c) {
-                ax[c] = 0.f;
-                ay[c] = 0.f;
-                if (c0 + c < k && m0 < M) {
-                    const uint4 u = __ldcs(reinterpret_cast<const uint4*>(Qr + (long long)(c0 + c) * ldr + m0));
-                    float qv[8];
-                    bf16x8(u, qv);
-#pragma unroll
-                    for (int q = 0; q < RR_ROWS; ++q) {
-                        ax[c] = fmaf(qv[q], r[q].x, ax[c]);
-                        ay[c] = fmaf(qv[q], r[q].y, ay[c]);
-                    }
-                }
-            }
-#pragma unroll
-            for (int c = 0; c < RR_KC; ++c)
-                for (int o = 16; o > 0; o >>= 1) {
-                    ax[c] += __shfl_xor_sync(0xffffffffu, ax[c], o);
-                    ay[c] += __shfl_xor_sync(0xffffffffu, ay[c], o);
-                }
-            if (lane == 0)
-#pragma unroll
-                for (int c = 0; c < RR_KC; ++c)
-                    if (c0 + c < k) {
-                        sacc[warp][c0 + c].x += ax[c];
-                        sacc[warp][c0 + c].y += ay[c];
-                    }
-        }
-    }
-    __syncthreads();
-    for (int j = threadIdx.x; j < k; j += RR_T) {
-        float2 t = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int w = 0; w < NW; ++w) t = cadd(t, sacc[w][j]);
-        partials[(long long)blockIdx.x * k + j] = t;
+// the residual that the restriction projects, where the pair layout does not apply (odd n,
+// 2D, unaligned vectors) or the sweep leaves residual on both colours: RED, the red row of
+// every node pair (M = ceil(N / 2) rows); else every row (M = N; z may be null: v itself).
+// Zero on masked nodes.  Consecutive rows on consecutive lanes, so the neighbour loads
+// coalesce; forming the residual inside the projection (81 blocks at 97^3) took 30 us,
+// the two launches 6 + 5 us.
+template <bool RED>
+__global__ void __launch_bounds__(256) k_residual32(Op<float> op, const float2* __restrict__ v,
+                                                    const float2* __restrict__ z, int conj, float2* __restrict__ r,
+                                                    long long M) {
+    for (long long m = blockIdx.x * 256LL + threadIdx.x; m < M; m += gridDim.x * 256LL) {
+        if (RED || z) r[m] = row_residual32(op, v, z, RED ? 2 * m + node_colour(2 * m, op.n) : m, conj);
+        else r[m] = op.mask[m] ? make_float2(0.f, 0.f) : v[m];
     }
 }
 
-// c = Q_red^T r_red from a stored red-row residual: a tall-skinny product.  A warp
+// c = Q^T r from a stored residual (red rows or all rows): a tall-skinny product.  A warp
 // owns RQ_COLS columns and one range of RQ_RANGE rows; per 256 rows each lane loads
 // its 8 consecutive residual rows and then all its 16-byte basis pieces (one per
 // column, issued together) before the FMAs, and keeps the complex sums in
@@ -1080,7 +933,7 @@ __global__ void __launch_bounds__(RR_T, 4) k_restrict32_red(Op<float> op, const 
 // and lane 0 writes partials[range][j].  Deterministic.
 constexpr int RQ_COLS = 8;
 constexpr int RQ_RANGE = 1024;
-__global__ void __launch_bounds__(256) k_restrict32_rr(const __nv_bfloat16* __restrict__ Qr, long long ldr, int k,
+__global__ void __launch_bounds__(256) k_restrict32(const __nv_bfloat16* __restrict__ Qr, long long ldr, int k,
                                                        const float2* __restrict__ r, long long M,
                                                        float2* __restrict__ partials, int S) {
     const int lane = threadIdx.x & 31;
@@ -1254,18 +1107,12 @@ void launch_gauss_jordan(const double* C, int ldc, int k, double2* Ainv, double2
     k_gauss_jordan<<<1, 1024, 0, s>>>(C, ldc, k, Ainv, work, flag);
 }
 
-int restrict_blocks(long long N) {
-    long long b = (N + RS_TILE - 1) / RS_TILE;
-    return (int)(b < 2 * 152 ? (b < 1 ? 1 : b) : 2 * 152);
-}
-
 void launch_coarse_apply(const double2* partials, int nblk, int k, const double2* Ainv, int conj, double2* y,
                          double2* cbuf, cudaStream_t s) {
     // two small launches spread over k SMs (FP64 is 2 FMA/clk per SM: one CTA would serialise)
     k_coarse_reduce<<<k, 64, 0, s>>>(partials, nblk, k, cbuf);
     k_coarse_gemv<<<k, 64, 0, s>>>(Ainv, k, conj, cbuf, y);
 }
-
 
 int project_blocks(long long N) {
     long long b = (N + PJ_TILE - 1) / PJ_TILE;
@@ -1356,47 +1203,22 @@ void launch_red_rows_bf16(const void* Q, long long ldq, int k, long long N, int 
                                             static_cast<__nv_bfloat16*>(Qr), ldr);
 }
 
-int restrict32_red_blocks(long long N) {
-    const long long M = (N + 1) / 2;
-    const long long wtiles = ((M + RR_ROWS - 1) / RR_ROWS + 31) / 32;
-    const long long b = (wtiles + RR_T / 32 - 1) / (RR_T / 32);
-    return (int)(b < 4 * 152 ? (b < 1 ? 1 : b) : 4 * 152);
+void launch_residual32(const Op<float>& op, const float2* v, const float2* z, bool red, int conj, float2* r,
+                       cudaStream_t s) {
+    const long long M = red ? (op.N + 1) / 2 : op.N;
+    const unsigned b = (unsigned)std::min<long long>((M + 255) / 256, 16 * 152);
+    if (red) k_residual32<true><<<b, 256, 0, s>>>(op, v, z, conj, r, M);
+    else k_residual32<false><<<b, 256, 0, s>>>(op, v, z, conj, r, M);
 }
 
-int launch_restrict32_red(const Op<float>& op, const void* Qr, long long ldr, int k, const float2* v,
-                          const float2* z, int conj, float2* partials, cudaStream_t s) {
-    const int nb = restrict32_red_blocks(op.N);
-    k_restrict32_red<<<nb, RR_T, 0, s>>>(op, static_cast<const __nv_bfloat16*>(Qr), ldr, k, v, z, conj, partials,
-                                         (op.N + 1) / 2);
-    return nb;
-}
+int restrict32_ranges(long long M) { return (int)std::max<long long>(1, (M + RQ_RANGE - 1) / RQ_RANGE); }
 
-int restrict32_rr_ranges(long long N) {
-    const long long M = (N + 1) / 2;
-    return (int)std::max<long long>(1, (M + RQ_RANGE - 1) / RQ_RANGE);
-}
-
-int launch_restrict32_rr(const void* Qr, long long ldr, int k, const float2* r_red, long long M, float2* partials,
-                         long long N, cudaStream_t s) {
-    const int S = restrict32_rr_ranges(N);
+int launch_restrict32(const void* Q, long long ld, int k, const float2* r, long long M, float2* partials,
+                      cudaStream_t s) {
+    const int S = restrict32_ranges(M);
     const dim3 g((S + 7) / 8, (k + RQ_COLS - 1) / RQ_COLS);
-    k_restrict32_rr<<<g, 256, 0, s>>>(static_cast<const __nv_bfloat16*>(Qr), ldr, k, r_red, M, partials, S);
+    k_restrict32<<<g, 256, 0, s>>>(static_cast<const __nv_bfloat16*>(Q), ld, k, r, M, partials, S);
     return S;
-}
-
-void launch_restrict32(const Op<float>& op, const void* Qv, long long ldq, int k, const float2* v, const float2* z,
-                       int conj, float2* partials, int nblk, cudaStream_t s) {
-    const __nv_bfloat16* Q = static_cast<const __nv_bfloat16*>(Qv);
-    long long rows = (op.N + nblk - 1) / nblk;
-    const int kpw = (k + 7) / 8;
-#define RS_CASE(K) k_restrict32<K><<<nblk, RS_T, 0, s>>>(op, Q, ldq, k, v, z, conj, partials, rows)
-    if (kpw <= 1) RS_CASE(1);
-    else if (kpw <= 2) RS_CASE(2);
-    else if (kpw <= 4) RS_CASE(4);
-    else if (kpw <= 8) RS_CASE(8);
-    else if (kpw <= 16) RS_CASE(16);
-    else RS_CASE(32);
-#undef RS_CASE
 }
 
 void launch_coarse_apply32(const float2* partials, int nblk, int k, const double2* Ainv, int conj, float2* y,
