@@ -1169,9 +1169,8 @@ void fill_tables(helm_handle* h) {
         const float2 re = split(o.invd_tab[m].x), im = split(o.invd_tab[m].y);
         t.invd[m] = make_float4(re.x, re.y, im.x, im.y);
     }
-    // the fused sweep's launch shape queries the occupancy once per row width: here,
-    // outside any stream capture
-    (void)rbgs_sweep32_ok(f, nullptr, nullptr, nullptr);
+    o.ncl = f.ncl = h->ncl;
+    plan_sweep32(f);
 }
 
 // A_c = Q^T (A Q) and its inverse from a node-major copy of Q (N x ldq)
@@ -1283,6 +1282,7 @@ helm_status helm_create(int dim, int n, double k0, int layer_cells, double layer
     }
     if (dalloc(h, &h->lidx, (size_t)N) != HELM_OK) return bail(HELM_OUT_OF_MEMORY);
     if (dalloc(h, &h->nbm, (size_t)N) != HELM_OK) return bail(HELM_OUT_OF_MEMORY);
+    if (dim == 3 && n % 2 == 0 && n <= 256 && dalloc(h, &h->ncl, (size_t)N) != HELM_OK) return bail(HELM_OUT_OF_MEMORY);
     fill_tables(h);
     launch_layer_index(h->op64, h->lidx, nullptr);
     if (k2) {
@@ -1297,6 +1297,7 @@ helm_status helm_create(int dim, int n, double k0, int layer_cells, double layer
     if (cudaDeviceSynchronize() != cudaSuccess) return bail(HELM_CUDA_ERROR);
     if (bad) return bail(HELM_BAD_ARG);
     launch_nbr_code(h->op64, h->nbm, nullptr);
+    if (h->ncl) launch_node_pack(h->op32, h->ncl, nullptr);
     if (cudaDeviceSynchronize() != cudaSuccess) return bail(HELM_CUDA_ERROR);
     cudaEventCreate(&h->ev0);
     cudaEventCreate(&h->ev1);
@@ -1382,7 +1383,7 @@ helm_status helm_destroy(helm_handle* h) {
     if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
     for (helm_handle* c : h->mg) helm_destroy(c);
     h->mg.clear();
-    dfree(h->mask); dfree(h->lidx); dfree(h->nbm); dfree(h->face); dfree(h->k2); dfree(h->invd); dfree(h->k2f);
+    dfree(h->mask); dfree(h->lidx); dfree(h->nbm); dfree(h->ncl); dfree(h->face); dfree(h->k2); dfree(h->invd); dfree(h->k2f);
     dfree(h->invdf);
     dfree(h->red); dfree(h->sc); dfree(h->dflag); dfree(h->counter); dfree(h->fparts);
     if (h->hpin) cudaFreeHost(h->hpin);

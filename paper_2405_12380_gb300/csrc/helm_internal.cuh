@@ -119,6 +119,8 @@ struct Op {
     const uint8_t* mask;
     const uint8_t* lidx;     // per-node layer index m (flat-index kernels; avoids index division)
     const uint8_t* nbm;      // per-node neighbour code: bit q = neighbour q fluid, 0x80 = masked node
+    const uint16_t* ncl;     // code | layer index << 8 (3D grids of the fused complex64 sweep) or nullptr
+    int sw_rows, sw_zc;      // launch shape of the fused sweep (plan_sweep32; 0 rows: not used)
     const C* k2;             // stored k^2 field or nullptr
     const C* invd;           // per-node 1/diag for the stored field, or nullptr
     // Sommerfeld / Neumann outer boundary (helm_create_bvp) or nullptr: per node
@@ -176,6 +178,8 @@ void launch_rbgs_half(const Op<R>& op, int colour, const typename CT<R>::T* f, t
 bool launch_rbgs_sweep32(const Op<float>& op, int c0, const float2* f, const float2* xin, float2* xout, int conj,
                          double omega, cudaStream_t s);
 bool rbgs_sweep32_ok(const Op<float>& op, const void* f, const void* x, const void* tmp);
+void plan_sweep32(Op<float>& op);     // sets op.sw_rows, op.sw_zc (occupancy queries: outside stream capture)
+void launch_node_pack(const Op<float>& op, uint16_t* ncl, cudaStream_t s);
 // r_red[q] = (f - A x) at the red node of pair q (the pair layout: 3D, n even; the
 // red rows in the order of the red-row basis copy), zero on masked nodes; false
 // without launching where the pair layout does not apply
@@ -394,6 +398,7 @@ struct helm_handle {
     uint8_t* mask = nullptr;
     uint8_t* lidx = nullptr;
     uint8_t* nbm = nullptr;
+    uint16_t* ncl = nullptr;        // packed tables of the fused complex64 sweep (3D, even n <= 256)
     uint8_t* face = nullptr;        // outer-boundary problem (helm_create_bvp): face bytes
     int bvp = 0, neumann_top = 0;
     double2* k2 = nullptr;

@@ -557,43 +557,54 @@ __global__ void __launch_bounds__(BX * BY) k_rbgs_c64(Op<float> op, int zc, int 
 
 // ---- one full red-black sweep per launch (complex64, 3D, n even, pair layout)
 //
-// Colour c0 on every node, then colour 1 - c0, read from xin and written to xout
-// (out of place).  A block owns whole x-rows: blockDim.x threads over the n/2
-// pairs of a row (a multiple of 32), blockDim.y = BYI + 2 rows, of which the first
-// and last are halo rows: they compute the colour-c0 values of the rows just
-// outside the block, which the block's own second-colour nodes need, instead of
-// waiting for the neighbouring block.  Each thread marches in z over its pair.
+// Colour A (c0) on every node, then colour B (1 - c0), read from xin and written to xout
+// (out of place).  A block owns whole x-rows: blockDim.x threads over the n/2 pairs of a
+// row (a multiple of 32), blockDim.y = BYI + 2 rows, of which the first and last are halo
+// rows: they compute the colour-A values of the rows just outside the block, which the
+// block's own colour-B nodes need, instead of waiting for the neighbouring block.  Each
+// thread marches in z over its pair; blocks split z into chunks and recompute the
+// colour-A planes just outside their chunk.
 //
-// Old values are staged in shared memory: a ring of five z-planes of the block's rows
-// plus one more row on each side (the y-neighbours of the halo rows), filled by
-// asynchronous copies (cp.async, 16 bytes per thread and row) issued two planes
-// ahead, so that no neighbour read waits on global memory and the staging holds no
-// registers.  At step t a thread updates colour c0 at plane t from the staged planes
-// t - 1, t, t + 1 and puts the new value in a ring of three shared planes; after one
-// barrier it updates colour 1 - c0 at plane t - 1 from the new colour-c0 values
-// (x and y neighbours from the shared plane, z neighbours from its registers) and
-// writes the pair.  Blocks split z into chunks and recompute the colour-c0 planes
-// just outside their chunk.  1/diag of the layer comes from a shared copy of the
-// per-layer table.  Every node value comes from the arithmetic of k_rbgs_c64
-// (gs_value) with the neighbour sums in the same order, so one launch equals two
-// half-sweeps.
-__device__ __forceinline__ float2 pair_node(float4 v, int a) { return a ? hi2(v) : lo2(v); }
+// The kernel is bound by instruction issue before it is bound by HBM, so everything is
+// kept split by colour rather than by position in the pair: which of a pair's two nodes is
+// colour A alternates with row and plane, and only the loads of f and the tables and the
+// store of the result swap by it.  All six neighbours of a node have the other colour, so
+//  - only the colour-B half of xin is ever a neighbour: it is staged in shared memory, 8
+//    bytes a pair, by asynchronous copies issued three planes ahead (a ring of four planes
+//    of the block's rows plus one more row on each side);
+//  - new colour-A values go to a ring of three shared planes; after one barrier the thread
+//    updates colour B one plane behind;
+//  - in both, one x-neighbour is the thread's own pair, the other the pair to the left or
+//    right (alternating with the plane), y-neighbours are one row away, z-neighbours are
+//    the thread's own values of the planes before and after.
+// Old values of the swept nodes themselves are read only for SOR.  A node with all six
+// neighbours fluid (the common case) takes no selects.  Every node value comes from the
+// arithmetic of k_rbgs_c64 with the neighbour sums in the same order, so one launch equals
+// two half-sweeps.  Measured against the form that staged whole pairs and selected by
+// position (431 instructions a pair at 256^3; ncu, cold): 256^3 133 -> 83 us a sweep (5.3
+// TB/s of the 26 B a node), 128^3 20.5 -> 15.2 us, 64^3 13.2 -> 6.3 us.  The launch shape
+// is chosen by plan_sweep32.
 
-// neighbour sum of one node from its six neighbour values (code bits select the
-// fluid ones), in the order of pair_sums
-__device__ __forceinline__ float2 six_sum(unsigned c, float2 xm, float2 xp, float2 ym, float2 yp, float2 zm,
+// neighbour sum of the node at position a of its pair: own, the pair's other node; side, the
+// node across the pair's end (code bits select the fluid ones); the order of pair_sums
+__device__ __forceinline__ float2 six_sum(unsigned c, int a, float2 own, float2 side, float2 ym, float2 yp, float2 zm,
                                           float2 zp) {
-    if ((c & 0x3Fu) == 0x3Fu) return cadd(cadd(cadd(xm, xp), cadd(ym, yp)), cadd(zm, zp));
-    return cadd(cadd(cadd(pick(c, 1u, xm), pick(c, 2u, xp)), cadd(pick(c, 4u, ym), pick(c, 8u, yp))),
-                cadd(pick(c, 16u, zm), pick(c, 32u, zp)));
+    if ((c & 0x3Fu) != 0x3Fu) {
+        own = pick(c, a ? 1u : 2u, own);
+        side = pick(c, a ? 2u : 1u, side);
+        ym = pick(c, 4u, ym);
+        yp = pick(c, 8u, yp);
+        zm = pick(c, 16u, zm);
+        zp = pick(c, 32u, zp);
+    }
+    return cadd(cadd(cadd(own, side), cadd(ym, yp)), cadd(zm, zp));
 }
 
-// 16-byte asynchronous copy global -> shared (L2 only); valid = false fills zeros
-// without reading (src must still be a mapped address)
-__device__ __forceinline__ void cp_async16(void* dst, const void* src, bool valid) {
+// 8-byte asynchronous copy global -> shared; valid = false fills zeros without reading
+// (src must still be a mapped address)
+__device__ __forceinline__ void cp_async8(void* dst, const void* src, bool valid) {
     const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(d), "l"(src), "r"(valid ? 16 : 0)
-                 : "memory");
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(d), "l"(src), "r"(valid ? 8 : 0) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 // wait until at most N of this thread's copy groups are still in flight
@@ -603,33 +614,20 @@ __device__ __forceinline__ void cp_async_wait() {
 }
 
 constexpr int kSweepMaxThreads = 1024;
-constexpr int kSweepXPlanes = 5;     // staged old-value planes: t - 1, t, t + 1, and two in flight
-
-// 1/diag of node a of the pair at pair index l with layer byte m: the stored field's
-// per-node value, or the shared copy of the layer table (conjugated already)
-__device__ __forceinline__ float2 sweep_invd(const Op<float>& op, const float2* stab, int l, int a, unsigned m,
-                                             int conj) {
-    if (op.k2) {
-        const float4 iv = reinterpret_cast<const float4*>(op.invd)[HCHK(l, op.N >> 1)];
-        float2 id = a ? hi2(iv) : lo2(iv);
-        if (conj) id.y = -id.y;
-        return id;
-    }
-    return stab[HCHK(m, kMaxLayerCells + 1)];
-}
+constexpr int kSweepXPlanes = 4;     // staged planes: t, t + 1, and two in flight
 
 // dynamic shared memory of k_sweep_c64 for a block of txt x tyt threads
 __host__ __device__ constexpr size_t sweep_smem_bytes(int txt, int tyt, bool xzero) {
-    return (xzero ? 0 : (size_t)kSweepXPlanes * (tyt + 2) * txt * sizeof(float4)) +
-           (size_t)3 * tyt * txt * sizeof(float2) + (size_t)(kMaxLayerCells + 1) * sizeof(float2);
+    return ((xzero ? 0 : (size_t)kSweepXPlanes * (tyt + 2) * txt) + (size_t)3 * tyt * txt + kMaxLayerCells + 1) *
+           sizeof(float2);
 }
 
-template <bool XZERO>
+template <bool XZERO, bool SOR, bool K2>
 __global__ void __launch_bounds__(kSweepMaxThreads, 1)
-    k_sweep_c64(Op<float> op, int zc, int c0, const float4* __restrict__ f, const float4* __restrict__ xin,
+    k_sweep_c64(Op<float> op, int zc, int c0, const float4* __restrict__ f, const float2* __restrict__ xin,
                 float4* __restrict__ xout, int conj, float omega) {
-    extern __shared__ float4 sweep_smem[];
-    constexpr unsigned kMM = kMasked | (kMasked << 8);
+    extern __shared__ __align__(16) float2 sweep_smem[];
+    constexpr unsigned kOut = kMasked | (kMasked << 16);   // (code, layer) byte pairs of two masked nodes
     const int n = op.n, h = n >> 1;
     const int TXT = blockDim.x, TYT = blockDim.y, BYI = TYT - 2;
     const int i2 = threadIdx.x, ty = threadIdx.y;
@@ -642,130 +640,148 @@ __global__ void __launch_bounds__(kSweepMaxThreads, 1)
     [[maybe_unused]] const long long NP = op.N >> 1;
     const int RS = TYT + 2;                                // staged rows j0 - 2 .. j0 + BYI + 1
     const int PX = RS * TXT, PR = TYT * TXT;
-    float4* xs = sweep_smem;                               // [5][RS][TXT] old pairs (not with XZERO)
-    float2* ring = reinterpret_cast<float2*>(sweep_smem + (XZERO ? 0 : kSweepXPlanes * PX));   // [3][TYT][TXT]
+    float2* xs = sweep_smem;                               // [4][RS][TXT] old colour-B values (not with XZERO)
+    float2* ring = sweep_smem + (XZERO ? 0 : kSweepXPlanes * PX);   // [3][TYT][TXT] new colour-A values
     float2* stab = ring + 3 * PR;                          // 1/diag by layer index
     const int me = ty * TXT + i2;                          // this thread in a ring plane
-    const int mx = (ty + 1) * TXT + i2;                    // this thread's row in a staged plane
-    const int im1 = i2 > 0 ? -1 : 0, ip1 = i2 + 1 < TXT ? 1 : 0;
-    const unsigned short* code2 = reinterpret_cast<const unsigned short*>(op.nbm);
-    const unsigned short* lidx2 = reinterpret_cast<const unsigned short*>(op.lidx);
-    const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    const int mx = me + TXT;                               // this thread's row in a staged plane
+    const unsigned* cl2 = reinterpret_cast<const unsigned*>(op.ncl);
     const float2 z2 = make_float2(0.f, 0.f);
     const int lrow = i2 + h * j;
-    for (int q = ty * TXT + i2; q <= op.L && q <= kMaxLayerCells; q += TXT * TYT) {
-        float2 v = op.invd_tab[q];
-        if (conj) v.y = -v.y;
-        stab[q] = v;
-    }
-    // staged rows of this thread: its own, and the outer row next to a halo row
-    const int jx = ty == 0 ? j0 - 2 : (ty == TYT - 1 ? j0 + BYI + 1 : -1);
-    const int mo = (ty == 0 ? 0 : RS - 1) * TXT + i2;
-    // stage plane p (zeros outside the grid) into the staged plane at offset so
-    const bool out_ok = jx != -1 && i2 < h && jx >= 0 && jx < n;
-    const int lout = i2 + h * jx;
-    auto stage = [&](int p, int so) {
-        const bool pin = p >= 0 && p < n;
-        cp_async16(xs + so + mx, xin + HCHK(pin && row_ok ? lrow + sz * p : 0, NP), pin && row_ok);
-        if (jx != -1) cp_async16(xs + so + mo, xin + HCHK(pin && out_ok ? lout + sz * p : 0, NP), pin && out_ok);
-    };
+    if (!K2)
+        for (int q = me; q <= op.L && q <= kMaxLayerCells; q += PR) {
+            float2 v = op.invd_tab[q];
+            if (conj) v.y = -v.y;
+            stab[q] = v;
+        }
     int t = k0 - 1;
-    auto in_t = [&](int q) { return row_ok && q >= 0 && q < n; };
-    // offsets of the staged planes t - 1, t, t + 1, t + 2 (in flight) and of the free
-    // slot that plane t + 3 goes to (rotated every step: no index arithmetic per access)
-    int o_m1 = 0, o_0 = PX, o_p1 = 2 * PX, o_p2 = 3 * PX, o_p3 = 4 * PX;
+    int ar = c0 ^ ((j + t) & 1);                           // position of the colour-A node at plane t
+    // staged rows of this thread: its own, and the outer row next to a halo row
+    const int jx = ty == 0 ? j0 - 2 : j0 + BYI + 1;
+    const bool halo = !XZERO && (ty == 0 || ty == TYT - 1);
+    const bool out_ok = halo && i2 < h && jx >= 0 && jx < n;
+    const int mo = (ty == 0 ? 0 : RS - 1) * TXT + i2;
+    const int lout = i2 + h * jx;
+    // stage plane p (zeros outside the grid) at offset so; a: position of colour A there
+    auto stage = [&](int p, int so, int a) {
+        const bool pin = p >= 0 && p < n;
+        cp_async8(xs + so + mx, xin + HCHK(pin && row_ok ? 2 * (lrow + sz * p) + (a ^ 1) : 0, op.N), pin && row_ok);
+        if (halo) cp_async8(xs + so + mo, xin + HCHK(pin && out_ok ? 2 * (lout + sz * p) + a : 0, op.N), pin && out_ok);
+    };
+    int o_0 = 0, o_p1 = PX, o_p2 = 2 * PX, o_p3 = 3 * PX;
     if (!XZERO) {
-        stage(t - 1, o_m1);
-        stage(t, o_0);
-        stage(t + 1, o_p1);
+        stage(t, o_0, ar);
+        stage(t + 1, o_p1, ar ^ 1);
         cp_async_commit();
-        stage(t + 2, o_p2);
+        stage(t + 2, o_p2, ar);
         cp_async_commit();
         cp_async_wait<1>();
     }
-    float4 fc = in_t(t) ? f[HCHK(lrow + sz * t, NP)] : z4;
-    unsigned cc = in_t(t) ? (unsigned)code2[HCHK(lrow + sz * t, NP)] : kMM;
-    unsigned lc = in_t(t) ? (unsigned)lidx2[HCHK(lrow + sz * t, NP)] : 0u;
-    float2 rm2 = z2, rm = z2;                              // new colour-c0 values at planes t-2, t-1
-    // the colour-(1 - c0) node of this thread's pair at plane t - 1: f, old value,
-    // code and layer bytes (kept from the previous step)
-    float2 fb = z2, xob = z2;
-    unsigned cb = kMasked, lb = 0u;
-    int rs = 0, rs_m = 2;                                  // ring slots of planes t and t - 1
-    __syncthreads();
-    for (; t <= k1; ++t) {
+    // this plane's f, tables, 1/diag (K2) and old colour-A value (SOR), by position
+    const bool in0 = row_ok && t >= 0;
+    float4 fc = make_float4(0.f, 0.f, 0.f, 0.f), ic = fc;
+    unsigned cl = kOut;
+    float2 xa = z2;
+    if (in0) {
         const int l = lrow + sz * t;
-        float4 fn = z4;
-        unsigned cn = kMM, ln = 0u;
-        if (in_t(t + 1)) {
+        fc = f[HCHK(l, NP)];
+        cl = cl2[HCHK(l, NP)];
+        if (K2) ic = reinterpret_cast<const float4*>(op.invd)[HCHK(l, NP)];
+        if (SOR && !XZERO) xa = xin[HCHK(2 * l + ar, op.N)];
+    }
+    // the pair to the left / right of this one (itself at the ends of the row: those nodes
+    // lie on the masked ring and have no such neighbour)
+    const int dl = i2 > 0 ? -1 : 0, dr = i2 + 1 < TXT ? 1 : 0;
+    float2 am2 = z2, am1 = z2;                             // new colour-A values at planes t - 2, t - 1
+    float2 fb = z2, xb = z2, ib = z2;                      // colour B of plane t - 1: f, old value, 1/diag
+    unsigned cb = kMasked;                                 // its code and layer bytes
+    float2 bm1 = z2, b0 = z2;                              // own old colour-B values at planes t - 1, t
+    if (!XZERO && row_ok && t >= 1) bm1 = xin[HCHK(2 * (lrow + sz * (t - 1)) + ar, op.N)];
+    __syncthreads();
+    if (!XZERO) b0 = xs[o_0 + mx];
+    int rs = 0, rs_m = 2 * PR;                             // ring planes of t and t - 1
+    int l = lrow + sz * t;
+#pragma unroll 2
+    for (; t <= k1; ++t, l += sz, ar ^= 1) {
+        float4 fn = make_float4(0.f, 0.f, 0.f, 0.f), in = fn;
+        unsigned cn = kOut;
+        float2 xan = z2;
+        if (row_ok && t + 1 < n) {
             fn = f[HCHK(l + sz, NP)];
-            cn = code2[HCHK(l + sz, NP)];
-            ln = lidx2[HCHK(l + sz, NP)];
+            cn = cl2[HCHK(l + sz, NP)];
+            if (K2) in = reinterpret_cast<const float4*>(op.invd)[HCHK(l + sz, NP)];
+            if (SOR && !XZERO) xan = xin[HCHK(2 * (l + sz) + (ar ^ 1), op.N)];
         }
-        // colour c0 at plane t (old neighbours from the staged planes)
-        const int ar = c0 ^ ((j + t) & 1);                 // the colour-c0 node of the pair
-        const unsigned ca = ar ? (cc >> 8) : (cc & 0xffu);
-        float2 rc = z2;
-        float4 own = z4;                                   // this thread's old pair at plane t
-        if (!XZERO) own = xs[o_0 + mx];
-        if (in_t(t)) {
-            float2 sa = z2;
-            if (!XZERO && !(ca & kMasked)) {
-                const float4* P = xs + o_0;
-                // the y and z neighbours: node ar of the neighbouring pairs, read as one
-                // complex64 value each (an offset, not a select)
-                const float2* P2 = reinterpret_cast<const float2*>(xs) + ar;
-                const float2 xm = ar ? lo2(own) : hi2(P[mx + im1]);
-                const float2 xp = ar ? lo2(P[mx + ip1]) : hi2(own);
-                const float2 ym = P2[2 * (o_0 + mx - TXT)];
-                const float2 yp = P2[2 * (o_0 + mx + TXT)];
-                const float2 zm = P2[2 * (o_m1 + mx)];
-                const float2 zp = P2[2 * (o_p1 + mx)];
-                sa = six_sum(ca, xm, xp, ym, yp, zm, zp);
+        const int dx = ar ? dr : dl;
+        // colour A at plane t
+        const float2 fa = ar ? hi2(fc) : lo2(fc);
+        const unsigned ca = (ar ? cl >> 16 : cl) & 0xffffu;
+        float2 bp1 = z2;
+        if (!XZERO) bp1 = xs[o_p1 + mx];
+        float2 na;
+        if ((ca & 0xffu) == kMasked) {
+            na = fa;
+        } else {
+            float2 id;
+            if (K2) {
+                id = ar ? hi2(ic) : lo2(ic);
+                if (conj) id.y = -id.y;
+            } else {
+                id = stab[HCHK(ca >> 8, kMaxLayerCells + 1)];
             }
-            const float2 id = (ca & kMasked) ? z2 : sweep_invd(op, stab, l, ar, ar ? (lc >> 8) : (lc & 0xffu), conj);
-            rc = gs_value(op, ca, pair_node(fc, ar), sa, id, pair_node(own, ar), omega, XZERO);
+            if (XZERO) {
+                na = cmul(id, fa);
+            } else {
+                const float2* P = xs + o_0 + mx;
+                const float2 bx = P[dx];
+                const float2 s = six_sum(ca, ar, b0, bx, P[-TXT], P[TXT], bm1, bp1);
+                na = cmul(id, make_float2(fa.x - op.hinv2 * s.x, fa.y - op.hinv2 * s.y));
+            }
         }
-        ring[rs * PR + me] = rc;
+        if (SOR) na = XZERO ? cscale(omega, na) : cadd(xa, cscale(omega, csub(na, xa)));
+        ring[rs + me] = na;
         if (!XZERO) {
-            // plane t + 3 into the slot of plane t - 2 (last read in the previous step);
-            // plane t + 2 (issued one step ago) must have landed before the barrier
-            stage(t + 3, o_p3);
+            // plane t + 3 into the slot of plane t - 1 (last read before the previous step's
+            // barrier); plane t + 2 (issued one step ago) must have landed before this one
+            stage(t + 3, o_p3, ar ^ 1);
             cp_async_commit();
             cp_async_wait<1>();
         }
         __syncthreads();
-        // colour 1 - c0 at plane t - 1 (new colour-c0 neighbours)
+        // colour B at plane t - 1 (its position there is that of colour A at plane t)
         if (inner && t - 1 >= k0 && t - 1 < k1) {
-            const int lmi = l - sz;
-            const int a = ar;                              // (c0 ^ 1) ^ ((j + t - 1) & 1)
-            float2 b;
-            if (cb & kMasked) {
-                b = gs_value(op, cb, fb, z2, z2, xob, omega, false);
+            float2 nb;
+            if ((cb & 0xffu) == kMasked) {
+                nb = fb;
             } else {
-                const float2* R = ring + rs_m * PR;
-                const float2 xm = a ? rm : R[me + im1];
-                const float2 xp = a ? R[me + ip1] : rm;
-                const float2 sb = six_sum(cb, xm, xp, R[me - TXT], R[me + TXT], rm2, rc);
-                const float2 id = sweep_invd(op, stab, lmi, a, lb, conj);
-                b = gs_value(op, cb, fb, sb, id, xob, omega, false);
+                const float2* R = ring + rs_m + me;
+                const float2 ax = R[dx];
+                const float2 s = six_sum(cb, ar, am1, ax, R[-TXT], R[TXT], am2, na);
+                float2 id = ib;
+                if (!K2) id = stab[HCHK(cb >> 8, kMaxLayerCells + 1)];
+                else if (conj) id.y = -id.y;
+                nb = cmul(id, make_float2(fb.x - op.hinv2 * s.x, fb.y - op.hinv2 * s.y));
             }
-            xout[HCHK(lmi, NP)] = a ? make_float4(rm.x, rm.y, b.x, b.y) : make_float4(b.x, b.y, rm.x, rm.y);
+            // (from zero only colour A starts from zero: colour B's own old value is zero too)
+            if (SOR) nb = cadd(xb, cscale(omega, csub(nb, xb)));
+            xout[HCHK(l - sz, NP)] = ar ? make_float4(am1.x, am1.y, nb.x, nb.y) : make_float4(nb.x, nb.y, am1.x, am1.y);
         }
-        rm2 = rm;
-        rm = rc;
-        // the other node of the pair at plane t (element 1 - ar) is swept next step
+        am2 = am1;
+        am1 = na;
+        // the colour-B node at plane t is swept next step
         fb = ar ? lo2(fc) : hi2(fc);
-        xob = ar ? lo2(own) : hi2(own);
-        cb = ar ? (cc & 0xffu) : (cc >> 8);
-        lb = ar ? (lc & 0xffu) : (lc >> 8);
+        cb = (ar ? cl : cl >> 16) & 0xffffu;
+        if (K2) ib = ar ? lo2(ic) : hi2(ic);
+        if (SOR) xb = b0;
+        bm1 = b0;
+        b0 = bp1;
         fc = fn;
-        cc = cn;
-        lc = ln;
+        cl = cn;
+        if (K2) ic = in;
+        if (SOR) xa = xan;
         rs_m = rs;
-        rs = rs == 2 ? 0 : rs + 1;
-        const int o_free = o_m1;
-        o_m1 = o_0;
+        rs = rs == 2 * PR ? 0 : rs + PR;
+        const int o_free = o_0;
         o_0 = o_p1;
         o_p1 = o_p2;
         o_p2 = o_p3;
@@ -1521,6 +1537,13 @@ __global__ void k_nbr_code(Op<double> op, uint8_t* __restrict__ code) {
     code[l] = (uint8_t)c;
 }
 
+// ncl[l] = neighbour code | layer index << 8: one load a pair for both tables
+__global__ void k_node_pack(const uint8_t* __restrict__ code, const uint8_t* __restrict__ lidx,
+                            uint16_t* __restrict__ ncl, long long N) {
+    for (long long l = blockIdx.x * (long long)blockDim.x + threadIdx.x; l < N; l += (long long)gridDim.x * blockDim.x)
+        ncl[l] = (uint16_t)(code[l] | (lidx[l] << 8));
+}
+
 // face byte of a node: (number of boundary faces << 4) | axis bits
 __global__ void k_face_code(Op<double> op, uint8_t* __restrict__ face) {
     const int i = blockIdx.x * BX + threadIdx.x;
@@ -1798,67 +1821,80 @@ int launch_apply32_bicg(const Op<float>& op, int mode, const float2* x, float2* 
 
 namespace {
 
-// launch shape of k_sweep_c64 on an n^3 grid: whole rows per block (n/2 pairs, at
-// most 128), as many rows as fill 1024 threads (8 to 32) including the two halo rows;
-// z chunks of 4..16 planes, as many as fill the resident block slots once
-struct SweepShape {
-    dim3 g, b;
-    int zc;
-    size_t smem, smem0;         // dynamic shared memory: from xin, from zero
-};
-
-bool sweep_shape(int n, SweepShape& sh) {
-    const int h = n / 2;
-    if (n % 2 != 0 || h < 1 || h > 128) return false;
-    const int txt = (h + 31) / 32 * 32;
-    const int tyt = std::max(8, std::min(32, kSweepMaxThreads / txt));
-    const int byi = tyt - 2;
-    sh.b = dim3(txt, tyt);
-    sh.smem = sweep_smem_bytes(txt, tyt, false);
-    sh.smem0 = sweep_smem_bytes(txt, tyt, true);
-    static int sms = 0;
-    static int occ[5] = {0, 0, 0, 0, 0};
-    const int w = txt / 32;
-    if (sms == 0) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        // the largest block shape (128 x 8 threads) needs about 127 KB
-        cudaFuncSetAttribute(k_sweep_c64<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 136 * 1024);
-        cudaFuncSetAttribute(k_sweep_c64<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 136 * 1024);
-    }
-    if (occ[w] == 0) {
-        int o0 = 0, o1 = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o0, k_sweep_c64<false>, txt * tyt, sh.smem);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o1, k_sweep_c64<true>, txt * tyt, sh.smem0);
-        occ[w] = std::max(1, std::min(o0, o1));
-    }
-    const int gy = (n + byi - 1) / byi;
-    const long long slots = (long long)std::max(sms, 1) * occ[w];
-    const int chunks = (int)std::max<long long>(1, slots / gy);
-    sh.zc = std::max(4, std::min(16, (n + chunks - 1) / chunks));
-    sh.g = dim3(1, gy, (n + sh.zc - 1) / sh.zc);
-    return true;
+using SweepFn = void (*)(Op<float>, int, int, const float4*, const float2*, float4*, int, float);
+SweepFn sweep_fn(bool xzero, bool sor, bool k2) {
+    if (xzero) return sor ? (k2 ? k_sweep_c64<true, true, true> : k_sweep_c64<true, true, false>)
+                          : (k2 ? k_sweep_c64<true, false, true> : k_sweep_c64<true, false, false>);
+    return sor ? (k2 ? k_sweep_c64<false, true, true> : k_sweep_c64<false, true, false>)
+               : (k2 ? k_sweep_c64<false, false, true> : k_sweep_c64<false, false, false>);
 }
 
 }  // namespace
 
+// Launch shape of k_sweep_c64 on an n^3 grid: whole rows per block (n/2 pairs, at most
+// 128), 8, 16 or 32 rows (two of them halo) and a z chunk, by the shortest estimate of
+//   waves of blocks x (planes per block + 5) x time of a step,
+// where a step takes 500 clocks (its loads, barrier and shared-memory round trips) or the
+// issue time of the threads resident on the SM, whichever is longer, and 5 stands for the
+// two recomputed planes and the start of a block.  Small grids so get short chunks and few
+// rows (64^3: 2 chunks of 30 rows left 122 of 152 SMs idle), large ones whole waves
+// (256^3: 4.53 waves of 16-plane chunks cost 5).
+void plan_sweep32(Op<float>& op) {
+    op.sw_rows = op.sw_zc = 0;
+    const int n = op.n, h = n / 2;
+    if (op.dim != 3 || n % 2 != 0 || h < 1 || h > 128 || op.face || !op.ncl) return;
+    const int txt = (h + 31) / 32 * 32;
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 152;
+    double best = 0;
+    if (cudaFuncSetAttribute(k_sweep_c64<false, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024) !=
+        cudaSuccess)
+        return;
+    for (int tyt = 8; tyt <= 32 && tyt * txt <= kSweepMaxThreads; tyt *= 2) {
+        int occ = 0;
+        const size_t smem = sweep_smem_bytes(txt, tyt, false);
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_sweep_c64<false, false, false>, txt * tyt, smem) !=
+                cudaSuccess ||
+            occ < 1)
+            continue;
+        const int gy = (n + tyt - 3) / (tyt - 2);
+        for (int chunks = 1; chunks <= (n + 1) / 2; ++chunks) {
+            const int zc = (n + chunks - 1) / chunks;
+            const long long blocks = (long long)gy * ((n + zc - 1) / zc), slots = (long long)sms * occ;
+            const long long waves = (blocks + slots - 1) / slots;
+            const double resident = (double)std::min<long long>(occ, (blocks + sms - 1) / sms) * txt * tyt;
+            const double cost = (double)waves * (zc + 5) * std::max(500.0, 0.8 * resident);
+            if (op.sw_rows == 0 || cost < best) {
+                best = cost;
+                op.sw_rows = tyt;
+                op.sw_zc = zc;
+            }
+        }
+    }
+}
+
 bool rbgs_sweep32_ok(const Op<float>& op, const void* f, const void* x, const void* tmp) {
-    SweepShape sh;
-    const bool shape = op.dim == 3 && sweep_shape(op.n, sh);      // (also fills the occupancy cache)
-    return shape && pair_ok(op, f, x, tmp) && x != tmp;
+    return op.sw_rows > 0 && pair_ok(op, f, x, tmp) && x != tmp;
 }
 
 bool launch_rbgs_sweep32(const Op<float>& op, int c0, const float2* f, const float2* xin, float2* xout, int conj,
                          double omega, cudaStream_t s) {
-    SweepShape sh;
-    if (!pair_ok(op, f, xin, xout) || !sweep_shape(op.n, sh) || xin == xout) return false;
-    const float4* f4 = reinterpret_cast<const float4*>(f);
-    const float4* x4 = reinterpret_cast<const float4*>(xin);
-    float4* y4 = reinterpret_cast<float4*>(xout);
-    if (xin) k_sweep_c64<false><<<sh.g, sh.b, sh.smem, s>>>(op, sh.zc, c0, f4, x4, y4, conj, (float)omega);
-    else k_sweep_c64<true><<<sh.g, sh.b, sh.smem0, s>>>(op, sh.zc, c0, f4, x4, y4, conj, (float)omega);
+    if (!rbgs_sweep32_ok(op, f, xin, xout)) return false;
+    const int txt = (op.n / 2 + 31) / 32 * 32, tyt = op.sw_rows;
+    const dim3 g(1, (op.n + tyt - 3) / (tyt - 2), (op.n + op.sw_zc - 1) / op.sw_zc), b(txt, tyt);
+    const size_t smem = sweep_smem_bytes(txt, tyt, xin == nullptr);   // at most 78 KB
+    const SweepFn fn = sweep_fn(xin == nullptr, omega != 1.0, op.k2 != nullptr);
+    if (smem > 48 * 1024 &&
+        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024) != cudaSuccess)
+        return false;
+    fn<<<g, b, smem, s>>>(op, op.sw_zc, c0, reinterpret_cast<const float4*>(f), xin, reinterpret_cast<float4*>(xout), conj,
+                          (float)omega);
     return true;
+}
+
+void launch_node_pack(const Op<float>& op, uint16_t* ncl, cudaStream_t s) {
+    k_node_pack<<<4 * 152, 256, 0, s>>>(op.nbm, op.lidx, ncl, op.N);
 }
 
 void launch_apply_bicg_df(const Op<double>& op, const DfTab& t, int mode, const float4* x, double2* y,
