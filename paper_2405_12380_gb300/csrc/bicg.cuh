@@ -26,31 +26,42 @@ __device__ __forceinline__ bool last_block_done(unsigned* counter, unsigned nblo
     return s_last;
 }
 
+// v[q] summed over the block's kFusedThreads threads (flat index tid) in a fixed order,
+// valid in thread 0: halves are added through shared memory, so that 255 additions a value
+// take 12 FP64 instructions of a warp.  (Butterflies in every warp take 45, and an FP64
+// instruction holds a scheduler's pipe for 64 clocks whatever its lanes do: with a few
+// nodes per thread they were a third of a fused kernel's FP64 work.)
+template <int W>
+__device__ __forceinline__ void block_tree(double* v, int tid) {
+    __shared__ double red[W][kFusedThreads / 2];
+#pragma unroll
+    for (int h = kFusedThreads / 2; h >= 32; h >>= 1) {
+        if (tid >= h && tid < 2 * h)
+#pragma unroll
+            for (int q = 0; q < W; ++q) red[q][tid - h] = v[q];
+        __syncthreads();
+        if (tid < h)
+#pragma unroll
+            for (int q = 0; q < W; ++q) v[q] += red[q][tid];
+        __syncthreads();
+    }
+    if (tid < 32)
+#pragma unroll
+        for (int q = 0; q < W; ++q)
+            for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_down_sync(0xffffffffu, v[q], o);
+}
+
 // fixed-order sum of nparts partials of W doubles (stride W) by a block of
 // kFusedThreads threads (flat thread index tid); result valid in tid 0
 template <int W>
 __device__ __forceinline__ void sum_parts(const double* parts, int nparts, int tid, double* out) {
-    __shared__ double red[W][kFusedThreads / 32];
-    double v[W];
 #pragma unroll
-    for (int q = 0; q < W; ++q) v[q] = 0.0;
+    for (int q = 0; q < W; ++q) out[q] = 0.0;
+#pragma unroll 4
     for (int b = tid; b < nparts; b += kFusedThreads)
 #pragma unroll
-        for (int q = 0; q < W; ++q) v[q] += __ldcg(parts + (long long)b * W + q);
-#pragma unroll
-    for (int q = 0; q < W; ++q)
-        for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
-    if ((tid & 31) == 0)
-#pragma unroll
-        for (int q = 0; q < W; ++q) red[q][tid >> 5] = v[q];
-    __syncthreads();
-    if (tid == 0)
-#pragma unroll
-        for (int q = 0; q < W; ++q) {
-            double s = 0.0;
-            for (int w = 0; w < kFusedThreads / 32; ++w) s += red[q][w];
-            out[q] = s;
-        }
+        for (int q = 0; q < W; ++q) out[q] += __ldcg(parts + (long long)b * W + q);
+    block_tree<W>(out, tid);
 }
 
 // --- recurrences (one thread), slots S_* of helm_internal.cuh ----------------

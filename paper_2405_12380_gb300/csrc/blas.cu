@@ -23,46 +23,23 @@ __device__ __forceinline__ double2 warp_sum(double2 v) {
     return v;
 }
 
-// block-wide sum (TB threads); result valid in thread 0
-__device__ __forceinline__ double block_sum(double v) {
-    __shared__ double red[TB / 32];
-    v = warp_sum(v);
-    int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    __syncthreads();
-    if (lane == 0) red[w] = v;
-    __syncthreads();
-    if (w == 0) {
-        v = lane < TB / 32 ? red[lane] : 0.0;
-        v = warp_sum(v);
-    }
-    return v;
-}
-__device__ __forceinline__ double2 block_sum(double2 v) {
-    double a = block_sum(v.x);
-    double b = block_sum(v.y);
-    return make_double2(a, b);
-}
-
 __global__ void __launch_bounds__(TB) k_dot(const double2* __restrict__ a, const double2* __restrict__ b,
                                             long long N, double2* partials) {
     double2 acc = make_double2(0, 0);
     for (long long l = blockIdx.x * (long long)TB + threadIdx.x; l < N; l += (long long)gridDim.x * TB) {
-        double2 u = a[l], v = b[l];
-        acc.x += u.x * v.x + u.y * v.y;
-        acc.y += u.x * v.y - u.y * v.x;
+        acc = cfmac(a[l], b[l], acc);
     }
-    acc = block_sum(acc);
-    if (threadIdx.x == 0) partials[blockIdx.x] = acc;
+    double v[2] = {acc.x, acc.y};
+    block_tree<2>(v, threadIdx.x);
+    if (threadIdx.x == 0) partials[blockIdx.x] = make_double2(v[0], v[1]);
 }
 
 __global__ void __launch_bounds__(TB) k_norm2(const double2* __restrict__ a, long long N, double* partials) {
-    double acc = 0;
-    for (long long l = blockIdx.x * (long long)TB + threadIdx.x; l < N; l += (long long)gridDim.x * TB) {
-        double2 u = a[l];
-        acc += u.x * u.x + u.y * u.y;
-    }
-    acc = block_sum(acc);
-    if (threadIdx.x == 0) partials[blockIdx.x] = acc;
+    double acc[1] = {0.0};
+    for (long long l = blockIdx.x * (long long)TB + threadIdx.x; l < N; l += (long long)gridDim.x * TB)
+        acc[0] = cnorm2(a[l], acc[0]);
+    block_tree<1>(acc, threadIdx.x);
+    if (threadIdx.x == 0) partials[blockIdx.x] = acc[0];
 }
 
 // fixed-order sum of partials by one block of kFinThreads threads
@@ -115,8 +92,7 @@ __global__ void __launch_bounds__(TB) k_bicg_p(const double2* __restrict__ r, co
                                                double2* __restrict__ p, const double2* __restrict__ sc, long long N) {
     const double2 beta = sc[S_BETA], omega = sc[S_OMEGA];
     for (long long l = blockIdx.x * (long long)TB + threadIdx.x; l < N; l += (long long)gridDim.x * TB) {
-        double2 t = csub(p[l], cmul(omega, v[l]));
-        p[l] = cadd(r[l], cmul(beta, t));
+        p[l] = cfma(beta, cfma(make_double2(-omega.x, -omega.y), v[l], p[l]), r[l]);
     }
 }
 
@@ -124,15 +100,15 @@ __global__ void __launch_bounds__(TB) k_bicg_p(const double2* __restrict__ r, co
 __global__ void __launch_bounds__(kFusedThreads) k_bicg_s_fused(const double2* __restrict__ r, const double2* __restrict__ v,
                                                                 double2* __restrict__ s, double2* sc, long long N,
                                                                 double* parts, unsigned* counter, double tol_abs) {
-    const double2 alpha = sc[S_ALPHA];
-    double acc = 0;
+    const double2 na = make_double2(-sc[S_ALPHA].x, -sc[S_ALPHA].y);
+    double acc[1] = {0.0};
     for (long long l = blockIdx.x * (long long)kFusedThreads + threadIdx.x; l < N; l += (long long)gridDim.x * kFusedThreads) {
-        const double2 q = csub(r[l], cmul(alpha, v[l]));
+        const double2 q = cfma(na, v[l], r[l]);
         s[l] = q;
-        acc += q.x * q.x + q.y * q.y;
+        acc[0] = cnorm2(q, acc[0]);
     }
-    acc = block_sum(acc);
-    if (threadIdx.x == 0) parts[blockIdx.x] = acc;
+    block_tree<1>(acc, threadIdx.x);
+    if (threadIdx.x == 0) parts[blockIdx.x] = acc[0];
     if (last_block_done(counter, gridDim.x)) {
         double tot[1];
         sum_parts<1>(parts, gridDim.x, threadIdx.x, tot);
@@ -159,22 +135,18 @@ __global__ void __launch_bounds__(kFusedThreads) k_bicg_xr_fused(double2* __rest
     double2 rho = make_double2(0, 0);
     for (long long l = blockIdx.x * (long long)kFusedThreads + threadIdx.x; l < N && !skip;
          l += (long long)gridDim.x * kFusedThreads) {
-        double2 xv = cadd(x[l], cmul(alpha, phat[l]));
-        xv = cadd(xv, cmul(omega, shat[l]));
-        x[l] = xv;
-        const double2 q = csub(s[l], cmul(omega, t[l]));
+        x[l] = cfma(omega, shat[l], cfma(alpha, phat[l], x[l]));
+        const double2 q = cfma(make_double2(-omega.x, -omega.y), t[l], s[l]);
         r[l] = q;
-        rn += q.x * q.x + q.y * q.y;
-        const double2 h = rhat[l];
-        rho.x += h.x * q.x + h.y * q.y;
-        rho.y += h.x * q.y - h.y * q.x;
+        rn = cnorm2(q, rn);
+        rho = cfmac(rhat[l], q, rho);
     }
-    rn = block_sum(rn);
-    rho = block_sum(rho);
+    double v[3] = {rn, rho.x, rho.y};
+    block_tree<3>(v, threadIdx.x);
     if (threadIdx.x == 0) {
-        parts[3 * blockIdx.x + 0] = rn;
-        parts[3 * blockIdx.x + 1] = rho.x;
-        parts[3 * blockIdx.x + 2] = rho.y;
+        parts[3 * blockIdx.x + 0] = v[0];
+        parts[3 * blockIdx.x + 1] = v[1];
+        parts[3 * blockIdx.x + 2] = v[2];
     }
     if (last_block_done(counter, gridDim.x)) {
         double tot[3];
@@ -260,9 +232,7 @@ __global__ void __launch_bounds__(TB) k_mupdate(const double2* __restrict__ V, i
         double2 s = w[l];
 #pragma unroll 4
         for (int i = 0; i < nv; ++i) {
-            double2 v = V[(long long)i * N + l];
-            s.x += c[i].x * v.x - c[i].y * v.y;
-            s.y += c[i].x * v.y + c[i].y * v.x;
+            s = cfma(c[i], V[(long long)i * N + l], s);
         }
         w[l] = s;
     }
@@ -279,9 +249,7 @@ __global__ void __launch_bounds__(TB) k_mupdate32(const float2* __restrict__ V, 
 #pragma unroll 4
         for (int i = 0; i < nv; ++i) {
             float2 vf = V[(long long)i * N + l];
-            double2 v = make_double2(vf.x, vf.y);
-            s.x += c[i].x * v.x - c[i].y * v.y;
-            s.y += c[i].x * v.y + c[i].y * v.x;
+            s = cfma(c[i], make_double2(vf.x, vf.y), s);
         }
         w[l] = s;
     }

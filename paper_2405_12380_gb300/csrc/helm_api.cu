@@ -1139,6 +1139,8 @@ void fill_tables(helm_handle* h) {
     f.hinv2 = (float)o.hinv2;
     o.dre = h->k0 * h->k0 - 2.0 * h->dim / (h->h * h->h);
     f.dre = (float)o.dre;
+    o.dsub = 2.0 * h->dim * o.hinv2;
+    f.dsub = (float)(2 * h->dim) * f.hinv2;
     o.mask = f.mask = h->mask;
     o.lidx = f.lidx = h->lidx;
     o.nbm = f.nbm = h->nbm;

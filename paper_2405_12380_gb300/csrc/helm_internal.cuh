@@ -104,6 +104,45 @@ __host__ __device__ __forceinline__ double2 cdiv(double2 a, double2 b) {
     return make_double2((a.x * b.x + a.y * b.y) / d, (a.y * b.x - a.x * b.y) / d);
 }
 
+// ------------------------------------------------- FP32 pairs <-> FP64
+// value = hi + lo with hi = the nearest FP32 number and lo the nearest to the rest.  A
+// conversion between the formats runs on the FP64 pipe (64 clocks of a scheduler's pipe
+// per warp, like every FP64 instruction): four per component for a split, two and an add
+// for a join.  Both are instead formed with integer instructions, bit for bit the same;
+// values outside the range where that holds (subnormal in FP32, near its largest, not
+// finite) take the conversions.
+__device__ __forceinline__ float2 f64_to_pair(double v) {
+    const unsigned h = (unsigned)__double2hiint(v), l = (unsigned)__double2loint(v);
+    const unsigned ed = (h >> 20) & 0x7ffu;                // biased exponent
+    if (ed - 949u <= 1150u - 949u) {                       // 2^-74 <= |v| < 2^128
+        // the magnitude's leading 24 bits, rounded to nearest even at bit 29
+        unsigned top = ((h & 0x7fffffffu) << 3) | (l >> 29);
+        const unsigned frac = l & 0x1fffffffu;
+        const bool up = frac > 0x10000000u || (frac == 0x10000000u && (top & 1u));
+        top += up ? 1u : 0u;
+        const int rest = (int)frac - (up ? 0x20000000 : 0);            // units of 2^(e - 52)
+        const unsigned sign = h & 0x80000000u;
+        const float hi = __uint_as_float((top - (896u << 23)) | sign);
+        const float scale = __uint_as_float(((ed - 948u) << 23) | sign);   // +- 2^(e - 52)
+        if ((__float_as_uint(hi) & 0x7f800000u) != 0x7f800000u) return make_float2(hi, (float)rest * scale);
+    }
+    const float hi = __double2float_rn(v);
+    return make_float2(hi, v == 0.0 ? 0.f : __double2float_rn(v - (double)hi));
+}
+// hi + lo rounded to FP64
+__device__ __forceinline__ double pair_to_f64(float hi, float lo) {
+    const unsigned b = __float_as_uint(hi), e = (b >> 23) & 0xffu;
+    const float units = lo * __uint_as_float(((306u - e) & 0xffu) << 23);             // lo in units of 2^(e - 52)
+    // (at a power of two the unit below is half; a pair that is not normalised converts)
+    if (e - 53u <= 254u - 53u && (b & 0x7fffffu) && fabsf(units) <= 536870912.f) {
+        const int rest = __float2int_rn(units);
+        const unsigned hw = ((b & 0x7fffffffu) >> 3) + (896u << 20), lw = b << 29;
+        const long long mag = (long long)(((unsigned long long)hw << 32) | lw) + ((int)b < 0 ? -rest : rest);
+        return __longlong_as_double(mag | ((long long)(b & 0x80000000u) << 32));
+    }
+    return (double)hi + (double)lo;
+}
+
 // ------------------------------------------------------ operator description
 // Everything a stencil kernel needs, passed by value.  The absorbing layer is
 // tabulated by the layer index m = max_a max(0, L - dist_a) in 0..L, so k^2 and
@@ -116,6 +155,7 @@ struct Op {
     long long N;
     R hinv2;                 // h^-2
     R dre;                   // k0^2 - 2 d h^-2 (real part of the diagonal, layer form)
+    R dsub;                  // 2 d h^-2 (the diagonal of a stored field is k^2 - dsub)
     const uint8_t* mask;
     const uint8_t* lidx;     // per-node layer index m (flat-index kernels; avoids index division)
     const uint8_t* nbm;      // per-node neighbour code: bit q = neighbour q fluid, 0x80 = masked node
@@ -193,6 +233,7 @@ bool launch_red_residual32(const Op<float>& op, const float2* f, const float2* x
 int launch_apply32_bicg(const Op<float>& op, int mode, const float2* x, float2* y, const float2* w, int conj,
                         const double2* sc, float* parts, cudaStream_t s);
 int apply_grid_blocks(int dim, int n);
+int noalloc_grid_blocks(int dim, int n);   // of them, what the table-free operator may write
 int bicg_grid_blocks(int dim, int n);
 void launch_rhs(const Op<double>& op, const double2* src, const double2* g, double2* b, cudaStream_t s);
 void launch_layer_k2(const Op<double>& op, double k0, double strength, const double* scale,

@@ -61,7 +61,7 @@ extern "C" helm_status helm_residual_noalloc(int dim, int n, double k0, int laye
     long long N = 1;
     for (int a = 0; a < dim; ++a) N *= n;
     if (N >= (1LL << 31) || n > 65535) return HELM_BAD_ARG;
-    if ((long long)apply_grid_blocks(dim, n) > kScratchDoubles) return HELM_SCRATCH_TOO_SMALL;
+    if ((long long)noalloc_grid_blocks(dim, n) > kScratchDoubles) return HELM_SCRATCH_TOO_SMALL;
     double* scratch = nullptr;
     int* flag = nullptr;
     helm_status st = scratch_for_current_device(&scratch, &flag);
@@ -76,6 +76,7 @@ extern "C" helm_status helm_residual_noalloc(int dim, int n, double k0, int laye
     op.N = N;
     op.hinv2 = 1.0 / (h * h);
     op.dre = k0 * k0 - 2.0 * dim / (h * h);
+    op.dsub = 2.0 * dim * op.hinv2;
     op.mask = mask;
     op.k2 = reinterpret_cast<const double2*>(k2);
     op.invd = nullptr;

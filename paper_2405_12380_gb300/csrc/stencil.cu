@@ -49,7 +49,7 @@ __device__ __forceinline__ typename CT<R>::T diag_of(const Op<R>& op, long long 
     typename CT<R>::T d;
     if (op.k2) {
         d = op.k2[l];
-        d.x -= (R)(2 * op.dim) * op.hinv2;
+        d.x -= op.dsub;
     } else {
         d.x = op.dre;
         d.y = op.im[m];
@@ -145,13 +145,12 @@ __device__ __forceinline__ void block_reduce_store(double v, double* out) {
     }
 }
 
-// y = A x, or y = f - A x (resid), at one node; returns |y_l|^2
+// y = A x, or y = f - A x (resid), at one node; returns y_l
 template <typename R, bool RESID>
-__device__ __forceinline__ double apply_point(const Op<R>& op, const typename CT<R>::T* __restrict__ x,
+__device__ __forceinline__ typename CT<R>::T apply_point(const Op<R>& op, const typename CT<R>::T* __restrict__ x,
                                               const typename CT<R>::T* __restrict__ f, typename CT<R>::T* __restrict__ y,
-                                              int conj, int i, int j, int k) {
+                                              int conj, int i, int j, int k, long long l) {
     using C = typename CT<R>::T;
-    const long long l = i + (long long)op.n * (j + (long long)op.n * k);
     const C xc = x[l];
     const unsigned code = node_code(op, l);
     C out;
@@ -165,31 +164,35 @@ __device__ __forceinline__ double apply_point(const Op<R>& op, const typename CT
     }
     if (RESID) out = csub(f[l], out);
     y[l] = out;
-    return (double)out.x * out.x + (double)out.y * out.y;
+    return out;
 }
+__device__ __forceinline__ double norm_acc(double2 a, double s) { return cnorm2(a, s); }
+__device__ __forceinline__ double norm_acc(float2 a, double s) { return s + ((double)a.x * a.x + (double)a.y * a.y); }
 
-// 3D operator marching in z: a block owns a 32 x 8 tile of (x, y) and walks zc
-// planes (zc chosen so that the grid still has a few blocks per SM).  The
-// z-neighbours come from registers (each plane of x is loaded once, two planes
-// ahead of its use), the x-neighbours from warp shuffles (a warp is one row of 32
-// consecutive nodes; the two row ends load from memory), the y-neighbours from L1.
-constexpr int ZC = 16;      // largest z chunk
+// 3D operator marching in z: a block owns 256 consecutive nodes of a plane (whatever rows
+// they lie in, so that every lane has a node: with one row per warp a 129-node row filled
+// four fifths of its lanes, and an FP64 instruction costs the same however few are active)
+// and walks zc planes.  The z-neighbours come from registers (each plane of x is loaded
+// once, two planes ahead of its use), the x-neighbours from warp shuffles (fluid nodes are
+// interior, so theirs are the neighbours in the plane's order; the two ends of the warp
+// load from memory), the y-neighbours from L1 or L2.  Bound by the FP64 pipe in complex128
+// (16 instructions a node, 20 with the residual and its norm).
+constexpr int AZ = 256;
 
 template <typename R, bool RESID, bool NORM>
-__global__ void __launch_bounds__(BX * BY) k_apply_z(Op<R> op, int zc, const typename CT<R>::T* __restrict__ x,
-                                                     const typename CT<R>::T* __restrict__ f,
-                                                     typename CT<R>::T* __restrict__ y, double* partials, int conj) {
+__global__ void __launch_bounds__(AZ) k_apply_z(Op<R> op, int zc, const typename CT<R>::T* __restrict__ x,
+                                                const typename CT<R>::T* __restrict__ f,
+                                                typename CT<R>::T* __restrict__ y, double* partials, int conj) {
     using C = typename CT<R>::T;
-    const int i = blockIdx.x * BX + threadIdx.x;
-    const int j = blockIdx.y * BY + threadIdx.y;
-    const int k0 = blockIdx.z * zc;
+    const int sy = op.n, sz = op.n * op.n;                 // (N < 2^31)
+    const int q = blockIdx.x * AZ + threadIdx.x;           // index in the plane
+    const int k0 = blockIdx.y * zc;
     const int k1 = min(op.n, k0 + zc);
-    const bool valid = i < op.n && j < op.n;
-    const long long sy = op.n, sz = (long long)op.n * op.n;
-    const int lane = threadIdx.x;
+    const bool valid = q < sz;
+    const int lane = threadIdx.x & 31;
     C zero;
     zero.x = 0; zero.y = 0;
-    long long l = i + (long long)op.n * (j + (long long)op.n * k0);
+    long long l = q + (long long)sz * k0;
     C prev = (valid && k0 > 0) ? x[l - sz] : zero;
     C cur = valid ? x[l] : zero;
     C next = (valid && k0 + 1 < op.n) ? x[l + sz] : zero;
@@ -203,13 +206,14 @@ __global__ void __launch_bounds__(BX * BY) k_apply_z(Op<R> op, int zc, const typ
         const C next2 = (more && k + 2 < op.n) ? x[l + 2 * sz] : zero;
         const unsigned code_n = more ? (unsigned)op.nbm[l + sz] : kMasked;
         const int li_n = more ? (int)op.lidx[l + sz] : 0;
-        C xm, xp;
+        C xm, xp, fv = zero;
+        if (RESID && valid) fv = f[l];
         xm.x = __shfl_up_sync(0xffffffffu, cur.x, 1);
         xm.y = __shfl_up_sync(0xffffffffu, cur.y, 1);
         xp.x = __shfl_down_sync(0xffffffffu, cur.x, 1);
         xp.y = __shfl_down_sync(0xffffffffu, cur.y, 1);
         if (lane == 0 && (code & 1u)) xm = x[l - 1];
-        if (lane == BX - 1 && (code & 2u)) xp = x[l + 1];
+        if (lane == 31 && (code & 2u)) xp = x[l + 1];
         C out;
         if (code & kMasked) {
             out = cur;
@@ -226,9 +230,9 @@ __global__ void __launch_bounds__(BX * BY) k_apply_z(Op<R> op, int zc, const typ
             out.y = op.hinv2 * s.y + (dg.x * cur.y + dg.y * cur.x);
         }
         if (valid) {
-            if (RESID) out = csub(f[l], out);
+            if (RESID) out = csub(fv, out);
             y[l] = out;
-            if (NORM) acc += (double)out.x * out.x + (double)out.y * out.y;
+            if (NORM) acc = norm_acc(out, acc);
         }
         prev = cur;
         cur = next;
@@ -237,7 +241,9 @@ __global__ void __launch_bounds__(BX * BY) k_apply_z(Op<R> op, int zc, const typ
         li = li_n;
     }
     if (NORM) {
-        block_reduce_store<R>(acc, partials + (blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z)));
+        double v[1] = {acc};
+        block_tree<1>(v, threadIdx.x);
+        if (threadIdx.x == 0) partials[blockIdx.x + gridDim.x * blockIdx.y] = v[0];
     }
 }
 
@@ -803,65 +809,53 @@ __global__ void __launch_bounds__(BX * BY) k_apply(Op<R> op, int zc, const typen
     const int k1 = op.dim == 3 ? min(op.n, k0 + zc) : 1;
     double acc = 0.0;
     if (i < op.n && j < op.n)
-        for (int kk = k0; kk < k1; ++kk) acc += apply_point<R, RESID>(op, x, f, y, conj, i, j, kk);
+        for (int kk = k0; kk < k1; ++kk)
+            acc = norm_acc(apply_point<R, RESID>(op, x, f, y, conj, i, j, kk, i + (long long)op.n * (j + (long long)op.n * kk)),
+                           acc);
     if (NORM) {
         block_reduce_store<R>(acc, partials + (blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z)));
     }
 }
 
-// y = A x with a BiCGStab reduction in the epilogue and its scalar update in the
-// last block.  mode 1: <w, y> -> alpha = rho / <rhat, v> (w = rhat);
-// mode 2: <y, w>, <y, y> -> omega (w = s).
+// the end of a BiCGStab operator kernel: the block's sums a (and c) into parts, and in the
+// last block the scalar update
 template <int MODE>
-__global__ void __launch_bounds__(BX * BY) k_apply_bicg(Op<double> op, const double2* __restrict__ x,
-                                                        double2* __restrict__ y, const double2* __restrict__ w,
-                                                        int conj, double2* sc, double* parts, unsigned* counter) {
-    const int i = blockIdx.x * BX + threadIdx.x;
-    const int j = blockIdx.y * BY + threadIdx.y;
-    const int k0 = op.dim == 3 ? 2 * blockIdx.z : 0;
-    double a = 0, b = 0, c = 0;
-    if (i < op.n && j < op.n) {
-        for (int kk = k0; kk < (op.dim == 3 ? min(k0 + 2, op.n) : 1); ++kk) {
-            apply_point<double, false>(op, x, nullptr, y, conj, i, j, kk);
-            const long long l = i + (long long)op.n * (j + (long long)op.n * kk);
-            const double2 yv = y[l], wv = w[l];
-            if (MODE == 1) {          // conj(w) y
-                a += wv.x * yv.x + wv.y * yv.y;
-                b += wv.x * yv.y - wv.y * yv.x;
-            } else {                  // conj(y) w and |y|^2
-                a += yv.x * wv.x + yv.y * wv.y;
-                b += yv.x * wv.y - yv.y * wv.x;
-                c += yv.x * yv.x + yv.y * yv.y;
-            }
-        }
-    }
-    const int tid = threadIdx.x + BX * threadIdx.y;
-    const unsigned nblk = gridDim.x * gridDim.y * gridDim.z;
-    const unsigned bid = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
-    __shared__ double red[3][BX * BY / 32];
-    for (int o = 16; o > 0; o >>= 1) {
-        a += __shfl_xor_sync(0xffffffffu, a, o);
-        b += __shfl_xor_sync(0xffffffffu, b, o);
-        c += __shfl_xor_sync(0xffffffffu, c, o);
-    }
-    if ((tid & 31) == 0) { red[0][tid >> 5] = a; red[1][tid >> 5] = b; red[2][tid >> 5] = c; }
-    __syncthreads();
-    if (tid == 0) {
-        double sa = 0, sb = 0, scc = 0;
-        for (int q = 0; q < BX * BY / 32; ++q) { sa += red[0][q]; sb += red[1][q]; scc += red[2][q]; }
-        parts[3 * bid + 0] = sa;
-        parts[3 * bid + 1] = sb;
-        parts[3 * bid + 2] = scc;
-    }
-    if (last_block_done(counter, nblk)) {
-        double tot[3];
-        sum_parts<3>(parts, nblk, tid, tot);
+__device__ __forceinline__ void bicg_finish(double2 a, double c, int tid, double2* sc, double* parts, unsigned* counter) {
+    constexpr int W = MODE == 1 ? 2 : 3;
+    double v[3] = {a.x, a.y, c};
+    block_tree<W>(v, tid);
+    if (tid == 0)
+        for (int q = 0; q < W; ++q) parts[W * blockIdx.x + q] = v[q];
+    if (last_block_done(counter, gridDim.x)) {
+        sum_parts<W>(parts, gridDim.x, tid, v);
         if (tid == 0) {
-            if (MODE == 1) bicg_alpha(sc, make_double2(tot[0], tot[1]));
-            else bicg_omega(sc, make_double2(tot[0], tot[1]), tot[2]);
+            if (MODE == 1) bicg_alpha(sc, make_double2(v[0], v[1]));
+            else bicg_omega(sc, make_double2(v[0], v[1]), v[2]);
             *counter = 0;
         }
     }
+}
+
+// y = A x with a BiCGStab reduction in the epilogue and its scalar update in the
+// last block.  mode 1: <w, y> -> alpha = rho / <rhat, v> (w = rhat);
+// mode 2: <y, w>, <y, y> -> omega (w = s).  Two nodes per thread, 512 consecutive ones
+// per block (every lane busy whatever the row length).
+constexpr int BN = 2;                 // nodes per thread
+template <int MODE>
+__global__ void __launch_bounds__(kFusedThreads) k_apply_bicg(Op<double> op, const double2* __restrict__ x,
+                                                              double2* __restrict__ y, const double2* __restrict__ w,
+                                                              int conj, double2* sc, double* parts, unsigned* counter) {
+    double2 a = make_double2(0, 0);
+    double c = 0;
+#pragma unroll
+    for (int u = 0; u < BN; ++u) {
+        const long long l = (blockIdx.x * (long long)BN + u) * kFusedThreads + threadIdx.x;
+        if (l >= op.N) break;
+        const double2 yv = apply_point<double, false>(op, x, nullptr, y, conj, 0, 0, 0, l), wv = w[l];
+        a = MODE == 1 ? cfmac(wv, yv, a) : cfmac(yv, wv, a);
+        if (MODE == 2) c = cnorm2(yv, c);
+    }
+    bicg_finish<MODE>(a, c, threadIdx.x, sc, parts, counter);
 }
 
 // one damped-Jacobi sweep: xout = xin + omega D^-1 (f - A xin), evaluated on a
@@ -870,11 +864,10 @@ __global__ void __launch_bounds__(BX * BY) k_apply_bicg(Op<double> op, const dou
 template <typename R, bool XZERO>
 __device__ __forceinline__ void jacobi_point(const Op<R>& op, R omega, const typename CT<R>::T* __restrict__ f,
                                              const typename CT<R>::T* __restrict__ xin,
-                                             typename CT<R>::T* __restrict__ xout, int conj, int i, int j, int k) {
+                                             typename CT<R>::T* __restrict__ xout, int conj, long long l) {
     using C = typename CT<R>::T;
-    const long long l = i + (long long)op.n * (j + (long long)op.n * k);
     const C fl = f[l];
-    const unsigned code = node_code(op, l);
+    const unsigned code = op.nbm[l];
     C out;
     if (code & kMasked) {
         if (XZERO) {
@@ -884,7 +877,7 @@ __device__ __forceinline__ void jacobi_point(const Op<R>& op, R omega, const typ
             out = cadd(xc, cscale(omega, csub(fl, xc)));
         }
     } else {
-        C id = invd_of(op, l, node_lidx(op, l, i, j, k), conj);
+        C id = invd_of(op, l, op.lidx[l], conj);
         if (XZERO) {
             out = cscale(omega, cmul(id, fl));
         } else {
@@ -902,17 +895,14 @@ __device__ __forceinline__ void jacobi_point(const Op<R>& op, R omega, const typ
     xout[l] = out;
 }
 
-// Two z-planes per thread (independent points: more FP64 work in flight per warp).
+// One node per thread in the flat order: every lane has a node whatever the row length
+// (as in k_apply_z and the red-black kernels below).
 template <typename R, bool XZERO>
 __global__ void __launch_bounds__(BX * BY) k_jacobi(Op<R> op, R omega, const typename CT<R>::T* __restrict__ f,
                                                     const typename CT<R>::T* __restrict__ xin,
                                                     typename CT<R>::T* __restrict__ xout, int conj) {
-    const int i = blockIdx.x * BX + threadIdx.x;
-    const int j = blockIdx.y * BY + threadIdx.y;
-    const int k0 = op.dim == 3 ? 2 * blockIdx.z : 0;
-    if (i >= op.n || j >= op.n) return;
-    jacobi_point<R, XZERO>(op, omega, f, xin, xout, conj, i, j, k0);
-    if (op.dim == 3 && k0 + 1 < op.n) jacobi_point<R, XZERO>(op, omega, f, xin, xout, conj, i, j, k0 + 1);
+    const long long l = blockIdx.x * (long long)(BX * BY) + threadIdx.x;
+    if (l < op.N) jacobi_point<R, XZERO>(op, omega, f, xin, xout, conj, l);
 }
 
 // Several damped-Jacobi sweeps of a 2D grid in one launch (small grids, where a sweep
@@ -978,16 +968,15 @@ __global__ void k_jacobi_tile(Op<R> op, R omega, int S, const typename CT<R>::T*
 // SOR (omega != 1): x_l + omega (that value - x_l)
 template <typename R, bool XZERO>
 __device__ __forceinline__ void rbgs_point(const Op<R>& op, const typename CT<R>::T* __restrict__ f,
-                                           typename CT<R>::T* x, int conj, int i, int j, int k, R omega) {
+                                           typename CT<R>::T* x, int conj, long long l, R omega, bool sor) {
     using C = typename CT<R>::T;
-    const long long l = i + (long long)op.n * (j + (long long)op.n * k);
     const C fl = f[l];
-    const unsigned code = node_code(op, l);
+    const unsigned code = op.nbm[l];
     C out;
     if (code & kMasked) {
         out = fl;
     } else {
-        const C id = invd_of(op, l, node_lidx(op, l, i, j, k), conj);
+        const C id = invd_of(op, l, op.lidx[l], conj);
         if (XZERO) {
             out = cmul(id, fl);
         } else {
@@ -998,7 +987,7 @@ __device__ __forceinline__ void rbgs_point(const Op<R>& op, const typename CT<R>
             out = cmul(id, g);
         }
     }
-    if (omega != (R)1) {
+    if (sor) {
         if (XZERO) {
             out = cscale(omega, out);
         } else {
@@ -1009,38 +998,48 @@ __device__ __forceinline__ void rbgs_point(const Op<R>& op, const typename CT<R>
     x[l] = out;
 }
 
-template <typename R, bool XZERO>
-__global__ void __launch_bounds__(BX * BY) k_rbgs(Op<R> op, int colour, const typename CT<R>::T* __restrict__ f,
-                                                  typename CT<R>::T* x, int conj, R omega) {
-    const int j = blockIdx.y * BY + threadIdx.y;
-    const int k = op.dim == 3 ? blockIdx.z : 0;
-    if (j >= op.n) return;
-    const int i = 2 * (blockIdx.x * BX + threadIdx.x) + ((j + k + colour) & 1);
-    if (i < op.n) rbgs_point<R, XZERO>(op, f, x, conj, i, j, k, omega);
+// colour of node l: (i + j + k) mod 2
+__device__ __forceinline__ int colour_of(long long l, int n) {
+    const unsigned ul = (unsigned)l, un = (unsigned)n;
+    const unsigned r = ul / un;          // row index j + n k
+    const unsigned kk = r / un;
+    return (int)(((ul - r * un) + (r - kk * un) + kk) & 1u);
 }
 
-// r_red[l / 2] = (v - A z)_l at the red nodes l (one per node pair (2m, 2m + 1))
+// One thread per node pair (2m, 2m + 1), which holds one node of each colour (rows of even
+// length start on even l; for odd n the colour is the parity of l), in the flat order, so
+// that every lane has a node: one row per warp left a quarter of the lanes of 96-node rows
+// idle, and the kernel is bound by the FP64 pipe (16 instructions a node).  96^3: 24.2 us
+// a half-sweep before.
+template <typename R, bool XZERO>
+__global__ void __launch_bounds__(BX * BY) k_rbgs(Op<R> op, int colour, const typename CT<R>::T* __restrict__ f,
+                                                  typename CT<R>::T* x, int conj, R omega, bool sor) {
+    const long long m2 = 2 * (blockIdx.x * (long long)(BX * BY) + threadIdx.x);
+    if (m2 >= op.N) return;
+    const long long l = m2 + (colour_of(m2, op.n) != colour);
+    if (l < op.N) rbgs_point<R, XZERO>(op, f, x, conj, l, omega, sor);
+}
+
+// r_red[m] = (v - A z) at the red node of pair (2m, 2m + 1)
 __global__ void __launch_bounds__(BX * BY) k_residual_red(Op<double> op, const double2* __restrict__ z,
                                                           const double2* __restrict__ v,
                                                           double2* __restrict__ r_red, int conj) {
-    const int j = blockIdx.y * BY + threadIdx.y;
-    const int k = op.dim == 3 ? blockIdx.z : 0;
-    if (j >= op.n) return;
-    const int i = 2 * (blockIdx.x * BX + threadIdx.x) + ((j + k) & 1);
-    if (i >= op.n) return;
-    const long long l = i + (long long)op.n * (j + (long long)op.n * k);
+    const long long m = blockIdx.x * (long long)(BX * BY) + threadIdx.x;
+    if (2 * m >= op.N) return;
+    const long long l = 2 * m + colour_of(2 * m, op.n);
+    if (l >= op.N) return;
     const double2 xc = z[l];
-    const unsigned code = node_code(op, l);
+    const unsigned code = op.nbm[l];
     double2 out;
     if (code & kMasked) {
         out = xc;
     } else {
         const double2 s = nbr_sum(op, z, l, code);
-        const double2 d = diag_of(op, l, node_lidx(op, l, i, j, k), conj);
+        const double2 d = diag_of(op, l, op.lidx[l], conj);
         out.x = op.hinv2 * s.x + (d.x * xc.x - d.y * xc.y);
         out.y = op.hinv2 * s.y + (d.x * xc.y + d.y * xc.x);
     }
-    r_red[l >> 1] = csub(v[l], out);
+    r_red[m] = csub(v[l], out);
 }
 
 // ---- double-float red-black Gauss-Seidel for FP64 handles.  The sweeps of the
@@ -1069,10 +1068,7 @@ __device__ __forceinline__ float2 df_mul(float2 a, float2 b) {
     e = fmaf(a.y, b.x, e);
     return df_norm(p, e);
 }
-__device__ __forceinline__ float2 df_split(double v) {
-    const float h = __double2float_rn(v);
-    return make_float2(h, __double2float_rn(v - (double)h));
-}
+__device__ __forceinline__ float2 df_split(double v) { return f64_to_pair(v); }
 
 struct Cdf {          // complex double-float
     float2 re, im;
@@ -1205,67 +1201,34 @@ __device__ __forceinline__ Cdf nbr_sum_any(const Op<double>& op, const XT* __res
 }
 
 template <int MODE, typename XT>
-__global__ void __launch_bounds__(BX * BY) k_apply_bicg_df(Op<double> op, DfTab t, const XT* __restrict__ x,
-                                                           double2* __restrict__ y, const double2* __restrict__ w,
-                                                           int conj, double2* sc, double* parts, unsigned* counter) {
-    const int i = blockIdx.x * BX + threadIdx.x;
-    const int j = blockIdx.y * BY + threadIdx.y;
-    const int k0 = op.dim == 3 ? 2 * blockIdx.z : 0;
-    double a = 0, b = 0, c = 0;
-    if (i < op.n && j < op.n) {
-        for (int kk = k0; kk < (op.dim == 3 ? min(k0 + 2, op.n) : 1); ++kk) {
-            const long long l = i + (long long)op.n * (j + (long long)op.n * kk);
-            const unsigned code = node_code(op, l);
-            const Cdf X = cdf_load(x, l);
-            Cdf out;
-            if (code & kMasked) {
-                out = X;
-            } else {
-                const Cdf sum = nbr_sum_any(op, x, l, code);
-                const int m = node_lidx(op, l, i, j, kk);
-                const Cdf d = {t.dre, conj ? df_neg(t.im[m]) : t.im[m]};
-                out = cdf_add(cdf_scale(t.hinv2, sum), cdf_mul(d, X));
-            }
-            const double2 yv = make_double2((double)out.re.x + (double)out.re.y, (double)out.im.x + (double)out.im.y);
-            y[l] = yv;
-            const double2 wv = w[l];
-            if (MODE == 1) {          // conj(w) y
-                a += wv.x * yv.x + wv.y * yv.y;
-                b += wv.x * yv.y - wv.y * yv.x;
-            } else {                  // conj(y) w and |y|^2
-                a += yv.x * wv.x + yv.y * wv.y;
-                b += yv.x * wv.y - yv.y * wv.x;
-                c += yv.x * yv.x + yv.y * yv.y;
-            }
+__global__ void __launch_bounds__(kFusedThreads) k_apply_bicg_df(Op<double> op, DfTab t, const XT* __restrict__ x,
+                                                                 double2* __restrict__ y, const double2* __restrict__ w,
+                                                                 int conj, double2* sc, double* parts,
+                                                                 unsigned* counter) {
+    double2 a = make_double2(0, 0);
+    double c = 0;
+#pragma unroll
+    for (int u = 0; u < BN; ++u) {
+        const long long l = (blockIdx.x * (long long)BN + u) * kFusedThreads + threadIdx.x;
+        if (l >= op.N) break;
+        const unsigned code = op.nbm[l];
+        const Cdf X = cdf_load(x, l);
+        const double2 wv = w[l];
+        Cdf out;
+        if (code & kMasked) {
+            out = X;
+        } else {
+            const Cdf sum = nbr_sum_any(op, x, l, code);
+            const int m = op.lidx[l];
+            const Cdf d = {t.dre, conj ? df_neg(t.im[m]) : t.im[m]};
+            out = cdf_add(cdf_scale(t.hinv2, sum), cdf_mul(d, X));
         }
+        const double2 yv = make_double2(pair_to_f64(out.re.x, out.re.y), pair_to_f64(out.im.x, out.im.y));
+        y[l] = yv;
+        a = MODE == 1 ? cfmac(wv, yv, a) : cfmac(yv, wv, a);
+        if (MODE == 2) c = cnorm2(yv, c);
     }
-    const int tid = threadIdx.x + BX * threadIdx.y;
-    const unsigned nblk = gridDim.x * gridDim.y * gridDim.z;
-    const unsigned bid = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
-    __shared__ double red[3][BX * BY / 32];
-    for (int o = 16; o > 0; o >>= 1) {
-        a += __shfl_xor_sync(0xffffffffu, a, o);
-        b += __shfl_xor_sync(0xffffffffu, b, o);
-        c += __shfl_xor_sync(0xffffffffu, c, o);
-    }
-    if ((tid & 31) == 0) { red[0][tid >> 5] = a; red[1][tid >> 5] = b; red[2][tid >> 5] = c; }
-    __syncthreads();
-    if (tid == 0) {
-        double sa = 0, sb = 0, scc = 0;
-        for (int q = 0; q < BX * BY / 32; ++q) { sa += red[0][q]; sb += red[1][q]; scc += red[2][q]; }
-        parts[3 * bid + 0] = sa;
-        parts[3 * bid + 1] = sb;
-        parts[3 * bid + 2] = scc;
-    }
-    if (last_block_done(counter, nblk)) {
-        double tot[3];
-        sum_parts<3>(parts, nblk, tid, tot);
-        if (tid == 0) {
-            if (MODE == 1) bicg_alpha(sc, make_double2(tot[0], tot[1]));
-            else bicg_omega(sc, make_double2(tot[0], tot[1]), tot[2]);
-            *counter = 0;
-        }
-    }
+    bicg_finish<MODE>(a, c, threadIdx.x, sc, parts, counter);
 }
 
 // ---- the red-black part of the trunk-basis hybrid cycle in one cooperative
@@ -1321,13 +1284,6 @@ __device__ __forceinline__ void grid_barrier(const GridBar& b) {
     __syncthreads();
 }
 
-__device__ __forceinline__ int colour_of(long long l, int n) {
-    const unsigned ul = (unsigned)l, un = (unsigned)n;
-    const unsigned r = ul / un;          // row index j + n k
-    const unsigned kk = r / un;
-    return (int)(((ul - r * un) + (r - kk * un) + kk) & 1u);
-}
-
 __device__ __forceinline__ Cdf cdf_load_cg(const float4* p, long long l) {
     const float4 v = __ldcg(p + l);
     return {make_float2(v.x, v.y), make_float2(v.z, v.w)};
@@ -1373,13 +1329,12 @@ __global__ void __launch_bounds__(kCycleThreads, 1) k_cycle_df(Op<double> op, Df
         if (PRE == 0) {
             fv = f[l];
         } else if (PRE == 1) {
-            const double2 tt = csub(w[l], cmul(c2, v[l]));
-            fv = cadd(f[l], cmul(c1, tt));
+            fv = cfma(c1, cfma(make_double2(-c2.x, -c2.y), v[l], w[l]), f[l]);
             w[l] = fv;
         } else {
-            fv = csub(f[l], cmul(c1, v[l]));
+            fv = cfma(make_double2(-c1.x, -c1.y), v[l], f[l]);
             w[l] = fv;
-            acc += fv.x * fv.x + fv.y * fv.y;
+            acc = cnorm2(fv, acc);
         }
         const Cdf F = {df_split(fv.x), df_split(fv.y)};
         __stcg(fs + l, cdf_pack(F));
@@ -1391,21 +1346,25 @@ __global__ void __launch_bounds__(kCycleThreads, 1) k_cycle_df(Op<double> op, Df
         __stcg(xs + l, cdf_pack(x));
     }
     if (PRE == 2) {
-        __shared__ double red[kCycleThreads / 32];
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double b = 0.0;
-            for (int q = 0; q < kCycleThreads / 32; ++q) b += red[q];
-            parts[blockIdx.x] = b;
+        // fixed-order tree over the block (see block_tree for why not butterflies)
+        __shared__ double red[kCycleThreads / 2];
+        for (int h = kCycleThreads / 2; h >= 32; h >>= 1) {
+            if ((int)threadIdx.x >= h && (int)threadIdx.x < 2 * h) red[threadIdx.x - h] = acc;
+            __syncthreads();
+            if ((int)threadIdx.x < h) acc += red[threadIdx.x];
+            __syncthreads();
+        }
+        if (threadIdx.x < 32) {
+            for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+            if (threadIdx.x == 0) parts[blockIdx.x] = acc;
         }
     }
     grid_barrier(bar);
-    if (PRE == 2 && blockIdx.x == 0 && threadIdx.x == 0) {
+    if (PRE == 2 && blockIdx.x == 0 && threadIdx.x < 32) {
         double sn = 0.0;
-        for (unsigned b = 0; b < gridDim.x; ++b) sn += __ldcg(parts + b);
-        bicg_snorm(sc, sn, tol_abs);
+        for (unsigned b = threadIdx.x; b < gridDim.x; b += 32) sn += __ldcg(parts + b);
+        for (int o = 16; o > 0; o >>= 1) sn += __shfl_down_sync(0xffffffffu, sn, o);
+        if (threadIdx.x == 0) bicg_snorm(sc, sn, tol_abs);
     }
     for (int q = 0; q < n_r; ++q) {
         for (int colour = (q == 0 ? 1 : 0); colour < 2; ++colour) {
@@ -1640,10 +1599,17 @@ dim3 grid_for(int dim, int n, int xdiv = 1, int zdiv = 1) {
 
 }  // namespace
 
+namespace {
+long long node_count(int dim, int n) { return dim == 3 ? (long long)n * n * n : (long long)n * n; }
+// blocks of BX * BY threads, one element each
+unsigned flat_blocks(long long count) { return (unsigned)((count + BX * BY - 1) / (BX * BY)); }
+}  // namespace
+
 int bicg_grid_blocks(int dim, int n) {
-    dim3 g = grid_for(dim, n, 1, 2);
-    return g.x * g.y * g.z;
+    return (int)((node_count(dim, n) + BN * kFusedThreads - 1) / (BN * kFusedThreads));
 }
+
+constexpr int ZC = 16;      // largest z chunk
 
 // z chunk of a 3D marching grid with xy blocks per plane: the largest of 16, 8,
 // 4, 2, 1 that leaves at least four blocks per SM
@@ -1656,6 +1622,25 @@ int march_zc(long long xy, int n) {
 int apply_zc(int dim, int n) {
     if (dim != 3) return 1;
     return march_zc((long long)((n + BX - 1) / BX) * ((n + BY - 1) / BY), n);
+}
+
+// grid of k_apply_z: the z chunk for which the busiest SM walks the fewest planes (its
+// share of the blocks, times their planes and one for the start of each), so that the
+// blocks come out in whole rounds (129^3: 765 blocks for 608 slots were two rounds)
+dim3 applyz_grid(int n, int* zc) {
+    const long long per = ((long long)n * n + AZ - 1) / AZ;
+    long long best = 0;
+    *zc = 1;
+    for (int chunks = 1; chunks <= n; ++chunks) {
+        const int z = (n + chunks - 1) / chunks;
+        if (z < 4 && chunks > 1) break;
+        const long long blocks = per * ((n + z - 1) / z), cost = (blocks + 151) / 152 * (z + 1);
+        if (best == 0 || cost < best) {
+            best = cost;
+            *zc = z;
+        }
+    }
+    return dim3((unsigned)per, (n + *zc - 1) / *zc);
 }
 
 // grid of the two-nodes-per-thread complex64 kernels
@@ -1674,14 +1659,25 @@ bool pair_ok(const Op<float>& op, const void* a, const void* b, const void* c) {
            aligned16(op.k2) && aligned16(op.invd);
 }
 
-// an upper bound on the partial sums any operator launch writes (buffer sizing)
-int apply_grid_blocks(int dim, int n) {
+// blocks of the table-free operator (one partial sum each)
+int noalloc_grid_blocks(int dim, int n) {
     dim3 g = grid_for(dim, n, 1, apply_zc(dim, n));
     long long b = (long long)g.x * g.y * g.z;
     if (dim == 3 && n % 2 == 0) {
         int zc;
         dim3 p = pair_grid(n, &zc);
         b = std::max(b, (long long)p.x * p.y * p.z);
+    }
+    return (int)b;
+}
+
+// an upper bound on the partial sums any operator launch writes (buffer sizing)
+int apply_grid_blocks(int dim, int n) {
+    long long b = noalloc_grid_blocks(dim, n);
+    if (dim == 3) {
+        int zc;
+        const dim3 g = applyz_grid(n, &zc);
+        b = std::max(b, (long long)g.x * g.y);
     }
     return (int)b;
 }
@@ -1706,18 +1702,20 @@ int launch_apply(const Op<R>& op, const typename CT<R>::T* x, const typename CT<
             return (int)(g.x * g.y * g.z);
         }
     }
+    if (op.dim == 3 && op.nbm && op.lidx && !op.face) {
+        int zc;
+        const dim3 g = applyz_grid(op.n, &zc);
+        if (resid) {
+            if (partials) k_apply_z<R, true, true><<<g, AZ, 0, s>>>(op, zc, x, f, y, partials, conj);
+            else k_apply_z<R, true, false><<<g, AZ, 0, s>>>(op, zc, x, f, y, partials, conj);
+        } else {
+            if (partials) k_apply_z<R, false, true><<<g, AZ, 0, s>>>(op, zc, x, f, y, partials, conj);
+            else k_apply_z<R, false, false><<<g, AZ, 0, s>>>(op, zc, x, f, y, partials, conj);
+        }
+        return (int)(g.x * g.y);
+    }
     const int zc = apply_zc(op.dim, op.n);
     dim3 g = grid_for(op.dim, op.n, 1, zc), b(BX, BY);
-    if (op.dim == 3 && op.nbm && op.lidx && !op.face) {
-        if (resid) {
-            if (partials) k_apply_z<R, true, true><<<g, b, 0, s>>>(op, zc, x, f, y, partials, conj);
-            else k_apply_z<R, true, false><<<g, b, 0, s>>>(op, zc, x, f, y, partials, conj);
-        } else {
-            if (partials) k_apply_z<R, false, true><<<g, b, 0, s>>>(op, zc, x, f, y, partials, conj);
-            else k_apply_z<R, false, false><<<g, b, 0, s>>>(op, zc, x, f, y, partials, conj);
-        }
-        return (int)(g.x * g.y * g.z);
-    }
     // 2D, or an operator without the per-node tables (the allocation-free path)
     if (resid) {
         if (partials) k_apply<R, true, true><<<g, b, 0, s>>>(op, zc, x, f, y, partials, conj);
@@ -1744,9 +1742,9 @@ void launch_jacobi(const Op<R>& op, double omega, const typename CT<R>::T* f, co
             return;
         }
     }
-    dim3 g = grid_for(op.dim, op.n, 1, 2), b(BX, BY);
-    if (xzero) k_jacobi<R, true><<<g, b, 0, s>>>(op, (R)omega, f, xin, xout, conj);
-    else k_jacobi<R, false><<<g, b, 0, s>>>(op, (R)omega, f, xin, xout, conj);
+    const unsigned g = flat_blocks(op.N);
+    if (xzero) k_jacobi<R, true><<<g, BX * BY, 0, s>>>(op, (R)omega, f, xin, xout, conj);
+    else k_jacobi<R, false><<<g, BX * BY, 0, s>>>(op, (R)omega, f, xin, xout, conj);
 }
 
 // sweeps per launch of the tiled form for this operator, 0 where it does not apply (3D,
@@ -1790,9 +1788,10 @@ void launch_rbgs_half(const Op<R>& op, int colour, const typename CT<R>::T* f, t
             return;
         }
     }
-    dim3 g = grid_for(op.dim, op.n, 2, 1), b(BX, BY);
-    if (xzero) k_rbgs<R, true><<<g, b, 0, s>>>(op, colour, f, x, conj, (R)omega);
-    else k_rbgs<R, false><<<g, b, 0, s>>>(op, colour, f, x, conj, (R)omega);
+    const unsigned g = flat_blocks((op.N + 1) / 2);
+    const bool sor = (R)omega != (R)1;
+    if (xzero) k_rbgs<R, true><<<g, BX * BY, 0, s>>>(op, colour, f, x, conj, (R)omega, sor);
+    else k_rbgs<R, false><<<g, BX * BY, 0, s>>>(op, colour, f, x, conj, (R)omega, sor);
 }
 
 bool launch_red_residual32(const Op<float>& op, const float2* f, const float2* x, float2* r_red, int conj,
@@ -1899,14 +1898,14 @@ void launch_node_pack(const Op<float>& op, uint16_t* ncl, cudaStream_t s) {
 
 void launch_apply_bicg_df(const Op<double>& op, const DfTab& t, int mode, const float4* x, double2* y,
                           const double2* w, int conj, double2* sc, double* parts, unsigned* counter, cudaStream_t s) {
-    dim3 g = grid_for(op.dim, op.n, 1, 2), b(BX, BY);
+    const int g = bicg_grid_blocks(op.dim, op.n), b = kFusedThreads;
     if (mode == 1) k_apply_bicg_df<1, float4><<<g, b, 0, s>>>(op, t, x, y, w, conj, sc, parts, counter);
     else k_apply_bicg_df<2, float4><<<g, b, 0, s>>>(op, t, x, y, w, conj, sc, parts, counter);
 }
 
 void launch_apply_bicg(const Op<double>& op, int mode, const double2* x, double2* y, const double2* w, int conj,
                        double2* sc, double* parts, unsigned* counter, cudaStream_t s) {
-    dim3 g = grid_for(op.dim, op.n, 1, 2), b(BX, BY);
+    const int g = bicg_grid_blocks(op.dim, op.n), b = kFusedThreads;
     if (mode == 1) k_apply_bicg<1><<<g, b, 0, s>>>(op, x, y, w, conj, sc, parts, counter);
     else k_apply_bicg<2><<<g, b, 0, s>>>(op, x, y, w, conj, sc, parts, counter);
 }
@@ -1926,7 +1925,7 @@ template void launch_rbgs_half<float>(const Op<float>&, int, const float2*, floa
 
 void launch_residual_red(const Op<double>& op, const double2* z, const double2* v, double2* r_red, int conj,
                          cudaStream_t s) {
-    k_residual_red<<<grid_for(op.dim, op.n, 2, 1), dim3(BX, BY), 0, s>>>(op, z, v, r_red, conj);
+    k_residual_red<<<flat_blocks((op.N + 1) / 2), BX * BY, 0, s>>>(op, z, v, r_red, conj);
 }
 
 void launch_rbgs_df_first(const Op<double>& op, const DfTab& t, const double2* f, float4* fs, float4* xs, int conj,

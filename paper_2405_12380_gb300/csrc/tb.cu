@@ -446,8 +446,9 @@ __global__ void __launch_bounds__(1024) k_gauss_jordan(const double* __restrict_
 // converted back to FP64 once per sum.
 
 __device__ __forceinline__ void split_f64(double x, float& hi, float& lo) {
-    hi = __double2float_rn(x);
-    lo = __double2float_rn(x - (double)hi);
+    const float2 p = f64_to_pair(x);
+    hi = p.x;
+    lo = p.y;
 }
 
 // (sh, sl) += (ah + al) * (bh + bl), dropping al*bl (~2^-48 relative)
@@ -538,7 +539,7 @@ __global__ void __launch_bounds__(PJ_T, 2) k_project_df(const float2* __restrict
         pair_warp_sum(acc[c][2], acc[c][3]);
         if (lane == 0 && j < k)
             partials[(long long)blockIdx.x * k + j] =
-                make_double2((double)acc[c][0] + (double)acc[c][1], (double)acc[c][2] + (double)acc[c][3]);
+                make_double2(pair_to_f64(acc[c][0], acc[c][1]), pair_to_f64(acc[c][2], acc[c][3]));
     }
 }
 
@@ -675,14 +676,14 @@ __global__ void __launch_bounds__(256) k_prolong_df(const float2* __restrict__ Q
             float s1 = b.z + a2;
             bb = s1 - b.z;
             const float e1 = (b.z - (s1 - bb)) + (a2 - bb) + (b.w + a3);
-            z[l] = make_double2((double)s0 + (double)e0, (double)s1 + (double)e1);
+            z[l] = make_double2(pair_to_f64(s0, e0), pair_to_f64(s1, e1));
             if (zdf) {
                 const float h0 = s0 + e0, h1 = s1 + e1;
                 zdf[l] = make_float4(h0, e0 - (h0 - s0), h1, e1 - (h1 - s1));
             }
         } else {
             double2 zz = z[l];
-            z[l] = make_double2(zz.x + ((double)a0 + (double)a1), zz.y + ((double)a2 + (double)a3));
+            z[l] = make_double2(zz.x + pair_to_f64(a0, a1), zz.y + pair_to_f64(a2, a3));
         }
     }
 }
