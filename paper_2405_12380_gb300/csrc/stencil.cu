@@ -176,7 +176,8 @@ __device__ __forceinline__ double norm_acc(float2 a, double s) { return s + ((do
 // once, two planes ahead of its use), the x-neighbours from warp shuffles (fluid nodes are
 // interior, so theirs are the neighbours in the plane's order; the two ends of the warp
 // load from memory), the y-neighbours from L1 or L2.  Bound by the FP64 pipe in complex128
-// (16 instructions a node, 20 with the residual and its norm).
+// (16 instructions a node, 20 with the residual and its norm): the residual with its norm
+// at 129^3 141 -> 102 us (ncu, cold), 68 us at the pipe's rate.
 constexpr int AZ = 256;
 
 template <typename R, bool RESID, bool NORM>
@@ -1009,8 +1010,8 @@ __device__ __forceinline__ int colour_of(long long l, int n) {
 // One thread per node pair (2m, 2m + 1), which holds one node of each colour (rows of even
 // length start on even l; for odd n the colour is the parity of l), in the flat order, so
 // that every lane has a node: one row per warp left a quarter of the lanes of 96-node rows
-// idle, and the kernel is bound by the FP64 pipe (16 instructions a node).  96^3: 24.2 us
-// a half-sweep before.
+// idle, and the kernel is bound by the FP64 pipe (16 instructions a node).  96^3: 24.2 ->
+// 19.1 us a half-sweep (ncu, cold).
 template <typename R, bool XZERO>
 __global__ void __launch_bounds__(BX * BY) k_rbgs(Op<R> op, int colour, const typename CT<R>::T* __restrict__ f,
                                                   typename CT<R>::T* x, int conj, R omega, bool sor) {
