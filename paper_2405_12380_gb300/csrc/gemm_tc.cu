@@ -2,18 +2,28 @@
 // for the dense layers of the DeepONet (App. B): C = alpha op(A) op(B) + beta C with
 // FP32 row-major operands, as nn_gemm, but with op(A) and op(B) rounded to BF16.
 //
-// Structure (one CTA per 128 x 128 tile of C, 64-deep K steps, a four-stage ring):
-//  - the operands are first converted to BF16 "K-major" copies (op(A) as M x K rows,
-//    op(B)^T as N x K rows), zero-padded to multiples of 128 rows and 64 columns so
-//    that every TMA box lies inside the copy and starts on a 16-byte boundary;
-//  - warp 0: one elected thread loads the A and B boxes of a stage with
-//    cp.async.bulk.tensor (128-byte swizzle) onto the stage's "full" mbarrier;
-//  - warp 1: one elected thread issues tcgen05.mma.kind::f16 (M = 128, N = 128,
-//    K = 16 per instruction, four per stage) into a TMEM accumulator and commits
-//    each stage to its "empty" mbarrier, the last one to the "done" mbarrier;
-//  - warp 2 allocates and frees the 128 TMEM columns;
+// Structure:
+//  - both operands are first converted to BF16 "K-major" copies (op(B)^T as N x K rows,
+//    op(A) as M x K rows) in one launch, zero-padded to multiples of 128 rows and 64
+//    columns so that every TMA box lies inside the copy and starts on a 16-byte boundary;
+//  - a CTA owns 128 columns of C (the M = 128 side of the MMA, so that the 32 lanes of an
+//    epilogue warp hold neighbouring columns and its stores coalesce) and TN rows of C (the
+//    N side): 16 to 128, as few as leave about one CTA per SM.  K is not split: the sum of
+//    each value stays one chain, whatever the tile;
+//  - warp 0: one elected thread loads the two boxes of a 64-deep K step with
+//    cp.async.bulk.tensor (128-byte swizzle) onto the stage's "full" mbarrier; the ring has
+//    as many stages as K has steps, up to what 200 KB hold (11 with TN = 16);
+//  - warp 1: one elected thread issues tcgen05.mma.kind::f16 (K = 16 per instruction, four
+//    per stage) into a TMEM accumulator and commits each stage to its "empty" mbarrier, the
+//    last one to the "done" mbarrier;
+//  - warp 2 allocates and frees the TMEM columns;
 //  - warps 4-7 (one per quarter of the TMEM lanes) read the accumulator with
 //    tcgen05.ld and write alpha D + beta C for the valid rows and columns.
+// What bounds it: the branch's first layer (64 x 256 x 128000 at 40^3) is a chain of 8000
+// dependent MMAs per value on 8 CTAs; it takes about 80 ns a link, 0.9 -> 0.66 ms (ncu,
+// cold).  Splitting K would shorten it but change the last bits of the activations, which
+// the next layer rounds to BF16.  Its weight gradient (K = 64, 256 x 128000 values) is
+// bound by the stores: 197 -> 32 us with lanes along C's rows.
 // Every mbarrier wait is bounded: a wait that runs out records an error flag and the
 // thread goes on (the result is then garbage but the launch ends); the host reads
 // the flag with nn_gemm_bf16_status.
@@ -21,6 +31,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "helm_internal.cuh"
@@ -29,9 +40,9 @@ namespace helm {
 
 namespace {
 
-constexpr int TBM = 128, TBN = 128, TBK = 64, STAGES = 4;
+constexpr int TBM = 128, TBK = 64, MAX_STAGES = 16;
 constexpr int TC_THREADS = 256;
-constexpr unsigned kStageBytes = (TBM + TBN) * TBK * 2;        // 32 KiB
+constexpr unsigned kRingBytes = 200 * 1024;                    // shared memory of the stages, at most
 constexpr unsigned kWaitLimit = 1u << 26;
 
 __device__ int g_tc_error;
@@ -53,12 +64,16 @@ __device__ __forceinline__ bool mbar_try(uint64_t* b, unsigned parity) {
         : "memory");
     return ok != 0;
 }
-// bounded wait for the phase of the given parity; false (and the error flag) on a timeout
+// bounded wait for the phase of the given parity; false (and the error flag) on a timeout.
+// Once a wait of the launch has given up the others do so too, at their next look at the
+// flag.  They look only while waiting in vain: the flag lies in global memory, and a look
+// before every wait cost the MMA thread 0.4 us per K step (0.46 us a step whatever the
+// tile or the number of stages).
 __device__ __forceinline__ bool mbar_wait(uint64_t* b, unsigned parity) {
-    // after one timeout in the launch the other waits give up at once
-    if (*reinterpret_cast<volatile int*>(&g_tc_error)) return false;
-    for (unsigned it = 0; it < kWaitLimit; ++it)
+    for (unsigned it = 1; it <= kWaitLimit; ++it) {
         if (mbar_try(b, parity)) return true;
+        if ((it & 1023u) == 0 && *reinterpret_cast<volatile int*>(&g_tc_error)) return false;
+    }
     atomicExch(&g_tc_error, 1);
     return false;
 }
@@ -82,21 +97,26 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int m, int n) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
 
-__global__ void __launch_bounds__(TC_THREADS, 1)
-    k_gemm_bf16_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, int M, int N,
-                   int Kp, float alpha, float beta, float* __restrict__ C, int ldc) {
+// C (M x N) = alpha A B^T + beta C from the K-major copies; mapN: op(B)^T, mapM: op(A)
+template <int TN>
+__global__ void __launch_bounds__(TC_THREADS)
+    k_gemm_bf16_tc(const __grid_constant__ CUtensorMap mapN, const __grid_constant__ CUtensorMap mapM, int M, int N,
+                   int Kp, int stages, float alpha, float beta, float* __restrict__ C, int ldc) {
+    constexpr unsigned kNBytes = TBM * TBK * 2, kMBytes = TN * TBK * 2;
+    constexpr unsigned kCols = TN < 32 ? 32 : TN;          // TMEM columns (at least 32 are allocated)
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     // 1024-byte alignment of the stage buffers (the swizzle atom)
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint8_t* sA = smem;
-    uint8_t* sB = smem + STAGES * TBM * TBK * 2;
-    __shared__ uint64_t full[STAGES], empty[STAGES], done;
+    uint8_t* sN = smem;
+    uint8_t* sM = smem + stages * kNBytes;
+    __shared__ uint64_t full[MAX_STAGES], empty[MAX_STAGES], done;
     __shared__ uint32_t tmem_base;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int m0 = blockIdx.y * TBM, n0 = blockIdx.x * TBN;
+    const int tiles_m = (M + TN - 1) / TN;
+    const int m0 = (blockIdx.x % tiles_m) * TN, n0 = (blockIdx.x / tiles_m) * TBM;
     const int nk = Kp / TBK;
     if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES; ++s) {
+        for (int s = 0; s < stages; ++s) {
             mbar_init(&full[s], 1);
             mbar_init(&empty[s], 1);
         }
@@ -106,7 +126,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     }
     if (warp == 2) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(&tmem_base)),
-                     "r"(TBN)
+                     "r"(kCols)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -117,21 +137,27 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 
     if (warp == 0 && lane == 0) {
         // producer
+        int s = 0;
+        unsigned parity = 1;                               // (the first round finds every stage empty)
         for (int kb = 0; kb < nk; ++kb) {
-            const int s = kb % STAGES;
-            if (kb >= STAGES) mbar_wait(&empty[s], ((kb / STAGES) - 1) & 1);
-            mbar_expect_tx(&full[s], kStageBytes);
-            tma_load_2d(sA + s * TBM * TBK * 2, &mapA, kb * TBK, m0, &full[s]);
-            tma_load_2d(sB + s * TBN * TBK * 2, &mapB, kb * TBK, n0, &full[s]);
+            if (kb >= stages) mbar_wait(&empty[s], parity);
+            mbar_expect_tx(&full[s], kNBytes + kMBytes);
+            tma_load_2d(sN + s * kNBytes, &mapN, kb * TBK, n0, &full[s]);
+            tma_load_2d(sM + s * kMBytes, &mapM, kb * TBK, m0, &full[s]);
+            if (++s == stages) {
+                s = 0;
+                parity ^= 1u;
+            }
         }
     } else if (warp == 1 && lane == 0) {
         // MMA issuer
-        constexpr uint32_t idesc = idesc_bf16(TBM, TBN);
+        constexpr uint32_t idesc = idesc_bf16(TBM, TN);
+        int s = 0;
+        unsigned parity = 0;
         for (int kb = 0; kb < nk; ++kb) {
-            const int s = kb % STAGES;
-            mbar_wait(&full[s], (kb / STAGES) & 1);
+            mbar_wait(&full[s], parity);
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint64_t da = smem_desc(sA + s * TBM * TBK * 2), db = smem_desc(sB + s * TBN * TBK * 2);
+            const uint64_t da = smem_desc(sN + s * kNBytes), db = smem_desc(sM + s * kMBytes);
 #pragma unroll
             for (int k = 0; k < TBK / 16; ++k) {
                 // K = 16 BF16 = 32 bytes further along the swizzled 128-byte rows
@@ -146,37 +172,38 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                              su32(&empty[s]))
                          : "memory");
+            if (++s == stages) {
+                s = 0;
+                parity ^= 1u;
+            }
         }
         asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(su32(&done))
                      : "memory");
     } else if (warp >= 4) {
-        // epilogue: warp 4 + q reads TMEM lanes 32 q .. 32 q + 31 (rows of the tile)
+        // epilogue: warp 4 + q reads TMEM lanes 32 q .. 32 q + 31 (columns n of the tile)
         const int q = warp - 4;
         mbar_wait(&done, 0);
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const int row = m0 + 32 * q + lane;
-        for (int c0 = 0; c0 < TBN; c0 += 32) {
-            uint32_t v[32];
+        const int n = n0 + 32 * q + lane;
+        for (int c0 = 0; c0 < TN; c0 += 16) {
+            uint32_t v[16];
             const uint32_t taddr = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)c0;
             asm volatile(
-                "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
-                "%14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+                "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
+                "%14, %15}, [%16];"
                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-                  "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
-                  "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]),
-                  "=r"(v[23]), "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]),
-                  "=r"(v[30]), "=r"(v[31])
+                  "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
                 : "r"(taddr)
                 : "memory");
             asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            if (row < M) {
-                float* Cr = C + (long long)row * ldc;
+            if (n < N) {
 #pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    const int col = n0 + c0 + j;
-                    if (col < N) {
+                for (int j = 0; j < 16; ++j) {
+                    const int m = m0 + c0 + j;
+                    if (m < M) {
+                        float* c = C + (long long)m * ldc + n;
                         const float d = __uint_as_float(v[j]);
-                        Cr[col] = beta == 0.f ? alpha * d : fmaf(alpha, d, beta * Cr[col]);
+                        *c = beta == 0.f ? alpha * d : fmaf(alpha, d, beta * *c);
                     }
                 }
             }
@@ -185,21 +212,85 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (warp == 2) {
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TBN) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kCols) : "memory");
     }
 }
 
-// dst (rows_p x Kp, BF16, row-major, zero padding) from the FP32 operand: element
-// (r, k) of op(X) is X[r * ld + k] (trans = 0) or X[k * ld + r] (trans = 1)
-__global__ void k_to_bf16_kmajor(const float* __restrict__ X, int ld, int trans, int rows, int K,
-                                 __nv_bfloat16* __restrict__ dst, int rows_p, int Kp) {
-    const long long total = (long long)rows_p * Kp;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
-         e += (long long)gridDim.x * blockDim.x) {
-        const int r = (int)(e / Kp), k = (int)(e - (long long)r * Kp);
-        float v = 0.f;
-        if (r < rows && k < K) v = trans ? X[(long long)k * ld + r] : X[(long long)r * ld + k];
-        dst[e] = __float2bfloat16_rn(v);
+// one operand to convert: dst (rows_p x Kp, BF16, row-major, zero padding); element (r, k)
+// is X[r * ld + k] (kc) or X[k * ld + r]; vec: 16-byte rows and base
+struct PackOp {
+    const float* X;
+    __nv_bfloat16* dst;
+    int ld, rows, rows_p, kc, vec;
+};
+
+__device__ __forceinline__ uint4 bf16x8_of(const float* v) {
+    uint4 u;
+    __nv_bfloat162 p[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) p[q] = __floats2bfloat162_rn(v[2 * q], v[2 * q + 1]);
+    u.x = *reinterpret_cast<const uint32_t*>(&p[0]);
+    u.y = *reinterpret_cast<const uint32_t*>(&p[1]);
+    u.z = *reinterpret_cast<const uint32_t*>(&p[2]);
+    u.w = *reinterpret_cast<const uint32_t*>(&p[3]);
+    return u;
+}
+
+// four values along the contiguous side, zeros past n
+__device__ __forceinline__ float4 load4(const float* p, int n, bool vec) {
+    if (n >= 4 && vec) return __ldg(reinterpret_cast<const float4*>(p));
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (n > 0) v.x = __ldg(p);
+    if (n > 1) v.y = __ldg(p + 1);
+    if (n > 2) v.z = __ldg(p + 2);
+    if (n > 3) v.w = __ldg(p + 3);
+    return v;
+}
+
+// Both operands to K-major BF16, 64 rows x 64 k a block, 16 bytes per load and store: the
+// copies stream at HBM's rate.  An operand stored with its rows contiguous goes through
+// shared memory.  22 launches of a training step at 40^3 take about 180 us; as 44 launches
+// with one element per thread, a 64-bit division each and reads a whole row apart, 476 us.
+__global__ void __launch_bounds__(256) k_pack_bf16(PackOp a, PackOp b, int K, int Kp, long long blocks_a) {
+    __shared__ float tile[64][65];
+    const bool second = blockIdx.x >= blocks_a;
+    const PackOp o = second ? b : a;
+    const long long blk = blockIdx.x - (second ? blocks_a : 0);
+    const int kt = Kp / TBK;
+    const int r0 = (int)(blk / kt) * 64, k0 = (int)(blk % kt) * TBK, t = threadIdx.x;
+    const int c = t & 7;                                   // chunk of eight k of the rows t / 8, t / 8 + 32
+    float v[2][8];
+    if (o.kc) {
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int r = r0 + (t >> 3) + 32 * u, k = k0 + 8 * c;
+            const int n = r < o.rows ? K - k : 0;
+            const float* p = o.X + (long long)r * o.ld + k;
+            const float4 x = load4(p, n, o.vec), y = load4(p + 4, n - 4, o.vec);
+            v[u][0] = x.x; v[u][1] = x.y; v[u][2] = x.z; v[u][3] = x.w;
+            v[u][4] = y.x; v[u][5] = y.y; v[u][6] = y.z; v[u][7] = y.w;
+        }
+    } else {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int k = (t >> 4) + 16 * u, r = 4 * (t & 15);
+            const int n = k0 + k < K ? o.rows - (r0 + r) : 0;
+            const float4 x = load4(o.X + (long long)(k0 + k) * o.ld + r0 + r, n, o.vec);
+            tile[r][k] = x.x;
+            tile[r + 1][k] = x.y;
+            tile[r + 2][k] = x.z;
+            tile[r + 3][k] = x.w;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+            for (int q = 0; q < 8; ++q) v[u][q] = tile[(t >> 3) + 32 * u][8 * c + q];
+    }
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        const int r = r0 + (t >> 3) + 32 * u;
+        if (r < o.rows_p) *reinterpret_cast<uint4*>(o.dst + (long long)r * Kp + k0 + 8 * c) = bf16x8_of(v[u]);
     }
 }
 
@@ -221,25 +312,43 @@ EncodeFn encode_fn() {
     return fn;
 }
 
-bool make_map(CUtensorMap* map, const void* base, int rows_p, int Kp) {
+bool make_map(CUtensorMap* map, const void* base, int rows_p, int Kp, int box_rows) {
     EncodeFn fn = encode_fn();
     if (!fn) return false;
     const cuuint64_t dims[2] = {(cuuint64_t)Kp, (cuuint64_t)rows_p};
     const cuuint64_t strides[1] = {(cuuint64_t)Kp * 2};
-    const cuuint32_t box[2] = {TBK, TBM};
+    const cuuint32_t box[2] = {TBK, (cuuint32_t)box_rows};
     const cuuint32_t estr[2] = {1, 1};
     return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// per-device workspace of the BF16 copies (grown on demand, held until exit)
+// per-device workspace of the BF16 copies (grown on demand, held until exit).  Each call
+// first waits for the last one's event, so that calls on different streams take turns (not
+// while being captured: a captured call is ordered by its graph)
 struct Ws {
     void* p = nullptr;
     size_t bytes = 0;
+    cudaEvent_t ev = nullptr;
+    bool used = false;
 };
 std::mutex g_ws_mutex;
 Ws g_ws[64];
+
+template <int TN>
+cudaError_t gemm_tc(const CUtensorMap& mn, const CUtensorMap& mm, int M, int N, int Kp, float alpha, float beta, float* C,
+                    int ldc, cudaStream_t s) {
+    constexpr unsigned stage = (TBM + TN) * TBK * 2;
+    const int stages = std::min(std::min(Kp / TBK, MAX_STAGES), (int)(kRingBytes / stage));
+    const size_t smem = (size_t)stages * stage + 1024;
+    const cudaError_t e =
+        cudaFuncSetAttribute(k_gemm_bf16_tc<TN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kRingBytes + 1024));
+    if (e != cudaSuccess) return e;
+    const long long tiles = (long long)((M + TN - 1) / TN) * ((N + TBM - 1) / TBM);
+    k_gemm_bf16_tc<TN><<<(unsigned)tiles, TC_THREADS, smem, s>>>(mn, mm, M, N, Kp, stages, alpha, beta, C, ldc);
+    return cudaGetLastError();
+}
 
 }  // namespace
 
@@ -252,7 +361,7 @@ extern "C" helm_status nn_gemm_bf16(int transA, int transB, int M, int N, int K,
     if (M < 0 || N < 0 || K < 0 || !A || !B || !C || ldc < N) return HELM_BAD_ARG;
     if (M == 0 || N == 0) return HELM_OK;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const int Mp = (M + TBM - 1) / TBM * TBM, Np = (N + TBN - 1) / TBN * TBN;
+    const int Mp = (M + TBM - 1) / TBM * TBM, Np = (N + TBM - 1) / TBM * TBM;
     const int Kp = K == 0 ? TBK : (K + TBK - 1) / TBK * TBK;
     const size_t need = ((size_t)Mp + Np) * Kp * 2;
     int dev = 0;
@@ -272,24 +381,35 @@ extern "C" helm_status nn_gemm_bf16(int transA, int transB, int M, int N, int K,
         }
         w.bytes = need;
     }
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) return HELM_CUDA_ERROR;
+    const bool ordered = cap == cudaStreamCaptureStatusNone;
+    if (!w.ev && cudaEventCreateWithFlags(&w.ev, cudaEventDisableTiming) != cudaSuccess) return HELM_CUDA_ERROR;
+    if (ordered && w.used && cudaStreamWaitEvent(s, w.ev, 0) != cudaSuccess) return HELM_CUDA_ERROR;
     __nv_bfloat16* Ab = static_cast<__nv_bfloat16*>(w.p);
     __nv_bfloat16* Bb = Ab + (size_t)Mp * Kp;
-    k_to_bf16_kmajor<<<4 * 152, 256, 0, s>>>(A, lda, transA, M, K, Ab, Mp, Kp);
+    auto vec = [](const float* p, int ld) { return ld % 4 == 0 && (reinterpret_cast<uintptr_t>(p) & 15u) == 0; };
     // op(B) is K x N; its K-major copy holds op(B)^T (N x K): element (n, k) = op(B)(k, n)
-    k_to_bf16_kmajor<<<4 * 152, 256, 0, s>>>(B, ldb, !transB, N, K, Bb, Np, Kp);
-    CUtensorMap ma, mb;
-    if (!make_map(&ma, Ab, Mp, Kp) || !make_map(&mb, Bb, Np, Kp)) return HELM_CUDA_ERROR;
-    const size_t smem = (size_t)STAGES * kStageBytes + 1024;
-    static bool attr = false;
-    if (!attr) {
-        if (cudaFuncSetAttribute(k_gemm_bf16_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-            cudaSuccess)
-            return HELM_CUDA_ERROR;
-        attr = true;
+    const PackOp pa{A, Ab, lda, M, Mp, !transA, vec(A, lda)}, pb{B, Bb, ldb, N, Np, transB != 0, vec(B, ldb)};
+    const long long ka = (long long)(Mp / 64) * (Kp / TBK), kb = (long long)(Np / 64) * (Kp / TBK);
+    if (ka + kb > 0x7fffffffLL) return HELM_BAD_ARG;
+    k_pack_bf16<<<(unsigned)(ka + kb), 256, 0, s>>>(pa, pb, K, Kp, ka);
+    // the tallest tile (fewest reads of op(B)) that still gives about one CTA per SM
+    const long long nt = Np / TBM;
+    int tn = 128;
+    while (tn > 16 && nt * ((M + tn - 1) / tn) < 128) tn /= 2;
+    while (tn > 16 && tn / 2 >= M) tn /= 2;                // (no taller than the rows there are)
+    CUtensorMap mn, mm;
+    if (!make_map(&mn, Bb, Np, Kp, TBM) || !make_map(&mm, Ab, Mp, Kp, tn)) return HELM_CUDA_ERROR;
+    const cudaError_t e = tn == 128  ? gemm_tc<128>(mn, mm, M, N, Kp, alpha, beta, C, ldc, s)
+                          : tn == 64 ? gemm_tc<64>(mn, mm, M, N, Kp, alpha, beta, C, ldc, s)
+                          : tn == 32 ? gemm_tc<32>(mn, mm, M, N, Kp, alpha, beta, C, ldc, s)
+                                     : gemm_tc<16>(mn, mm, M, N, Kp, alpha, beta, C, ldc, s);
+    if (ordered) {
+        if (cudaEventRecord(w.ev, s) != cudaSuccess) return HELM_CUDA_ERROR;
+        w.used = true;
     }
-    dim3 grid(Np / TBN, Mp / TBM);
-    k_gemm_bf16_tc<<<grid, TC_THREADS, smem, s>>>(ma, mb, M, N, Kp, alpha, beta, C, ldc);
-    return cudaGetLastError() == cudaSuccess ? HELM_OK : HELM_CUDA_ERROR;
+    return e == cudaSuccess ? HELM_OK : HELM_CUDA_ERROR;
 }
 
 extern "C" helm_status nn_gemm_bf16_status(int* timed_out) {

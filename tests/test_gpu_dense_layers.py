@@ -127,3 +127,31 @@ def test_gemm_tiles(ta, tb, M, N, K):
         bound = (K + 4) * U * 1.5 * (np.abs(opA) @ np.abs(opB)) + 4 * U * abs(beta) * np.abs(C0[:, :N])
         assert np.all(np.abs(got[:, :N] - ref) <= bound)
         assert np.array_equal(got[:, N:], C0[:, N:])      # nothing outside the matrix
+
+
+@pytest.mark.parametrize("ta,tb", [(0, 0), (0, 1), (1, 0), (1, 1)])
+@pytest.mark.parametrize("M,N,K", [(1, 1, 1), (16, 128, 64), (17, 129, 65), (33, 300, 128), (65, 128, 1000), (129, 20000, 64),
+                                   (3, 5, 5000)])
+def test_gemm_bf16_tiles(ta, tb, M, N, K):
+    """Edges of the BF16 product's tiles (16 to 128 rows of C by 128 columns), of the
+    conversion's 64 x 64 blocks and of the ring (fewer K steps than stages, and wrapping
+    it), leading dimensions with and without 16-byte rows, beta 0 with NaN in C and general:
+    |C - exact| <= 4 K 2^-24 (|A| |B|) on the rounded operands, as in test_gpu_gemm_tc.py."""
+    from oracle.tb import bf16_round
+    rng = np.random.default_rng(M + 3 * N + 7 * K)
+    for pad, beta in ((0, 0.0), (1, -0.75)):
+        A = rng.standard_normal((K, M + pad) if ta else (M, K + pad)).astype(np.float32)
+        B = rng.standard_normal((N, K + pad) if tb else (K, N + pad)).astype(np.float32)
+        C0 = rng.standard_normal((M, N + pad)).astype(np.float32)
+        opA = bf16_round((A[:, :M].T if ta else A[:, :K]).astype(np.float64))
+        opB = bf16_round((B[:, :K].T if tb else B[:, :N]).astype(np.float64))
+        Ad, Bd, Cd = _off(A, pad), to_dev(B), to_dev(C0)
+        if beta == 0.0:
+            Cd[:, :N] = float("nan")
+        assert _lib().nn_gemm_bf16(ta, tb, M, N, K, 1.5, _p(Ad), A.shape[1], _p(Bd), B.shape[1], beta, _p(Cd), N + pad, None) == 0
+        got = Cd.cpu().numpy()
+        bound = 4 * K * U * 1.5 * (np.abs(opA) @ np.abs(opB)) + 4 * U * abs(beta) * np.abs(C0[:, :N]) + 1e-30
+        assert np.all(np.abs(got[:, :N] - (1.5 * (opA @ opB) + beta * C0[:, :N])) <= bound)
+        assert np.array_equal(got[:, N:], C0[:, N:])
+    flag = C.c_int(-1)
+    assert _lib().nn_gemm_bf16_status(C.byref(flag)) == 0 and flag.value == 0
