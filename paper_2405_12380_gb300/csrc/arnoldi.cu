@@ -121,6 +121,7 @@ __global__ void __launch_bounds__(GT) k_gs(const double2* __restrict__ V, int nv
                                            const float2* __restrict__ w32, double2* w, const double2* __restrict__ coef,
                                            int lrt, double2* partials, unsigned* counter, double2* Hcol,
                                            double2* coef_out, GivensArgs ga) {
+    pdl_begin();
     extern __shared__ double2 gs_smem[];
     const int RT = 1 << lrt, t = threadIdx.x;
     double2* vs = gs_smem;                                 // [nv][RT + 1]
@@ -208,6 +209,7 @@ __global__ void __launch_bounds__(GT) k_gs(const double2* __restrict__ V, int nv
 // a restart cycle)
 __global__ void __launch_bounds__(256) k_gs_scale(const double2* w, double2* v, float2* __restrict__ v32,
                                                   const double* __restrict__ norm, long long N, double2* g, int m1) {
+    pdl_begin();
     double inv;
     if (g) {
         const double nn = sqrt(norm[0]);
@@ -229,6 +231,7 @@ __global__ void __launch_bounds__(256) k_gs_scale(const double2* w, double2* v, 
 // walking memory took 54 us at k = 15)
 __global__ void __launch_bounds__(64) k_hsolve(const double2* __restrict__ H, int ldh, int k, const double2* __restrict__ g,
                                                double2* __restrict__ y) {
+    pdl_begin();
     extern __shared__ double2 hs_smem[];
     double2* R = hs_smem;                                  // [k][k] column-major
     double2* b = hs_smem + k * k;
@@ -271,7 +274,7 @@ cudaError_t gs(const double2* V, int nv, long long N, const float2* w32, double2
     // a tile is loaded, then used: another block on the SM fills the wait (two; with more the
     // last block's sums over the blocks cost what the overlap gains)
     const unsigned nb = (unsigned)std::min<long long>(tiles, kRedBlocks);
-    k_gs<MODE, W32><<<nb, GT, smem, s>>>(V, nv, N, w32, w, coef, lrt, partials, counter, Hcol, coef_out, ga);
+    launch_after(k_gs<MODE, W32>, nb, GT, smem, s, V, nv, N, w32, w, coef, lrt, partials, counter, Hcol, coef_out, ga);
     return cudaSuccess;
 }
 
@@ -294,7 +297,7 @@ cudaError_t launch_arnoldi(const double2* V, int j, long long N, const float2* w
 void launch_gs_scale(const double2* w, double2* v, float2* v32, const double* norm2, long long N, double2* g, int m1,
                      cudaStream_t s) {
     const long long b = (N + 255) / 256;
-    k_gs_scale<<<(unsigned)std::min<long long>(b, 4 * kRedBlocks), 256, 0, s>>>(w, v, v32, norm2, N, g, m1);
+    launch_after(k_gs_scale, (unsigned)std::min<long long>(b, 4 * kRedBlocks), 256, 0, s, w, v, v32, norm2, N, g, m1);
 }
 
 cudaError_t launch_hsolve(const double2* H, int ldh, int k, const double2* g, double2* y, cudaStream_t s) {
@@ -304,7 +307,7 @@ cudaError_t launch_hsolve(const double2* H, int ldh, int k, const double2* g, do
                                                    (kMaxRestart * kMaxRestart + kMaxRestart) * (int)sizeof(double2));
         if (e != cudaSuccess) return e;
     }
-    k_hsolve<<<1, 64, smem, s>>>(H, ldh, k, g, y);
+    launch_after(k_hsolve, 1, 64, smem, s, H, ldh, k, g, y);
     return cudaSuccess;
 }
 

@@ -115,6 +115,7 @@ __device__ __forceinline__ void st2(float2* a, long long q, bool half, float4 v)
 // p = r + beta (p - omega v)
 __global__ void __launch_bounds__(kB32Threads) k32_update_p(const float2* __restrict__ r, const float2* __restrict__ v,
                                                             float2* __restrict__ p, const double2* sc, long long N) {
+    pdl_begin();
     if (stopped(sc)) return;
     __shared__ float2 s_beta, s_omega;                     // converted once per block
     if (threadIdx.x == 0) {
@@ -134,6 +135,7 @@ __global__ void __launch_bounds__(kB32Threads) k32_update_p(const float2* __rest
 // alpha = rho / <rhat, v>
 __global__ void __launch_bounds__(kB32Threads) k32_alpha(const float2* __restrict__ rhat, const float2* __restrict__ v,
                                                          double2* sc, long long N, double* parts, unsigned* counter) {
+    pdl_begin();
     if (stopped(sc)) return;
     float re = 0.f, im = 0.f;
     for_pairs(N, [&](long long q, bool half) {
@@ -163,6 +165,7 @@ template <bool DOT>
 __global__ void __launch_bounds__(kB32Threads) k32_s(const float2* __restrict__ r, const float2* __restrict__ v,
                                                      float2* __restrict__ s, double2* sc, long long N, double* parts,
                                                      unsigned* counter, const float* aparts, int na) {
+    pdl_begin();
     if (stopped(sc)) return;
     // the scalar in one thread, shared with the block (FP64 division is slow here)
     __shared__ float2 s_alpha;
@@ -207,6 +210,7 @@ __global__ void __launch_bounds__(kB32Threads) k32_s(const float2* __restrict__ 
 // omega = <t, s> / <t, t>
 __global__ void __launch_bounds__(kB32Threads) k32_omega(const float2* __restrict__ t, const float2* __restrict__ s,
                                                          double2* sc, long long N, double* parts, unsigned* counter) {
+    pdl_begin();
     if (stopped(sc)) return;
     float re = 0.f, im = 0.f, tt = 0.f;
     for_pairs(N, [&](long long q, bool half) {
@@ -243,6 +247,7 @@ __global__ void __launch_bounds__(kB32Threads, 4) k32_xr(float2* __restrict__ xl
                                                       const float2* __restrict__ s, const float2* __restrict__ t,
                                                       const float2* __restrict__ rhat, double2* sc, long long N,
                                                       double* parts, unsigned* counter, const float* oparts, int no) {
+    pdl_begin();
     // the scalars in one thread, shared with the block (FP64 division is slow here)
     __shared__ float2 s_alpha, s_omega;
     __shared__ int s_skip;
@@ -325,6 +330,7 @@ __global__ void __launch_bounds__(kB32Threads, 4) k32_xr(float2* __restrict__ xl
 // fold); 3: x -= xl, xl = 0 (undo a trial fold)
 __global__ void __launch_bounds__(kB32Threads) k32_fold(double2* __restrict__ x, float2* __restrict__ xl, long long N,
                                                         int mode) {
+    pdl_begin();
     for (long long l = blockIdx.x * (long long)kB32Threads + threadIdx.x; l < N;
          l += (long long)gridDim.x * kB32Threads) {
         if (mode != 1) {
@@ -344,6 +350,7 @@ __global__ void __launch_bounds__(kB32Threads) k32_replace(const double2* __rest
                                                            float2* __restrict__ rhat, float2* __restrict__ p,
                                                            float2* __restrict__ v, int restart, double2* sc,
                                                            long long N, double* parts, unsigned* counter) {
+    pdl_begin();
     float re = 0.f, im = 0.f;
     for (long long l = blockIdx.x * (long long)kB32Threads + threadIdx.x; l < N;
          l += (long long)gridDim.x * kB32Threads) {
@@ -382,7 +389,8 @@ __global__ void __launch_bounds__(kB32Threads) k32_replace(const double2* __rest
     }
 }
 
-__global__ void k32_set_tol(double2* sc, double tol_abs) { sc[S_TOLS] = make_double2(tol_abs, 0.0); }
+__global__ void k32_set_tol(double2* sc, double tol_abs) {
+    pdl_begin(); sc[S_TOLS] = make_double2(tol_abs, 0.0); }
 
 }  // namespace
 
@@ -398,42 +406,42 @@ int bicg32_blocks() {
 }
 
 void launch_b32_update_p(const float2* r, const float2* v, float2* p, const double2* sc, long long N, cudaStream_t s) {
-    k32_update_p<<<bicg32_blocks(), kB32Threads, 0, s>>>(r, v, p, sc, N);
+    launch_after(k32_update_p, bicg32_blocks(), kB32Threads, 0, s, r, v, p, sc, N);
 }
 void launch_b32_alpha(const float2* rhat, const float2* v, double2* sc, long long N, double* parts, unsigned* counter,
                       cudaStream_t s) {
-    k32_alpha<<<bicg32_blocks(), kB32Threads, 0, s>>>(rhat, v, sc, N, parts, counter);
+    launch_after(k32_alpha, bicg32_blocks(), kB32Threads, 0, s, rhat, v, sc, N, parts, counter);
 }
 void launch_b32_s(const float2* r, const float2* v, float2* sv, double2* sc, long long N, double* parts,
                   unsigned* counter, cudaStream_t s) {
-    k32_s<false><<<bicg32_blocks(), kB32Threads, 0, s>>>(r, v, sv, sc, N, parts, counter, nullptr, 0);
+    launch_after(k32_s<false>, bicg32_blocks(), kB32Threads, 0, s, r, v, sv, sc, N, parts, counter, nullptr, 0);
 }
 void launch_b32_s_dot(const float2* r, const float2* v, float2* sv, double2* sc, long long N, double* parts,
                       unsigned* counter, const float* aparts, int na, cudaStream_t s) {
-    k32_s<true><<<bicg32_blocks(), kB32Threads, 0, s>>>(r, v, sv, sc, N, parts, counter, aparts, na);
+    launch_after(k32_s<true>, bicg32_blocks(), kB32Threads, 0, s, r, v, sv, sc, N, parts, counter, aparts, na);
 }
-void launch_b32_set_tol(double2* sc, double tol_abs, cudaStream_t s) { k32_set_tol<<<1, 1, 0, s>>>(sc, tol_abs); }
+void launch_b32_set_tol(double2* sc, double tol_abs, cudaStream_t s) { launch_after(k32_set_tol, 1, 1, 0, s, sc, tol_abs); }
 void launch_b32_omega(const float2* t, const float2* sv, double2* sc, long long N, double* parts, unsigned* counter,
                       cudaStream_t s) {
-    k32_omega<<<bicg32_blocks(), kB32Threads, 0, s>>>(t, sv, sc, N, parts, counter);
+    launch_after(k32_omega, bicg32_blocks(), kB32Threads, 0, s, t, sv, sc, N, parts, counter);
 }
 void launch_b32_xr(float2* xl, float2* r, const float2* phat, const float2* shat, const float2* sv, const float2* t,
                    const float2* rhat, double2* sc, long long N, double* parts, unsigned* counter, cudaStream_t s) {
-    k32_xr<false><<<bicg32_blocks(), kB32Threads, 0, s>>>(xl, r, phat, shat, sv, t, rhat, sc, N, parts, counter,
+    launch_after(k32_xr<false>, bicg32_blocks(), kB32Threads, 0, s, xl, r, phat, shat, sv, t, rhat, sc, N, parts, counter,
                                                           nullptr, 0);
 }
 void launch_b32_xr_dot(float2* xl, float2* r, const float2* phat, const float2* shat, const float2* sv,
                        const float2* t, const float2* rhat, double2* sc, long long N, double* parts, unsigned* counter,
                        const float* oparts, int no, cudaStream_t s) {
-    k32_xr<true><<<bicg32_blocks(), kB32Threads, 0, s>>>(xl, r, phat, shat, sv, t, rhat, sc, N, parts, counter,
+    launch_after(k32_xr<true>, bicg32_blocks(), kB32Threads, 0, s, xl, r, phat, shat, sv, t, rhat, sc, N, parts, counter,
                                                          oparts, no);
 }
 void launch_b32_fold(double2* x, float2* xl, long long N, cudaStream_t s, int mode) {
-    k32_fold<<<bicg32_blocks(), kB32Threads, 0, s>>>(x, xl, N, mode);
+    launch_after(k32_fold, bicg32_blocks(), kB32Threads, 0, s, x, xl, N, mode);
 }
 void launch_b32_replace(const double2* r64, float2* r, float2* rhat, float2* p, float2* v, int restart, double2* sc,
                         long long N, double* parts, unsigned* counter, cudaStream_t s) {
-    k32_replace<<<bicg32_blocks(), kB32Threads, 0, s>>>(r64, r, rhat, p, v, restart, sc, N, parts, counter);
+    launch_after(k32_replace, bicg32_blocks(), kB32Threads, 0, s, r64, r, rhat, p, v, restart, sc, N, parts, counter);
 }
 
 }  // namespace helm

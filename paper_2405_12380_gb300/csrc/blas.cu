@@ -25,6 +25,7 @@ __device__ __forceinline__ double2 warp_sum(double2 v) {
 
 __global__ void __launch_bounds__(TB) k_dot(const double2* __restrict__ a, const double2* __restrict__ b,
                                             long long N, double2* partials) {
+    pdl_begin();
     double2 acc = make_double2(0, 0);
     for (long long l = blockIdx.x * (long long)TB + threadIdx.x; l < N; l += (long long)gridDim.x * TB) {
         acc = cfmac(a[l], b[l], acc);
@@ -35,6 +36,7 @@ __global__ void __launch_bounds__(TB) k_dot(const double2* __restrict__ a, const
 }
 
 __global__ void __launch_bounds__(TB) k_norm2(const double2* __restrict__ a, long long N, double* partials) {
+    pdl_begin();
     double acc[1] = {0.0};
     for (long long l = blockIdx.x * (long long)TB + threadIdx.x; l < N; l += (long long)gridDim.x * TB)
         acc[0] = cnorm2(a[l], acc[0]);
@@ -83,6 +85,7 @@ __device__ __forceinline__ double2 fin_sum_c(const double2* p, int nparts, int s
 }
 
 __global__ void __launch_bounds__(kFinThreads) k_sum_real(const double* partials, int nparts, double* out) {
+    pdl_begin();
     double v = fin_sum_d(partials, nparts);
     if (threadIdx.x == 0) *out = v;
 }
@@ -90,6 +93,7 @@ __global__ void __launch_bounds__(kFinThreads) k_sum_real(const double* partials
 
 __global__ void __launch_bounds__(TB) k_bicg_p(const double2* __restrict__ r, const double2* __restrict__ v,
                                                double2* __restrict__ p, const double2* __restrict__ sc, long long N) {
+    pdl_begin();
     const double2 beta = sc[S_BETA], omega = sc[S_OMEGA];
     for (long long l = blockIdx.x * (long long)TB + threadIdx.x; l < N; l += (long long)gridDim.x * TB) {
         p[l] = cfma(beta, cfma(make_double2(-omega.x, -omega.y), v[l], p[l]), r[l]);
@@ -100,6 +104,7 @@ __global__ void __launch_bounds__(TB) k_bicg_p(const double2* __restrict__ r, co
 __global__ void __launch_bounds__(kFusedThreads) k_bicg_s_fused(const double2* __restrict__ r, const double2* __restrict__ v,
                                                                 double2* __restrict__ s, double2* sc, long long N,
                                                                 double* parts, unsigned* counter, double tol_abs) {
+    pdl_begin();
     const double2 na = make_double2(-sc[S_ALPHA].x, -sc[S_ALPHA].y);
     double acc[1] = {0.0};
     for (long long l = blockIdx.x * (long long)kFusedThreads + threadIdx.x; l < N; l += (long long)gridDim.x * kFusedThreads) {
@@ -129,6 +134,7 @@ __global__ void __launch_bounds__(kFusedThreads) k_bicg_xr_fused(double2* __rest
                                                                  const double2* __restrict__ rhat, double2* sc,
                                                                  long long N, double* parts, unsigned* counter,
                                                                  double tol, double bnorm) {
+    pdl_begin();
     const double2 alpha = sc[S_ALPHA], omega = sc[S_OMEGA];
     const bool skip = sc[S_FLAGS].y == 1.0 || sc[S_STOP].x != 0.0;
     double rn = 0;
@@ -168,6 +174,7 @@ __global__ void __launch_bounds__(kFusedThreads) k_bicg_xr_fused(double2* __rest
 // recipes: 0 = rho & beta (complex partials), 1 = alpha, 2 = ||s||^2, 3 = omega, 4 = ||r||^2, 5 = reset
 __global__ void __launch_bounds__(kFinThreads) k_bicg_scalar(int recipe, const double* partials, int nparts,
                                                              double2* sc, double tol_abs) {
+    pdl_begin();
     if (recipe == 0 || recipe == 1) {
         double2 d = fin_sum_c(reinterpret_cast<const double2*>(partials), nparts);
         if (threadIdx.x != 0) return;
@@ -225,6 +232,7 @@ __global__ void __launch_bounds__(kFinThreads) k_bicg_scalar(int recipe, const d
 // w += sign * sum_i V_i coef_i (the solution update of FGMRES)
 __global__ void __launch_bounds__(TB) k_mupdate(const double2* __restrict__ V, int nv, const double2* __restrict__ coef,
                                                 double sign, double2* __restrict__ w, long long N) {
+    pdl_begin();
     __shared__ double2 c[kMaxRestart + 1];
     for (int i = threadIdx.x; i < nv; i += TB) c[i] = cscale(sign, coef[i]);
     __syncthreads();
@@ -241,6 +249,7 @@ __global__ void __launch_bounds__(TB) k_mupdate(const double2* __restrict__ V, i
 // w += sign * sum_i V_i coef_i with complex64 vectors V (FP64 accumulation)
 __global__ void __launch_bounds__(TB) k_mupdate32(const float2* __restrict__ V, int nv, const double2* __restrict__ coef,
                                                   double sign, double2* __restrict__ w, long long N) {
+    pdl_begin();
     __shared__ double2 c[kMaxRestart + 1];
     for (int i = threadIdx.x; i < nv; i += TB) c[i] = cscale(sign, coef[i]);
     __syncthreads();
@@ -257,15 +266,18 @@ __global__ void __launch_bounds__(TB) k_mupdate32(const float2* __restrict__ V, 
 
 __global__ void __launch_bounds__(TB) k_set_masked(double2* __restrict__ x, const double2* __restrict__ f,
                                                    const uint8_t* __restrict__ mask, long long N) {
+    pdl_begin();
     for (long long l = blockIdx.x * (long long)TB + threadIdx.x; l < N; l += (long long)gridDim.x * TB)
         if (mask[l]) x[l] = f[l];
 }
 
 __global__ void __launch_bounds__(TB) k_cvt64to32(const double2* __restrict__ a, float2* __restrict__ b, long long N) {
+    pdl_begin();
     for (long long l = blockIdx.x * (long long)TB + threadIdx.x; l < N; l += (long long)gridDim.x * TB)
         b[l] = make_float2((float)a[l].x, (float)a[l].y);
 }
 __global__ void __launch_bounds__(TB) k_cvt32to64(const float2* __restrict__ a, double2* __restrict__ b, long long N) {
+    pdl_begin();
     for (long long l = blockIdx.x * (long long)TB + threadIdx.x; l < N; l += (long long)gridDim.x * TB)
         b[l] = make_double2((double)a[l].x, (double)a[l].y);
 }
@@ -278,48 +290,48 @@ int stream_blocks(long long N) {
 }  // namespace
 
 void launch_dot(const double2* a, const double2* b, long long N, double2* partials, cudaStream_t s) {
-    k_dot<<<kRedBlocks, TB, 0, s>>>(a, b, N, partials);
+    launch_after(k_dot, kRedBlocks, TB, 0, s, a, b, N, partials);
 }
 void launch_norm2(const double2* a, long long N, double* partials, cudaStream_t s) {
-    k_norm2<<<kRedBlocks, TB, 0, s>>>(a, N, partials);
+    launch_after(k_norm2, kRedBlocks, TB, 0, s, a, N, partials);
 }
 void launch_sum_real(const double* partials, int nparts, double* out, cudaStream_t s) {
-    k_sum_real<<<1, kFinThreads, 0, s>>>(partials, nparts, out);
+    launch_after(k_sum_real, 1, kFinThreads, 0, s, partials, nparts, out);
 }
 void launch_bicg_update_p(const double2* r, const double2* v, double2* p, const double2* sc, long long N,
                           cudaStream_t s) {
-    k_bicg_p<<<stream_blocks(N), TB, 0, s>>>(r, v, p, sc, N);
+    launch_after(k_bicg_p, stream_blocks(N), TB, 0, s, r, v, p, sc, N);
 }
 void launch_bicg_s_fused(const double2* r, const double2* v, double2* sv, double2* sc, long long N, double* parts,
                          unsigned* counter, double tol_abs, cudaStream_t s) {
-    k_bicg_s_fused<<<kRedBlocks, kFusedThreads, 0, s>>>(r, v, sv, sc, N, parts, counter, tol_abs);
+    launch_after(k_bicg_s_fused, kRedBlocks, kFusedThreads, 0, s, r, v, sv, sc, N, parts, counter, tol_abs);
 }
 void launch_bicg_xr_fused(double2* x, double2* r, const double2* phat, const double2* shat, const double2* sv,
                           const double2* t, const double2* rhat, double2* sc, long long N, double* parts,
                           unsigned* counter, double tol, double bnorm, cudaStream_t s) {
-    k_bicg_xr_fused<<<kRedBlocks, kFusedThreads, 0, s>>>(x, r, phat, shat, sv, t, rhat, sc, N, parts, counter, tol,
+    launch_after(k_bicg_xr_fused, kRedBlocks, kFusedThreads, 0, s, x, r, phat, shat, sv, t, rhat, sc, N, parts, counter, tol,
                                                          bnorm);
 }
 void launch_bicg_scalar(int recipe, const double* partials, int nparts, double2* sc, double tol_abs,
                         cudaStream_t s) {
-    k_bicg_scalar<<<1, kFinThreads, 0, s>>>(recipe, partials, nparts, sc, tol_abs);
+    launch_after(k_bicg_scalar, 1, kFinThreads, 0, s, recipe, partials, nparts, sc, tol_abs);
 }
 void launch_mupdate(const double2* V, int nv, const double2* coef, double sign, double2* w, long long N,
                     cudaStream_t s) {
-    k_mupdate<<<stream_blocks(N), TB, 0, s>>>(V, nv, coef, sign, w, N);
+    launch_after(k_mupdate, stream_blocks(N), TB, 0, s, V, nv, coef, sign, w, N);
 }
 void launch_mupdate32(const float2* V, int nv, const double2* coef, double sign, double2* w, long long N,
                       cudaStream_t s) {
-    k_mupdate32<<<stream_blocks(N), TB, 0, s>>>(V, nv, coef, sign, w, N);
+    launch_after(k_mupdate32, stream_blocks(N), TB, 0, s, V, nv, coef, sign, w, N);
 }
 void launch_set_masked(double2* x, const double2* f, const uint8_t* mask, long long N, cudaStream_t s) {
-    k_set_masked<<<stream_blocks(N), TB, 0, s>>>(x, f, mask, N);
+    launch_after(k_set_masked, stream_blocks(N), TB, 0, s, x, f, mask, N);
 }
 void launch_cvt_f64_to_f32(const double2* a, float2* b, long long N, cudaStream_t s) {
-    k_cvt64to32<<<stream_blocks(N), TB, 0, s>>>(a, b, N);
+    launch_after(k_cvt64to32, stream_blocks(N), TB, 0, s, a, b, N);
 }
 void launch_cvt_f32_to_f64(const float2* a, double2* b, long long N, cudaStream_t s) {
-    k_cvt32to64<<<stream_blocks(N), TB, 0, s>>>(a, b, N);
+    launch_after(k_cvt32to64, stream_blocks(N), TB, 0, s, a, b, N);
 }
 
 }  // namespace helm

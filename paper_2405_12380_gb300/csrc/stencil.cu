@@ -184,6 +184,7 @@ template <typename R, bool RESID, bool NORM>
 __global__ void __launch_bounds__(AZ) k_apply_z(Op<R> op, int zc, const typename CT<R>::T* __restrict__ x,
                                                 const typename CT<R>::T* __restrict__ f,
                                                 typename CT<R>::T* __restrict__ y, double* partials, int conj) {
+    pdl_begin();
     using C = typename CT<R>::T;
     const int sy = op.n, sz = op.n * op.n;                 // (N < 2^31)
     const int q = blockIdx.x * AZ + threadIdx.x;           // index in the plane
@@ -294,6 +295,7 @@ __global__ void __launch_bounds__(BX * BY) k_march_c64(Op<float> op, int zc, flo
                                                        const float4* __restrict__ x, const float4* __restrict__ f,
                                                        float4* __restrict__ y, double* partials, int conj,
                                                        Dot32 dot = Dot32{}) {
+    pdl_begin();
     static_assert(DOT == 0 || (KIND == 0 && !FLAG && !NORM), "the fused reduction follows y = A x only");
     constexpr bool NBR = !(KIND == 1 && FLAG);             // neighbours (and x) are read
     constexpr bool RHS = KIND >= 1 || FLAG;                // f is read
@@ -491,6 +493,7 @@ __device__ __forceinline__ float2 gs_value(const Op<float>& op, unsigned c, floa
 template <bool XZERO>
 __global__ void __launch_bounds__(BX * BY) k_rbgs_c64(Op<float> op, int zc, int colour, const float4* __restrict__ f,
                                                       float4* x, int conj, float omega) {
+    pdl_begin();
     constexpr unsigned kMM = kMasked | (kMasked << 8);
     const int n = op.n, h = n >> 1;
     const int i2 = blockIdx.x * BX + threadIdx.x;
@@ -633,6 +636,7 @@ template <bool XZERO, bool SOR, bool K2>
 __global__ void __launch_bounds__(kSweepMaxThreads, 1)
     k_sweep_c64(Op<float> op, int zc, int c0, const float4* __restrict__ f, const float2* __restrict__ xin,
                 float4* __restrict__ xout, int conj, float omega) {
+    pdl_begin();
     extern __shared__ __align__(16) float2 sweep_smem[];
     constexpr unsigned kOut = kMasked | (kMasked << 16);   // (code, layer) byte pairs of two masked nodes
     const int n = op.n, h = n >> 1;
@@ -803,6 +807,7 @@ __global__ void __launch_bounds__(BX * BY) k_apply(Op<R> op, int zc, const typen
                                                    const typename CT<R>::T* __restrict__ f,
                                                    typename CT<R>::T* __restrict__ y, double* partials,
                                                    int conj) {
+    pdl_begin();
     const int i = blockIdx.x * BX + threadIdx.x;
     const int j = blockIdx.y * BY + threadIdx.y;
     // 3D: zc planes per block (the grid of k_apply_z, so partial counts agree)
@@ -846,6 +851,7 @@ template <int MODE>
 __global__ void __launch_bounds__(kFusedThreads) k_apply_bicg(Op<double> op, const double2* __restrict__ x,
                                                               double2* __restrict__ y, const double2* __restrict__ w,
                                                               int conj, double2* sc, double* parts, unsigned* counter) {
+    pdl_begin();
     double2 a = make_double2(0, 0);
     double c = 0;
 #pragma unroll
@@ -902,6 +908,7 @@ template <typename R, bool XZERO>
 __global__ void __launch_bounds__(BX * BY) k_jacobi(Op<R> op, R omega, const typename CT<R>::T* __restrict__ f,
                                                     const typename CT<R>::T* __restrict__ xin,
                                                     typename CT<R>::T* __restrict__ xout, int conj) {
+    pdl_begin();
     const long long l = blockIdx.x * (long long)(BX * BY) + threadIdx.x;
     if (l < op.N) jacobi_point<R, XZERO>(op, omega, f, xin, xout, conj, l);
 }
@@ -919,6 +926,7 @@ template <typename R>
 __global__ void k_jacobi_tile(Op<R> op, R omega, int S, const typename CT<R>::T* __restrict__ f,
                               const typename CT<R>::T* __restrict__ xin, typename CT<R>::T* __restrict__ xout,
                               int conj) {
+    pdl_begin();
     using C = typename CT<R>::T;
     extern __shared__ __align__(16) unsigned char jt_smem[];
     const int E = blockDim.x, TI = E - 2 * S, tx = threadIdx.x, ty = threadIdx.y, t = ty * E + tx;
@@ -1015,6 +1023,7 @@ __device__ __forceinline__ int colour_of(long long l, int n) {
 template <typename R, bool XZERO>
 __global__ void __launch_bounds__(BX * BY) k_rbgs(Op<R> op, int colour, const typename CT<R>::T* __restrict__ f,
                                                   typename CT<R>::T* x, int conj, R omega, bool sor) {
+    pdl_begin();
     const long long m2 = 2 * (blockIdx.x * (long long)(BX * BY) + threadIdx.x);
     if (m2 >= op.N) return;
     const long long l = m2 + (colour_of(m2, op.n) != colour);
@@ -1025,6 +1034,7 @@ __global__ void __launch_bounds__(BX * BY) k_rbgs(Op<R> op, int colour, const ty
 __global__ void __launch_bounds__(BX * BY) k_residual_red(Op<double> op, const double2* __restrict__ z,
                                                           const double2* __restrict__ v,
                                                           double2* __restrict__ r_red, int conj) {
+    pdl_begin();
     const long long m = blockIdx.x * (long long)(BX * BY) + threadIdx.x;
     if (2 * m >= op.N) return;
     const long long l = 2 * m + colour_of(2 * m, op.n);
@@ -1206,6 +1216,7 @@ __global__ void __launch_bounds__(kFusedThreads) k_apply_bicg_df(Op<double> op, 
                                                                  double2* __restrict__ y, const double2* __restrict__ w,
                                                                  int conj, double2* sc, double* parts,
                                                                  unsigned* counter) {
+    pdl_begin();
     double2 a = make_double2(0, 0);
     double c = 0;
 #pragma unroll
@@ -1694,11 +1705,11 @@ int launch_apply(const Op<R>& op, const typename CT<R>::T* x, const typename CT<
             const float4* f4 = reinterpret_cast<const float4*>(f);
             float4* y4 = reinterpret_cast<float4*>(y);
             if (resid) {
-                if (partials) k_march_c64<0, true, true><<<g, b, 0, s>>>(op, zc, 0.f, x4, f4, y4, partials, conj);
-                else k_march_c64<0, true, false><<<g, b, 0, s>>>(op, zc, 0.f, x4, f4, y4, partials, conj);
+                if (partials) launch_after(k_march_c64<0, true, true>, g, b, 0, s, op, zc, 0.f, x4, f4, y4, partials, conj, Dot32{});
+                else launch_after(k_march_c64<0, true, false>, g, b, 0, s, op, zc, 0.f, x4, f4, y4, partials, conj, Dot32{});
             } else {
-                if (partials) k_march_c64<0, false, true><<<g, b, 0, s>>>(op, zc, 0.f, x4, f4, y4, partials, conj);
-                else k_march_c64<0, false, false><<<g, b, 0, s>>>(op, zc, 0.f, x4, f4, y4, partials, conj);
+                if (partials) launch_after(k_march_c64<0, false, true>, g, b, 0, s, op, zc, 0.f, x4, f4, y4, partials, conj, Dot32{});
+                else launch_after(k_march_c64<0, false, false>, g, b, 0, s, op, zc, 0.f, x4, f4, y4, partials, conj, Dot32{});
             }
             return (int)(g.x * g.y * g.z);
         }
@@ -1707,11 +1718,11 @@ int launch_apply(const Op<R>& op, const typename CT<R>::T* x, const typename CT<
         int zc;
         const dim3 g = applyz_grid(op.n, &zc);
         if (resid) {
-            if (partials) k_apply_z<R, true, true><<<g, AZ, 0, s>>>(op, zc, x, f, y, partials, conj);
-            else k_apply_z<R, true, false><<<g, AZ, 0, s>>>(op, zc, x, f, y, partials, conj);
+            if (partials) launch_after(k_apply_z<R, true, true>, g, AZ, 0, s, op, zc, x, f, y, partials, conj);
+            else launch_after(k_apply_z<R, true, false>, g, AZ, 0, s, op, zc, x, f, y, partials, conj);
         } else {
-            if (partials) k_apply_z<R, false, true><<<g, AZ, 0, s>>>(op, zc, x, f, y, partials, conj);
-            else k_apply_z<R, false, false><<<g, AZ, 0, s>>>(op, zc, x, f, y, partials, conj);
+            if (partials) launch_after(k_apply_z<R, false, true>, g, AZ, 0, s, op, zc, x, f, y, partials, conj);
+            else launch_after(k_apply_z<R, false, false>, g, AZ, 0, s, op, zc, x, f, y, partials, conj);
         }
         return (int)(g.x * g.y);
     }
@@ -1719,11 +1730,11 @@ int launch_apply(const Op<R>& op, const typename CT<R>::T* x, const typename CT<
     dim3 g = grid_for(op.dim, op.n, 1, zc), b(BX, BY);
     // 2D, or an operator without the per-node tables (the allocation-free path)
     if (resid) {
-        if (partials) k_apply<R, true, true><<<g, b, 0, s>>>(op, zc, x, f, y, partials, conj);
-        else k_apply<R, true, false><<<g, b, 0, s>>>(op, zc, x, f, y, partials, conj);
+        if (partials) launch_after(k_apply<R, true, true>, g, b, 0, s, op, zc, x, f, y, partials, conj);
+        else launch_after(k_apply<R, true, false>, g, b, 0, s, op, zc, x, f, y, partials, conj);
     } else {
-        if (partials) k_apply<R, false, true><<<g, b, 0, s>>>(op, zc, x, f, y, partials, conj);
-        else k_apply<R, false, false><<<g, b, 0, s>>>(op, zc, x, f, y, partials, conj);
+        if (partials) launch_after(k_apply<R, false, true>, g, b, 0, s, op, zc, x, f, y, partials, conj);
+        else launch_after(k_apply<R, false, false>, g, b, 0, s, op, zc, x, f, y, partials, conj);
     }
     return (int)(g.x * g.y * g.z);
 }
@@ -1738,14 +1749,14 @@ void launch_jacobi(const Op<R>& op, double omega, const typename CT<R>::T* f, co
             const float4* x4 = reinterpret_cast<const float4*>(xin);
             const float4* f4 = reinterpret_cast<const float4*>(f);
             float4* y4 = reinterpret_cast<float4*>(xout);
-            if (xzero) k_march_c64<1, true, false><<<g, b, 0, s>>>(op, zc, (float)omega, x4, f4, y4, nullptr, conj);
-            else k_march_c64<1, false, false><<<g, b, 0, s>>>(op, zc, (float)omega, x4, f4, y4, nullptr, conj);
+            if (xzero) launch_after(k_march_c64<1, true, false>, g, b, 0, s, op, zc, (float)omega, x4, f4, y4, nullptr, conj, Dot32{});
+            else launch_after(k_march_c64<1, false, false>, g, b, 0, s, op, zc, (float)omega, x4, f4, y4, nullptr, conj, Dot32{});
             return;
         }
     }
     const unsigned g = flat_blocks(op.N);
-    if (xzero) k_jacobi<R, true><<<g, BX * BY, 0, s>>>(op, (R)omega, f, xin, xout, conj);
-    else k_jacobi<R, false><<<g, BX * BY, 0, s>>>(op, (R)omega, f, xin, xout, conj);
+    if (xzero) launch_after(k_jacobi<R, true>, g, BX * BY, 0, s, op, (R)omega, f, xin, xout, conj);
+    else launch_after(k_jacobi<R, false>, g, BX * BY, 0, s, op, (R)omega, f, xin, xout, conj);
 }
 
 // sweeps per launch of the tiled form for this operator, 0 where it does not apply (3D,
@@ -1765,7 +1776,7 @@ void launch_jacobi_tile(const Op<R>& op, double omega, int sweeps, const typenam
     // node per thread)
     const int TI = std::max(6, std::min(16, (op.n + 11) / 12)), E = TI + 2 * sweeps;
     const dim3 g((op.n + TI - 1) / TI, (op.n + TI - 1) / TI), b(E, E);
-    k_jacobi_tile<R><<<g, b, 2 * (size_t)E * E * sizeof(typename CT<R>::T), s>>>(op, (R)omega, sweeps, f, xin, xout, conj);
+    launch_after(k_jacobi_tile<R>, g, b, 2 * (size_t)E * E * sizeof(typename CT<R>::T), s, op, (R)omega, sweeps, f, xin, xout, conj);
 }
 
 template int jacobi_tile_sweeps<double>(const Op<double>&);
@@ -1784,15 +1795,15 @@ void launch_rbgs_half(const Op<R>& op, int colour, const typename CT<R>::T* f, t
             const dim3 g = pair_grid(op.n, &zc), b(BX, BY);
             const float4* f4 = reinterpret_cast<const float4*>(f);
             float4* x4 = reinterpret_cast<float4*>(x);
-            if (xzero) k_rbgs_c64<true><<<g, b, 0, s>>>(op, zc, colour, f4, x4, conj, (float)omega);
-            else k_rbgs_c64<false><<<g, b, 0, s>>>(op, zc, colour, f4, x4, conj, (float)omega);
+            if (xzero) launch_after(k_rbgs_c64<true>, g, b, 0, s, op, zc, colour, f4, x4, conj, (float)omega);
+            else launch_after(k_rbgs_c64<false>, g, b, 0, s, op, zc, colour, f4, x4, conj, (float)omega);
             return;
         }
     }
     const unsigned g = flat_blocks((op.N + 1) / 2);
     const bool sor = (R)omega != (R)1;
-    if (xzero) k_rbgs<R, true><<<g, BX * BY, 0, s>>>(op, colour, f, x, conj, (R)omega, sor);
-    else k_rbgs<R, false><<<g, BX * BY, 0, s>>>(op, colour, f, x, conj, (R)omega, sor);
+    if (xzero) launch_after(k_rbgs<R, true>, g, BX * BY, 0, s, op, colour, f, x, conj, (R)omega, sor);
+    else launch_after(k_rbgs<R, false>, g, BX * BY, 0, s, op, colour, f, x, conj, (R)omega, sor);
 }
 
 bool launch_red_residual32(const Op<float>& op, const float2* f, const float2* x, float2* r_red, int conj,
@@ -1800,9 +1811,9 @@ bool launch_red_residual32(const Op<float>& op, const float2* f, const float2* x
     if (!pair_ok(op, f, x, r_red)) return false;
     int zc;
     const dim3 g = pair_grid(op.n, &zc), b(BX, BY);
-    k_march_c64<2, false, false><<<g, b, 0, s>>>(op, zc, 0.f, reinterpret_cast<const float4*>(x),
+    launch_after(k_march_c64<2, false, false>, g, b, 0, s, op, zc, 0.f, reinterpret_cast<const float4*>(x),
                                                  reinterpret_cast<const float4*>(f), reinterpret_cast<float4*>(r_red),
-                                                 nullptr, conj);
+                                                 nullptr, conj, Dot32{});
     return true;
 }
 
@@ -1814,8 +1825,8 @@ int launch_apply32_bicg(const Op<float>& op, int mode, const float2* x, float2* 
     const Dot32 d{reinterpret_cast<const float4*>(w), const_cast<double2*>(sc), parts};
     const float4* x4 = reinterpret_cast<const float4*>(x);
     float4* y4 = reinterpret_cast<float4*>(y);
-    if (mode == 1) k_march_c64<0, false, false, 1><<<g, b, 0, s>>>(op, zc, 0.f, x4, nullptr, y4, nullptr, conj, d);
-    else k_march_c64<0, false, false, 2><<<g, b, 0, s>>>(op, zc, 0.f, x4, nullptr, y4, nullptr, conj, d);
+    if (mode == 1) launch_after(k_march_c64<0, false, false, 1>, g, b, 0, s, op, zc, 0.f, x4, nullptr, y4, nullptr, conj, d);
+    else launch_after(k_march_c64<0, false, false, 2>, g, b, 0, s, op, zc, 0.f, x4, nullptr, y4, nullptr, conj, d);
     return (int)(g.x * g.y * g.z);
 }
 
@@ -1888,9 +1899,8 @@ bool launch_rbgs_sweep32(const Op<float>& op, int c0, const float2* f, const flo
     if (smem > 48 * 1024 &&
         cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024) != cudaSuccess)
         return false;
-    fn<<<g, b, smem, s>>>(op, op.sw_zc, c0, reinterpret_cast<const float4*>(f), xin, reinterpret_cast<float4*>(xout), conj,
-                          (float)omega);
-    return true;
+    return launch_after(fn, g, b, smem, s, op, op.sw_zc, c0, reinterpret_cast<const float4*>(f), xin,
+                        reinterpret_cast<float4*>(xout), conj, (float)omega) == cudaSuccess;
 }
 
 void launch_node_pack(const Op<float>& op, uint16_t* ncl, cudaStream_t s) {
@@ -1900,15 +1910,15 @@ void launch_node_pack(const Op<float>& op, uint16_t* ncl, cudaStream_t s) {
 void launch_apply_bicg_df(const Op<double>& op, const DfTab& t, int mode, const float4* x, double2* y,
                           const double2* w, int conj, double2* sc, double* parts, unsigned* counter, cudaStream_t s) {
     const int g = bicg_grid_blocks(op.dim, op.n), b = kFusedThreads;
-    if (mode == 1) k_apply_bicg_df<1, float4><<<g, b, 0, s>>>(op, t, x, y, w, conj, sc, parts, counter);
-    else k_apply_bicg_df<2, float4><<<g, b, 0, s>>>(op, t, x, y, w, conj, sc, parts, counter);
+    if (mode == 1) launch_after(k_apply_bicg_df<1, float4>, g, b, 0, s, op, t, x, y, w, conj, sc, parts, counter);
+    else launch_after(k_apply_bicg_df<2, float4>, g, b, 0, s, op, t, x, y, w, conj, sc, parts, counter);
 }
 
 void launch_apply_bicg(const Op<double>& op, int mode, const double2* x, double2* y, const double2* w, int conj,
                        double2* sc, double* parts, unsigned* counter, cudaStream_t s) {
     const int g = bicg_grid_blocks(op.dim, op.n), b = kFusedThreads;
-    if (mode == 1) k_apply_bicg<1><<<g, b, 0, s>>>(op, x, y, w, conj, sc, parts, counter);
-    else k_apply_bicg<2><<<g, b, 0, s>>>(op, x, y, w, conj, sc, parts, counter);
+    if (mode == 1) launch_after(k_apply_bicg<1>, g, b, 0, s, op, x, y, w, conj, sc, parts, counter);
+    else launch_after(k_apply_bicg<2>, g, b, 0, s, op, x, y, w, conj, sc, parts, counter);
 }
 
 template int launch_apply<double>(const Op<double>&, const double2*, const double2*, double2*, double*, int,
@@ -1926,7 +1936,7 @@ template void launch_rbgs_half<float>(const Op<float>&, int, const float2*, floa
 
 void launch_residual_red(const Op<double>& op, const double2* z, const double2* v, double2* r_red, int conj,
                          cudaStream_t s) {
-    k_residual_red<<<flat_blocks((op.N + 1) / 2), BX * BY, 0, s>>>(op, z, v, r_red, conj);
+    launch_after(k_residual_red, flat_blocks((op.N + 1) / 2), BX * BY, 0, s, op, z, v, r_red, conj);
 }
 
 void launch_rbgs_df_first(const Op<double>& op, const DfTab& t, const double2* f, float4* fs, float4* xs, int conj,

@@ -487,6 +487,7 @@ template <int KPW, bool SPLIT>
 __global__ void __launch_bounds__(PJ_T, 2) k_project_df(const float2* __restrict__ Q, long long ld, int k,
                                                      const void* __restrict__ rv_, long long N,
                                                      double2* __restrict__ partials, long long rows_per_block) {
+    pdl_begin();
     __shared__ float4 rs[PJ_TILE];       // (re hi, re lo, im hi, im lo)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     constexpr int NW = PJ_T / 32;
@@ -546,6 +547,7 @@ __global__ void __launch_bounds__(PJ_T, 2) k_project_df(const float2* __restrict
 // c_j = fixed-order sum of the block partials, one block per column
 __global__ void __launch_bounds__(64) k_coarse_reduce(const double2* __restrict__ partials, int nblk, int k,
                                                       double2* __restrict__ c) {
+    pdl_begin();
     __shared__ double2 red[2];
     const int j = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     double sx = 0, sy = 0;
@@ -564,6 +566,7 @@ __global__ void __launch_bounds__(64) k_coarse_reduce(const double2* __restrict_
 // y_i = sum_j A_c^-1[i][j] c_j (conj: conj(A_c^-1)), one block per row
 __global__ void __launch_bounds__(64) k_coarse_gemv(const double2* __restrict__ Ainv, int k, int conj,
                                                     const double2* __restrict__ c, double2* __restrict__ y) {
+    pdl_begin();
     __shared__ double2 red[2];
     const int i = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     double sx = 0, sy = 0;
@@ -589,6 +592,7 @@ __global__ void __launch_bounds__(64) k_coarse_gemv(const double2* __restrict__ 
 // (FP64 adds and shuffles run at a small fraction of the FP32 rate on this GPU)
 __global__ void __launch_bounds__(256) k_coarse32_reduce(const float2* __restrict__ partials, int nblk, int k,
                                                          double2* __restrict__ c) {
+    pdl_begin();
     __shared__ float2 red[8];
     const int j = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     float sx = 0.f, sy = 0.f;
@@ -615,6 +619,7 @@ __global__ void __launch_bounds__(256) k_coarse32_reduce(const float2* __restric
 
 __global__ void __launch_bounds__(64) k_coarse32_gemv(const double2* __restrict__ Ainv, int k, int conj,
                                                       const double2* __restrict__ c, float2* __restrict__ y) {
+    pdl_begin();
     __shared__ double2 red[2];
     const int i = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     double sx = 0, sy = 0;
@@ -640,6 +645,7 @@ __global__ void __launch_bounds__(256) k_prolong_df(const float2* __restrict__ Q
                                                     const double2* __restrict__ y, double2* __restrict__ z,
                                                     const float4* __restrict__ base, float4* __restrict__ zdf,
                                                     long long N) {
+    pdl_begin();
     __shared__ float4 ys[kMaxP];
     for (int j = threadIdx.x; j < k; j += blockDim.x) {
         float4 t;
@@ -839,6 +845,7 @@ __global__ void k_rm_to_cm_bf16(const double* __restrict__ A, int ld, int k, __n
 
 __global__ void __launch_bounds__(256) k_prolong32(const __nv_bfloat16* __restrict__ Q, long long ldq, int k,
                                                    const float2* __restrict__ y, float2* __restrict__ z, long long N) {
+    pdl_begin();
     __shared__ float2 ys[kMaxP];
     for (int j = threadIdx.x; j < k; j += blockDim.x) ys[j] = y[j];
     __syncthreads();
@@ -920,6 +927,7 @@ template <bool RED>
 __global__ void __launch_bounds__(256) k_residual32(Op<float> op, const float2* __restrict__ v,
                                                     const float2* __restrict__ z, int conj, float2* __restrict__ r,
                                                     long long M) {
+    pdl_begin();
     for (long long m = blockIdx.x * 256LL + threadIdx.x; m < M; m += gridDim.x * 256LL) {
         if (RED || z) r[m] = row_residual32(op, v, z, RED ? 2 * m + node_colour(2 * m, op.n) : m, conj);
         else r[m] = op.mask[m] ? make_float2(0.f, 0.f) : v[m];
@@ -937,6 +945,7 @@ constexpr int RQ_RANGE = 1024;
 __global__ void __launch_bounds__(256) k_restrict32(const __nv_bfloat16* __restrict__ Qr, long long ldr, int k,
                                                        const float2* __restrict__ r, long long M,
                                                        float2* __restrict__ partials, int S) {
+    pdl_begin();
     const int lane = threadIdx.x & 31;
     const int rg = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int c0 = blockIdx.y * RQ_COLS;
@@ -996,6 +1005,7 @@ __global__ void __launch_bounds__(256) k_restrict32(const __nv_bfloat16* __restr
 __global__ void __launch_bounds__(256) k_prolong32v(const __nv_bfloat16* __restrict__ Q, long long ldq, int k,
                                                     const float2* __restrict__ y, float2* __restrict__ z,
                                                     long long N) {
+    pdl_begin();
     __shared__ float2 ys[kMaxP];
     for (int j = threadIdx.x; j < k; j += blockDim.x) ys[j] = y[j];
     __syncthreads();
@@ -1111,8 +1121,8 @@ void launch_gauss_jordan(const double* C, int ldc, int k, double2* Ainv, double2
 void launch_coarse_apply(const double2* partials, int nblk, int k, const double2* Ainv, int conj, double2* y,
                          double2* cbuf, cudaStream_t s) {
     // two small launches spread over k SMs (FP64 is 2 FMA/clk per SM: one CTA would serialise)
-    k_coarse_reduce<<<k, 64, 0, s>>>(partials, nblk, k, cbuf);
-    k_coarse_gemv<<<k, 64, 0, s>>>(Ainv, k, conj, cbuf, y);
+    launch_after(k_coarse_reduce, k, 64, 0, s, partials, nblk, k, cbuf);
+    launch_after(k_coarse_gemv, k, 64, 0, s, Ainv, k, conj, cbuf, y);
 }
 
 int project_blocks(long long N) {
@@ -1124,7 +1134,7 @@ void launch_project_df(const float2* Q, long long ld, int k, const double2* r, l
                        int nblk, cudaStream_t s) {
     long long rows = (N + nblk - 1) / nblk;
     const int kpw = (k + 15) / 16;
-#define PJ_CASE(K) k_project_df<K, false><<<nblk, PJ_T, 0, s>>>(Q, ld, k, r, N, partials, rows)
+#define PJ_CASE(K) launch_after(k_project_df<K, false>, nblk, PJ_T, 0, s, Q, ld, k, r, N, partials, rows)
     if (kpw <= 1) PJ_CASE(1);
     else if (kpw <= 2) PJ_CASE(2);
     else if (kpw <= 4) PJ_CASE(4);
@@ -1136,20 +1146,20 @@ void launch_project_df(const float2* Q, long long ld, int k, const double2* r, l
 void launch_prolong_df(const float2* Q, long long ld, int k, const double2* y, double2* z, long long N,
                        cudaStream_t s) {
     long long b = (N + 255) / 256;
-    k_prolong_df<false><<<(unsigned)(b < 8 * 152 ? b : 8 * 152), 256, 0, s>>>(Q, ld, k, y, z, nullptr, nullptr, N);
+    launch_after(k_prolong_df<false>, (unsigned)(b < 8 * 152 ? b : 8 * 152), 256, 0, s, Q, ld, k, y, z, nullptr, nullptr, N);
 }
 
 void launch_prolong_df_base(const float2* Q, long long ld, int k, const double2* y, const float4* base, double2* z,
                             float4* zdf, long long N, cudaStream_t s) {
     long long b = (N + 255) / 256;
-    k_prolong_df<true><<<(unsigned)(b < 8 * 152 ? b : 8 * 152), 256, 0, s>>>(Q, ld, k, y, z, base, zdf, N);
+    launch_after(k_prolong_df<true>, (unsigned)(b < 8 * 152 ? b : 8 * 152), 256, 0, s, Q, ld, k, y, z, base, zdf, N);
 }
 
 void launch_project_df_split(const float2* Q, long long ld, int k, const float4* r, long long N, double2* partials,
                              int nblk, cudaStream_t s) {
     long long rows = (N + nblk - 1) / nblk;
     const int kpw = (k + 15) / 16;
-#define PJ_CASE(K) k_project_df<K, true><<<nblk, PJ_T, 0, s>>>(Q, ld, k, r, N, partials, rows)
+#define PJ_CASE(K) launch_after(k_project_df<K, true>, nblk, PJ_T, 0, s, Q, ld, k, r, N, partials, rows)
     if (kpw <= 1) PJ_CASE(1);
     else if (kpw <= 2) PJ_CASE(2);
     else if (kpw <= 4) PJ_CASE(4);
@@ -1208,8 +1218,8 @@ void launch_residual32(const Op<float>& op, const float2* v, const float2* z, bo
                        cudaStream_t s) {
     const long long M = red ? (op.N + 1) / 2 : op.N;
     const unsigned b = (unsigned)std::min<long long>((M + 255) / 256, 16 * 152);
-    if (red) k_residual32<true><<<b, 256, 0, s>>>(op, v, z, conj, r, M);
-    else k_residual32<false><<<b, 256, 0, s>>>(op, v, z, conj, r, M);
+    if (red) launch_after(k_residual32<true>, b, 256, 0, s, op, v, z, conj, r, M);
+    else launch_after(k_residual32<false>, b, 256, 0, s, op, v, z, conj, r, M);
 }
 
 int restrict32_ranges(long long M) { return (int)std::max<long long>(1, (M + RQ_RANGE - 1) / RQ_RANGE); }
@@ -1218,25 +1228,25 @@ int launch_restrict32(const void* Q, long long ld, int k, const float2* r, long 
                       cudaStream_t s) {
     const int S = restrict32_ranges(M);
     const dim3 g((S + 7) / 8, (k + RQ_COLS - 1) / RQ_COLS);
-    k_restrict32<<<g, 256, 0, s>>>(static_cast<const __nv_bfloat16*>(Q), ld, k, r, M, partials, S);
+    launch_after(k_restrict32, g, 256, 0, s, static_cast<const __nv_bfloat16*>(Q), ld, k, r, M, partials, S);
     return S;
 }
 
 void launch_coarse_apply32(const float2* partials, int nblk, int k, const double2* Ainv, int conj, float2* y,
                            double2* cbuf, cudaStream_t s) {
-    k_coarse32_reduce<<<k, 256, 0, s>>>(partials, nblk, k, cbuf);
-    k_coarse32_gemv<<<k, 64, 0, s>>>(Ainv, k, conj, cbuf, y);
+    launch_after(k_coarse32_reduce, k, 256, 0, s, partials, nblk, k, cbuf);
+    launch_after(k_coarse32_gemv, k, 64, 0, s, Ainv, k, conj, cbuf, y);
 }
 
 void launch_prolong32(const void* Q, long long ldq, int k, const float2* y, float2* z, long long N, cudaStream_t s) {
     const __nv_bfloat16* Qb = static_cast<const __nv_bfloat16*>(Q);
     if ((reinterpret_cast<uintptr_t>(z) & 15u) == 0 && (reinterpret_cast<uintptr_t>(Q) & 15u) == 0 && ldq % 8 == 0) {
         const long long b = ((N + 7) / 8 + 255) / 256;
-        k_prolong32v<<<(unsigned)(b < 8 * 152 ? b : 8 * 152), 256, 0, s>>>(Qb, ldq, k, y, z, N);
+        launch_after(k_prolong32v, (unsigned)(b < 8 * 152 ? b : 8 * 152), 256, 0, s, Qb, ldq, k, y, z, N);
         return;
     }
     long long b = (N + 255) / 256;
-    k_prolong32<<<(unsigned)(b < 8 * 152 ? b : 8 * 152), 256, 0, s>>>(Qb, ldq, k, y, z, N);
+    launch_after(k_prolong32, (unsigned)(b < 8 * 152 ? b : 8 * 152), 256, 0, s, Qb, ldq, k, y, z, N);
 }
 
 }  // namespace helm
