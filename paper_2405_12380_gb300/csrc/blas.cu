@@ -4,6 +4,8 @@
 // partial per block, and a single block sums the partials in a fixed order.
 // Scalars (rho, alpha, omega, beta, norms, Hessenberg columns, Givens
 // rotations) stay in device memory; the host only reads a status word.
+#include <algorithm>
+
 #include "bicg.cuh"
 #include "helm_internal.cuh"
 
@@ -35,13 +37,21 @@ __global__ void __launch_bounds__(TB) k_dot(const double2* __restrict__ a, const
     if (threadIdx.x == 0) partials[blockIdx.x] = make_double2(v[0], v[1]);
 }
 
-__global__ void __launch_bounds__(TB) k_norm2(const double2* __restrict__ a, long long N, double* partials) {
+__global__ void __launch_bounds__(TB) k_norm2(const double2* __restrict__ a, long long N, double* partials,
+                                              double* out, unsigned* counter) {
     pdl_begin();
     double acc[1] = {0.0};
     for (long long l = blockIdx.x * (long long)TB + threadIdx.x; l < N; l += (long long)gridDim.x * TB)
         acc[0] = cnorm2(a[l], acc[0]);
     block_tree<1>(acc, threadIdx.x);
     if (threadIdx.x == 0) partials[blockIdx.x] = acc[0];
+    if (last_block_done(counter, gridDim.x)) {
+        sum_parts<1>(partials, gridDim.x, threadIdx.x, acc);
+        if (threadIdx.x == 0) {
+            *out = acc[0];
+            *counter = 0;
+        }
+    }
 }
 
 // fixed-order sum of partials by one block of kFinThreads threads
@@ -292,8 +302,10 @@ int stream_blocks(long long N) {
 void launch_dot(const double2* a, const double2* b, long long N, double2* partials, cudaStream_t s) {
     launch_after(k_dot, kRedBlocks, TB, 0, s, a, b, N, partials);
 }
-void launch_norm2(const double2* a, long long N, double* partials, cudaStream_t s) {
-    launch_after(k_norm2, kRedBlocks, TB, 0, s, a, N, partials);
+void launch_norm2(const double2* a, long long N, double* partials, double* out, unsigned* counter, cudaStream_t s) {
+    // (no more blocks than the vector fills: each costs the last one a partial)
+    const unsigned nb = (unsigned)std::min<long long>(kRedBlocks, (N + TB - 1) / TB);
+    launch_after(k_norm2, nb, TB, 0, s, a, N, partials, out, counter);
 }
 void launch_sum_real(const double* partials, int nparts, double* out, cudaStream_t s) {
     launch_after(k_sum_real, 1, kFinThreads, 0, s, partials, nparts, out);

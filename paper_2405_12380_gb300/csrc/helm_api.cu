@@ -112,19 +112,22 @@ double hs(const helm_handle* h, int slot, int im = 0) { return h->hpin[2 * slot 
 // a grid-barrier wait of the cooperative cycle gave up (flag 4 in S_FLAGS.y, read by poll)
 bool barrier_timed_out(const helm_handle* h) { return hs(h, S_FLAGS, 1) == 4.0; }
 
+// the block counter of a launch that finishes a norm: each takes the next of 64, so that
+// launches on two streams (a handle whose stream was changed without waiting) cannot leave
+// each other's counter off zero
+unsigned* norm_counter(helm_handle* h) { return h->counter + 16 + (h->norm_launch++ & 63u); }
+
 // ||f - A x||^2 into slot (FP64)
 helm_status residual_norm(helm_handle* h, const double2* f, const double2* x, double2* r, int conj, int slot) {
-    const int nb = launch_apply<double>(h->op64, x, f, r, h->red, conj, true, h->stream);
-    launch_sum_real(h->red, nb, scal(h, slot), h->stream);
-    h->launches += 2;
+    launch_apply<double>(h->op64, x, f, r, h->red, conj, true, h->stream, scal(h, slot), norm_counter(h));
+    h->launches += 1;
     CKL();
     return HELM_OK;
 }
 
 helm_status norm2_into(helm_handle* h, const double2* a, int slot) {
-    launch_norm2(a, h->N, h->red, h->stream);
-    launch_sum_real(h->red, kRedBlocks, scal(h, slot), h->stream);
-    h->launches += 2;
+    launch_norm2(a, h->N, h->red, scal(h, slot), norm_counter(h), h->stream);
+    h->launches += 1;
     CKL();
     return HELM_OK;
 }
@@ -1264,12 +1267,12 @@ helm_status helm_create(int dim, int n, double k0, int layer_cells, double layer
     if (dalloc(h, &h->red, (size_t)h->red_len) != HELM_OK) return bail(HELM_OUT_OF_MEMORY);
     if (dalloc(h, &h->sc, (size_t)S_NSLOTS) != HELM_OK) return bail(HELM_OUT_OF_MEMORY);
     if (dalloc(h, &h->dflag, 8) != HELM_OK) return bail(HELM_OUT_OF_MEMORY);
-    if (dalloc(h, &h->counter, 4) != HELM_OK) return bail(HELM_OUT_OF_MEMORY);
+    if (dalloc(h, &h->counter, kCounters) != HELM_OK) return bail(HELM_OUT_OF_MEMORY);
     if (dalloc(h, &h->fparts,
                (size_t)4 * std::max<long long>(std::max(apply_grid_blocks(dim, n), bicg_grid_blocks(dim, n)),
                                                kRedBlocks)) != HELM_OK)
         return bail(HELM_OUT_OF_MEMORY);
-    if (cudaMemset(h->counter, 0, 4 * sizeof(unsigned)) != cudaSuccess) return bail(HELM_CUDA_ERROR);
+    if (cudaMemset(h->counter, 0, kCounters * sizeof(unsigned)) != cudaSuccess) return bail(HELM_CUDA_ERROR);
     if (cudaMallocHost((void**)&h->hpin, sizeof(double2) * S_NSLOTS) != cudaSuccess) return bail(HELM_OUT_OF_MEMORY);
     if (cudaMallocHost((void**)&h->hring, 2 * sizeof(double2) * S_NSLOTS) != cudaSuccess)
         return bail(HELM_OUT_OF_MEMORY);
@@ -1345,12 +1348,12 @@ helm_status helm_create_bvp(int dim, int n, double k0, const uint8_t* mask, cons
     if (cudaMemcpy(h->mask, mask, (size_t)N, cudaMemcpyDefault) != cudaSuccess) return bail(HELM_CUDA_ERROR);
     h->red_len = std::max<long long>(apply_grid_blocks(dim, n), 4LL * kRedBlocks) * 2;
     if (dalloc(h, &h->red, (size_t)h->red_len) != HELM_OK || dalloc(h, &h->sc, (size_t)S_NSLOTS) != HELM_OK ||
-        dalloc(h, &h->dflag, 8) != HELM_OK || dalloc(h, &h->counter, 4) != HELM_OK ||
+        dalloc(h, &h->dflag, 8) != HELM_OK || dalloc(h, &h->counter, kCounters) != HELM_OK ||
         dalloc(h, &h->fparts, (size_t)4 * std::max<long long>(std::max(apply_grid_blocks(dim, n),
                                                                         bicg_grid_blocks(dim, n)),
                                                                kRedBlocks)) != HELM_OK)
         return bail(HELM_OUT_OF_MEMORY);
-    if (cudaMemset(h->counter, 0, 4 * sizeof(unsigned)) != cudaSuccess) return bail(HELM_CUDA_ERROR);
+    if (cudaMemset(h->counter, 0, kCounters * sizeof(unsigned)) != cudaSuccess) return bail(HELM_CUDA_ERROR);
     if (cudaMemset(h->dflag, 0, 8 * sizeof(int)) != cudaSuccess) return bail(HELM_CUDA_ERROR);
     if (cudaMallocHost((void**)&h->hpin, sizeof(double2) * S_NSLOTS) != cudaSuccess ||
         cudaMallocHost((void**)&h->hring, 2 * sizeof(double2) * S_NSLOTS) != cudaSuccess)
@@ -1485,16 +1488,15 @@ helm_status helm_residual(helm_handle* h, const void* f, const void* x, void* r,
                           int dtype) {
     if (!h || !f || !x || !r) return fail(h, HELM_BAD_ARG, "null argument");
     double* part = norm2 ? h->red : nullptr;
-    int nb = 0;
+    unsigned* counter = norm2 ? norm_counter(h) : nullptr;
     if (dtype == HELM_C128)
-        nb = launch_apply<double>(h->op64, (const double2*)x, (const double2*)f, (double2*)r, part, conj, true,
-                                  h->stream);
+        launch_apply<double>(h->op64, (const double2*)x, (const double2*)f, (double2*)r, part, conj, true, h->stream,
+                             norm2, counter);
     else if (dtype == HELM_C64)
-        nb = launch_apply<float>(h->op32, (const float2*)x, (const float2*)f, (float2*)r, part, conj, true,
-                                 h->stream);
+        launch_apply<float>(h->op32, (const float2*)x, (const float2*)f, (float2*)r, part, conj, true, h->stream, norm2,
+                            counter);
     else
         return fail(h, HELM_BAD_ARG, "dtype");
-    if (norm2) launch_sum_real(h->red, nb, norm2, h->stream);
     CKL();
     return HELM_OK;
 }

@@ -68,6 +68,7 @@ constexpr int kMaxP = 256;          // trunk basis functions
 constexpr int kMaxRestart = 64;     // FGMRES(m)
 constexpr int kRedBlocks = 304;     // blocks of the fixed-grid reductions (2 per SM)
 constexpr int kFinThreads = 1024;
+constexpr int kCounters = 80;       // block counters of a handle
 
 // ------------------------------------------------------------ complex helpers
 template <typename R> struct CT;
@@ -223,10 +224,12 @@ cudaError_t launch_after(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t s
 
 // ------------------------------------------------------------ kernel launchers
 // stencil.cu
-// returns the number of per-block partial sums written to `partials` (when given)
+// returns the number of per-block partial sums of ||y||^2 written to `partials` (when
+// given); with a counter (zero between uses) the last block also sums them into *norm
 template <typename R>
 int launch_apply(const Op<R>& op, const typename CT<R>::T* x, const typename CT<R>::T* f,
-                 typename CT<R>::T* y, double* partials, int conj, bool resid, cudaStream_t s);
+                 typename CT<R>::T* y, double* partials, int conj, bool resid, cudaStream_t s,
+                 double* norm = nullptr, unsigned* counter = nullptr);
 template <typename R>
 void launch_jacobi(const Op<R>& op, double omega, const typename CT<R>::T* f,
                    const typename CT<R>::T* xin, typename CT<R>::T* xout, int conj, bool xzero,
@@ -320,7 +323,7 @@ void launch_b32_replace(const double2* r64, float2* r, float2* rhat, float2* p, 
 // blas.cu
 // partial reductions over a fixed grid of kRedBlocks blocks
 void launch_dot(const double2* a, const double2* b, long long N, double2* partials, cudaStream_t s);
-void launch_norm2(const double2* a, long long N, double* partials, cudaStream_t s);
+void launch_norm2(const double2* a, long long N, double* partials, double* out, unsigned* counter, cudaStream_t s);
 void launch_sum_real(const double* partials, int nparts, double* out, cudaStream_t s);
 // BiCGStab pieces (scalars live in device memory, see blas.cu)
 void launch_bicg_update_p(const double2* r, const double2* v, double2* p, const double2* sc, long long N,
@@ -485,7 +488,10 @@ struct helm_handle {
     double* hring = nullptr;        // two pinned snapshots of the scalars (lagged BiCGStab polling)
     cudaEvent_t evring[2] = {nullptr, nullptr};
     int* dflag = nullptr;           // device int flags
-    unsigned* counter = nullptr;    // block counter of the fused reductions (zero between kernels)
+    // block counters, zero between kernels: 0 the fused reductions of the solvers, 2 and 3
+    // the grid barrier, 16 .. 79 the norms (see norm_counter)
+    unsigned* counter = nullptr;
+    unsigned norm_launch = 0;
     double* fparts = nullptr;       // partials of the fused reductions
     // general temporaries (N complex128 each)
     std::vector<double2*> tmp;

@@ -105,6 +105,24 @@ __device__ __forceinline__ typename CT<R>::T nbr_sum(const Op<R>& op, const type
 
 constexpr unsigned kMasked = 0x80u;
 
+// The end of a kernel that left one partial of ||r||^2 per block: the last block sums them
+// in a fixed order into *out (no launch of its own; without a counter they are left).
+struct NormTail {
+    double* out;
+    unsigned* counter;
+};
+__device__ __forceinline__ void norm_tail(const NormTail& t, const double* partials, unsigned nblocks, int tid) {
+    if (!t.counter) return;
+    if (last_block_done(t.counter, nblocks)) {
+        double v[1];
+        sum_parts<1>(partials, (int)nblocks, tid, v);
+        if (tid == 0) {
+            *t.out = v[0];
+            *t.counter = 0;
+        }
+    }
+}
+
 // neighbour code and layer index of a node: from the handle's tables, or from the
 // mask and the indices when the operator carries no tables (no-allocation path)
 template <typename R>
@@ -183,7 +201,8 @@ constexpr int AZ = 256;
 template <typename R, bool RESID, bool NORM>
 __global__ void __launch_bounds__(AZ) k_apply_z(Op<R> op, int zc, const typename CT<R>::T* __restrict__ x,
                                                 const typename CT<R>::T* __restrict__ f,
-                                                typename CT<R>::T* __restrict__ y, double* partials, int conj) {
+                                                typename CT<R>::T* __restrict__ y, double* partials, int conj,
+                                                NormTail tail) {
     pdl_begin();
     using C = typename CT<R>::T;
     const int sy = op.n, sz = op.n * op.n;                 // (N < 2^31)
@@ -246,6 +265,7 @@ __global__ void __launch_bounds__(AZ) k_apply_z(Op<R> op, int zc, const typename
         double v[1] = {acc};
         block_tree<1>(v, threadIdx.x);
         if (threadIdx.x == 0) partials[blockIdx.x + gridDim.x * blockIdx.y] = v[0];
+        norm_tail(tail, partials, gridDim.x * gridDim.y, threadIdx.x);
     }
 }
 
@@ -294,7 +314,7 @@ template <int KIND, bool FLAG, bool NORM, int DOT = 0>
 __global__ void __launch_bounds__(BX * BY) k_march_c64(Op<float> op, int zc, float omega,
                                                        const float4* __restrict__ x, const float4* __restrict__ f,
                                                        float4* __restrict__ y, double* partials, int conj,
-                                                       Dot32 dot = Dot32{}) {
+                                                       Dot32 dot = Dot32{}, NormTail tail = NormTail{}) {
     pdl_begin();
     static_assert(DOT == 0 || (KIND == 0 && !FLAG && !NORM), "the fused reduction follows y = A x only");
     constexpr bool NBR = !(KIND == 1 && FLAG);             // neighbours (and x) are read
@@ -440,6 +460,7 @@ __global__ void __launch_bounds__(BX * BY) k_march_c64(Op<float> op, int zc, flo
     }
     if (NORM) {
         block_reduce_store<float>((double)acc, partials + (blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z)));
+        norm_tail(tail, partials, gridDim.x * gridDim.y * gridDim.z, threadIdx.x + BX * threadIdx.y);
     }
     if (DOT) {
         // S_STOP was set, if at all, by an earlier launch: every block takes the same
@@ -806,7 +827,7 @@ template <typename R, bool RESID, bool NORM>
 __global__ void __launch_bounds__(BX * BY) k_apply(Op<R> op, int zc, const typename CT<R>::T* __restrict__ x,
                                                    const typename CT<R>::T* __restrict__ f,
                                                    typename CT<R>::T* __restrict__ y, double* partials,
-                                                   int conj) {
+                                                   int conj, NormTail tail) {
     pdl_begin();
     const int i = blockIdx.x * BX + threadIdx.x;
     const int j = blockIdx.y * BY + threadIdx.y;
@@ -820,6 +841,7 @@ __global__ void __launch_bounds__(BX * BY) k_apply(Op<R> op, int zc, const typen
                            acc);
     if (NORM) {
         block_reduce_store<R>(acc, partials + (blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z)));
+        norm_tail(tail, partials, gridDim.x * gridDim.y * gridDim.z, threadIdx.x + BX * threadIdx.y);
     }
 }
 
@@ -1696,7 +1718,8 @@ int apply_grid_blocks(int dim, int n) {
 
 template <typename R>
 int launch_apply(const Op<R>& op, const typename CT<R>::T* x, const typename CT<R>::T* f, typename CT<R>::T* y,
-                 double* partials, int conj, bool resid, cudaStream_t s) {
+                 double* partials, int conj, bool resid, cudaStream_t s, double* norm, unsigned* counter) {
+    const NormTail tail{norm, counter};
     if constexpr (std::is_same<R, float>::value) {
         if (pair_ok(op, x, resid ? f : nullptr, y)) {
             int zc;
@@ -1705,11 +1728,11 @@ int launch_apply(const Op<R>& op, const typename CT<R>::T* x, const typename CT<
             const float4* f4 = reinterpret_cast<const float4*>(f);
             float4* y4 = reinterpret_cast<float4*>(y);
             if (resid) {
-                if (partials) launch_after(k_march_c64<0, true, true>, g, b, 0, s, op, zc, 0.f, x4, f4, y4, partials, conj, Dot32{});
-                else launch_after(k_march_c64<0, true, false>, g, b, 0, s, op, zc, 0.f, x4, f4, y4, partials, conj, Dot32{});
+                if (partials) launch_after(k_march_c64<0, true, true>, g, b, 0, s, op, zc, 0.f, x4, f4, y4, partials, conj, Dot32{}, tail);
+                else launch_after(k_march_c64<0, true, false>, g, b, 0, s, op, zc, 0.f, x4, f4, y4, partials, conj, Dot32{}, tail);
             } else {
-                if (partials) launch_after(k_march_c64<0, false, true>, g, b, 0, s, op, zc, 0.f, x4, f4, y4, partials, conj, Dot32{});
-                else launch_after(k_march_c64<0, false, false>, g, b, 0, s, op, zc, 0.f, x4, f4, y4, partials, conj, Dot32{});
+                if (partials) launch_after(k_march_c64<0, false, true>, g, b, 0, s, op, zc, 0.f, x4, f4, y4, partials, conj, Dot32{}, tail);
+                else launch_after(k_march_c64<0, false, false>, g, b, 0, s, op, zc, 0.f, x4, f4, y4, partials, conj, Dot32{}, tail);
             }
             return (int)(g.x * g.y * g.z);
         }
@@ -1718,11 +1741,11 @@ int launch_apply(const Op<R>& op, const typename CT<R>::T* x, const typename CT<
         int zc;
         const dim3 g = applyz_grid(op.n, &zc);
         if (resid) {
-            if (partials) launch_after(k_apply_z<R, true, true>, g, AZ, 0, s, op, zc, x, f, y, partials, conj);
-            else launch_after(k_apply_z<R, true, false>, g, AZ, 0, s, op, zc, x, f, y, partials, conj);
+            if (partials) launch_after(k_apply_z<R, true, true>, g, AZ, 0, s, op, zc, x, f, y, partials, conj, tail);
+            else launch_after(k_apply_z<R, true, false>, g, AZ, 0, s, op, zc, x, f, y, partials, conj, tail);
         } else {
-            if (partials) launch_after(k_apply_z<R, false, true>, g, AZ, 0, s, op, zc, x, f, y, partials, conj);
-            else launch_after(k_apply_z<R, false, false>, g, AZ, 0, s, op, zc, x, f, y, partials, conj);
+            if (partials) launch_after(k_apply_z<R, false, true>, g, AZ, 0, s, op, zc, x, f, y, partials, conj, tail);
+            else launch_after(k_apply_z<R, false, false>, g, AZ, 0, s, op, zc, x, f, y, partials, conj, tail);
         }
         return (int)(g.x * g.y);
     }
@@ -1730,11 +1753,11 @@ int launch_apply(const Op<R>& op, const typename CT<R>::T* x, const typename CT<
     dim3 g = grid_for(op.dim, op.n, 1, zc), b(BX, BY);
     // 2D, or an operator without the per-node tables (the allocation-free path)
     if (resid) {
-        if (partials) launch_after(k_apply<R, true, true>, g, b, 0, s, op, zc, x, f, y, partials, conj);
-        else launch_after(k_apply<R, true, false>, g, b, 0, s, op, zc, x, f, y, partials, conj);
+        if (partials) launch_after(k_apply<R, true, true>, g, b, 0, s, op, zc, x, f, y, partials, conj, tail);
+        else launch_after(k_apply<R, true, false>, g, b, 0, s, op, zc, x, f, y, partials, conj, tail);
     } else {
-        if (partials) launch_after(k_apply<R, false, true>, g, b, 0, s, op, zc, x, f, y, partials, conj);
-        else launch_after(k_apply<R, false, false>, g, b, 0, s, op, zc, x, f, y, partials, conj);
+        if (partials) launch_after(k_apply<R, false, true>, g, b, 0, s, op, zc, x, f, y, partials, conj, tail);
+        else launch_after(k_apply<R, false, false>, g, b, 0, s, op, zc, x, f, y, partials, conj, tail);
     }
     return (int)(g.x * g.y * g.z);
 }
@@ -1749,8 +1772,8 @@ void launch_jacobi(const Op<R>& op, double omega, const typename CT<R>::T* f, co
             const float4* x4 = reinterpret_cast<const float4*>(xin);
             const float4* f4 = reinterpret_cast<const float4*>(f);
             float4* y4 = reinterpret_cast<float4*>(xout);
-            if (xzero) launch_after(k_march_c64<1, true, false>, g, b, 0, s, op, zc, (float)omega, x4, f4, y4, nullptr, conj, Dot32{});
-            else launch_after(k_march_c64<1, false, false>, g, b, 0, s, op, zc, (float)omega, x4, f4, y4, nullptr, conj, Dot32{});
+            if (xzero) launch_after(k_march_c64<1, true, false>, g, b, 0, s, op, zc, (float)omega, x4, f4, y4, nullptr, conj, Dot32{}, NormTail{});
+            else launch_after(k_march_c64<1, false, false>, g, b, 0, s, op, zc, (float)omega, x4, f4, y4, nullptr, conj, Dot32{}, NormTail{});
             return;
         }
     }
@@ -1813,7 +1836,7 @@ bool launch_red_residual32(const Op<float>& op, const float2* f, const float2* x
     const dim3 g = pair_grid(op.n, &zc), b(BX, BY);
     launch_after(k_march_c64<2, false, false>, g, b, 0, s, op, zc, 0.f, reinterpret_cast<const float4*>(x),
                                                  reinterpret_cast<const float4*>(f), reinterpret_cast<float4*>(r_red),
-                                                 nullptr, conj, Dot32{});
+                                                 nullptr, conj, Dot32{}, NormTail{});
     return true;
 }
 
@@ -1825,8 +1848,8 @@ int launch_apply32_bicg(const Op<float>& op, int mode, const float2* x, float2* 
     const Dot32 d{reinterpret_cast<const float4*>(w), const_cast<double2*>(sc), parts};
     const float4* x4 = reinterpret_cast<const float4*>(x);
     float4* y4 = reinterpret_cast<float4*>(y);
-    if (mode == 1) launch_after(k_march_c64<0, false, false, 1>, g, b, 0, s, op, zc, 0.f, x4, nullptr, y4, nullptr, conj, d);
-    else launch_after(k_march_c64<0, false, false, 2>, g, b, 0, s, op, zc, 0.f, x4, nullptr, y4, nullptr, conj, d);
+    if (mode == 1) launch_after(k_march_c64<0, false, false, 1>, g, b, 0, s, op, zc, 0.f, x4, nullptr, y4, nullptr, conj, d, NormTail{});
+    else launch_after(k_march_c64<0, false, false, 2>, g, b, 0, s, op, zc, 0.f, x4, nullptr, y4, nullptr, conj, d, NormTail{});
     return (int)(g.x * g.y * g.z);
 }
 
@@ -1922,9 +1945,9 @@ void launch_apply_bicg(const Op<double>& op, int mode, const double2* x, double2
 }
 
 template int launch_apply<double>(const Op<double>&, const double2*, const double2*, double2*, double*, int,
-                                  bool, cudaStream_t);
+                                  bool, cudaStream_t, double*, unsigned*);
 template int launch_apply<float>(const Op<float>&, const float2*, const float2*, float2*, double*, int, bool,
-                                 cudaStream_t);
+                                 cudaStream_t, double*, unsigned*);
 template void launch_jacobi<double>(const Op<double>&, double, const double2*, const double2*, double2*, int,
                                     bool, cudaStream_t);
 template void launch_jacobi<float>(const Op<float>&, double, const float2*, const float2*, float2*, int, bool,

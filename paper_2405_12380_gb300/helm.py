@@ -133,7 +133,7 @@ class Problem:
 
     def residual(self, f, x, conj=False, want_norm=True):
         r = torch.empty_like(x)
-        nrm = torch.zeros(1, dtype=torch.float64, device="cuda") if want_norm else None
+        nrm = torch.empty(1, dtype=torch.float64, device="cuda") if want_norm else None
         self._check(self.lib.helm_residual(self.h, _ptr(f), _ptr(x), _ptr(r), _ptr(nrm), int(conj),
                                            _dtype_code(x)), "residual")
         return (r, nrm) if want_norm else r
