@@ -248,9 +248,12 @@ void launch_rbgs_half(const Op<R>& op, int colour, const typename CT<R>::T* f, t
 // one full red-black sweep, colour c0 on every node then colour 1 - c0, from xin
 // (nullptr: from zero) into xout (a different buffer) in one launch; returns false
 // without launching where the fused kernel does not apply (2D, odd n, n > 256,
-// outer-boundary rows, unaligned vectors)
+// outer-boundary rows, unaligned vectors).  cin / cout (omega 1 only): xin / xout hold
+// the nodes of colour 1 - c0 alone, N / 2 values
 bool launch_rbgs_sweep32(const Op<float>& op, int c0, const float2* f, const float2* xin, float2* xout, int conj,
-                         double omega, cudaStream_t s);
+                         double omega, bool cin, bool cout, cudaStream_t s);
+// out[pair] = the node of that colour (3D, n even)
+void launch_pack_colour(const Op<float>& op, int colour, const float2* x, float2* out, cudaStream_t s);
 bool rbgs_sweep32_ok(const Op<float>& op, const void* f, const void* x, const void* tmp);
 void plan_sweep32(Op<float>& op);     // sets op.sw_rows, op.sw_zc (occupancy queries: outside stream capture)
 void launch_node_pack(const Op<float>& op, uint16_t* ncl, cudaStream_t s);

@@ -608,7 +608,10 @@ __global__ void __launch_bounds__(BX * BY) k_rbgs_c64(Op<float> op, int zc, int 
 //  - in both, one x-neighbour is the thread's own pair, the other the pair to the left or
 //    right (alternating with the plane), y-neighbours are one row away, z-neighbours are
 //    the thread's own values of the planes before and after.
-// Old values of the swept nodes themselves are read only for SOR.  A node with all six
+// Old values of the swept nodes themselves are read only for SOR; without it the next sweep
+// in the same order needs the colour-B nodes alone, so sweeps in a row pass just those on
+// (CIN, COUT: xin, xout hold one float2 per pair; 18 B a node of reads and writes between
+// two others, 22 at the ends of a run, instead of 26).  A node with all six
 // neighbours fluid (the common case) takes no selects.  Every node value comes from the
 // arithmetic of k_rbgs_c64 with the neighbour sums in the same order, so one launch equals
 // two half-sweeps.  Measured against the form that staged whole pairs and selected by
@@ -653,11 +656,12 @@ __host__ __device__ constexpr size_t sweep_smem_bytes(int txt, int tyt, bool xze
            sizeof(float2);
 }
 
-template <bool XZERO, bool SOR, bool K2>
+template <bool XZERO, bool SOR, bool K2, bool CIN, bool COUT>
 __global__ void __launch_bounds__(kSweepMaxThreads, 1)
     k_sweep_c64(Op<float> op, int zc, int c0, const float4* __restrict__ f, const float2* __restrict__ xin,
-                float4* __restrict__ xout, int conj, float omega) {
+                float2* __restrict__ xout, int conj, float omega) {
     pdl_begin();
+    static_assert(!(SOR && (CIN || COUT)) && !(XZERO && CIN), "SOR reads the old values of both colours");
     extern __shared__ __align__(16) float2 sweep_smem[];
     constexpr unsigned kOut = kMasked | (kMasked << 16);   // (code, layer) byte pairs of two masked nodes
     const int n = op.n, h = n >> 1;
@@ -697,8 +701,9 @@ __global__ void __launch_bounds__(kSweepMaxThreads, 1)
     // stage plane p (zeros outside the grid) at offset so; a: position of colour A there
     auto stage = [&](int p, int so, int a) {
         const bool pin = p >= 0 && p < n;
-        cp_async8(xs + so + mx, xin + HCHK(pin && row_ok ? 2 * (lrow + sz * p) + (a ^ 1) : 0, op.N), pin && row_ok);
-        if (halo) cp_async8(xs + so + mo, xin + HCHK(pin && out_ok ? 2 * (lout + sz * p) + a : 0, op.N), pin && out_ok);
+        auto at = [&](int q, int pos) { return CIN ? q : 2 * q + pos; };
+        cp_async8(xs + so + mx, xin + HCHK(pin && row_ok ? at(lrow + sz * p, a ^ 1) : 0, CIN ? NP : op.N), pin && row_ok);
+        if (halo) cp_async8(xs + so + mo, xin + HCHK(pin && out_ok ? at(lout + sz * p, a) : 0, CIN ? NP : op.N), pin && out_ok);
     };
     int o_0 = 0, o_p1 = PX, o_p2 = 2 * PX, o_p3 = 3 * PX;
     if (!XZERO) {
@@ -728,7 +733,10 @@ __global__ void __launch_bounds__(kSweepMaxThreads, 1)
     float2 fb = z2, xb = z2, ib = z2;                      // colour B of plane t - 1: f, old value, 1/diag
     unsigned cb = kMasked;                                 // its code and layer bytes
     float2 bm1 = z2, b0 = z2;                              // own old colour-B values at planes t - 1, t
-    if (!XZERO && row_ok && t >= 1) bm1 = xin[HCHK(2 * (lrow + sz * (t - 1)) + ar, op.N)];
+    if (!XZERO && row_ok && t >= 1) {
+        const int q = lrow + sz * (t - 1);
+        bm1 = xin[HCHK(CIN ? q : 2 * q + ar, CIN ? NP : op.N)];
+    }
     __syncthreads();
     if (!XZERO) b0 = xs[o_0 + mx];
     int rs = 0, rs_m = 2 * PR;                             // ring planes of t and t - 1
@@ -796,7 +804,11 @@ __global__ void __launch_bounds__(kSweepMaxThreads, 1)
             }
             // (from zero only colour A starts from zero: colour B's own old value is zero too)
             if (SOR) nb = cadd(xb, cscale(omega, csub(nb, xb)));
-            xout[HCHK(l - sz, NP)] = ar ? make_float4(am1.x, am1.y, nb.x, nb.y) : make_float4(nb.x, nb.y, am1.x, am1.y);
+            if (COUT)
+                xout[HCHK(l - sz, NP)] = nb;
+            else
+                reinterpret_cast<float4*>(xout)[HCHK(l - sz, NP)] =
+                    ar ? make_float4(am1.x, am1.y, nb.x, nb.y) : make_float4(nb.x, nb.y, am1.x, am1.y);
         }
         am2 = am1;
         am1 = na;
@@ -1855,12 +1867,25 @@ int launch_apply32_bicg(const Op<float>& op, int mode, const float2* x, float2* 
 
 namespace {
 
-using SweepFn = void (*)(Op<float>, int, int, const float4*, const float2*, float4*, int, float);
-SweepFn sweep_fn(bool xzero, bool sor, bool k2) {
-    if (xzero) return sor ? (k2 ? k_sweep_c64<true, true, true> : k_sweep_c64<true, true, false>)
-                          : (k2 ? k_sweep_c64<true, false, true> : k_sweep_c64<true, false, false>);
-    return sor ? (k2 ? k_sweep_c64<false, true, true> : k_sweep_c64<false, true, false>)
-               : (k2 ? k_sweep_c64<false, false, true> : k_sweep_c64<false, false, false>);
+using SweepFn = void (*)(Op<float>, int, int, const float4*, const float2*, float2*, int, float);
+template <bool K2>
+SweepFn sweep_fn(bool xzero, bool sor, bool cin, bool cout) {
+    if (sor) return xzero ? k_sweep_c64<true, true, K2, false, false> : k_sweep_c64<false, true, K2, false, false>;
+    if (xzero) return cout ? k_sweep_c64<true, false, K2, false, true> : k_sweep_c64<true, false, K2, false, false>;
+    if (cin) return cout ? k_sweep_c64<false, false, K2, true, true> : k_sweep_c64<false, false, K2, true, false>;
+    return cout ? k_sweep_c64<false, false, K2, false, true> : k_sweep_c64<false, false, K2, false, false>;
+}
+
+// the nodes of one colour, one float2 per pair
+__global__ void __launch_bounds__(256) k_pack_colour(int n, int colour, const float4* __restrict__ x,
+                                                     float2* __restrict__ out, unsigned npairs) {
+    pdl_begin();
+    const unsigned h = n / 2;
+    for (unsigned q = blockIdx.x * 256 + threadIdx.x; q < npairs; q += gridDim.x * 256) {
+        const unsigned row = q / h, k = row / n, j = row - k * n;
+        const float4 v = x[q];
+        out[q] = ((j + k + colour) & 1) ? hi2(v) : lo2(v);
+    }
 }
 
 }  // namespace
@@ -1882,13 +1907,13 @@ void plan_sweep32(Op<float>& op) {
     cudaGetDevice(&dev);
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 152;
     double best = 0;
-    if (cudaFuncSetAttribute(k_sweep_c64<false, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024) !=
+    if (cudaFuncSetAttribute(k_sweep_c64<false, false, false, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024) !=
         cudaSuccess)
         return;
     for (int tyt = 8; tyt <= 32 && tyt * txt <= kSweepMaxThreads; tyt *= 2) {
         int occ = 0;
         const size_t smem = sweep_smem_bytes(txt, tyt, false);
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_sweep_c64<false, false, false>, txt * tyt, smem) !=
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_sweep_c64<false, false, false, false, false>, txt * tyt, smem) !=
                 cudaSuccess ||
             occ < 1)
             continue;
@@ -1913,17 +1938,23 @@ bool rbgs_sweep32_ok(const Op<float>& op, const void* f, const void* x, const vo
 }
 
 bool launch_rbgs_sweep32(const Op<float>& op, int c0, const float2* f, const float2* xin, float2* xout, int conj,
-                         double omega, cudaStream_t s) {
-    if (!rbgs_sweep32_ok(op, f, xin, xout)) return false;
+                         double omega, bool cin, bool cout, cudaStream_t s) {
+    if (!rbgs_sweep32_ok(op, f, xin, xout) || (omega != 1.0 && (cin || cout)) || (cin && !xin)) return false;
     const int txt = (op.n / 2 + 31) / 32 * 32, tyt = op.sw_rows;
     const dim3 g(1, (op.n + tyt - 3) / (tyt - 2), (op.n + op.sw_zc - 1) / op.sw_zc), b(txt, tyt);
     const size_t smem = sweep_smem_bytes(txt, tyt, xin == nullptr);   // at most 78 KB
-    const SweepFn fn = sweep_fn(xin == nullptr, omega != 1.0, op.k2 != nullptr);
+    const SweepFn fn = (op.k2 ? sweep_fn<true> : sweep_fn<false>)(xin == nullptr, omega != 1.0, cin, cout);
     if (smem > 48 * 1024 &&
         cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024) != cudaSuccess)
         return false;
-    return launch_after(fn, g, b, smem, s, op, op.sw_zc, c0, reinterpret_cast<const float4*>(f), xin,
-                        reinterpret_cast<float4*>(xout), conj, (float)omega) == cudaSuccess;
+    return launch_after(fn, g, b, smem, s, op, op.sw_zc, c0, reinterpret_cast<const float4*>(f), xin, xout, conj,
+                        (float)omega) == cudaSuccess;
+}
+
+void launch_pack_colour(const Op<float>& op, int colour, const float2* x, float2* out, cudaStream_t s) {
+    const long long np = op.N / 2;
+    launch_after(k_pack_colour, dim3((unsigned)std::min<long long>((np + 255) / 256, 8 * 152)), dim3(256), 0, s, op.n,
+                 colour, reinterpret_cast<const float4*>(x), out, (unsigned)np);
 }
 
 void launch_node_pack(const Op<float>& op, uint16_t* ncl, cudaStream_t s) {
