@@ -10,20 +10,25 @@
 //    epilogue warp hold neighbouring columns and its stores coalesce) and TN rows of C (the
 //    N side): 16 to 128, as few as leave about one CTA per SM.  K is not split: the sum of
 //    each value stays one chain, whatever the tile;
-//  - warp 0: one elected thread loads the two boxes of a 64-deep K step with
-//    cp.async.bulk.tensor (128-byte swizzle) onto the stage's "full" mbarrier; the ring has
-//    as many stages as K has steps, up to what 200 KB hold (11 with TN = 16);
+//  - warp 0: one elected thread loads the two boxes of every 64-deep K step with
+//    cp.async.bulk.tensor (128-byte swizzle); a stage is SUB such steps on one "full"
+//    mbarrier, and the ring has as many stages as K fills, up to what 222 KB hold (three);
 //  - warp 1: one elected thread issues tcgen05.mma.kind::f16 (K = 16 per instruction, four
-//    per stage) into a TMEM accumulator and commits each stage to its "empty" mbarrier, the
-//    last one to the "done" mbarrier;
+//    per step) into a TMEM accumulator and commits each stage to its "empty" mbarrier, the
+//    last one to the "done" mbarrier as well;
 //  - warp 2 allocates and frees the TMEM columns;
 //  - warps 4-7 (one per quarter of the TMEM lanes) read the accumulator with
 //    tcgen05.ld and write alpha D + beta C for the valid rows and columns.
 // What bounds it: the branch's first layer (64 x 256 x 128000 at 40^3) is a chain of 8000
-// dependent MMAs per value on 8 CTAs; it takes about 80 ns a link, 0.9 -> 0.66 ms (ncu,
-// cold).  Splitting K would shorten it but change the last bits of the activations, which
-// the next layer rounds to BF16.  Its weight gradient (K = 64, 256 x 128000 values) is
-// bound by the stores: 197 -> 32 us with lanes along C's rows.
+// dependent MMAs per value on 8 CTAs.  An MMA takes about 27 ns whatever its width, and one
+// round of wait and commit about 150 ns of the issuing thread (measured with the loads, the
+// MMAs and the commits left out in turn), so a stage holds as many K steps as still leave
+// three stages: per step 330 ns with one step a stage and a lane == 0 branch, 251 elected,
+// 178 with two steps, 146 with three, 131 with four (145 with six, which leaves two stages).
+// Looking at the next stage's barrier before the MMAs gains with one or two steps and loses
+// with more.  64 x 256 x 128000: 660 -> 262 us.  Splitting K would shorten it further but
+// change the last bits of the activations, which the next layer rounds to BF16.  The weight
+// gradient (K = 64, 256 x 128000 values) is bound by the stores: 32 us.
 // Every mbarrier wait is bounded: a wait that runs out records an error flag and the
 // thread goes on (the result is then garbage but the launch ends); the host reads
 // the flag with nn_gemm_bf16_status.
@@ -42,7 +47,7 @@ namespace {
 
 constexpr int TBM = 128, TBK = 64, MAX_STAGES = 16;
 constexpr int TC_THREADS = 256;
-constexpr unsigned kRingBytes = 200 * 1024;                    // shared memory of the stages, at most
+constexpr unsigned kRingBytes = 222 * 1024;                    // shared memory of the stages, at most
 constexpr unsigned kWaitLimit = 1u << 26;
 
 __device__ int g_tc_error;
@@ -78,6 +83,15 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* b, unsigned parity) {
     return false;
 }
 
+// true in one lane of the warp (all lanes arrive).  The issuing instructions take their
+// operands from uniform registers; inside a lane == 0 branch the compiler moves every one
+// there through a loop over the lanes.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+    return p != 0;
+}
+
 __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
     asm volatile(
         "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
@@ -98,7 +112,7 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int m, int n) {
 }
 
 // C (M x N) = alpha A B^T + beta C from the K-major copies; mapN: op(B)^T, mapM: op(A)
-template <int TN>
+template <int TN, int SUB>
 __global__ void __launch_bounds__(TC_THREADS)
     k_gemm_bf16_tc(const __grid_constant__ CUtensorMap mapN, const __grid_constant__ CUtensorMap mapM, int M, int N,
                    int Kp, int stages, float alpha, float beta, float* __restrict__ C, int ldc) {
@@ -108,7 +122,7 @@ __global__ void __launch_bounds__(TC_THREADS)
     // 1024-byte alignment of the stage buffers (the swizzle atom)
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint8_t* sN = smem;
-    uint8_t* sM = smem + stages * kNBytes;
+    uint8_t* sM = smem + min(stages * SUB, Kp / TBK) * kNBytes;
     __shared__ uint64_t full[MAX_STAGES], empty[MAX_STAGES], done;
     __shared__ uint32_t tmem_base;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -135,50 +149,68 @@ __global__ void __launch_bounds__(TC_THREADS)
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_base;
 
-    if (warp == 0 && lane == 0) {
+    if (warp == 0) {
         // producer
         int s = 0;
         unsigned parity = 1;                               // (the first round finds every stage empty)
-        for (int kb = 0; kb < nk; ++kb) {
-            if (kb >= stages) mbar_wait(&empty[s], parity);
-            mbar_expect_tx(&full[s], kNBytes + kMBytes);
-            tma_load_2d(sN + s * kNBytes, &mapN, kb * TBK, n0, &full[s]);
-            tma_load_2d(sM + s * kMBytes, &mapM, kb * TBK, m0, &full[s]);
+        for (int kb = 0, g = 0; kb < nk; kb += SUB, ++g) {
+            if (g >= stages) mbar_wait(&empty[s], parity);
+            if (elect_one()) {
+                const int sub = min(SUB, nk - kb);
+                mbar_expect_tx(&full[s], sub * (kNBytes + kMBytes));
+#pragma unroll
+                for (int u = 0; u < SUB; ++u)
+                    if (u < sub) {
+                        tma_load_2d(sN + (s * SUB + u) * kNBytes, &mapN, (kb + u) * TBK, n0, &full[s]);
+                        tma_load_2d(sM + (s * SUB + u) * kMBytes, &mapM, (kb + u) * TBK, m0, &full[s]);
+                    }
+            }
             if (++s == stages) {
                 s = 0;
                 parity ^= 1u;
             }
         }
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
         // MMA issuer
         constexpr uint32_t idesc = idesc_bf16(TBM, TN);
+        const uint64_t dn0 = smem_desc(sN), dm0 = smem_desc(sM);
         int s = 0;
         unsigned parity = 0;
-        for (int kb = 0; kb < nk; ++kb) {
+        for (int kb = 0; kb < nk; kb += SUB) {
             mbar_wait(&full[s], parity);
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint64_t da = smem_desc(sN + s * kNBytes), db = smem_desc(sM + s * kMBytes);
+            if (elect_one()) {
 #pragma unroll
-            for (int k = 0; k < TBK / 16; ++k) {
-                // K = 16 BF16 = 32 bytes further along the swizzled 128-byte rows
-                const uint64_t koff = (uint64_t)((k * 32) >> 4);
-                const uint32_t acc = (kb > 0 || k > 0) ? 1u : 0u;
-                asm volatile(
-                    "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                    " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
-                    "l"(da + koff), "l"(db + koff), "r"(idesc), "r"(acc)
-                    : "memory");
+                for (int u = 0; u < SUB; ++u) {
+                    if (kb + u < nk) {
+                        const uint64_t da = dn0 + (uint64_t)((s * SUB + u) * (kNBytes >> 4));
+                        const uint64_t db = dm0 + (uint64_t)((s * SUB + u) * (kMBytes >> 4));
+#pragma unroll
+                        for (int k = 0; k < TBK / 16; ++k) {
+                            // K = 16 BF16 = 32 bytes further along the swizzled 128-byte rows
+                            const uint64_t koff = (uint64_t)((k * 32) >> 4);
+                            const uint32_t acc = (kb > 0 || u > 0 || k > 0) ? 1u : 0u;
+                            asm volatile(
+                                "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+                                " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
+                                "l"(da + koff), "l"(db + koff), "r"(idesc), "r"(acc)
+                                : "memory");
+                        }
+                    }
+                }
+                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                                 su32(&empty[s]))
+                             : "memory");
+                if (kb + SUB >= nk)
+                    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                                     su32(&done))
+                                 : "memory");
             }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                             su32(&empty[s]))
-                         : "memory");
             if (++s == stages) {
                 s = 0;
                 parity ^= 1u;
             }
         }
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(su32(&done))
-                     : "memory");
     } else if (warp >= 4) {
         // epilogue: warp 4 + q reads TMEM lanes 32 q .. 32 q + 31 (columns n of the tile)
         const int q = warp - 4;
@@ -336,17 +368,17 @@ struct Ws {
 std::mutex g_ws_mutex;
 Ws g_ws[64];
 
-template <int TN>
+template <int TN, int SUB>
 cudaError_t gemm_tc(const CUtensorMap& mn, const CUtensorMap& mm, int M, int N, int Kp, float alpha, float beta, float* C,
                     int ldc, cudaStream_t s) {
-    constexpr unsigned stage = (TBM + TN) * TBK * 2;
-    const int stages = std::min(std::min(Kp / TBK, MAX_STAGES), (int)(kRingBytes / stage));
-    const size_t smem = (size_t)stages * stage + 1024;
+    constexpr unsigned stage = (TBM + TN) * TBK * 2 * SUB;
+    const int stages = std::min(std::min((Kp / TBK + SUB - 1) / SUB, MAX_STAGES), (int)(kRingBytes / stage));
+    const size_t smem = (size_t)std::min(stages * SUB, Kp / TBK) * (stage / SUB) + 1024;
     const cudaError_t e =
-        cudaFuncSetAttribute(k_gemm_bf16_tc<TN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kRingBytes + 1024));
+        cudaFuncSetAttribute(k_gemm_bf16_tc<TN, SUB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kRingBytes + 1024));
     if (e != cudaSuccess) return e;
     const long long tiles = (long long)((M + TN - 1) / TN) * ((N + TBM - 1) / TBM);
-    k_gemm_bf16_tc<TN><<<(unsigned)tiles, TC_THREADS, smem, s>>>(mn, mm, M, N, Kp, stages, alpha, beta, C, ldc);
+    k_gemm_bf16_tc<TN, SUB><<<(unsigned)tiles, TC_THREADS, smem, s>>>(mn, mm, M, N, Kp, stages, alpha, beta, C, ldc);
     return cudaGetLastError();
 }
 
@@ -401,10 +433,10 @@ extern "C" helm_status nn_gemm_bf16(int transA, int transB, int M, int N, int K,
     while (tn > 16 && tn / 2 >= M) tn /= 2;                // (no taller than the rows there are)
     CUtensorMap mn, mm;
     if (!make_map(&mn, Bb, Np, Kp, TBM) || !make_map(&mm, Ab, Mp, Kp, tn)) return HELM_CUDA_ERROR;
-    const cudaError_t e = tn == 128  ? gemm_tc<128>(mn, mm, M, N, Kp, alpha, beta, C, ldc, s)
-                          : tn == 64 ? gemm_tc<64>(mn, mm, M, N, Kp, alpha, beta, C, ldc, s)
-                          : tn == 32 ? gemm_tc<32>(mn, mm, M, N, Kp, alpha, beta, C, ldc, s)
-                                     : gemm_tc<16>(mn, mm, M, N, Kp, alpha, beta, C, ldc, s);
+    const cudaError_t e = tn == 128  ? gemm_tc<128, 2>(mn, mm, M, N, Kp, alpha, beta, C, ldc, s)
+                          : tn == 64 ? gemm_tc<64, 3>(mn, mm, M, N, Kp, alpha, beta, C, ldc, s)
+                          : tn == 32 ? gemm_tc<32, 3>(mn, mm, M, N, Kp, alpha, beta, C, ldc, s)
+                                     : gemm_tc<16, 4>(mn, mm, M, N, Kp, alpha, beta, C, ldc, s);
     if (ordered) {
         if (cudaEventRecord(w.ev, s) != cudaSuccess) return HELM_CUDA_ERROR;
         w.used = true;

@@ -155,3 +155,19 @@ def test_gemm_bf16_tiles(ta, tb, M, N, K):
         assert np.array_equal(got[:, N:], C0[:, N:])
     flag = C.c_int(-1)
     assert _lib().nn_gemm_bf16_status(C.byref(flag)) == 0 and flag.value == 0
+
+
+@pytest.mark.parametrize("N", [256, 4096, 8192, 16384])   # tiles of 16, 32, 64 and 128 rows
+@pytest.mark.parametrize("K", [100, 192, 450, 833])        # 2, 3, 8 and 14 K steps: stages filled, part filled, reused
+def test_gemm_bf16_stages(N, K):
+    """Stages of several K steps, the last one part filled: bound as in test_gemm_bf16_tiles."""
+    from oracle.tb import bf16_round
+    M = 128
+    rng = np.random.default_rng(N + K)
+    A, B = rng.standard_normal((M, K)).astype(np.float32), rng.standard_normal((N, K)).astype(np.float32)
+    opA, opB = bf16_round(A.astype(np.float64)), bf16_round(B.T.astype(np.float64))
+    Ad, Bd, Cd = to_dev(A), to_dev(B), to_dev(np.full((M, N), np.nan, np.float32))
+    assert _lib().nn_gemm_bf16(0, 1, M, N, K, 1.0, _p(Ad), K, _p(Bd), K, 0.0, _p(Cd), N, None) == 0
+    assert np.all(np.abs(Cd.cpu().numpy() - opA @ opB) <= 4 * K * U * (np.abs(opA) @ np.abs(opB)) + 1e-30)
+    flag = C.c_int(-1)
+    assert _lib().nn_gemm_bf16_status(C.byref(flag)) == 0 and flag.value == 0
