@@ -316,7 +316,7 @@ def kernel_entries(w, st_prof, N, k, hbm, hbm_src, workload):
                     "timing": "CUDA events around every launch, one profiled solve after the timed solves"})
 
     if mixed:
-        add("restrict", "k_march_c64<2> + k_restrict32_rr", "n_restrict", "restrict_ms", (k + 26.0) * N,
+        add("restrict", "k_march_c64<2> + k_restrict32", "n_restrict", "restrict_ms", (k + 26.0) * N,
             "c = Q_red^T (v - A z) on the red rows: red residual, then BF16 tall-skinny product")
         add("prolong", "k_prolong32v", "n_prolong", "prolong_ms", (2.0 * k + 16.0) * N, "z += Q y, BF16 Q")
         nr = max(1, w["n_r"])

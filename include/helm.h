@@ -315,6 +315,7 @@ helm_status helm_set_k2(helm_handle* h, const double* k2);
  *   ReLU (slope 0.01) (bias may be NULL).
  * nn_act_backward: dX *= act'(Y), Y the activation output.
  * nn_bias_grad: db[c] = sum_r dY[r][c].
+ * nn_bias_grad_rows: the same, each sum taken in the order of the rows.
  * nn_adam: Adam with bias correction, step t >= 1.
  * nn_rel_l2: per-sample ||pred - target||^2 / ||target||^2 over P2 values and the
  *   gradient of the batch mean with respect to pred.
@@ -336,6 +337,7 @@ helm_status nn_gemm(int transA, int transB, int M, int N, int K, float alpha, co
 helm_status nn_bias_act(int rows, int cols, float* X, const float* bias, int act, void* stream);
 helm_status nn_act_backward(long long n, float* dX, const float* Y, int act, void* stream);
 helm_status nn_bias_grad(int rows, int cols, const float* dY, float* db, void* stream);
+helm_status nn_bias_grad_rows(int rows, int cols, const float* dY, float* db, void* stream);
 helm_status nn_adam(long long n, float* p, const float* g, float* m, float* v, float lr, float beta1,
                     float beta2, float eps, int t, void* stream);
 helm_status nn_rel_l2(int B, int P2, const float* pred, const float* target, float* dpred, float* loss,

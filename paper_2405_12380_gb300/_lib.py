@@ -87,6 +87,7 @@ SIGNATURES = {
     "nn_bias_act": (i32, [i32, i32, vp, vp, i32, vp]),
     "nn_act_backward": (i32, [i64, vp, vp, i32, vp]),
     "nn_bias_grad": (i32, [i32, i32, vp, vp, vp]),
+    "nn_bias_grad_rows": (i32, [i32, i32, vp, vp, vp]),
     "nn_adam": (i32, [i64, vp, vp, vp, vp, C.c_float, C.c_float, C.c_float, C.c_float, i32, vp]),
     "nn_rel_l2": (i32, [i32, i32, vp, vp, vp, vp, vp]),
     "nn_gather": (i32, [i32, i32, vp, i64, vp, vp, vp, vp]),

@@ -135,7 +135,9 @@ def _backward_mlp(layers, acts, dout, act, stream, need_input_grad=False):
         if i < len(layers) - 1:
             _ck(lib.nn_act_backward(d.numel(), _p(d), _p(acts[i + 1]), act, stream), "nn_act_backward")
         _ck(_gemm(lib, 1, 0, fout, fin, rows, 1.0, _p(d), fout, _p(acts[i]), fin, 0.0, _p(l.gW), fin, stream), "dW")
-        _ck(lib.nn_bias_grad(rows, fout, _p(d), _p(l.gb), stream), "db")
+        # (in the order of the rows where the next step's products round to BF16)
+        db = lib.nn_bias_grad_rows if _TENSOR_CORES else lib.nn_bias_grad
+        _ck(db(rows, fout, _p(d), _p(l.gb), stream), "db")
         if i > 0 or need_input_grad:
             dn = torch.empty(rows, fin, dtype=torch.float32, device="cuda")
             _ck(_gemm(lib, 0, 0, rows, fin, fout, 1.0, _p(d), fout, _p(l.W), fin, 0.0, _p(dn), fin, stream), "dX")

@@ -171,3 +171,30 @@ def test_gemm_bf16_stages(N, K):
     assert np.all(np.abs(Cd.cpu().numpy() - opA @ opB) <= 4 * K * U * (np.abs(opA) @ np.abs(opB)) + 1e-30)
     flag = C.c_int(-1)
     assert _lib().nn_gemm_bf16_status(C.byref(flag)) == 0 and flag.value == 0
+
+
+@pytest.mark.parametrize("rows,cols", [(0, 5), (1, 1), (31, 8), (33, 9), (1024, 100), (1025, 33), (5000, 20)])
+def test_bias_grad_rows_keeps_the_order(rows, cols):
+    """The sums in the order of the rows, bit for bit (one tile of 1024 rows, its edges, several)."""
+    dY = np.random.default_rng(rows + cols).standard_normal((max(rows, 1), cols)).astype(np.float32)
+    ref = np.zeros(cols, np.float32)
+    for r in range(rows):
+        ref += dY[r]
+    Dd, db = to_dev(dY), to_dev(np.full(cols, np.nan, np.float32))
+    assert _lib().nn_bias_grad_rows(rows, cols, _p(Dd), _p(db), None) == 0
+    assert np.array_equal(db.cpu().numpy(), ref)
+
+
+def test_adam_same_bits_on_every_path():
+    """Values in 16-byte groups, in the tail and in arrays off 16 bytes take the same step."""
+    rng = np.random.default_rng(9)
+    a = [rng.standard_normal(4099).astype(np.float32) for _ in range(3)] + [rng.random(4099).astype(np.float32)]
+    out = []
+    for off in (0, 1):
+        for n in (4099, 4096):
+            d = [_off(x[-n:], off) for x in a]
+            assert _lib().nn_adam(n, _p(d[0]), _p(d[1]), _p(d[2]), _p(d[3]), 1e-3, 0.9, 0.999, 1e-8, 4, None) == 0
+            out.append([t.cpu().numpy()[-4096:] for t in d])
+    for o in out[1:]:
+        for x, y in zip(out[0], o):
+            assert np.array_equal(x, y)
