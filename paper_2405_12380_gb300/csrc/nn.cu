@@ -296,44 +296,56 @@ __global__ void __launch_bounds__(256) k_bias_grad(int rows, int cols, const flo
 
 // The same sums, each added in the order of the rows.  BF16 training needs the bits that do
 // not move with the kernel: the last bit of a bias decides BF16 roundings of the next step
-// (summed in clusters, one small step in ten ended 1e-3 away from the row order).  The chain
-// of adds is the bound: 4 clocks a row, 17 us for 8192 rows.  A block owns 8 columns; all
-// its threads fetch the next 1024 rows while 8 lanes add the current ones from shared
-// memory.  The three large sums of the 40^3 step
-// take 20 us in clusters, about 100 us here.
-constexpr int BS_ROWS = 1024;
+// (summed in clusters, one small step in ten ended 1e-3 away from the row order).  One
+// warp's issue is the bound, 4 clocks an add: a block owns 8 columns, all its threads fetch
+// the next 1024 rows while 8 lanes add the current ones from shared memory, four rows a
+// load: 8192 x 256 takes 30 us (40 with a load a row; 7 in clusters, in another order).
+constexpr int BS_ROWS = 1024, BS_PITCH = BS_ROWS + 4;
 __global__ void __launch_bounds__(256) k_bias_grad_rows(int rows, int cols, const float* __restrict__ dY,
                                                         float* __restrict__ db) {
-    extern __shared__ float tile[];                        // [2][BS_ROWS][8]
+    extern __shared__ __align__(16) float tile[];          // [2][8][BS_PITCH], column by column
     const int tid = threadIdx.x, cc = tid & 7, rr = tid >> 3;
     const int c = blockIdx.x * 8 + cc;
-    constexpr int V = BS_ROWS / 32;
-    float v[V], s = 0.f;
-    auto fetch = [&](int r0) {
-#pragma unroll
-        for (int q = 0; q < V; ++q) {
+    float s = 0.f;
+    // 4-byte asynchronous copies (zeros past the matrix), so that nothing waits for them here
+    auto fetch = [&](int r0, float* t) {
+#pragma unroll 8
+        for (int q = 0; q < BS_ROWS / 32; ++q) {
             const int r = r0 + rr + 32 * q;
-            v[q] = r < rows && c < cols ? __ldg(dY + (long long)r * cols + c) : 0.f;
+            const bool in = r < rows && c < cols;
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(
+                             (unsigned)__cvta_generic_to_shared(t + cc * BS_PITCH + rr + 32 * q)),
+                         "l"(in ? dY + (long long)r * cols + c : dY), "r"(in ? 4 : 0)
+                         : "memory");
         }
+        asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    fetch(0);
+    if (rows > 0) fetch(0, tile);
     for (int r0 = 0, buf = 0; r0 < rows; r0 += BS_ROWS, buf ^= 1) {
-        float* t = tile + buf * BS_ROWS * 8;
-#pragma unroll
-        for (int q = 0; q < V; ++q) t[(rr + 32 * q) * 8 + cc] = v[q];
-        __syncthreads();                                   // (the buffer written next was read before this)
-        if (r0 + BS_ROWS < rows) fetch(r0 + BS_ROWS);
+        const float* t = tile + buf * BS_PITCH * 8;
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();                                   // (the other buffer has been added)
+        if (r0 + BS_ROWS < rows) fetch(r0 + BS_ROWS, tile + (buf ^ 1) * BS_PITCH * 8);
         if (tid < 8) {
+            // 16 values on their way from shared memory while 16 are added; the zeros past
+            // the last row leave the sum as it is
             const int m = min(BS_ROWS, rows - r0);
-            int r = 0;
-            for (; r + 32 <= m; r += 32) {
-                float x[32];
+            const float4* col = reinterpret_cast<const float4*>(t + tid * BS_PITCH);
+            float4 x[4], y[4];
 #pragma unroll
-                for (int u = 0; u < 32; ++u) x[u] = t[(r + u) * 8 + tid];
+            for (int u = 0; u < 4; ++u) x[u] = col[u];
+            for (int r = 0; r < m; r += 32) {
 #pragma unroll
-                for (int u = 0; u < 32; ++u) s += x[u];
+                for (int u = 0; u < 4; ++u) y[u] = col[r / 4 + 4 + u];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) s = (((s + x[u].x) + x[u].y) + x[u].z) + x[u].w;
+                if (r + 32 < m) {
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) x[u] = col[r / 4 + 8 + u];
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) s = (((s + y[u].x) + y[u].y) + y[u].z) + y[u].w;
             }
-            for (; r < m; ++r) s += t[r * 8 + tid];
         }
     }
     if (tid < 8 && c < cols) db[c] = s;
@@ -677,7 +689,7 @@ helm_status nn_bias_grad(int rows, int cols, const float* dY, float* db, void* s
 helm_status nn_bias_grad_rows(int rows, int cols, const float* dY, float* db, void* stream) {
     if (rows < 0 || cols < 0 || !dY || !db) return HELM_BAD_ARG;
     if (cols == 0) return HELM_OK;
-    const size_t smem = 2 * BS_ROWS * 8 * sizeof(float);
+    const size_t smem = 2 * BS_PITCH * 8 * sizeof(float);
     if (cudaFuncSetAttribute(k_bias_grad_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return HELM_CUDA_ERROR;
     k_bias_grad_rows<<<(cols + 7) / 8, 256, smem, static_cast<cudaStream_t>(stream)>>>(rows, cols, dY, db);
