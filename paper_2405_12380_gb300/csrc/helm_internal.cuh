@@ -94,6 +94,15 @@ __device__ __forceinline__ double2 cfmac(double2 a, double2 b, double2 c) {
     return make_double2(fma(a.x, b.x, fma(a.y, b.y, c.x)), fma(a.x, b.y, fma(-a.y, b.x, c.y)));
 }
 __device__ __forceinline__ double cnorm2(double2 a, double s) { return fma(a.x, a.x, fma(a.y, a.y, s)); }
+// a b in FP32 with the fused multiply-adds spelled out: written as a.x b.y + a.y b.x the
+// compiler fuses one product or the other, in each kernel as it likes.  cmul_n fuses the
+// product with a.x in both components, cmul_t the one with a.y in the imaginary part
+__device__ __forceinline__ float2 cmul_n(float2 a, float2 b) {
+    return make_float2(fmaf(a.x, b.x, -__fmul_rn(a.y, b.y)), fmaf(a.x, b.y, __fmul_rn(a.y, b.x)));
+}
+__device__ __forceinline__ float2 cmul_t(float2 a, float2 b) {
+    return make_float2(fmaf(a.x, b.x, -__fmul_rn(a.y, b.y)), fmaf(a.y, b.x, __fmul_rn(a.x, b.y)));
+}
 __host__ __device__ __forceinline__ double2 cadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
 __host__ __device__ __forceinline__ double2 csub(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
 __host__ __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }

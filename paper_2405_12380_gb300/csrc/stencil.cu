@@ -614,7 +614,10 @@ __global__ void __launch_bounds__(BX * BY) k_rbgs_c64(Op<float> op, int zc, int 
 // two others, 22 at the ends of a run, instead of 26).  A node with all six
 // neighbours fluid (the common case) takes no selects.  Every node value comes from the
 // arithmetic of k_rbgs_c64 with the neighbour sums in the same order, so one launch equals
-// two half-sweeps.  Measured against the form that staged whole pairs and selected by
+// two half-sweeps.  The roundings are spelled out (sor_step, cmul_n; cmul_t for colour A
+// from zero), the same in every instantiation: left to the compiler they moved from one to
+// the next by 2e-8, which the trunk-basis correction and eight FGMRES steps can raise to
+// 1e-5 of the solution.  Measured against the form that staged whole pairs and selected by
 // position (431 instructions a pair at 256^3; ncu, cold): 256^3 133 -> 83 us a sweep (5.3
 // TB/s of the 26 B a node), 128^3 20.5 -> 15.2 us, 64^3 13.2 -> 6.3 us.  The launch shape
 // is chosen by plan_sweep32.
@@ -632,6 +635,11 @@ __device__ __forceinline__ float2 six_sum(unsigned c, int a, float2 own, float2 
         zp = pick(c, 32u, zp);
     }
     return cadd(cadd(cadd(own, side), cadd(ym, yp)), cadd(zm, zp));
+}
+
+// x + omega (v - x)
+__device__ __forceinline__ float2 sor_step(float2 x, float2 v, float omega) {
+    return make_float2(fmaf(omega, v.x - x.x, x.x), fmaf(omega, v.y - x.y, x.y));
 }
 
 // 8-byte asynchronous copy global -> shared; valid = false fills zeros without reading
@@ -770,15 +778,15 @@ __global__ void __launch_bounds__(kSweepMaxThreads, 1)
                 id = stab[HCHK(ca >> 8, kMaxLayerCells + 1)];
             }
             if (XZERO) {
-                na = cmul(id, fa);
+                na = cmul_t(id, fa);
             } else {
                 const float2* P = xs + o_0 + mx;
                 const float2 bx = P[dx];
                 const float2 s = six_sum(ca, ar, b0, bx, P[-TXT], P[TXT], bm1, bp1);
-                na = cmul(id, make_float2(fa.x - op.hinv2 * s.x, fa.y - op.hinv2 * s.y));
+                na = cmul_n(id, make_float2(fmaf(-op.hinv2, s.x, fa.x), fmaf(-op.hinv2, s.y, fa.y)));
             }
         }
-        if (SOR) na = XZERO ? cscale(omega, na) : cadd(xa, cscale(omega, csub(na, xa)));
+        if (SOR) na = XZERO ? cscale(omega, na) : sor_step(xa, na, omega);
         ring[rs + me] = na;
         if (!XZERO) {
             // plane t + 3 into the slot of plane t - 1 (last read before the previous step's
@@ -800,10 +808,10 @@ __global__ void __launch_bounds__(kSweepMaxThreads, 1)
                 float2 id = ib;
                 if (!K2) id = stab[HCHK(cb >> 8, kMaxLayerCells + 1)];
                 else if (conj) id.y = -id.y;
-                nb = cmul(id, make_float2(fb.x - op.hinv2 * s.x, fb.y - op.hinv2 * s.y));
+                nb = cmul_n(id, make_float2(fmaf(-op.hinv2, s.x, fb.x), fmaf(-op.hinv2, s.y, fb.y)));
             }
             // (from zero only colour A starts from zero: colour B's own old value is zero too)
-            if (SOR) nb = cadd(xb, cscale(omega, csub(nb, xb)));
+            if (SOR) nb = sor_step(xb, nb, omega);
             if (COUT)
                 xout[HCHK(l - sz, NP)] = nb;
             else
