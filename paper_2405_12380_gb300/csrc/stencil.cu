@@ -959,17 +959,20 @@ __global__ void __launch_bounds__(BX * BY) k_jacobi(Op<R> op, R omega, const typ
 // costs its launch: 5.3 us at 64 x 64 against 0.1 us of FP64 arithmetic).  A block owns
 // TI x TI nodes and recomputes a halo of S nodes around them, one node per thread
 // (blockDim = TI + 2 S per side): S sweeps run in shared memory, each on a region one
-// node smaller per side, and only the block's own nodes are written.  The sweep is
+// node smaller per side, and only the block's own nodes are written.  In FP64 the sweep is
 // x <- (1 - omega) x + omega D^-1 f - omega h^-2 D^-1 s with the two products of D^-1
 // formed once per node (12 FP64 instructions a sweep against 16 when D^-1 (f - h^-2 s)
-// is formed each time); a masked node has s's factor zero, and is zero to its
-// neighbours.  xin = nullptr: from zero.
+// is formed each time).  In FP32, where instructions are cheap and a cycle's last bits show
+// in the fifth digit of a mixed-precision solution, it is jacobi_point's formula with the
+// same roundings, so that the tiled sweeps equal single ones bit for bit.  A masked node is
+// zero to its neighbours.  xin = nullptr: from zero.
 template <typename R>
 __global__ void k_jacobi_tile(Op<R> op, R omega, int S, const typename CT<R>::T* __restrict__ f,
                               const typename CT<R>::T* __restrict__ xin, typename CT<R>::T* __restrict__ xout,
                               int conj) {
     pdl_begin();
     using C = typename CT<R>::T;
+    constexpr bool kSplit = std::is_same<R, double>::value;
     extern __shared__ __align__(16) unsigned char jt_smem[];
     const int E = blockDim.x, TI = E - 2 * S, tx = threadIdx.x, ty = threadIdx.y, t = ty * E + tx;
     C* buf = reinterpret_cast<C*>(jt_smem);                // [2][E * E]
@@ -984,12 +987,17 @@ __global__ void k_jacobi_tile(Op<R> op, R omega, int S, const typename CT<R>::T*
         fluid = !(op.nbm[HCHK(l, op.N)] & kMasked);
         const C fv = f[HCHK(l, op.N)];
         if (xin) x = xin[HCHK(l, op.N)];
-        if (fluid) {
-            const C id = cscale(omega, invd_of(op, l, op.lidx[HCHK(l, op.N)], conj));
-            fp = cmul(id, fv);
-            c = cscale(op.hinv2, id);
-        } else {
-            fp = cscale(omega, fv);
+        if (kSplit) {                                      // fp: omega D^-1 f, c: omega h^-2 D^-1
+            if (fluid) {
+                const C id = cscale(omega, invd_of(op, l, op.lidx[HCHK(l, op.N)], conj));
+                fp = cmul(id, fv);
+                c = cscale(op.hinv2, id);
+            } else {
+                fp = cscale(omega, fv);
+            }
+        } else {                                           // fp: f, c: D^-1
+            fp = fv;
+            if (fluid) c = invd_of(op, l, op.lidx[HCHK(l, op.N)], conj);
         }
     }
     const int rim = min(min(tx, E - 1 - tx), min(ty, E - 1 - ty));
@@ -999,15 +1007,23 @@ __global__ void k_jacobi_tile(Op<R> op, R omega, int S, const typename CT<R>::T*
         b[t] = fluid ? x : zero;
         __syncthreads();
         if (rim > q) {
-            C y;
-            y.x = fp.x + w1 * x.x;
-            y.y = fp.y + w1 * x.y;
-            if (fluid) {
-                const C s = cadd(cadd(b[t - 1], b[t + 1]), cadd(b[t - E], b[t + E]));
-                y.x -= c.x * s.x - c.y * s.y;
-                y.y -= c.x * s.y + c.y * s.x;
+            C s = zero;
+            if (fluid) s = cadd(cadd(b[t - 1], b[t + 1]), cadd(b[t - E], b[t + E]));
+            if constexpr (kSplit) {
+                C y;
+                y.x = fp.x + w1 * x.x;
+                y.y = fp.y + w1 * x.y;
+                if (fluid) {
+                    y.x -= c.x * s.x - c.y * s.y;
+                    y.y -= c.x * s.y + c.y * s.x;
+                }
+                x = y;
+            } else if (fluid) {
+                const C d = cmul_n(c, make_float2(fmaf(-op.hinv2, s.x, fp.x), fmaf(-op.hinv2, s.y, fp.y)));
+                x = make_float2(fmaf(w1, x.x, __fmul_rn(omega, d.x)), fmaf(w1, x.y, __fmul_rn(omega, d.y)));
+            } else {
+                x = sor_step(x, fp, omega);
             }
-            x = y;
         }
     }
     if (rim >= S && in) xout[HCHK(l, op.N)] = x;

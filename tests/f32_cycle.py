@@ -80,3 +80,14 @@ class Op32:
                 x = tuple(np.where(self.colour == c, p, q) for p, q in zip(v, x))
                 zero = False
         return x
+
+    def jacobi(self, omega, count, f, x=None, conj=False):
+        """damped-Jacobi sweeps: (1 - omega) x + omega D^-1 (f - h^-2 sum of neighbours)"""
+        om = f32(omega)
+        w1 = f32(1) - om
+        invd = self.conj(self.invd, conj)
+        x = tuple(np.zeros_like(p) for p in f) if x is None else x
+        for _ in range(count):
+            v = cmul(invd, self.rhs_minus_nbrs(f, x))
+            x = tuple(np.where(self.fluid, fma(w1, q, om * p), fma(om, g - q, q)) for p, q, g in zip(v, x, f))
+        return x
