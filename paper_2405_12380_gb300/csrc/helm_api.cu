@@ -363,9 +363,13 @@ helm_status precond32(helm_handle* h, const helm_solve_opts* o, const float2* v,
         const bool red = !no_relax && o->relax == HELM_RBGS;
         const long long M = red ? (h->N + 1) / 2 : h->N;
         TRY(ensure_tmp32(h, 4));
-        if (!red || !launch_red_residual32(h->op32, v, z, h->tmp32[3], conj, s))
+        Rows32 rows = red ? Rows32::kPairs : Rows32::kAll;
+        if (!red || !launch_red_residual32(h->op32, v, z, h->tmp32[3], conj, s)) {
+            if (red) rows = Rows32::kRed;
             launch_residual32(h->op32, v, no_relax ? nullptr : z, red, conj, h->tmp32[3], s);
-        const int nblk = launch_restrict32(red ? h->Qbr : h->Qbf, basis_ld(M), h->k, h->tmp32[3], M, h->partials32, s);
+        }
+        const int nblk =
+            launch_restrict32(rows, red ? h->Qbr : h->Qbf, basis_ld(M), h->k, h->tmp32[3], M, h->partials32, s);
         ev_mark(h, 0, 1);
         launch_coarse_apply32(h->partials32, nblk, h->k, h->Ainv, conj, h->y32, h->cbuf, s);
         ev_mark(h, 1, 0);
@@ -1673,7 +1677,7 @@ helm_status don_load(helm_handle* h, const double* weights, const int* widths, i
     STEP(dalloc(h, &h->coarse_partials, (size_t)project_blocks(N) * k));
     if (h->precision == HELM_MIXED) {
         dfree(h->partials32); dfree(h->y32);
-        STEP(dalloc(h, &h->partials32, (size_t)restrict32_ranges(N) * k));
+        STEP(dalloc(h, &h->partials32, (size_t)restrict32_parts(N) * k));
         STEP(dalloc(h, &h->y32, (size_t)kMaxP));
     }
     STEP(dalloc(h, &h->cbuf, (size_t)kMaxP));

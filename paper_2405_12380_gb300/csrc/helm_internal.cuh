@@ -444,11 +444,13 @@ void launch_red_rows_bf16(const void* Q, long long ldq, int k, long long N, int 
 // r = v - A z (zero on masked nodes; z may be null: v) on every row, or on the red row of
 // each node pair; then c partials = Q^T r over its M rows with the BF16 basis (all rows:
 // stride basis_ld(N); red rows: basis_ld(ceil(N / 2))): returns the number of partial
-// rows written, restrict32_ranges(M)
+// rows written, at most restrict32_parts(N).  The rows also say in which order they are
+// added: the red rows of the pair layout, those of other grids, or all rows
+enum class Rows32 { kPairs, kRed, kAll };
 void launch_residual32(const Op<float>& op, const float2* v, const float2* z, bool red, int conj, float2* r,
                        cudaStream_t s);
-int restrict32_ranges(long long M);
-int launch_restrict32(const void* Q, long long ld, int k, const float2* r, long long M, float2* partials,
+int restrict32_parts(long long N);
+int launch_restrict32(Rows32 rows, const void* Q, long long ld, int k, const float2* r, long long M, float2* partials,
                       cudaStream_t s);
 
 // mg.cu: grid transfers of the multigrid V-cycle (n_f = 2 n_c - 1, coarse node I at fine 2I)

@@ -907,22 +907,21 @@ __device__ __forceinline__ float2 row_residual32(const Op<float>& op, const floa
     float2 d;
     if (op.k2) {
         d = op.k2[l];
-        d.x -= 2.0f * op.dim * op.hinv2;
+        d.x -= op.dsub;
     } else {
         d = make_float2(op.dre, op.im[op.lidx[l]]);
     }
     if (conj) d.y = -d.y;
-    const float2 zc = z[l], vv = v[l];
-    return make_float2(vv.x - (op.hinv2 * s.x + (d.x * zc.x - d.y * zc.y)),
-                       vv.y - (op.hinv2 * s.y + (d.x * zc.y + d.y * zc.x)));
+    const float2 vv = v[l], dz = cmul_t(d, z[l]);
+    return make_float2(vv.x - fmaf(op.hinv2, s.x, dz.x), vv.y - fmaf(op.hinv2, s.y, dz.y));
 }
 
 // the residual that the restriction projects, where the pair layout does not apply (odd n,
 // 2D, unaligned vectors) or the sweep leaves residual on both colours: RED, the red row of
 // every node pair (M = ceil(N / 2) rows); else every row (M = N; z may be null: v itself).
 // Zero on masked nodes.  Consecutive rows on consecutive lanes, so the neighbour loads
-// coalesce; forming the residual inside the projection (81 blocks at 97^3) took 30 us,
-// the two launches 6 + 5 us.
+// coalesce.  helm_precond at 97^3, red-black sweeps and 53 columns: 166 us with the residual
+// formed inside the projection, 106 us with two launches.
 template <bool RED>
 __global__ void __launch_bounds__(256) k_residual32(Op<float> op, const float2* __restrict__ v,
                                                     const float2* __restrict__ z, int conj, float2* __restrict__ r,
@@ -934,17 +933,21 @@ __global__ void __launch_bounds__(256) k_residual32(Op<float> op, const float2* 
     }
 }
 
-// c = Q^T r from a stored residual (red rows or all rows): a tall-skinny product.  A warp
-// owns RQ_COLS columns and one range of RQ_RANGE rows; per 256 rows each lane loads
-// its 8 consecutive residual rows and then all its 16-byte basis pieces (one per
-// column, issued together) before the FMAs, and keeps the complex sums in
-// registers over the range; the lanes are added once at the end (fixed butterfly)
-// and lane 0 writes partials[range][j].  Deterministic.
+// c = Q^T r from the stored residual, a tall-skinny product in FP32, in one of three orders
+// of the sums (enum Rows32).  c goes through A_c^-1 into the next Krylov vector, and the
+// last bits of c come out a hundred times larger, or more, in a mixed-precision solution:
+// each kind of cycle keeps its order, whatever the kernel.  Deterministic.
+//
+// Pair layout.  A warp owns RQ_COLS columns and one range of RQ_RANGE rows; per 256 rows
+// each lane loads its 8 consecutive residual rows and then all its 16-byte basis pieces
+// (one per column, issued together) before the FMAs, and keeps the complex sums in
+// registers over the range; the lanes are added once at the end (fixed butterfly) and lane
+// 0 writes partials[range][j].
 constexpr int RQ_COLS = 8;
 constexpr int RQ_RANGE = 1024;
 __global__ void __launch_bounds__(256) k_restrict32(const __nv_bfloat16* __restrict__ Qr, long long ldr, int k,
-                                                       const float2* __restrict__ r, long long M,
-                                                       float2* __restrict__ partials, int S) {
+                                                    const float2* __restrict__ r, long long M,
+                                                    float2* __restrict__ partials, int S) {
     pdl_begin();
     const int lane = threadIdx.x & 31;
     const int rg = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -998,6 +1001,161 @@ __global__ void __launch_bounds__(256) k_restrict32(const __nv_bfloat16* __restr
 #pragma unroll
         for (int c = 0; c < RQ_COLS; ++c)
             if (c < nc) partials[(long long)rg * k + c0 + c] = make_float2(ax[c], ay[c]);
+}
+
+// the V values of every lane summed over the warp as by a butterfly of all of them (offsets
+// 16 to 1, the same bits), but a lane passes on the half it does not keep, so that 16 values
+// take 16 shuffles instead of 80.  Returns the sum of value lane / (32 / V).
+template <int V>
+__device__ __forceinline__ float scatter_sum(float* v, int lane) {
+#pragma unroll
+    for (int o = 16, n = V; o > 0; o >>= 1, n = n > 1 ? n / 2 : 1) {
+        if (n > 1) {
+            const bool up = lane & o;
+#pragma unroll
+            for (int i = 0; i < n / 2; ++i) {
+                const float keep = up ? v[i + n / 2] : v[i], send = up ? v[i] : v[i + n / 2];
+                v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+            }
+        } else {
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+        }
+    }
+    return v[0];
+}
+
+// Red rows of 2D and odd grids: a warp adds 256 rows (8 consecutive ones a lane), its tiles
+// one after the other, and a block its eight warps in order.  A block does RQ_COLS columns
+// (several groups one after the other, the next one's loads ahead: 8 us slower at 97^3).
+// Bound by the loads in flight: 64 registers leave 32 warps an SM, 2 and 5 us at 97^3 and
+// 127^3 faster than 24.
+constexpr int RR_WARPS = 8, RR_ROWS = 256;
+__global__ void __launch_bounds__(32 * RR_WARPS, 4)
+    k_restrict32_red(const __nv_bfloat16* __restrict__ Qr, long long ldr, int k, const float2* __restrict__ r, long long M,
+                     float2* __restrict__ partials) {
+    pdl_begin();
+    __shared__ float sums[RR_WARPS][2 * RQ_COLS];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int c0 = blockIdx.y * RQ_COLS, nc = min(RQ_COLS, k - c0);
+    const long long tiles = (M + RR_ROWS - 1) / RR_ROWS;
+    float acc = 0.f;
+    for (long long t = blockIdx.x * (long long)RR_WARPS + w; t < tiles; t += (long long)gridDim.x * RR_WARPS) {
+        const long long m0 = t * RR_ROWS + lane * 8;
+        uint4 u[RQ_COLS];
+#pragma unroll
+        for (int c = 0; c < RQ_COLS; ++c)
+            u[c] = c < nc && m0 < M ? __ldcs(reinterpret_cast<const uint4*>(
+                                          Qr + HCHK((long long)(c0 + c) * ldr + m0, (long long)k * ldr - 7)))
+                                    : make_uint4(0u, 0u, 0u, 0u);
+        float2 rv[8];
+        if (m0 + 8 <= M) {
+            const float4* r4 = reinterpret_cast<const float4*>(r + HCHK(m0, M - 7));
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float4 x = r4[q];
+                rv[2 * q] = make_float2(x.x, x.y);
+                rv[2 * q + 1] = make_float2(x.z, x.w);
+            }
+        } else {
+#pragma unroll
+            for (int q = 0; q < 8; ++q) rv[q] = m0 + q < M ? r[HCHK(m0 + q, M)] : make_float2(0.f, 0.f);
+        }
+        float v[2 * RQ_COLS];
+#pragma unroll
+        for (int c = 0; c < RQ_COLS; ++c) {
+            float qv[8], ax = 0.f, ay = 0.f;
+            bf16x8(u[c], qv);
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                ax = fmaf(qv[q], rv[q].x, ax);
+                ay = fmaf(qv[q], rv[q].y, ay);
+            }
+            v[2 * c] = ax;
+            v[2 * c + 1] = ay;
+        }
+        acc += scatter_sum<2 * RQ_COLS>(v, lane);
+    }
+    if ((lane & 1) == 0) sums[w][lane >> 1] = acc;
+    __syncthreads();
+    if (threadIdx.x < 2 * nc) {
+        float t = 0.f;
+#pragma unroll
+        for (int q = 0; q < RR_WARPS; ++q) t += sums[q][threadIdx.x];
+        reinterpret_cast<float*>(partials)[2 * ((long long)blockIdx.x * k + c0) + threadIdx.x] = t;
+    }
+}
+
+// All rows (cycles without red-black Gauss-Seidel): the rows are dealt in equal shares, one
+// partial row each; a lane adds every 32nd row of the share in one chain and the warp adds
+// its lanes at the end.  A warp does RA_COLS columns.  A share starts at any row, so the
+// basis goes through shared memory of the warp's own, RA_TILE rows a stage: 16-byte
+// asynchronous copies from the 8 rows that hold the first one on, single values out of it.
+// helm_precond at 96^3, two Jacobi sweeps and 52 columns: 99 us; 145 with single values
+// loaded straight from memory.  Eight columns a warp: 1 us faster there, 4 slower at 20 to
+// 30 columns.
+constexpr int RA_COLS = 4, RA_TILE = 256, RA_PITCH = RA_TILE + 8, RA_STAGES = 3, RA_WARPS = 8;
+constexpr size_t kRestrictAllSmem = (size_t)RA_WARPS * RA_STAGES * RA_COLS * RA_PITCH * 2;
+__global__ void __launch_bounds__(32 * RA_WARPS)
+    k_restrict32_all(const __nv_bfloat16* __restrict__ Q, long long ld, int k, const float2* __restrict__ r, long long N,
+                     int share, float2* __restrict__ partials) {
+    pdl_begin();
+    extern __shared__ __align__(16) unsigned short ra_smem[];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, c0 = (blockIdx.y * RA_WARPS + w) * RA_COLS;
+    if (c0 >= k) return;
+    const int nc = min(RA_COLS, k - c0);
+    unsigned short* buf = ra_smem + w * RA_STAGES * RA_COLS * RA_PITCH;
+    const long long r0 = min(N, blockIdx.x * (long long)share);
+    const int rows = (int)min((long long)share, N - r0), off = (int)(r0 & 7), tiles = (rows + RA_TILE - 1) / RA_TILE;
+    const __nv_bfloat16* Qc = Q + (long long)c0 * ld + (r0 - off);
+    auto stage = [&](int t) {
+        if (t < tiles) {
+            unsigned short* b = buf + (t % RA_STAGES) * RA_COLS * RA_PITCH;
+            for (int e = lane; e < RA_COLS * (RA_PITCH / 8); e += 32) {
+                const int c = e / (RA_PITCH / 8), i = t * RA_TILE + 8 * (e % (RA_PITCH / 8));
+                const bool in = c < nc && i < off + rows;  // (then the 8 rows lie in the column's padded length)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(
+                                 (unsigned)__cvta_generic_to_shared(b + 8 * e)),
+                             "l"(Qc + HCHK(in ? c * ld + i : 0, (k - c0) * ld - (r0 - off))), "r"(in ? 16 : 0)
+                             : "memory");
+            }
+        }
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+    };
+    auto load = [&](int t, float2* x) {
+#pragma unroll
+        for (int u = 0; u < RA_TILE / 32; ++u) {
+            const int i = t * RA_TILE + lane + 32 * u;
+            x[u] = i < rows ? r[HCHK(r0 + i, N)] : make_float2(0.f, 0.f);
+        }
+    };
+    float v[2 * RA_COLS];
+#pragma unroll
+    for (int c = 0; c < 2 * RA_COLS; ++c) v[c] = 0.f;
+    float2 x[RA_TILE / 32], xn[RA_TILE / 32];
+    stage(0);
+    stage(1);
+    load(0, x);
+    for (int t = 0; t < tiles; ++t) {
+        stage(t + 2);                                      // (its buffer was read in the previous round)
+        load(t + 1, xn);
+        asm volatile("cp.async.wait_group %0;\n" ::"n"(RA_STAGES - 1) : "memory");
+        __syncwarp();
+        const unsigned short* b = buf + (t % RA_STAGES) * RA_COLS * RA_PITCH + off + lane;
+#pragma unroll
+        for (int u = 0; u < RA_TILE / 32; ++u) {
+#pragma unroll
+            for (int c = 0; c < RA_COLS; ++c) {
+                const float q = __uint_as_float((unsigned)b[c * RA_PITCH + 32 * u] << 16);
+                v[2 * c] = fmaf(q, x[u].x, v[2 * c]);
+                v[2 * c + 1] = fmaf(q, x[u].y, v[2 * c + 1]);
+            }
+            x[u] = xn[u];
+        }
+        __syncwarp();                                      // (before the buffer is filled again)
+    }
+    const float t = scatter_sum<2 * RA_COLS>(v, lane);
+    const int idx = lane / (16 / RA_COLS);
+    if (lane % (16 / RA_COLS) == 0 && idx < 2 * nc) reinterpret_cast<float*>(partials)[2 * ((long long)blockIdx.x * k + c0) + idx] = t;
 }
 
 // z += Q y, eight consecutive rows per thread (16-byte basis loads, 64-byte z
@@ -1222,14 +1380,46 @@ void launch_residual32(const Op<float>& op, const float2* v, const float2* z, bo
     else launch_after(k_residual32<false>, b, 256, 0, s, op, v, z, conj, r, M);
 }
 
+namespace {
+
 int restrict32_ranges(long long M) { return (int)std::max<long long>(1, (M + RQ_RANGE - 1) / RQ_RANGE); }
 
-int launch_restrict32(const void* Q, long long ld, int k, const float2* r, long long M, float2* partials,
+// (with the order of the sums: a change of these numbers changes last bits)
+int restrict32_red_blocks(long long M) {
+    const long long b = (M + RR_ROWS * RR_WARPS - 1) / (RR_ROWS * RR_WARPS);
+    return (int)std::max<long long>(1, std::min<long long>(b, 4 * 152));
+}
+int restrict32_shares(long long N) { return (int)std::max<long long>(1, std::min<long long>((N + 255) / 256, 2 * 152)); }
+
+}  // namespace
+
+int restrict32_parts(long long N) {
+    const long long M = (N + 1) / 2;
+    return std::max(std::max(restrict32_ranges(M), restrict32_red_blocks(M)), restrict32_shares(N));
+}
+
+int launch_restrict32(Rows32 rows, const void* Qv, long long ld, int k, const float2* r, long long M, float2* partials,
                       cudaStream_t s) {
-    const int S = restrict32_ranges(M);
-    const dim3 g((S + 7) / 8, (k + RQ_COLS - 1) / RQ_COLS);
-    launch_after(k_restrict32, g, 256, 0, s, static_cast<const __nv_bfloat16*>(Q), ld, k, r, M, partials, S);
-    return S;
+    const __nv_bfloat16* Q = static_cast<const __nv_bfloat16*>(Qv);
+    const unsigned groups = (k + RQ_COLS - 1) / RQ_COLS;
+    if (rows == Rows32::kPairs) {
+        const int S = restrict32_ranges(M);
+        launch_after(k_restrict32, dim3((S + 7) / 8, groups), 256, 0, s, Q, ld, k, r, M, partials, S);
+        return S;
+    }
+    if (rows == Rows32::kRed) {
+        const int nb = restrict32_red_blocks(M);
+        launch_after(k_restrict32_red, dim3(nb, groups), 32 * RR_WARPS, 0, s, Q, ld, k, r, M, partials);
+        return nb;
+    }
+    const int nb = restrict32_shares(M), cols = RA_COLS * RA_WARPS;
+    static_assert(kRestrictAllSmem > 48 * 1024, "the attribute is needed");
+    if (cudaFuncSetAttribute(k_restrict32_all, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRestrictAllSmem) !=
+        cudaSuccess)
+        return nb;                                         // (the caller's check of the last error reports it)
+    launch_after(k_restrict32_all, dim3(nb, (k + cols - 1) / cols), 32 * RA_WARPS, kRestrictAllSmem, s, Q, ld, k, r, M,
+                 (int)((M + nb - 1) / nb), partials);
+    return nb;
 }
 
 void launch_coarse_apply32(const float2* partials, int nblk, int k, const double2* Ainv, int conj, float2* y,

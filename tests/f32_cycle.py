@@ -91,3 +91,101 @@ class Op32:
             v = cmul(invd, self.rhs_minus_nbrs(f, x))
             x = tuple(np.where(self.fluid, fma(w1, q, om * p), fma(om, g - q, q)) for p, q, g in zip(v, x, f))
         return x
+
+    def residual(self, v, z, conj=False):
+        """v - A z on fluid nodes, 0 on masked ones; neighbours added one after the other"""
+        dz = cmul(self.conj(self.diag, conj), z, turned=True)
+        out = []
+        for vv, zz, p in zip(v, z, dz):
+            s = np.zeros_like(zz)
+            for a in range(self.dim - 1, -1, -1):
+                for q in self.neighbours(zz, a):
+                    s = s + q
+            out.append(np.where(self.fluid, vv - fma(self.hinv2, s, p), f32(0)))
+        return tuple(out)
+
+    def red_rows(self):
+        """the red node of each pair (2m, 2m + 1); N where the last pair has none"""
+        m2 = 2 * np.arange((self.fluid.size + 1) // 2)
+        return m2 + self.colour[m2]
+
+    def cycle(self, Q, Ainv, v, z, red, conj=False):
+        """z + Q A_c^-1 Q^T (v - A z) (z None: no sweeps), the residual on the red rows alone
+        (`red`) or on all; Q: the BF16 basis, node-major"""
+        r = tuple(np.where(self.fluid, p, f32(0)) for p in v) if z is None else self.residual(v, z, conj)
+        z = tuple(np.zeros_like(p) for p in v) if z is None else z
+        Q = np.asarray(Q, f32)
+        if red:
+            rows = np.append(np.arange(self.fluid.size), 0)[self.red_rows()]
+            here = (self.red_rows() < self.fluid.size)
+            c = [coarse_sum(red_parts(np.where(here[:, None], Q[rows], f32(0)), np.where(here, p[rows], f32(0)))) for p in r]
+        else:
+            c = [coarse_sum(all_parts(Q, p)) for p in r]
+        y = (Ainv.conj() if conj else Ainv) @ (c[0].astype(np.float64) + 1j * c[1].astype(np.float64))
+        out = []
+        for p, q in zip(z, pair(y)):
+            a = np.zeros_like(p)
+            for j in range(Q.shape[1]):
+                a = fma(Q[:, j], q[j], a)
+            out.append(p + a)
+        return tuple(out)
+
+
+def butterfly(v):
+    """the 32 lanes (first axis) added pairwise at distances 16, 8, 4, 2, 1"""
+    for o in (16, 8, 4, 2, 1):
+        v = v + v[np.arange(32) ^ o]
+    return v[0]
+
+
+def chain(q, r):
+    """sum of q r along the first axis, one fused multiply-add after the other"""
+    a = np.zeros(np.broadcast(q[0], r[0]).shape, f32)
+    for p, x in zip(q, r):
+        a = fma(p, x, a)
+    return a
+
+
+def red_parts(Q, r):
+    """Q^T r of red rows: 8 rows a lane, 256 a warp, tiles 8 blocks apart added in order, the
+    block's eight warps in order"""
+    M, k = Q.shape
+    tiles = -(-M // 256)
+    blocks = min(608, -(-tiles // 8))
+    q, x = np.zeros((tiles * 256, k), f32), np.zeros(tiles * 256, f32)
+    q[:M], x[:M] = Q, r
+    t = butterfly(chain(q.reshape(tiles, 32, 8, k).transpose(2, 1, 0, 3), x.reshape(tiles, 32, 8, 1).transpose(2, 1, 0, 3)))
+    part = np.zeros((blocks, k), f32)
+    for b in range(blocks):
+        for w in range(8):
+            acc = np.zeros(k, f32)
+            for i in range(8 * b + w, tiles, 8 * blocks):
+                acc = acc + t[i]
+            part[b] = part[b] + acc
+    return part
+
+
+def all_parts(Q, r):
+    """Q^T r of all rows: equal shares of the rows, every 32nd row of one in a lane's chain"""
+    N, k = Q.shape
+    blocks = min(304, max(1, -(-N // 256)))
+    share = -(-N // blocks)
+    m = -(-share // 32)
+    part = np.zeros((blocks, k), f32)
+    for b in range(blocks):
+        q, x = np.zeros((m * 32, k), f32), np.zeros(m * 32, f32)
+        rows = slice(min(N, b * share), min(N, (b + 1) * share))
+        q[:rows.stop - rows.start], x[:rows.stop - rows.start] = Q[rows], r[rows]
+        part[b] = butterfly(chain(q.reshape(m, 32, k), x.reshape(m, 32, 1)))
+    return part
+
+
+def coarse_sum(part):
+    """the partial rows: every 256th in a thread, a butterfly a warp, the eight warps in order"""
+    v = np.zeros((256, part.shape[1]), f32)
+    for b in range(part.shape[0]):
+        v[b % 256] = v[b % 256] + part[b]
+    s = np.zeros(part.shape[1], f32)
+    for w in range(8):
+        s = s + butterfly(v[32 * w:32 * w + 32])
+    return s
