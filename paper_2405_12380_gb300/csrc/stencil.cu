@@ -195,7 +195,8 @@ __device__ __forceinline__ double norm_acc(float2 a, double s) { return s + ((do
 // interior, so theirs are the neighbours in the plane's order; the two ends of the warp
 // load from memory), the y-neighbours from L1 or L2.  Bound by the FP64 pipe in complex128
 // (16 instructions a node, 20 with the residual and its norm): the residual with its norm
-// at 129^3 141 -> 102 us (ncu, cold), 68 us at the pipe's rate.
+// at 129^3 151 -> 99 us, 68 us at the pipe's rate.  (In 32 x 8 tiles, whose y-neighbours
+// share an L1, the times are the same to 1% from 64^3 to 256^3.)
 constexpr int AZ = 256;
 
 template <typename R, bool RESID, bool NORM>
@@ -1694,17 +1695,20 @@ int apply_zc(int dim, int n) {
     return march_zc((long long)((n + BX - 1) / BX) * ((n + BY - 1) / BY), n);
 }
 
-// grid of k_apply_z: the z chunk for which the busiest SM walks the fewest planes (its
-// share of the blocks, times their planes and one for the start of each), so that the
-// blocks come out in whole rounds (129^3: 765 blocks for 608 slots were two rounds)
-dim3 applyz_grid(int n, int* zc) {
+// grid of k_apply_z: the z chunk of 2 to 8 planes for which the busiest SM walks the fewest
+// planes (its share of the blocks, times their planes and, with a norm, half a plane for the
+// sums of each), so that the blocks come out in whole rounds.  Not more than 8 planes: a
+// longer chunk reads fewer planes twice but leaves an SM too few blocks to cover their
+// loads, which the count of planes does not see.  Apply and residual in complex128, us,
+// with one plane for the start of a block and no limit, and by this rule: 192^3 (192 planes,
+// one block an SM) 307 and 400, 240 and 308; 256^3 (64 planes) 602 and 730, 556 and 705;
+// 129^3 (15) 82 and 104, 75 and 99; 96^3 (24) 36 and 46, 32 and 44.
+dim3 applyz_grid(int n, bool norm, int* zc) {
     const long long per = ((long long)n * n + AZ - 1) / AZ;
     long long best = 0;
     *zc = 1;
-    for (int chunks = 1; chunks <= n; ++chunks) {
-        const int z = (n + chunks - 1) / chunks;
-        if (z < 4 && chunks > 1) break;
-        const long long blocks = per * ((n + z - 1) / z), cost = (blocks + 151) / 152 * (z + 1);
+    for (int z = std::min(8, n); z >= std::min(2, n); --z) {
+        const long long blocks = per * ((n + z - 1) / z), cost = (blocks + 151) / 152 * (2 * z + (norm ? 1 : 0));
         if (best == 0 || cost < best) {
             best = cost;
             *zc = z;
@@ -1746,7 +1750,7 @@ int apply_grid_blocks(int dim, int n) {
     long long b = noalloc_grid_blocks(dim, n);
     if (dim == 3) {
         int zc;
-        const dim3 g = applyz_grid(n, &zc);
+        const dim3 g = applyz_grid(n, true, &zc);
         b = std::max(b, (long long)g.x * g.y);
     }
     return (int)b;
@@ -1775,7 +1779,7 @@ int launch_apply(const Op<R>& op, const typename CT<R>::T* x, const typename CT<
     }
     if (op.dim == 3 && op.nbm && op.lidx && !op.face) {
         int zc;
-        const dim3 g = applyz_grid(op.n, &zc);
+        const dim3 g = applyz_grid(op.n, partials != nullptr, &zc);
         if (resid) {
             if (partials) launch_after(k_apply_z<R, true, true>, g, AZ, 0, s, op, zc, x, f, y, partials, conj, tail);
             else launch_after(k_apply_z<R, true, false>, g, AZ, 0, s, op, zc, x, f, y, partials, conj, tail);
