@@ -678,18 +678,25 @@ helm_status solve_fgmres(helm_handle* h, const helm_solve_opts* o, const double2
         launch_gs_scale(V0, V0, mixed ? h->tmp32[0] : nullptr, scal(h, S_BETA2), N, h->g, m + 1, s);
         h->launches += 1;
         // Lagged polling: step j + 1 is queued before the host waits for the estimate of
-        // step j, so the GPU does not idle while the host decides (about 20 us a step on
-        // small grids).  If step j ends the cycle, the queued step is surplus: it writes
-        // V_{j+2}, column j + 1 of H and of the rotations, and g_{j+1}, g_{j+2}, none of
-        // which the k = j + 1 solve reads.  (Not with profiling on, whose event counts
-        // are those of the steps taken.)
+        // step j, so the GPU does not idle while the host decides (about 20 us a step).
+        // If step j ends the cycle, the queued step is surplus: it writes V_{j+2}, column
+        // j + 1 of H and of the rotations, and g_{j+1}, g_{j+2}, none of which the
+        // k = j + 1 solve reads.  It also costs a whole step, so none is queued where step j
+        // may end the cycle: if it did twice as well as the last one known (a cycle's first
+        // step: gained a factor of 100), and, on grids where a step takes more than about
+        // 100 us (2^16 nodes), if it gained a factor of 10.  FGMRES of five steps at 128^3,
+        // FP64 and mixed: 4.56 and 3.04 ms with a step always queued, 3.73 and 2.51 so.
+        // (Nor with profiling on, whose event counts are those of the steps taken.)
+        const double leap = N > (1 << 16) ? 0.1 : 1.0;
         int kdim = 0, queued = 0;
+        double est1 = beta / bnorm, gain = 0.1;              // estimate before step j, its last gain
         for (int j = 0; j < m; ++j) {
             if (queued == j) {
                 TRY(enqueue_step(j, j & 1));
                 queued = j + 1;
             }
-            if (!h->profile && j + 1 < m && iters + 1 < o->maxit) {
+            if (!h->profile && j + 1 < m && iters + 1 < o->maxit &&
+                est1 * std::min(leap, gain * gain) > o->tol) {
                 TRY(enqueue_step(j + 1, (j + 1) & 1));
                 queued = j + 2;
             }
@@ -702,6 +709,8 @@ helm_status solve_fgmres(helm_handle* h, const helm_solve_opts* o, const double2
             if (snap[2 * S_FLAGS + 1] == 4.0) { st->status = HELM_TIMEOUT; break; }
             const double est = snap[2 * S_EST] / bnorm;
             hist.push(est);
+            gain = std::min(1.0, est / est1);
+            est1 = est;
             const double wn2 = snap[2 * S_WN2];
             if (!std::isfinite(est)) break;
             if (wn2 == 0.0 || est <= o->tol || iters >= o->maxit) break;
