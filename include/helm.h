@@ -142,7 +142,9 @@ helm_status helm_create(int dim, int n, double k0, int layer_cells, double layer
 helm_status helm_create_bvp(int dim, int n, double k0, const uint8_t* mask, const double* k2, int neumann_top,
                             helm_handle** out);
 helm_status helm_destroy(helm_handle* h);
-/* stream: a cudaStream_t (NULL = legacy default stream). */
+/* stream: a cudaStream_t (NULL = legacy default stream).  The handle has one workspace: a
+ * new stream's first call must come after the old stream's last one (an event or a
+ * synchronisation between them), also where the calls were captured and are replayed. */
 helm_status helm_set_stream(helm_handle* h, void* stream);
 const char* helm_last_error(const helm_handle* h);
 

@@ -26,6 +26,16 @@ __device__ __forceinline__ bool last_block_done(unsigned* counter, unsigned nblo
     return s_last;
 }
 
+// the same for the norms, whose counter wraps to zero by itself
+__device__ __forceinline__ bool norm_block_done(unsigned* counter, unsigned nblocks) {
+    __shared__ bool s_last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0 && threadIdx.y == 0) s_last = atomicInc(counter, nblocks - 1) == nblocks - 1;
+    __syncthreads();
+    return s_last;
+}
+
 // v[q] summed over the block's kFusedThreads threads (flat index tid) in a fixed order,
 // valid in thread 0: halves are added through shared memory, so that 255 additions a value
 // take 12 FP64 instructions of a warp.  (Butterflies in every warp take 45, and an FP64

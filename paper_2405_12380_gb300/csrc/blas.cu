@@ -45,12 +45,9 @@ __global__ void __launch_bounds__(TB) k_norm2(const double2* __restrict__ a, lon
         acc[0] = cnorm2(a[l], acc[0]);
     block_tree<1>(acc, threadIdx.x);
     if (threadIdx.x == 0) partials[blockIdx.x] = acc[0];
-    if (last_block_done(counter, gridDim.x)) {
+    if (norm_block_done(counter, gridDim.x)) {
         sum_parts<1>(partials, gridDim.x, threadIdx.x, acc);
-        if (threadIdx.x == 0) {
-            *out = acc[0];
-            *counter = 0;
-        }
+        if (threadIdx.x == 0) *out = acc[0];
     }
 }
 
@@ -302,10 +299,10 @@ int stream_blocks(long long N) {
 void launch_dot(const double2* a, const double2* b, long long N, double2* partials, cudaStream_t s) {
     launch_after(k_dot, kRedBlocks, TB, 0, s, a, b, N, partials);
 }
-void launch_norm2(const double2* a, long long N, double* partials, double* out, unsigned* counter, cudaStream_t s) {
+void launch_norm2(const double2* a, long long N, double* partials, double* out, unsigned* counters, cudaStream_t s) {
     // (no more blocks than the vector fills: each costs the last one a partial)
     const unsigned nb = (unsigned)std::min<long long>(kRedBlocks, (N + TB - 1) / TB);
-    launch_after(k_norm2, nb, TB, 0, s, a, N, partials, out, counter);
+    launch_after(k_norm2, nb, TB, 0, s, a, N, partials, out, counters + kNormVector);
 }
 void launch_sum_real(const double* partials, int nparts, double* out, cudaStream_t s) {
     launch_after(k_sum_real, 1, kFinThreads, 0, s, partials, nparts, out);

@@ -112,21 +112,18 @@ double hs(const helm_handle* h, int slot, int im = 0) { return h->hpin[2 * slot 
 // a grid-barrier wait of the cooperative cycle gave up (flag 4 in S_FLAGS.y, read by poll)
 bool barrier_timed_out(const helm_handle* h) { return hs(h, S_FLAGS, 1) == 4.0; }
 
-// the block counter of a launch that finishes a norm: each takes the next of 64, so that
-// launches on two streams (a handle whose stream was changed without waiting) cannot leave
-// each other's counter off zero
-unsigned* norm_counter(helm_handle* h) { return h->counter + 16 + (h->norm_launch++ & 63u); }
+unsigned* norm_counters(helm_handle* h) { return h->counter + kNormCounters; }
 
 // ||f - A x||^2 into slot (FP64)
 helm_status residual_norm(helm_handle* h, const double2* f, const double2* x, double2* r, int conj, int slot) {
-    launch_apply<double>(h->op64, x, f, r, h->red, conj, true, h->stream, scal(h, slot), norm_counter(h));
+    launch_apply<double>(h->op64, x, f, r, h->red, conj, true, h->stream, scal(h, slot), norm_counters(h));
     h->launches += 1;
     CKL();
     return HELM_OK;
 }
 
 helm_status norm2_into(helm_handle* h, const double2* a, int slot) {
-    launch_norm2(a, h->N, h->red, scal(h, slot), norm_counter(h), h->stream);
+    launch_norm2(a, h->N, h->red, scal(h, slot), norm_counters(h), h->stream);
     h->launches += 1;
     CKL();
     return HELM_OK;
@@ -1512,13 +1509,13 @@ helm_status helm_residual(helm_handle* h, const void* f, const void* x, void* r,
                           int dtype) {
     if (!h || !f || !x || !r) return fail(h, HELM_BAD_ARG, "null argument");
     double* part = norm2 ? h->red : nullptr;
-    unsigned* counter = norm2 ? norm_counter(h) : nullptr;
+    unsigned* counters = norm2 ? norm_counters(h) : nullptr;
     if (dtype == HELM_C128)
         launch_apply<double>(h->op64, (const double2*)x, (const double2*)f, (double2*)r, part, conj, true, h->stream,
-                             norm2, counter);
+                             norm2, counters);
     else if (dtype == HELM_C64)
         launch_apply<float>(h->op32, (const float2*)x, (const float2*)f, (float2*)r, part, conj, true, h->stream, norm2,
-                            counter);
+                            counters);
     else
         return fail(h, HELM_BAD_ARG, "dtype");
     CKL();

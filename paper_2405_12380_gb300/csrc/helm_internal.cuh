@@ -68,7 +68,12 @@ constexpr int kMaxP = 256;          // trunk basis functions
 constexpr int kMaxRestart = 64;     // FGMRES(m)
 constexpr int kRedBlocks = 304;     // blocks of the fixed-grid reductions (2 per SM)
 constexpr int kFinThreads = 1024;
-constexpr int kCounters = 80;       // block counters of a handle
+constexpr int kNormCounters = 4, kCounters = 8;     // block counters of a handle
+// The launches that finish a norm, a counter each: all launches of a route have the same
+// number of blocks, and the counter wraps at it (norm_block_done), so that even launches
+// that overlap (a handle used on two streams at once: their norms are wrong, the partials
+// are the handle's) leave it at zero for the next one
+enum NormRoute { kNormZ = 0, kNormPairs, kNormFlat, kNormVector };
 
 // ------------------------------------------------------------ complex helpers
 template <typename R> struct CT;
@@ -234,11 +239,11 @@ cudaError_t launch_after(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t s
 // ------------------------------------------------------------ kernel launchers
 // stencil.cu
 // returns the number of per-block partial sums of ||y||^2 written to `partials` (when
-// given); with a counter (zero between uses) the last block also sums them into *norm
+// given); with the handle's norm counters the last block also sums them into *norm
 template <typename R>
 int launch_apply(const Op<R>& op, const typename CT<R>::T* x, const typename CT<R>::T* f,
                  typename CT<R>::T* y, double* partials, int conj, bool resid, cudaStream_t s,
-                 double* norm = nullptr, unsigned* counter = nullptr);
+                 double* norm = nullptr, unsigned* counters = nullptr);
 template <typename R>
 void launch_jacobi(const Op<R>& op, double omega, const typename CT<R>::T* f,
                    const typename CT<R>::T* xin, typename CT<R>::T* xout, int conj, bool xzero,
@@ -335,7 +340,7 @@ void launch_b32_replace(const double2* r64, float2* r, float2* rhat, float2* p, 
 // blas.cu
 // partial reductions over a fixed grid of kRedBlocks blocks
 void launch_dot(const double2* a, const double2* b, long long N, double2* partials, cudaStream_t s);
-void launch_norm2(const double2* a, long long N, double* partials, double* out, unsigned* counter, cudaStream_t s);
+void launch_norm2(const double2* a, long long N, double* partials, double* out, unsigned* counters, cudaStream_t s);
 void launch_sum_real(const double* partials, int nparts, double* out, cudaStream_t s);
 // BiCGStab pieces (scalars live in device memory, see blas.cu)
 void launch_bicg_update_p(const double2* r, const double2* v, double2* p, const double2* sc, long long N,
@@ -503,9 +508,8 @@ struct helm_handle {
     cudaEvent_t evring[2] = {nullptr, nullptr};
     int* dflag = nullptr;           // device int flags
     // block counters, zero between kernels: 0 the fused reductions of the solvers, 2 and 3
-    // the grid barrier, 16 .. 79 the norms (see norm_counter)
+    // the grid barrier, from kNormCounters on those of enum NormRoute
     unsigned* counter = nullptr;
-    unsigned norm_launch = 0;
     double* fparts = nullptr;       // partials of the fused reductions
     // general temporaries (N complex128 each)
     std::vector<double2*> tmp;

@@ -113,13 +113,10 @@ struct NormTail {
 };
 __device__ __forceinline__ void norm_tail(const NormTail& t, const double* partials, unsigned nblocks, int tid) {
     if (!t.counter) return;
-    if (last_block_done(t.counter, nblocks)) {
+    if (norm_block_done(t.counter, nblocks)) {
         double v[1];
         sum_parts<1>(partials, (int)nblocks, tid, v);
-        if (tid == 0) {
-            *t.out = v[0];
-            *t.counter = 0;
-        }
+        if (tid == 0) *t.out = v[0];
     }
 }
 
@@ -1758,8 +1755,8 @@ int apply_grid_blocks(int dim, int n) {
 
 template <typename R>
 int launch_apply(const Op<R>& op, const typename CT<R>::T* x, const typename CT<R>::T* f, typename CT<R>::T* y,
-                 double* partials, int conj, bool resid, cudaStream_t s, double* norm, unsigned* counter) {
-    const NormTail tail{norm, counter};
+                 double* partials, int conj, bool resid, cudaStream_t s, double* norm, unsigned* counters) {
+    auto tail_of = [&](NormRoute r) { return NormTail{norm, counters ? counters + r : nullptr}; };
     if constexpr (std::is_same<R, float>::value) {
         if (pair_ok(op, x, resid ? f : nullptr, y)) {
             int zc;
@@ -1767,6 +1764,7 @@ int launch_apply(const Op<R>& op, const typename CT<R>::T* x, const typename CT<
             const float4* x4 = reinterpret_cast<const float4*>(x);
             const float4* f4 = reinterpret_cast<const float4*>(f);
             float4* y4 = reinterpret_cast<float4*>(y);
+            const NormTail tail = tail_of(kNormPairs);
             if (resid) {
                 if (partials) launch_after(k_march_c64<0, true, true>, g, b, 0, s, op, zc, 0.f, x4, f4, y4, partials, conj, Dot32{}, tail);
                 else launch_after(k_march_c64<0, true, false>, g, b, 0, s, op, zc, 0.f, x4, f4, y4, partials, conj, Dot32{}, tail);
@@ -1780,6 +1778,7 @@ int launch_apply(const Op<R>& op, const typename CT<R>::T* x, const typename CT<
     if (op.dim == 3 && op.nbm && op.lidx && !op.face) {
         int zc;
         const dim3 g = applyz_grid(op.n, partials != nullptr, &zc);
+        const NormTail tail = tail_of(kNormZ);
         if (resid) {
             if (partials) launch_after(k_apply_z<R, true, true>, g, AZ, 0, s, op, zc, x, f, y, partials, conj, tail);
             else launch_after(k_apply_z<R, true, false>, g, AZ, 0, s, op, zc, x, f, y, partials, conj, tail);
@@ -1792,6 +1791,7 @@ int launch_apply(const Op<R>& op, const typename CT<R>::T* x, const typename CT<
     const int zc = apply_zc(op.dim, op.n);
     dim3 g = grid_for(op.dim, op.n, 1, zc), b(BX, BY);
     // 2D, or an operator without the per-node tables (the allocation-free path)
+    const NormTail tail = tail_of(kNormFlat);
     if (resid) {
         if (partials) launch_after(k_apply<R, true, true>, g, b, 0, s, op, zc, x, f, y, partials, conj, tail);
         else launch_after(k_apply<R, true, false>, g, b, 0, s, op, zc, x, f, y, partials, conj, tail);
