@@ -61,6 +61,14 @@ __device__ __forceinline__ void tree(double2* red, int t, int nv, int ng) {
     __syncthreads();
 }
 
+// (2^-e, 2^e), e the binary exponent of z's larger part (kept where both are normal numbers;
+// 0 for a part that is not finite)
+__device__ __forceinline__ double2 pow2_scale(double2 z) {
+    int e = max(__double2hiint(z.x) & 0x7fffffff, __double2hiint(z.y) & 0x7fffffff) >> 20;
+    e = e == 2047 ? 1023 : min(max(e, 1), 2045);
+    return make_double2(__hiloint2double((2046 - e) << 20, 0), __hiloint2double(e << 20, 0));
+}
+
 // Givens step for column j; the column and the earlier rotations are staged in shared
 // memory first (thread 0 walks them in a dependent chain: with each entry loaded from
 // memory inside the chain a step took 12 us at j = 7 and grew with j)
@@ -85,18 +93,20 @@ __device__ void givens(const GivensArgs& a, double wn2, double2* col, double2* s
         }
         // c = |x| / t, s = (x / |x|) ||w|| / t, r = (x / |x|) t with t^2 = |x|^2 + ||w||^2; the
         // square roots do not wait for one another (a hypot or a division apiece cost this
-        // one thread about a microsecond each)
-        const double ab2 = x.x * x.x + x.y * x.y, t2 = ab2 + wn2;
-        const double iab = rsqrt(ab2), it = rsqrt(t2), hn = wn2 * rsqrt(wn2);
+        // one thread about a microsecond each).  |x| and x / |x| come from x scaled to about
+        // 1, as hypot does it: below 1e-154 |x|^2 would lose its digits
+        const double2 sx = pow2_scale(x), xs = cscale(sx.x, x);
+        const double as2 = xs.x * xs.x + xs.y * xs.y, t2 = x.x * x.x + x.y * x.y + wn2;
+        const double ias = rsqrt(as2), it = rsqrt(t2), hn = wn2 * rsqrt(wn2);
         double c;
         double2 s, r;
         if (wn2 == 0) {
             c = 1; s = make_double2(0, 0); r = x;
-        } else if (ab2 == 0) {
+        } else if (as2 == 0) {
             c = 0; s = make_double2(1.0, 0.0); r = make_double2(hn, 0);
         } else {
-            const double2 ph = cscale(iab, x);
-            c = ab2 * iab * it;
+            const double2 ph = cscale(ias, xs);
+            c = as2 * ias * sx.y * it;
             s = cscale(hn * it, ph);
             r = cscale(t2 * it, ph);
         }
@@ -106,7 +116,8 @@ __device__ void givens(const GivensArgs& a, double wn2, double2* col, double2* s
         const double2 gj = a.g[j], gn = cscale(-1.0, cmulc(s, gj));
         a.g[j + 1] = gn;
         a.g[j] = cscale(c, gj);
-        *a.est = sqrt(gn.x * gn.x + gn.y * gn.y);
+        const double2 sg = pow2_scale(gn), gs = cscale(sg.x, gn);
+        *a.est = sqrt(gs.x * gs.x + gs.y * gs.y) * sg.y;
         a.wnorm2[0] = wn2;
         a.wnorm2[1] = wn2 == 0 ? 0.0 : rsqrt(wn2);
     }
