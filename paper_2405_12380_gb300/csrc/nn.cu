@@ -612,18 +612,24 @@ helm_status nn_gemm(int transA, int transB, int M, int N, int K, float alpha, co
         if (beta != 1.f) k_scale_matrix<<<grid_for((long long)M * N), 256, 0, s>>>(M, N, beta, C, ldc);
         return cudaGetLastError() == cudaSuccess ? HELM_OK : HELM_CUDA_ERROR;
     }
+    // K is split, and the parts added atomically in any order, only where K is long and C
+    // small: from 128 on and below 304 tiles of 64 x 64.  Other products are one chain a
+    // value, the same bits on every call
+    const auto up = [](long long a, long long b) { return (a + b - 1) / b; };
+    const bool split = K >= 128 && up(M, 64) * up(N, 64) < 2 * 152;
     // 128 x 128 tiles where M fills them; 32 rows for the batch-sized products (a row of
-    // the batch per 8 threads wastes nothing on padding), 256 columns wide while that
-    // still gives two blocks per SM with K unsplit or K is long enough to split
-    const int bm = M <= 64 ? 32 : 128;
-    const int bn = bm == 32 && N > 128 ? 256 : 128;
-    const long long tiles = (long long)((M + bm - 1) / bm) * ((N + bn - 1) / bn);
+    // the batch per 8 threads wastes nothing on padding), and for an unsplit product of few
+    // tiles: one 32 x 256 tile an SM (4864 x 256 x 256: 30.8 -> 22.6 us; with 188 of them
+    // 30.8 -> 32.9) or two 32 x 128 (9728 x 100 x 100: 16.4 -> 12.4).  256 columns for N > 128
+    const int wide = N > 128 ? 256 : 128;
+    const int bm = M <= 64 || (!split && up(M, 32) * up(N, wide) <= (wide == 256 ? 152 : 2 * 152)) ? 32 : 128;
+    const int bn = bm == 32 ? wide : 128;
+    const long long tiles = up(M, bm) * up(N, bn);
     if (tiles > 0x7fffffffLL) return HELM_BAD_ARG;
-    // K split until every SM holds its resident blocks once (2 of 256 threads, 3 of 128, 5
-    // of 64: a part of a second wave would cost a whole one), at least 2 slabs each; the
-    // split parts add into C atomically
+    // a split fills every SM's resident blocks once (2 of 256 threads, 3 of 128, 5 of 64: a
+    // part of a second wave would cost a whole one), at least 2 slabs each
     const long long want = (bm == 128 ? 2 : bn == 256 ? 3 : 5) * 152;
-    int splits = (int)std::max<long long>(1, std::min<long long>(want / tiles, K / (2 * SBK)));
+    int splits = split ? (int)std::max<long long>(1, std::min<long long>(want / tiles, K / (2 * SBK))) : 1;
     int kslice = ((K + splits - 1) / splits + SBK - 1) / SBK * SBK;
     splits = (K + kslice - 1) / kslice;
     int add = splits > 1 ? 2 : (beta != 0.f);
