@@ -226,9 +226,9 @@ helm_status jacobi_run(helm_handle* h, const Op<R>& op, double omega, int sweeps
                        typename CT<R>::T* x, typename CT<R>::T* tmp, int conj, bool from_zero, cudaStream_t s) {
     using C = typename CT<R>::T;
     if (sweeps <= 0) return HELM_OK;
-    const int per = jacobi_tile_sweeps(op);
+    const int per = sweeps > 1 ? jacobi_tile_sweeps(op) : 0;
     int L = per ? (sweeps + per - 1) / per : sweeps;
-    if (per && !from_zero && sweeps > 1) L += L & 1;
+    if (per && !from_zero) L += L & 1;
     // the last launch writes x, unless an odd number starts from x: then it writes tmp
     const bool to_tmp = !from_zero && (L & 1);
     const C* in = from_zero ? nullptr : x;

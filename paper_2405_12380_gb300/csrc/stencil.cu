@@ -1823,12 +1823,14 @@ void launch_jacobi(const Op<R>& op, double omega, const typename CT<R>::T* f, co
 }
 
 // sweeps per launch of the tiled form for this operator, 0 where it does not apply (3D,
-// outer-boundary rows, no tables) or does not pay: with the halo an FP64 node costs about
-// twice its arithmetic, so the tiles win while a sweep is bound by its launch (64^2: 5.3 us
-// a launch; a 512^2 FP64 sweep is already bound by the FP64 pipe)
+// outer-boundary rows, no tables) or does not pay: with the halo a node costs two to four
+// times its arithmetic, so the tiles win while a sweep is bound by its launch.  20 sweeps,
+// us, single ones and tiled: complex128 128^2 59.0 and 40.6, 192^2 58.1 and 59.6, 256^2
+// 86.8 and 111.9; complex64 64^2 40.3 and 10.0, 512^2 42.9 and 34.9, 768^2 71.6 and 68.3,
+// 900^2 87.1 and 94.6.  (One sweep is a launch either way: 768^2 complex64 8.3 and 10.4.)
 template <typename R>
 int jacobi_tile_sweeps(const Op<R>& op) {
-    const int limit = std::is_same<R, double>::value ? 384 : 768;
+    const int limit = std::is_same<R, double>::value ? 160 : 768;
     return (op.dim == 2 && op.nbm && op.lidx && !op.face && op.n <= limit) ? kJacobiTileSweeps : 0;
 }
 
