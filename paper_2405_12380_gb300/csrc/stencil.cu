@@ -914,7 +914,9 @@ __device__ __forceinline__ void jacobi_point(const Op<R>& op, R omega, const typ
                                              typename CT<R>::T* __restrict__ xout, int conj, long long l) {
     using C = typename CT<R>::T;
     const C fl = f[l];
-    const unsigned code = op.nbm[l];
+    // (by node_code, although every handle has the table: the compiler orders the loads better
+    // behind its test; read straight from the table 256^3 took 871 us, 1024^2 49.3 for 42.7)
+    const unsigned code = node_code(op, l);
     C out;
     if (code & kMasked) {
         if (XZERO) {
@@ -943,7 +945,8 @@ __device__ __forceinline__ void jacobi_point(const Op<R>& op, R omega, const typ
 }
 
 // One node per thread in the flat order: every lane has a node whatever the row length
-// (as in k_apply_z and the red-black kernels below).
+// (as in k_apply_z and the red-black kernels below).  In complex128, 32 x 8 tiles with two
+// planes a thread and this: 97^3 59.5 and 51.4 us, 128^3 108.8 and 104.9, 256^3 785 and 783.
 template <typename R, bool XZERO>
 __global__ void __launch_bounds__(BX * BY) k_jacobi(Op<R> op, R omega, const typename CT<R>::T* __restrict__ f,
                                                     const typename CT<R>::T* __restrict__ xin,
@@ -1825,8 +1828,8 @@ void launch_jacobi(const Op<R>& op, double omega, const typename CT<R>::T* f, co
 // sweeps per launch of the tiled form for this operator, 0 where it does not apply (3D,
 // outer-boundary rows, no tables) or does not pay: with the halo a node costs two to four
 // times its arithmetic, so the tiles win while a sweep is bound by its launch.  20 sweeps,
-// us, single ones and tiled: complex128 128^2 59.0 and 40.6, 192^2 58.1 and 59.6, 256^2
-// 86.8 and 111.9; complex64 64^2 40.3 and 10.0, 512^2 42.9 and 34.9, 768^2 71.6 and 68.3,
+// us, single ones and tiled: complex128 128^2 59.0 and 40.6, 192^2 56.6 and 59.6, 256^2
+// 82.0 and 111.9; complex64 64^2 40.3 and 10.0, 512^2 42.9 and 34.9, 768^2 71.6 and 68.3,
 // 900^2 87.1 and 94.6.  (One sweep is a launch either way: 768^2 complex64 8.3 and 10.4.)
 template <typename R>
 int jacobi_tile_sweeps(const Op<R>& op) {
