@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(BM * BN / 64, BM * BN / 64 >= 256 ? 2 : 3)
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     constexpr int WN = BN / 64;                            // warps along N
     const int rm = (w / WN) * 32 + (lane >> 3) * 4, rn = (w % WN) * 64 + (lane & 7) * 4;
-    const int tiles_m = (M + BM - 1) / BM;
+    const int tiles_m = (M - 1) / BM + 1;
     const int m0 = (blockIdx.x % tiles_m) * BM, n0 = (blockIdx.x / tiles_m) * BN;
     const int k0 = blockIdx.z * kslice, k1 = min(K, k0 + kslice);
     unsigned long long acc[8][4];
@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(BM * BN / 64, BM * BN / 64 >= 256 ? 2 : 3)
             float* c = C + (long long)gm * ldc + gn;
 #pragma unroll
             for (int q = 0; q < 4; ++q) v[q] *= alpha;
-            if (gn + 4 <= N && (vecs & 4)) {
+            if (gn <= N - 4 && (vecs & 4)) {
                 if (add == 2) {
                     asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(c), "f"(v[0]), "f"(v[1]),
                                  "f"(v[2]), "f"(v[3])
@@ -208,12 +208,12 @@ __device__ __forceinline__ float act_of(float v, int act) {
 template <int V>
 __global__ void __launch_bounds__(256) k_bias_act(int rows, int cols, float* __restrict__ X,
                                                   const float* __restrict__ bias, int act) {
-    const int c = (blockIdx.x * 64 + (threadIdx.x & 63)) * V;
+    const long long c = (blockIdx.x * 64LL + (threadIdx.x & 63)) * V;
     if (c >= cols) return;
     float b[V];
 #pragma unroll
     for (int q = 0; q < V; ++q) b[q] = bias ? bias[c + q] : 0.f;
-    for (int r = blockIdx.y * 4 + (threadIdx.x >> 6); r < rows; r += gridDim.y * 4) {
+    for (unsigned r = blockIdx.y * 4 + (threadIdx.x >> 6); r < (unsigned)rows; r += gridDim.y * 4) {
         float* x = X + (long long)r * cols + c;
         if (V == 4) {
             float4 t = *reinterpret_cast<float4*>(x);
@@ -263,15 +263,16 @@ __global__ void __launch_bounds__(256) k_bias_grad(int rows, int cols, const flo
     __shared__ float part[32][8];
     __shared__ float sums[8];
     const int tid = threadIdx.x, cc = tid & 7, rr = tid >> 3;
-    const int c = (blockIdx.x / CS) * 8 + cc, rank = CS == 1 ? 0 : (int)(blockIdx.x % CS);
+    const long long c = (blockIdx.x / CS) * 8LL + cc;
+    const int rank = CS == 1 ? 0 : (int)(blockIdx.x % CS);
     float s[4] = {0.f, 0.f, 0.f, 0.f};
     if (c < cols) {
         constexpr int STEP = 32 * CS;
-        int r = rank * 32 + rr;
-        for (; r + 3 * STEP < rows; r += 4 * STEP)
+        unsigned r = rank * 32 + rr;                       // (32 bits without the sign: r runs past rows)
+        for (; r + 3 * STEP < (unsigned)rows; r += 4 * STEP)
 #pragma unroll
             for (int u = 0; u < 4; ++u) s[u] += dY[(long long)(r + u * STEP) * cols + c];
-        for (; r < rows; r += STEP) s[0] += dY[(long long)r * cols + c];
+        for (; r < (unsigned)rows; r += STEP) s[0] += dY[(long long)r * cols + c];
     }
     part[rr][cc] = (s[0] + s[1]) + (s[2] + s[3]);
     __syncthreads();
@@ -305,14 +306,14 @@ __global__ void __launch_bounds__(256) k_bias_grad_rows(int rows, int cols, cons
                                                         float* __restrict__ db) {
     extern __shared__ __align__(16) float tile[];          // [2][8][BS_PITCH], column by column
     const int tid = threadIdx.x, cc = tid & 7, rr = tid >> 3;
-    const int c = blockIdx.x * 8 + cc;
+    const long long c = blockIdx.x * 8LL + cc;
     float s = 0.f;
     // 4-byte asynchronous copies (zeros past the matrix), so that nothing waits for them here
-    auto fetch = [&](int r0, float* t) {
+    auto fetch = [&](unsigned r0, float* t) {
 #pragma unroll 8
         for (int q = 0; q < BS_ROWS / 32; ++q) {
-            const int r = r0 + rr + 32 * q;
-            const bool in = r < rows && c < cols;
+            const unsigned r = r0 + rr + 32 * q;
+            const bool in = r < (unsigned)rows && c < cols;
             asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(
                              (unsigned)__cvta_generic_to_shared(t + cc * BS_PITCH + rr + 32 * q)),
                          "l"(in ? dY + (long long)r * cols + c : dY), "r"(in ? 4 : 0)
@@ -321,15 +322,16 @@ __global__ void __launch_bounds__(256) k_bias_grad_rows(int rows, int cols, cons
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
     if (rows > 0) fetch(0, tile);
-    for (int r0 = 0, buf = 0; r0 < rows; r0 += BS_ROWS, buf ^= 1) {
+    int buf = 0;
+    for (unsigned r0 = 0; r0 < (unsigned)rows; r0 += BS_ROWS, buf ^= 1) {
         const float* t = tile + buf * BS_PITCH * 8;
         asm volatile("cp.async.wait_group 0;" ::: "memory");
         __syncthreads();                                   // (the other buffer has been added)
-        if (r0 + BS_ROWS < rows) fetch(r0 + BS_ROWS, tile + (buf ^ 1) * BS_PITCH * 8);
+        if (r0 + BS_ROWS < (unsigned)rows) fetch(r0 + BS_ROWS, tile + (buf ^ 1) * BS_PITCH * 8);
         if (tid < 8) {
             // 16 values on their way from shared memory while 16 are added; the zeros past
             // the last row leave the sum as it is
-            const int m = min(BS_ROWS, rows - r0);
+            const int m = (int)min((unsigned)BS_ROWS, (unsigned)rows - r0);
             const float4* col = reinterpret_cast<const float4*>(t + tid * BS_PITCH);
             float4 x[4], y[4];
 #pragma unroll
@@ -411,7 +413,7 @@ __global__ void __launch_bounds__(256) k_rel_l2(int Bn, int P2, const float* __r
     if (rank == 0) {
         float num = 0.f, den = 0.f;
 #pragma unroll 16
-        for (int e = threadIdx.x; e < P2; e += 256) {
+        for (unsigned e = threadIdx.x; e < (unsigned)P2; e += 256) {
             const float t = tg[e], d = pr[e] - t;
             num = fmaf(d, d, num);
             den = fmaf(t, t, den);
@@ -439,10 +441,11 @@ __global__ void __launch_bounds__(256) k_rel_l2(int Bn, int P2, const float* __r
         c = cl.map_shared_rank(sums, 0)[1];
         cl.sync();                                         // the sums stay until every block has read them
     }
-    const int share = (P2 + CS - 1) / CS, e0 = min(P2, rank * share), e1 = min(P2, e0 + share);
+    const unsigned share = ((unsigned)P2 + CS - 1) / CS, e0 = min((unsigned)P2, rank * share);
+    const unsigned e1 = min((unsigned)P2, e0 + share);
     const float scale = 2.f / (c * Bn);
 #pragma unroll 4
-    for (int e = e0 + threadIdx.x; e < e1; e += 256) dpred[(long long)b * P2 + e] = scale * (pr[e] - tg[e]);
+    for (unsigned e = e0 + threadIdx.x; e < e1; e += 256) dpred[(long long)b * P2 + e] = scale * (pr[e] - tg[e]);
 }
 
 // dst[r][c] = src[ri[r]][ci[c]] (ri, ci may be null: identity)
@@ -668,8 +671,8 @@ helm_status nn_bias_act(int rows, int cols, float* X, const float* bias, int act
     if (rows == 0 || cols == 0) return HELM_OK;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const bool vec = cols % 4 == 0 && al16(X);
-    const int gx = (cols + (vec ? 255 : 63)) / (vec ? 256 : 64);
-    const dim3 g(gx, (unsigned)std::max(1, std::min((rows + 3) / 4, 8 * 152 / std::min(gx, 8 * 152))));
+    const int gx = (cols - 1) / (vec ? 256 : 64) + 1;
+    const dim3 g(gx, (unsigned)std::max(1, std::min((rows - 1) / 4 + 1, 8 * 152 / std::min(gx, 8 * 152))));
     if (vec) k_bias_act<4><<<g, 256, 0, s>>>(rows, cols, X, bias, act);
     else k_bias_act<1><<<g, 256, 0, s>>>(rows, cols, X, bias, act);
     return cudaGetLastError() == cudaSuccess ? HELM_OK : HELM_CUDA_ERROR;
@@ -686,7 +689,7 @@ helm_status nn_bias_grad(int rows, int cols, const float* dY, float* db, void* s
     if (rows < 0 || cols < 0 || !dY || !db) return HELM_BAD_ARG;
     if (cols == 0) return HELM_OK;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const unsigned groups = (unsigned)((cols + 7) / 8);
+    const unsigned groups = (unsigned)((cols - 1) / 8 + 1);
     if (rows < 256) k_bias_grad<1><<<groups, 256, 0, s>>>(rows, cols, dY, db);
     else if (launch_clustered(k_bias_grad<8>, 8 * groups, 8, s, rows, cols, dY, db) != cudaSuccess) return HELM_CUDA_ERROR;
     return cudaGetLastError() == cudaSuccess ? HELM_OK : HELM_CUDA_ERROR;
@@ -698,7 +701,7 @@ helm_status nn_bias_grad_rows(int rows, int cols, const float* dY, float* db, vo
     const size_t smem = 2 * BS_PITCH * 8 * sizeof(float);
     if (cudaFuncSetAttribute(k_bias_grad_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return HELM_CUDA_ERROR;
-    k_bias_grad_rows<<<(cols + 7) / 8, 256, smem, static_cast<cudaStream_t>(stream)>>>(rows, cols, dY, db);
+    k_bias_grad_rows<<<(cols - 1) / 8 + 1, 256, smem, static_cast<cudaStream_t>(stream)>>>(rows, cols, dY, db);
     return cudaGetLastError() == cudaSuccess ? HELM_OK : HELM_CUDA_ERROR;
 }
 
