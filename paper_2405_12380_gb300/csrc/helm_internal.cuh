@@ -123,7 +123,8 @@ __host__ __device__ __forceinline__ double2 cdiv(double2 a, double2 b) {
 // value = hi + lo with hi = the nearest FP32 number and lo the nearest to the rest.  A
 // conversion between the formats runs on the FP64 pipe (64 clocks of a scheduler's pipe
 // per warp, like every FP64 instruction): four per component for a split, two and an add
-// for a join.  Both are instead formed with integer instructions, bit for bit the same;
+// for a join.  Both are instead formed with integer instructions, bit for bit the same (but
+// for the sign of a zero lo, which is that of the value);
 // values outside the range where that holds (subnormal in FP32, near its largest, not
 // finite) take the conversions.  Operator kernels with their BiCGStab dots at 64^3: 20.5
 // and 23.7 -> 16.7 and 19.5 us (ncu, cold; with the tree sums of bicg.cuh).
