@@ -149,17 +149,17 @@ __global__ void __launch_bounds__(GT) k_gs(const double2* __restrict__ V, int nv
         __syncthreads();                                   // the previous tile is consumed
         for (int e = t; e < nv << lrt; e += GT) {
             const int i = e >> lrt, r = e & (RT - 1);
-            gs_copy16(vs + i * (RT + 1) + r, r < rows ? V + (long long)i * N + t0 + r : V, r < rows);
+            gs_copy16(vs + i * (RT + 1) + r, r < rows ? V + HCHK((long long)i * N + t0 + r, (long long)nv * N) : V, r < rows);
         }
         asm volatile("cp.async.commit_group;\n" ::: "memory");
         double2 wv = make_double2(0, 0);
         if (ig == 0 && own < rows) {
             if (W32) {
-                const float2 q = w32[t0 + own];
+                const float2 q = w32[HCHK(t0 + own, N)];
                 wv = make_double2(q.x, q.y);
-                w[t0 + own] = wv;
+                w[HCHK(t0 + own, N)] = wv;
             } else {
-                wv = w[t0 + own];
+                wv = w[HCHK(t0 + own, N)];
             }
         }
         if (MODE == GS_DOT && ig == 0) ws[own] = wv;
@@ -176,7 +176,7 @@ __global__ void __launch_bounds__(GT) k_gs(const double2* __restrict__ V, int nv
                     for (int q = 1; q < IG; ++q) s = cadd(s, red[q * RT + own]);
             }
             if (ig == 0) {
-                if (own < rows) w[t0 + own] = s;
+                if (own < rows) w[HCHK(t0 + own, N)] = s;
                 if (MODE == GS_UPDOT) ws[own] = s;
                 else acc.x = cnorm2(s, acc.x);             // (zero past the last row)
             }
@@ -231,9 +231,9 @@ __global__ void __launch_bounds__(256) k_gs_scale(const double2* w, double2* v, 
     }
     if (inv == 0) return;
     for (long long l = blockIdx.x * 256LL + threadIdx.x; l < N; l += gridDim.x * 256LL) {
-        const double2 q = cscale(inv, w[l]);
-        v[l] = q;
-        if (v32) v32[l] = make_float2((float)q.x, (float)q.y);
+        const double2 q = cscale(inv, w[HCHK(l, N)]);
+        v[HCHK(l, N)] = q;
+        if (v32) v32[HCHK(l, N)] = make_float2((float)q.x, (float)q.y);
     }
 }
 

@@ -212,9 +212,9 @@ __global__ void __launch_bounds__(AZ) k_apply_z(Op<R> op, int zc, const typename
     C zero;
     zero.x = 0; zero.y = 0;
     long long l = q + (long long)sz * k0;
-    C prev = (valid && k0 > 0) ? x[l - sz] : zero;
-    C cur = valid ? x[l] : zero;
-    C next = (valid && k0 + 1 < op.n) ? x[l + sz] : zero;
+    C prev = (valid && k0 > 0) ? x[HCHK(l - sz, op.N)] : zero;
+    C cur = valid ? x[HCHK(l, op.N)] : zero;
+    C next = (valid && k0 + 1 < op.n) ? x[HCHK(l + sz, op.N)] : zero;
     // the per-node tables are read one plane ahead as well, so that no load of
     // the loop is used in the iteration that issues it
     unsigned code = valid ? (unsigned)op.nbm[l] : kMasked;
@@ -222,17 +222,17 @@ __global__ void __launch_bounds__(AZ) k_apply_z(Op<R> op, int zc, const typename
     double acc = 0.0;
     for (int k = k0; k < k1; ++k, l += sz) {
         const bool more = valid && k + 1 < k1;
-        const C next2 = (more && k + 2 < op.n) ? x[l + 2 * sz] : zero;
-        const unsigned code_n = more ? (unsigned)op.nbm[l + sz] : kMasked;
-        const int li_n = more ? (int)op.lidx[l + sz] : 0;
+        const C next2 = (more && k + 2 < op.n) ? x[HCHK(l + 2 * sz, op.N)] : zero;
+        const unsigned code_n = more ? (unsigned)op.nbm[HCHK(l + sz, op.N)] : kMasked;
+        const int li_n = more ? (int)op.lidx[HCHK(l + sz, op.N)] : 0;
         C xm, xp, fv = zero;
-        if (RESID && valid) fv = f[l];
+        if (RESID && valid) fv = f[HCHK(l, op.N)];
         xm.x = __shfl_up_sync(0xffffffffu, cur.x, 1);
         xm.y = __shfl_up_sync(0xffffffffu, cur.y, 1);
         xp.x = __shfl_down_sync(0xffffffffu, cur.x, 1);
         xp.y = __shfl_down_sync(0xffffffffu, cur.y, 1);
-        if (lane == 0 && (code & 1u)) xm = x[l - 1];
-        if (lane == 31 && (code & 2u)) xp = x[l + 1];
+        if (lane == 0 && (code & 1u)) xm = x[HCHK(l - 1, op.N)];
+        if (lane == 31 && (code & 2u)) xp = x[HCHK(l + 1, op.N)];
         C out;
         if (code & kMasked) {
             out = cur;
@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(AZ) k_apply_z(Op<R> op, int zc, const typename
         }
         if (valid) {
             if (RESID) out = csub(fv, out);
-            y[l] = out;
+            y[HCHK(l, op.N)] = out;
             if (NORM) acc = norm_acc(out, acc);
         }
         prev = cur;
@@ -1916,8 +1916,8 @@ __global__ void __launch_bounds__(256) k_pack_colour(int n, int colour, const fl
     const unsigned h = n / 2;
     for (unsigned q = blockIdx.x * 256 + threadIdx.x; q < npairs; q += gridDim.x * 256) {
         const unsigned row = q / h, k = row / n, j = row - k * n;
-        const float4 v = x[q];
-        out[q] = ((j + k + colour) & 1) ? hi2(v) : lo2(v);
+        const float4 v = x[HCHK(q, npairs)];
+        out[HCHK(q, npairs)] = ((j + k + colour) & 1) ? hi2(v) : lo2(v);
     }
 }
 
