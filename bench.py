@@ -213,17 +213,19 @@ def source_hash(path):
 
 
 def traffic_for(workload, kernel):
-    """DRAM bytes per launch of `kernel` from the committed ncu summary of the
-    workload, if the kernel's source file is unchanged since the capture (else None)."""
+    """(DRAM bytes per launch of `kernel` from the committed ncu summary of the workload,
+    None) if the kernel's source files are unchanged since the capture, else (None, why)."""
     try:
         prof = json.load(open(os.path.join(ROOT, "profiles", f"traffic_{workload}.json")))
-        e = prof["kernels"][kernel]
     except Exception:
-        return None
-    src = os.path.join(ROOT, "paper_2405_12380_gb300", "csrc", e["source"])
-    if e.get("sha256_16") != source_hash(src):
-        return None
-    return e.get("dram_bytes_per_launch")
+        return None, "no capture of this workload"
+    e = prof["kernels"].get(kernel)
+    if e is None:
+        return None, "no capture of this kernel"
+    for src, sha in [(e["source"], e.get("sha256_16")), *e.get("also", {}).items()]:
+        if sha != source_hash(os.path.join(ROOT, "paper_2405_12380_gb300", "csrc", src)):
+            return None, f"{src} changed since the capture"
+    return e.get("dram_bytes_per_launch"), None
 
 
 def stencil_bench(hm, torch, n=256, reps=20):
@@ -295,8 +297,9 @@ def kernel_entries(w, st_prof, N, k, hbm, hbm_src, workload):
     per launch over the mean CUDA-event duration.  Mixed handles, per node:
     restriction k + 26 B (red-row residual: v and z in, 2 table bytes, the red
     residual out and in again; BF16 Q_red k B), prolongation 2k + 16 B (BF16 Q,
-    z in and out), fused red-black sweep 26 B from x (x and f in, x out, 2 table
-    bytes) and 18 B from zero, operator with the fused BiCGStab reduction 26 B (x and
+    z in and out), fused red-black sweeps of a cycle from zero 14 B the first (f and 2
+    table bytes in, the black half of x out), 18 B those between (the half in too) and
+    22 B the last (x out), a single one 18 B, operator with the fused BiCGStab reduction 26 B (x and
     the dot operand in, y out, 2 table bytes).  FP64 handles: FP32-pair basis 8k B
     per row."""
     mixed = w.get("precision") == "mixed"
@@ -308,9 +311,10 @@ def kernel_entries(w, st_prof, N, k, hbm, hbm_src, workload):
         if not n:
             return
         avg = ms / 1e3 / n
+        traffic, why = traffic_for(workload, kernel)
         out.append({"bound": "hbm", "kernel": kernel, "what": what, "achieved": bytes_per_launch / avg / 1e9,
                     "peak": hbm, "unit": "GB/s", "frac": bytes_per_launch / avg / 1e9 / hbm,
-                    "peak_source": hbm_src, "traffic": traffic_for(workload, kernel),
+                    "peak_source": hbm_src, "traffic": traffic, **({"traffic_note": why} if why else {}),
                     "algorithmic_bytes_per_launch": bytes_per_launch, "avg_launch_us": avg * 1e6,
                     "launches": n, "share_of_solve": ms / st_prof["ms"],
                     "timing": "CUDA events around every launch, one profiled solve after the timed solves"})
@@ -320,7 +324,8 @@ def kernel_entries(w, st_prof, N, k, hbm, hbm_src, workload):
             "c = Q_red^T (v - A z) on the red rows: red residual, then BF16 tall-skinny product")
         add("prolong", "k_prolong32v", "n_prolong", "prolong_ms", (2.0 * k + 16.0) * N, "z += Q y, BF16 Q")
         nr = max(1, w["n_r"])
-        add("sweep", "k_sweep_c64", "n_sweep", "sweep_ms", (18.0 + 26.0 * (nr - 1)) / nr * N,
+        cycle = 18.0 if nr == 1 else 14.0 + 18.0 * (nr - 2) + 22.0
+        add("sweep", "k_sweep_c64", "n_sweep", "sweep_ms", cycle / nr * N,
             "complex64 red-black full sweep (one launch), the first of each cycle from zero")
         add("apply", "k_march_c64<0,DOT>", "n_apply", "apply_ms", 26.0 * N,
             "complex64 y = A x with the BiCGStab reduction (alpha or omega) in its epilogue")

@@ -12,7 +12,7 @@
 //    each value stays one chain, whatever the tile;
 //  - warp 0: one elected thread loads the two boxes of every 64-deep K step with
 //    cp.async.bulk.tensor (128-byte swizzle); a stage is SUB such steps on one "full"
-//    mbarrier, and the ring has as many stages as K fills, up to what 222 KB hold (three);
+//    mbarrier, and the ring has as many stages as K fills, up to the three that 222 KB hold;
 //  - warp 1: one elected thread issues tcgen05.mma.kind::f16 (K = 16 per instruction, four
 //    per step) into a TMEM accumulator and commits each stage to its "empty" mbarrier, the
 //    last one to the "done" mbarrier as well;
@@ -45,7 +45,7 @@ namespace helm {
 
 namespace {
 
-constexpr int TBM = 128, TBK = 64, MAX_STAGES = 16;
+constexpr int TBM = 128, TBK = 64, MAX_STAGES = 3;       // (three stages of every tile fill the ring)
 constexpr int TC_THREADS = 256;
 constexpr unsigned kRingBytes = 222 * 1024;                    // shared memory of the stages, at most
 constexpr unsigned kWaitLimit = 1u << 26;
@@ -372,7 +372,8 @@ template <int TN, int SUB>
 cudaError_t gemm_tc(const CUtensorMap& mn, const CUtensorMap& mm, int M, int N, int Kp, float alpha, float beta, float* C,
                     int ldc, cudaStream_t s) {
     constexpr unsigned stage = (TBM + TN) * TBK * 2 * SUB;
-    const int stages = std::min(std::min((Kp / TBK + SUB - 1) / SUB, MAX_STAGES), (int)(kRingBytes / stage));
+    static_assert(MAX_STAGES * stage <= kRingBytes && (MAX_STAGES + 1) * stage > kRingBytes, "the ring holds MAX_STAGES");
+    const int stages = std::min((Kp / TBK + SUB - 1) / SUB, MAX_STAGES);
     const size_t smem = (size_t)std::min(stages * SUB, Kp / TBK) * (stage / SUB) + 1024;
     const cudaError_t e =
         cudaFuncSetAttribute(k_gemm_bf16_tc<TN, SUB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kRingBytes + 1024));

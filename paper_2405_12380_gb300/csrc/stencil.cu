@@ -1,6 +1,7 @@
 // Matrix-free Helmholtz operator, residual and relaxation sweeps (Eq. 1-2).
 //
-// Blocks of 32 x 8 threads over (x, y).  Per node two byte tables (neighbour code,
+// Blocks of 256 threads: 32 x 8 over (x, y), or (complex128, odd and 2D grids) 256 nodes or
+// node pairs in the flat order.  Per node two byte tables (neighbour code,
 // layer index) replace the mask loads and the index arithmetic; k^2 and 1/diag
 // come from per-layer tables in Op (or the stored field).  Kernel families:
 //   k_apply_z        3D operator/residual marching in z (planes in registers,
@@ -849,7 +850,7 @@ __global__ void __launch_bounds__(BX * BY) k_apply(Op<R> op, int zc, const typen
     pdl_begin();
     const int i = blockIdx.x * BX + threadIdx.x;
     const int j = blockIdx.y * BY + threadIdx.y;
-    // 3D: zc planes per block (the grid of k_apply_z, so partial counts agree)
+    // 3D: zc planes per block (noalloc_grid_blocks counts this grid's blocks)
     const int k0 = op.dim == 3 ? zc * blockIdx.z : 0;
     const int k1 = op.dim == 3 ? min(op.n, k0 + zc) : 1;
     double acc = 0.0;
@@ -957,7 +958,7 @@ __global__ void __launch_bounds__(BX * BY) k_jacobi(Op<R> op, R omega, const typ
 }
 
 // Several damped-Jacobi sweeps of a 2D grid in one launch (small grids, where a sweep
-// costs its launch: 5.3 us at 64 x 64 against 0.1 us of FP64 arithmetic).  A block owns
+// costs its launch: 3 us at 64 x 64 against 0.1 us of FP64 arithmetic).  A block owns
 // TI x TI nodes and recomputes a halo of S nodes around them, one node per thread
 // (blockDim = TI + 2 S per side): S sweeps run in shared memory, each on a region one
 // node smaller per side, and only the block's own nodes are written.  In FP64 the sweep is
