@@ -616,7 +616,8 @@ __global__ void __launch_bounds__(BX * BY) k_rbgs_c64(Op<float> op, int zc, int 
 // two half-sweeps.  The roundings are spelled out (sor_step, cmul_n; cmul_t for colour A
 // from zero), the same in every instantiation: left to the compiler they moved from one to
 // the next by 2e-8, which the trunk-basis correction and eight FGMRES steps can raise to
-// 1e-5 of the solution.  Measured against the form that staged whole pairs and selected by
+// 1e-5 of the solution.  (f - h^-2 s can be fused in one way only; as fmaf it cost 2% of
+// the sweep.)  Measured against the form that staged whole pairs and selected by
 // position (431 instructions a pair at 256^3; ncu, cold): 256^3 133 -> 83 us a sweep (5.3
 // TB/s of the 26 B a node), 128^3 20.5 -> 15.2 us, 64^3 13.2 -> 6.3 us.  The launch shape
 // is chosen by plan_sweep32.
@@ -782,7 +783,7 @@ __global__ void __launch_bounds__(kSweepMaxThreads, 1)
                 const float2* P = xs + o_0 + mx;
                 const float2 bx = P[dx];
                 const float2 s = six_sum(ca, ar, b0, bx, P[-TXT], P[TXT], bm1, bp1);
-                na = cmul_n(id, make_float2(fmaf(-op.hinv2, s.x, fa.x), fmaf(-op.hinv2, s.y, fa.y)));
+                na = cmul_n(id, make_float2(fa.x - op.hinv2 * s.x, fa.y - op.hinv2 * s.y));
             }
         }
         if (SOR) na = XZERO ? cscale(omega, na) : sor_step(xa, na, omega);
@@ -807,7 +808,7 @@ __global__ void __launch_bounds__(kSweepMaxThreads, 1)
                 float2 id = ib;
                 if (!K2) id = stab[HCHK(cb >> 8, kMaxLayerCells + 1)];
                 else if (conj) id.y = -id.y;
-                nb = cmul_n(id, make_float2(fmaf(-op.hinv2, s.x, fb.x), fmaf(-op.hinv2, s.y, fb.y)));
+                nb = cmul_n(id, make_float2(fb.x - op.hinv2 * s.x, fb.y - op.hinv2 * s.y));
             }
             // (from zero only colour A starts from zero: colour B's own old value is zero too)
             if (SOR) nb = sor_step(xb, nb, omega);
