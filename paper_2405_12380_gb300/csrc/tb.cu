@@ -1090,9 +1090,11 @@ __global__ void __launch_bounds__(32 * RR_WARPS, 4)
 // its lanes at the end.  A warp does RA_COLS columns.  A share starts at any row, so the
 // basis goes through shared memory of the warp's own, RA_TILE rows a stage: 16-byte
 // asynchronous copies from the 8 rows that hold the first one on, single values out of it.
-// helm_precond at 96^3, two Jacobi sweeps and 52 columns: 99 us; 145 with single values
-// loaded straight from memory.  Eight columns a warp: 1 us faster there, 4 slower at 20 to
-// 30 columns.
+// Bound by instruction issue beside HBM: a lane's chunks are the same in every tile, so their
+// addresses are formed once.  helm_precond at 96^3, two Jacobi sweeps and 52 columns: 97 us;
+// 99 with the addresses formed in every tile, 102 with the residual through shared memory
+// (a barrier a tile), 145 with single values loaded straight from memory.  Eight columns a
+// warp: the same there, 4 us slower at 20 to 30 columns.
 constexpr int RA_COLS = 4, RA_TILE = 256, RA_PITCH = RA_TILE + 8, RA_STAGES = 3, RA_WARPS = 8;
 constexpr size_t kRestrictAllSmem = (size_t)RA_WARPS * RA_STAGES * RA_COLS * RA_PITCH * 2;
 __global__ void __launch_bounds__(32 * RA_WARPS)
@@ -1107,16 +1109,27 @@ __global__ void __launch_bounds__(32 * RA_WARPS)
     const long long r0 = min(N, blockIdx.x * (long long)share);
     const int rows = (int)min((long long)share, N - r0), off = (int)(r0 & 7), tiles = (rows + RA_TILE - 1) / RA_TILE;
     const __nv_bfloat16* Qc = Q + (long long)c0 * ld + (r0 - off);
-    auto stage = [&](int t) {
+    // this lane's chunks of a stage: the same columns and rows of every tile
+    constexpr int CH = RA_PITCH / 8, NCH = (RA_COLS * CH + 31) / 32;
+    const __nv_bfloat16* src[NCH];
+    int first[NCH];
+#pragma unroll
+    for (int q = 0; q < NCH; ++q) {
+        const int e = lane + 32 * q, c = e / CH;
+        first[q] = c < nc && e < RA_COLS * CH ? 8 * (e % CH) : rows + RA_PITCH;
+        src[q] = Qc + (c < nc ? (long long)c * ld : 0) + 8 * (e % CH);
+    }
+    auto stage = [&](int t, int slot) {
         if (t < tiles) {
-            unsigned short* b = buf + (t % RA_STAGES) * RA_COLS * RA_PITCH;
-            for (int e = lane; e < RA_COLS * (RA_PITCH / 8); e += 32) {
-                const int c = e / (RA_PITCH / 8), i = t * RA_TILE + 8 * (e % (RA_PITCH / 8));
-                const bool in = c < nc && i < off + rows;  // (then the 8 rows lie in the column's padded length)
-                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(
-                                 (unsigned)__cvta_generic_to_shared(b + 8 * e)),
-                             "l"(Qc + HCHK(in ? c * ld + i : 0, (k - c0) * ld - (r0 - off))), "r"(in ? 16 : 0)
-                             : "memory");
+            const unsigned b = (unsigned)__cvta_generic_to_shared(buf + slot * RA_COLS * RA_PITCH + 8 * lane);
+#pragma unroll
+            for (int q = 0; q < NCH; ++q) {
+                // (then the 8 rows lie in the column's padded length)
+                const bool in = t * RA_TILE + first[q] < off + rows;
+                if (32 * q + 31 < RA_COLS * CH || lane + 32 * q < RA_COLS * CH)
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(b + 512 * q),
+                                 "l"(in ? Q + HCHK(src[q] + t * RA_TILE - Q, k * ld - 7) : Q), "r"(in ? 16 : 0)
+                                 : "memory");
             }
         }
         asm volatile("cp.async.commit_group;\n" ::: "memory");
@@ -1132,15 +1145,16 @@ __global__ void __launch_bounds__(32 * RA_WARPS)
 #pragma unroll
     for (int c = 0; c < 2 * RA_COLS; ++c) v[c] = 0.f;
     float2 x[RA_TILE / 32], xn[RA_TILE / 32];
-    stage(0);
-    stage(1);
+    stage(0, 0);
+    stage(1, 1);
     load(0, x);
+    int slot = 0, free = 2;
     for (int t = 0; t < tiles; ++t) {
-        stage(t + 2);                                      // (its buffer was read in the previous round)
+        stage(t + 2, free);                                // (read in the previous round)
         load(t + 1, xn);
         asm volatile("cp.async.wait_group %0;\n" ::"n"(RA_STAGES - 1) : "memory");
         __syncwarp();
-        const unsigned short* b = buf + (t % RA_STAGES) * RA_COLS * RA_PITCH + off + lane;
+        const unsigned short* b = buf + slot * RA_COLS * RA_PITCH + off + lane;
 #pragma unroll
         for (int u = 0; u < RA_TILE / 32; ++u) {
 #pragma unroll
@@ -1152,6 +1166,8 @@ __global__ void __launch_bounds__(32 * RA_WARPS)
             x[u] = xn[u];
         }
         __syncwarp();                                      // (before the buffer is filled again)
+        free = slot;
+        slot = slot == RA_STAGES - 1 ? 0 : slot + 1;
     }
     const float t = scatter_sum<2 * RA_COLS>(v, lane);
     const int idx = lane / (16 / RA_COLS);
